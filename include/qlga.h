@@ -259,11 +259,11 @@ qlga_status qlga_set_graph_steps(qlga_handle* h, int32_t steps);
 
 /* Which kernel runs a step on a 2D lattice.  Sec. VII.B's step is the same either way; the two
  * forms differ only in how the passes are grouped, and their results agree to rounding.
- *   QLGA_STEP2D_AUTO      (default) the fused single-pass kernel when nx is a multiple of 32 and,
- *                         in FP64, a cost estimate favours it (on small FP64 lattices each row
- *                         chunk's warm-up rows outweigh the saved pass);
- *   QLGA_STEP2D_FUSED     always the fused kernel (warp strips of 32 columns: nx % 32 == 0);
- *   QLGA_STEP2D_TWO_PASS  always two passes: x, then y with the potential.
+ *   QLGA_STEP2D_AUTO      (default) FP32: the fused single-pass kernel when nx is a multiple of 32;
+ *                         FP64: two passes, K (both axes, in integer fixed point from nx = 32 on) and U;
+ *   QLGA_STEP2D_FUSED     FP32: always the fused kernel (warp strips of 32 columns: nx % 32 == 0);
+ *                         FP64: the same passes as the default;
+ *   QLGA_STEP2D_TWO_PASS  FP32: always two passes, x, then y with the potential; FP64: the default.
  * Errors: QLGA_ERR_INVALID_ARG for an unknown mode, QLGA_ERR_UNSUPPORTED for QLGA_STEP2D_FUSED
  * on a 1D lattice or nx not a multiple of 32.  Changing the mode waits for the handle's stream
  * and drops captured step graphs.  qlga_get_step2d_kernel() reports the form the next step uses

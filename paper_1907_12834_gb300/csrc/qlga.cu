@@ -130,7 +130,9 @@ __device__ __forceinline__ void put_pq(float* X, int64_t pair, cpx<float> a, cpx
 // HELD_PQ: store the result as (P, Q) = (a + bt, a - bt), the form in which 1D lattices and the
 // fused 2D steps hold a state pending K (qlga_step2d.cuh); else in the resident layout (a, bt).
 template <class T, bool SPLIT, bool HELD_PQ = false>
-__global__ void __launch_bounds__(kThreads) k_potential(T* X, int64_t nsites, PotConst<T> PC,
+// FP64: 128 registers, so that 16 warps per SM cover the latency of the integer sums (0.41 ms at 1024^2
+// against 0.48 at 250 registers and 8 warps).
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 1) k_potential(T* X, int64_t nsites, PotConst<T> PC,
                                                         unsigned* status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t base = int64_t(blockIdx.x) * blockDim.x; base < nsites; base += stride) {
@@ -143,9 +145,17 @@ __global__ void __launch_bounds__(kThreads) k_potential(T* X, int64_t nsites, Po
 #pragma unroll
             for (int m = 0; m < 5; ++m) a[m] = b[m] = {T(0), T(0)};
         }
-        potential_site<T, SPLIT, kZframe64<T>>(a, b, PC, T(1), T(0.5), status);
+        if constexpr (std::is_same<T, double>::value) potential_f64<HELD_PQ>(a, b, PC, 1.0, 0.5, status);
+        else potential_site<T, SPLIT>(a, b, PC, T(1), T(0.5), status);
         if (active) {
-            if constexpr (HELD_PQ) {
+            if constexpr (HELD_PQ && std::is_same<T, double>::value) {
+#pragma unroll
+                for (int m = 0; m < 5; ++m) {
+                    double2* p = reinterpret_cast<double2*>(X) + 2 * (m * nsites + site);
+                    p[0] = make_double2(a[m].re, a[m].im);
+                    p[1] = make_double2(b[m].re, b[m].im);
+                }
+            } else if constexpr (HELD_PQ) {
 #pragma unroll
                 for (int m = 0; m < 5; ++m) put_pq(X, m * nsites + site, a[m], b[m]);
             } else {
@@ -213,7 +223,7 @@ __global__ void __launch_bounds__(kThreads) k_kinetic_axis(const T* __restrict__
             oa[m] = {sc * acc_a.re, sc * acc_a.im};
             ob[m] = {sc * acc_bt.im, -sc * acc_bt.re};  // b = -i bt
         }
-        if (POT) potential_site<T, std::is_same<T, float>::value, kZframe64<T>>(oa, ob, PC, T(1), T(0.5), status);
+        if (POT) potential_site<T, std::is_same<T, float>::value>(oa, ob, PC, T(1), T(0.5), status);
         if (active) SiteIO<T>::store(out, nsites, site, oa, ob);
     }
 }
@@ -681,12 +691,10 @@ inline int step2d_device(Step2dDevice* out) {
             return 1;
         d.per_sm = ctas > 0 ? ctas * kStep2dWarpsPerCta : 1;
         const int s64 = kStep2d64SmemBytes;
-        if (cudaFuncSetAttribute(k_step2d_f64<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f64<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f64<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f64<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_kinetic2d_f64<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_kinetic2d_f64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
         int ctas64 = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas64, k_step2d_f64<0, true>, kStep2d64WarpsPerCta * 32, s64) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas64, k_kinetic2d_f64<0>, kStep2d64WarpsPerCta * 32, s64) != cudaSuccess)
             return 1;
         d.per_sm64 = ctas64 > 0 ? ctas64 * kStep2d64WarpsPerCta : 1;
         if (cudaFuncSetAttribute(k_obs2d_f32<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
@@ -703,40 +711,17 @@ inline int step2d_device(Step2dDevice* out) {
     return 0;
 }
 
-// FP64: whether the fused kernel beats the two-pass form (x pass, then y pass + U) on an nx x ny
-// lattice (nx a multiple of 32).  The fused kernel costs the row-chunk estimate above; the
-// two-pass form has no warm-up rows but evaluates the y axis as a second nine-point stencil and
-// reads and writes the state twice: 1.135 fused row updates per row of a strip, spread over all
-// sub-partitions (calibrated on 4096^2, 56.0 vs 52.4 ms per step).  Short chunks on small lattices
-// favour the two-pass form (512^2: 0.93 vs 0.99 ms per step; 384 x 107: 0.21 vs 0.35 ms).
-inline bool step2d_f64_fused_preferred(int64_t nx, int64_t ny) {
-    Step2dDevice dv;
-    if (step2d_device(&dv)) return true;  // the launch reports the error
-    const int64_t strips = nx / kStep2dWarpCols;
-    const int64_t c = step2d_chunks(strips, ny, dv.sms, dv.per_sm64, false, 18);
-    const int64_t lanes = 4 * int64_t(dv.sms);
-    const double fused = double((strips * c + lanes - 1) / lanes) * (double((ny + c - 1) / c) + 1.8);
-    const double two_pass = 1.135 * double(strips * ny) / double(lanes);
-    return fused <= two_pass;
-}
-
-// FP64 form (qlga_step2d_f64.cuh); same contract as step2d_f32_launch.
-inline int step2d_f64_launch(const double* in, double* out, int64_t nx, int64_t ny, int variant, bool pot,
-                             PotConst<double> PC, unsigned* status, cudaStream_t stream) {
+// FP64 (qlga_step2d_f64.cuh): K of a state held pending K, as the true state; same contract as
+// step2d_f32_launch.
+inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64_t ny, int variant, cudaStream_t stream) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
-    const int64_t strips = nx / kStep2dWarpCols;
-    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm64, false, 18);
+    const int64_t strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
+    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm64, true, 70);  // a warm-up row costs 0.9 of a row
     const int grid = int((strips * chunks + kStep2d64WarpsPerCta - 1) / kStep2d64WarpsPerCta);
     const dim3 b(kStep2d64WarpsPerCta * 32);
-    const int smem = kStep2d64SmemBytes;
-    if (variant == 0) {
-        if (pot) k_step2d_f64<0, true><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-        else k_step2d_f64<0, false><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-    } else {
-        if (pot) k_step2d_f64<1, true><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-        else k_step2d_f64<1, false><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-    }
+    if (variant == 0) k_kinetic2d_f64<0><<<grid, b, kStep2d64SmemBytes, stream>>>(in, out, int(nx), int(ny), chunks);
+    else k_kinetic2d_f64<1><<<grid, b, kStep2d64SmemBytes, stream>>>(in, out, int(nx), int(ny), chunks);
     return cudaPeekAtLastError() != cudaSuccess;
 }
 
@@ -1037,9 +1022,18 @@ qlga_status launch_pot(qlga_handle* h, void* buf, double delta) {
 
 bool step2d_uses_fused(const qlga_handle* h);
 
-// Whether this handle holds its states pending K in the (P, Q) form: 1D lattices and the fused
-// 2D steps (the two-pass 2D form holds (a, bt)).
-bool held_pq(const qlga_handle* h) { return h->cfg.ndim == 1 || step2d_uses_fused(h); }
+// Whether K of this 2D lattice runs in the warp-strip kernels: the fused FP32 step, and FP64 from 32
+// columns on, where K is one pass and U the other whatever the mode.
+bool step2d_uses_strips(const qlga_handle* h) {
+    if (h->cfg.ndim != 2) return false;
+    if (h->cfg.precision == 64)
+        return h->cfg.nx >= kStep2dWarpCols && h->cfg.nx <= (int64_t(1) << 30) && h->cfg.ny <= (int64_t(1) << 30);
+    return step2d_uses_fused(h);
+}
+
+// Whether this handle holds its states pending K in the (P, Q) form: 1D lattices and the strip
+// kernels (the other 2D form holds (a, bt)).
+bool held_pq(const qlga_handle* h) { return h->cfg.ndim == 1 || step2d_uses_strips(h); }
 
 // U on a true state, leaving it held pending K (X = U psi, true state K X): the first half of a
 // step, in the form the handle's kinetic pass reads.
@@ -1303,7 +1297,7 @@ bool step2d_uses_fused(const qlga_handle* h) {
     if (h->cfg.ndim != 2 || !step2d_f32_supported(h->cfg.nx, h->cfg.ny)) return false;
     if (h->step2d_mode == QLGA_STEP2D_FUSED) return true;
     if (h->step2d_mode == QLGA_STEP2D_TWO_PASS) return false;
-    return h->cfg.precision == 32 || step2d_f64_fused_preferred(h->cfg.nx, h->cfg.ny);
+    return h->cfg.precision == 32;  // FP64 runs K and U as two passes
 }
 
 // Apply the full kinetic operator: in -> out (out may not alias in).  2D uses `mid` for the
@@ -1325,17 +1319,16 @@ qlga_status kinetic_into(qlga_handle* h, const void* in, void* out, void* mid, b
         }
         return tile_1d(h, in, out, pot);
     }
-    if (step2d_uses_fused(h) && (held || !held_pq(h))) {
+    if (step2d_uses_strips(h) && held) {
         const int err = h->cfg.precision == 32
             ? step2d_f32_launch(static_cast<const float*>(in), static_cast<float*>(out), h->cfg.nx, h->cfg.ny,
                                 h->cfg.kinetic_variant, pot, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
                                 h->stream)
-            : step2d_f64_launch(static_cast<const double*>(in), static_cast<double*>(out), h->cfg.nx, h->cfg.ny,
-                                h->cfg.kinetic_variant, pot, PotConst<double>(pot_params(h->cfg, 1.0)), h->status,
-                                h->stream);
+            : kinetic2d_f64_launch(static_cast<const double*>(in), static_cast<double*>(out), h->cfg.nx, h->cfg.ny,
+                                   h->cfg.kinetic_variant, h->stream);
         if (err) return cuda_fail(cudaGetLastError(), "step2d launch");
         h->launches += 1;
-        return QLGA_OK;
+        return pot && h->cfg.precision == 64 ? launch_pot_held(h, out) : QLGA_OK;
     }
     qlga_status s = launch_axis(h, in, mid, 0, false);
     if (s != QLGA_OK) return s;
@@ -2445,7 +2438,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_potential(T* X, const BatchT
             b[m] = {p.v[3], -p.v[2]};
         }
         const PotConst<T> C = consts[tile.run];
-        potential_site<T, sizeof(T) == 4, kZframe64<T>>(a, b, C, T(1), T(0.5), status);
+        potential_site<T, sizeof(T) == 4>(a, b, C, T(1), T(0.5), status);
         __syncwarp();
         if (j < run.L) {
             // every run (1D tiles, 2D warp strips) holds its state pending K as (P, Q)

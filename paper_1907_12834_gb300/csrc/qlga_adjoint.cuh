@@ -72,7 +72,7 @@ struct AdjConst {
     T dg2_5;         // delta g2 / 5
     T delta;
     AdjConst() = default;
-    __host__ __device__ explicit AdjConst(const PotParams& P)
+    __host__ explicit AdjConst(const PotParams& P)
         : pc(P), dg0(T(P.delta * P.g0)), dg1(T(P.delta * P.g1)), dg2_5(T(P.delta * P.g2 / 5.0)),
           delta(T(P.delta)) {}
 };

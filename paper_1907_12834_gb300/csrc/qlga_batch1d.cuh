@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
             batch_kinetic_at<T, VARIANT>(&sm[0][0], TW + 8, p, oa, ob);
             // d takes the degree of psi: one warp-uniform Horner loop (2-3% faster than a per-lane
             // degree for d on the 1D scattering batches and on config 1)
-            potential_site<T, false, kZframe64<T>>(oa, ob, C, T(1.0 / 256.0), T(0.5 / 16.0), status);
+            potential_site<T, false>(oa, ob, C, T(1.0 / 256.0), T(0.5 / 16.0), status);
 #pragma unroll
             for (int m = 0; m < 5; ++m)  // held pending K, as (P, Q)
                 mid[m][p] = Pair4<T>{{oa[m].re - ob[m].im, oa[m].im + ob[m].re, oa[m].re + ob[m].im, oa[m].im - ob[m].re}};
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
         if (POT) {
             // all lanes take part (the Taylor degree is a warp maximum); lanes past the run's end
             // work on a copy of a valid site and store nothing
-            potential_site<T, false, kZframe64<T>>(oa, ob, C, T(1.0 / 256.0), T(0.5 / 16.0), status);
+            potential_site<T, false>(oa, ob, C, T(1.0 / 256.0), T(0.5 / 16.0), status);
         } else {
 #pragma unroll
             for (int m = 0; m < 5; ++m) {

@@ -20,6 +20,8 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "qlga_fixed.cuh"
+
 namespace qlga {
 
 // ------------------------------------------------------------------ complex helpers
@@ -247,15 +249,15 @@ struct PotParams {
 
 // Constants of the potential in the arithmetic type, computed on the host from PotParams.
 template <class T>
-struct PotConst {
+struct PotConstBase {
     T cphase;  // delta (g0 + g2/10): e^{-i delta c} with c = (g0 + g2/10) rho
     T dz;      // delta g1: diagonal spin entry per unit F_z m
     T dr;      // delta g2 / 10: diagonal shift of the singlet term per unit rho
     T e0, e1;  // delta g1, delta g1 sqrt(3/2): off-diagonal spin entries per unit F_+
     T R;       // delta g2 / 5: singlet rank-one term
     T b1, b2;  // 2 |g1| delta, |g2| delta / 10: beta = b1 |F| + b2 rho
-    PotConst() = default;
-    __host__ __device__ explicit PotConst(const PotParams& P) {
+    PotConstBase() = default;
+    __host__ __device__ explicit PotConstBase(const PotParams& P) {
         cphase = T(P.delta * (P.g0 + P.g2 / 10.0));
         dz = T(P.delta * P.g1);
         dr = T(P.delta * P.g2 / 10.0);
@@ -265,6 +267,18 @@ struct PotConst {
         b1 = T(2.0 * fabs(P.g1) * P.delta);
         b2 = T(0.1 * fabs(P.g2) * P.delta);
     }
+};
+template <class T>
+struct PotConst : PotConstBase<T> {
+    PotConst() = default;
+    __host__ __device__ explicit PotConst(const PotParams& P) : PotConstBase<T>(P) {}
+};
+template <>
+struct PotConst<double> : PotConstBase<double> {
+    FixPot fx;  // the same for the fixed-point form
+    PotConst() = default;
+    __host__ explicit PotConst(const PotParams& P)
+        : PotConstBase<double>(P), fx(cphase, dz, dr, e0, R, b1, b2) {}
 };
 
 // 1/k, k = 0..kTaylorMax+1 (entry 0 unused): Taylor coefficients without divisions.
@@ -533,7 +547,7 @@ __device__ __forceinline__ void zframe_inner_fp32(const cpx<double> xp[5], const
 // zframe_inner_fp32); Kin = 0 in FP32.
 template <class T>
 __device__ __forceinline__ void potential_tail_zframe(cpx<T> a[5], cpx<T> b[5], const cpx<T> psi[5], const cpx<T> d[5],
-                                                      cpx<T> Fp, T rho, T Fz, int K, int Kd, const PotConst<T>& C,
+                                                      cpx<T> Fp, T rho, T Fz, int K, int Kd, const PotConstBase<T>& C,
                                                       T inv_sigma2, T out_scale, int Kin = 0) {
     const T fp2 = norm2(Fp);
     cpx<T> e = {T(1), T(0)};
@@ -645,25 +659,22 @@ __device__ __forceinline__ void potential_tail_zframe(cpx<T> a[5], cpx<T> b[5], 
     }
 }
 
-// FP64 kernels run the Taylor sums in the z frame too: with the FP64 tolerance the degree is
-// higher, and the frame made the fused and two-pass FP64 2D steps 9% faster (the interleaved
-// passes keep the plain form: more spills there).
-template <class T>
-constexpr bool kZframe64 = std::is_same<T, double>::value;
+// log2 of an exact power of two
+__device__ __forceinline__ int log2_exact(double v) { return int((unsigned(__double2hiint(v)) >> 20) & 0x7ffu) - 1023; }
 
-// Apply U to the pair (a, b) of one site in place.  SPLIT_D: pick the degree for d = a - b
-// from its size relative to psi (the FP32 interleaved passes, where delta is 1/8 and d's degree
-// is often lower: 15% faster there, and the FP32 per-site kernels); otherwise d uses the degree
-// of psi (FP64; the fused 2D and the tiled 1D FP32 kernels, where the one warp-uniform loop over
-// both vectors beats the saved Taylor terms: 0.80 vs 0.85 ms per 4096^2 step, 2-3% on 1D).  ZFRAME: run the
-// Taylor sums in the z frame (potential_tail_zframe).  The frame costs a fixed ~60 operations per
-// site and saves ~26 per vector and Taylor term, so it pays where the warp-uniform degree is about
-// 3 or more: the FP32 2D vortex states of the fused warp-strip kernels (2.4% faster at 4096^2)
-// and the FP64 kernels that call this function outside the interleaved passes (kZframe64), but
-// not the lower FP32 degrees of the 1D workloads (5% slower there).
+// Apply U to the pair (a, b) of one site in place, in the arithmetic of T.  SPLIT_D: pick the
+// degree for d = a - b from its size relative to psi (the FP32 interleaved passes, where delta is
+// 1/8 and d's degree is often lower: 15% faster there, and the FP32 per-site kernels); otherwise d
+// uses the degree of psi (FP64; the fused 2D and the tiled 1D FP32 kernels, where the one
+// warp-uniform loop over both vectors beats the saved Taylor terms: 0.80 vs 0.85 ms per 4096^2
+// step, 2-3% on 1D).  ZFRAME: run the Taylor sums in the z frame (potential_tail_zframe).  The
+// frame costs a fixed ~60 operations per site and saves ~26 per vector and Taylor term, so it pays
+// where the warp-uniform degree is about 3 or more: the FP32 2D vortex states of the fused
+// warp-strip kernels (2.4% faster at 4096^2) and FP64, but not the lower FP32 degrees of the 1D
+// workloads (5% slower there).
 template <class T, bool SPLIT_D, bool ZFRAME = false>
-__device__ __forceinline__ void potential_site(cpx<T> a[5], cpx<T> b[5], const PotConst<T>& C,
-                                               T inv_sigma2, T out_scale, unsigned* status) {
+__device__ __forceinline__ void potential_direct(cpx<T> a[5], cpx<T> b[5], const PotConstBase<T>& C,
+                                                 T inv_sigma2, T out_scale, unsigned* status) {
     cpx<T> psi[5], d[5];
     T n[5];
 #pragma unroll
@@ -739,6 +750,60 @@ __device__ __forceinline__ void potential_site(cpx<T> a[5], cpx<T> b[5], const P
         a[i] = cmul(ph, vp[i] + vd[i]);
         b[i] = cmul(ph, vp[i] - vd[i]);
     }
+}
+
+// The FP64 form of U for the warps that the fixed-point form leaves (a lane with beta > 1 or a
+// value that is not finite, so every site that sets the status word): a call, so that the kernels
+// keep the registers and the instruction cache for the other.
+__device__ __noinline__ void potential_direct_f64(cpx<double>* a, cpx<double>* b, const PotConstBase<double>* C,
+                                                  double inv_sigma2, double out_scale, unsigned* status) {
+    potential_direct<double, false, true>(a, b, *C, inv_sigma2, out_scale, status);
+}
+
+// Apply U to the pair (a, b) of one site in place in FP64; all lanes of the warp take part.  It runs
+// in integer fixed point (qlga_fixed.cuh).  PQ: (a, b) become (P, Q) = (a + i b, a - i b).
+template <bool PQ>
+__device__ __forceinline__ void potential_f64(cpx<double> a[5], cpx<double> b[5], const PotConst<double>& C,
+                                              double inv_sigma2, double out_scale, unsigned* status) {
+    double ar[5], ai[5], br[5], bi[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        ar[i] = a[i].re;
+        ai[i] = a[i].im;
+        br[i] = b[i].re;
+        bi[i] = b[i].im;
+    }
+    if (fx_potential<PQ>(ar, ai, br, bi, log2_exact(inv_sigma2) / 2, log2_exact(out_scale), C.fx)) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            a[i] = {ar[i], ai[i]};
+            b[i] = {br[i], bi[i]};
+        }
+        return;
+    }
+    cpx<double> ta[5], tb[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        ta[i] = a[i];
+        tb[i] = b[i];
+    }
+    const PotConstBase<double> base = C;
+    potential_direct_f64(ta, tb, &base, inv_sigma2, out_scale, status);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        a[i] = PQ ? cpx<double>{ta[i].re - tb[i].im, ta[i].im + tb[i].re} : ta[i];
+        b[i] = PQ ? cpx<double>{ta[i].re + tb[i].im, ta[i].im - tb[i].re} : tb[i];
+    }
+}
+
+// Apply U to the pair (a, b) of one site in place.
+template <class T, bool SPLIT_D, bool ZFRAME = false>
+__device__ __forceinline__ void potential_site(cpx<T> a[5], cpx<T> b[5], const PotConst<T>& C, T inv_sigma2,
+                                               T out_scale, unsigned* status) {
+    if constexpr (std::is_same<T, float>::value)
+        potential_direct<float, SPLIT_D, ZFRAME>(a, b, C, inv_sigma2, out_scale, status);
+    else
+        potential_f64<false>(a, b, C, inv_sigma2, out_scale, status);
 }
 
 // ------------------------------------------------------------------ observables

@@ -1,0 +1,671 @@
+// qlga_fixed.cuh -- the FP64 potential unitary in 64-bit integer fixed point.
+//
+// GB300 issues one FP64 instruction per SM sub-partition every 64-76 cycles (measured: DFMA 64, DADD and
+// DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4 and a
+// 64-bit addition every 2.4.  A
+// product of two fixed-point numbers takes three of the former, so U on a site costs a quarter of
+// its FP64 form (1024^2 sites of a vortex lattice: 0.41 ms, against about 1.7), at a finer
+// resolution: relative to the site's largest component the operands carry 2^-58, where FP64 rounds
+// every operation at 2^-53 of its own result.
+//
+// Numbers.  A site's psi = a + b and d = a - b are int64 with one exponent per vector, psi's largest
+// component in [2^57, 2^58).  An operand of a product is split as v = h 2^32 + l, l the low word
+// taken as signed; h h' and h l' + l h' are summed in two 64-bit accumulators and l l' (zero mean,
+// below 2^62) is dropped.  The entries of delta W and the phase are fixed point with 2^61 = 1, so a
+// dropped product is below 2 units of the vector.
+//
+// U = e^{-i delta c} exp(-i delta W) as in potential_site, by the plain Taylor sum: the terms
+// T_k = (-i delta W)^k x are formed in fixed point up to the order k0 - 1 whose successor is bounded
+// by beta^k0 / k0! <= 2^-31 and added as T_k / k!; the terms from k0 on, so small that FP32 carries
+// them to 2^-54 of the site, continue in FP32.  The phase is applied as v + (e^{-i delta c} - 1) v.
+//
+// Domain.  beta <= 0.3 and finite components below 2^60; a warp with a lane outside it (among them
+// every site that the status word reports) takes the FP64 code.  Components below 2^-59 of the
+// site's largest one, and sites below 2^-850, round to zero.
+#pragma once
+
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <cuda_runtime.h>
+
+namespace qlga {
+
+#define QLGA_HD __host__ __device__ __forceinline__
+
+using i64 = long long;
+
+// ------------------------------------------------------------------ numbers
+
+struct Limb {
+    int h, l;  // h 2^32 + l
+};
+
+QLGA_HD Limb fx_split(i64 v) {  // the low limb is the low word as it stands, the high one takes its sign
+    return {int(v >> 32) + int(unsigned(v) >> 31), int(unsigned(v))};
+}
+QLGA_HD Limb fx_neg(Limb a) { return {-a.h, -a.l}; }
+
+// s + a b, 32 x 32 bits: one instruction
+QLGA_HD i64 fx_mad(int a, int b, i64 s) {
+#ifdef __CUDA_ARCH__
+    i64 d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(s));
+    return d;
+#else
+    return s + i64(a) * b;
+#endif
+}
+
+// The running sum of products: hh 2^64 + mid 2^32
+struct FxAcc {
+    i64 hh, mid;
+};
+QLGA_HD void fx_mac(FxAcc& s, Limb a, Limb b) {
+    s.hh = fx_mad(a.h, b.h, s.hh);
+    s.mid = fx_mad(a.l, b.h, fx_mad(a.h, b.l, s.mid));
+}
+// Every sum is rounded to nearest, not down: half a unit a step would add up over a run's thousands.
+template <int N>
+QLGA_HD FxAcc fx_zero() { return {0, i64(1) << (N - 33)}; }
+template <int N>
+QLGA_HD i64 fx_sum(FxAcc s) {  // sum / 2^N, 32 < N < 64, of an accumulator that began as fx_zero<N>
+    return (s.hh << (64 - N)) + (s.mid >> (N - 32));
+}
+// a b / 2^N with l l' too, for factors that need not fill their limbs
+template <int N>
+QLGA_HD i64 fx_mul_full(Limb a, Limb b) {
+    FxAcc s = fx_zero<N>();
+    fx_mac(s, a, b);
+    s.mid += fx_mad(a.l, b.l, 0) >> 32;
+    return fx_sum<N>(s);
+}
+QLGA_HD i64 fx_mul(Limb a, Limb b) {  // a b / 2^61
+    FxAcc s = fx_zero<61>();
+    fx_mac(s, a, b);
+    return fx_sum<61>(s);
+}
+
+// v 2^n for n in [-63, 62], rounded to nearest (|v| < 2^62; the caller knows that it fits)
+QLGA_HD i64 fx_scale(i64 v, int n) {
+    const int nl = n > 0 ? n : 0, nr = n < 0 ? -n : 0;
+    return (((v << nl << 1) >> nr) + 1) >> 1;
+}
+
+template <class T>
+QLGA_HD int fx_clz(T v) {  // v != 0
+#ifdef __CUDA_ARCH__
+    return __clzll(v);
+#else
+    return __builtin_clzll(static_cast<unsigned long long>(v));
+#endif
+}
+
+// ------------------------------------------------------------------ constants
+
+// A coupling c = m 2^(ex - 60), m in [2^59, 2^60) (0: all zero)
+struct FxConst {
+    Limb m;
+    int ex;
+    FxConst() = default;
+    __host__ explicit FxConst(double c) : m{0, 0}, ex(0) {
+        if (c == 0.0) return;
+        int e;
+        const double f = std::frexp(c, &e);  // c = f 2^e, |f| in [1/2, 1)
+        m = fx_split(i64(std::ldexp(f, 60)));
+        ex = e;
+    }
+};
+
+// The potential's constants (those of PotConst, qlga_device.cuh) for the fixed-point form.
+struct FixPot {
+    FxConst cphase, dz, dr, e0, R;
+    float b1, b2, cphase_f, R_f;
+    FixPot() = default;
+    __host__ FixPot(double cphase_, double dz_, double dr_, double e0_, double R_, double b1_, double b2_)
+        : cphase(cphase_), dz(dz_), dr(dr_), e0(e0_), R(R_), b1(float(b1_)), b2(float(b2_)), cphase_f(float(cphase_)),
+          R_f(float(R_)) {}
+};
+
+struct FxCpxF {
+    float re, im;
+};
+
+// num / den in 2^61 = 1
+QLGA_HD constexpr i64 fx_ratio(i64 num, i64 den) { return ((num << 61) + den / 2) / den; }
+constexpr i64 kFxR32m1 = 518226390554926330LL;  // sqrt(3/2) - 1 in 2^61 = 1
+
+// 1/k! in 2^61 = 1, k = 0..kFxTerms
+constexpr int kFxTerms = 16;
+struct FxInvFact {
+    int h[kFxTerms + 1], l[kFxTerms + 1];
+};
+constexpr FxInvFact make_fx_inv_fact() {
+    FxInvFact t{};
+    i64 f = 1;
+    for (int k = 0; k <= kFxTerms; ++k) {
+        if (k) f *= k;
+        const i64 v = fx_ratio(1, f), h = (v + (i64(1) << 31)) >> 32;
+        t.h[k] = int(h);
+        t.l[k] = int(v - h * (i64(1) << 32));
+    }
+    return t;
+}
+static constexpr FxInvFact kFxInvFactHost = make_fx_inv_fact();
+__constant__ FxInvFact c_fx_inv_fact = make_fx_inv_fact();
+QLGA_HD Limb fx_inv_fact(int k) {
+#ifdef __CUDA_ARCH__
+    return {c_fx_inv_fact.h[k], c_fx_inv_fact.l[k]};
+#else
+    return {kFxInvFactHost.h[k], kFxInvFactHost.l[k]};
+#endif
+}
+
+// ------------------------------------------------------------------ double <-> fixed point
+
+QLGA_HD unsigned fx_hi(double x) {
+#ifdef __CUDA_ARCH__
+    return unsigned(__double2hiint(x));
+#else
+    unsigned long long u;
+    std::memcpy(&u, &x, 8);
+    return unsigned(u >> 32);
+#endif
+}
+QLGA_HD unsigned fx_lo(double x) {
+#ifdef __CUDA_ARCH__
+    return unsigned(__double2loint(x));
+#else
+    unsigned long long u;
+    std::memcpy(&u, &x, 8);
+    return unsigned(u);
+#endif
+}
+QLGA_HD double fx_bits(unsigned hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+    return __hiloint2double(int(hi), int(lo));
+#else
+    const unsigned long long u = (static_cast<unsigned long long>(hi) << 32) | lo;
+    double x;
+    std::memcpy(&x, &u, 8);
+    return x;
+#endif
+}
+QLGA_HD double fx_pow2(int e) { return fx_bits(unsigned(e + 1023) << 20, 0u); }  // 2^e, -1022 <= e <= 1023
+
+// The biased exponent that a set of doubles is converted with: m is the largest high word without
+// sign; every |x| < 2^(E - 1022).  kFxMinExp: smaller sets round to zero.
+constexpr int kFxMinExp = 1022 - 850;
+QLGA_HD int fx_exponent(unsigned m) {
+    const int e = int(m >> 20);
+    return e > kFxMinExp ? e : kFxMinExp;
+}
+
+// x 2^(BITS + 1022 - E), rounded to nearest: the fixed-point value, below 2^BITS, of a double of a set
+// with exponent E
+template <int BITS>
+QLGA_HD i64 fx_from_double(double x, int E) {
+    const unsigned hi = fx_hi(x), lo = fx_lo(x);
+    int dE = E - int((hi >> 20) & 0x7ffu);
+    dE = dE < 63 ? dE : 63;
+    const unsigned long long M = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const i64 v = (i64((M << (BITS - 52)) >> dE) + 1) >> 1;
+    const i64 s = i64(int(hi)) >> 63;
+    return (v ^ s) - s;
+}
+
+// v 2^e (|v| < 2^62, -1022 <= e): one rounding.  scale_hi = 2^(e + 32), scale_lo = 2^e,
+// off = -(2^52 + 2^31) 2^(e + 32) - 2^(e + 52).  Two FP64 instructions: they run beside the integer work.
+struct FxToDouble {
+    double hi, lo, off;
+    QLGA_HD explicit FxToDouble(int e) : hi(fx_pow2(e + 32)), lo(fx_pow2(e)) {
+        // 2^(e + 84) + 2^(e + 63) + 2^(e + 52): 33 bits
+        off = -fx_bits((unsigned(e + 84 + 1023) << 20), 0x80000000u + 0x00100000u) ;
+    }
+    QLGA_HD double operator()(i64 v) const {
+        const double dh = fx_bits(0x43300000u, unsigned(int(v >> 32)) ^ 0x80000000u);  // 2^52 + 2^31 + high word
+        const double dl = fx_bits(0x43300000u, unsigned(v));                           // 2^52 + low word
+        return fma(dl, lo, fma(dh, hi, off));
+    }
+};
+
+// ------------------------------------------------------------------ the site
+
+struct FxVec {
+    Limb re[5], im[5];
+};
+
+// Shift that brings the largest of the ten components of (re, im) to [2^57, 2^58): v -> v 2^(-n).
+// Returns n (components below 2^62; all zero: -57).
+QLGA_HD int fx_headroom(const i64 re[5], const i64 im[5]) {
+    unsigned long long m = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) m |= static_cast<unsigned long long>(re[i] ^ (re[i] >> 63)) | static_cast<unsigned long long>(im[i] ^ (im[i] >> 63));
+    return m ? 6 - fx_clz(m) : -57;  // 64 - clz bits now, 58 wanted
+}
+QLGA_HD i64 fx_shift(i64 v, int n) {  // v 2^(-n), n in [-57, 5], rounded to nearest (|v| < 2^(58 + n))
+    return ((v << (5 - n)) + 16) >> 5;
+}
+
+// delta W of a site in fixed point (2^61 = 1) and in FP32
+struct FxW {
+    Limb D[5];
+    Limb e0r, e0i, e1r, e1i, ne0i, ne1i;  // delta g1 F_+ times 1 and sqrt(3/2); n*: negated imaginary part
+    FxVec u;                              // u_j = (-1)^j psi_{4-j}
+    Limb R;                               // delta g2 / 5: G = R dot / 2^55
+    float Df[5], e0rf, e0if, e1rf, e1if, Rf;
+};
+
+// t <- -i delta W t
+QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
+    FxAcc tp = fx_zero<60>(), tn = {0, 0}, ti = fx_zero<60>();
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        fx_mac(tp, W.u.re[j], t.re[j]);
+        fx_mac(tn, W.u.im[j], t.im[j]);
+        fx_mac(ti, W.u.re[j], t.im[j]);
+        fx_mac(ti, W.u.im[j], t.re[j]);
+    }
+    const Limb Gr = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>({tp.hh - tn.hh, tp.mid - tn.mid}))));
+    const Limb Gi = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(ti))));
+    const Limb nGr = fx_neg(Gr);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        // y = (W t)_i; o = -i y: o.re = y.im, o.im = -y.re
+        FxAcc yr = fx_zero<61>(), yi = fx_zero<61>();
+        fx_mac(yr, W.D[i], t.re[i]);
+        fx_mac(yi, W.D[i], t.im[i]);
+        fx_mac(yr, W.u.re[i], Gr);  // conj(u) G
+        fx_mac(yr, W.u.im[i], Gi);
+        fx_mac(yi, W.u.re[i], Gi);
+        fx_mac(yi, W.u.im[i], nGr);
+        if (i > 0) {  // e t_{i-1}
+            const bool s = i == 1 || i == 4;
+            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i, ne = s ? W.ne0i : W.ne1i;
+            fx_mac(yr, er, t.re[i - 1]);
+            fx_mac(yr, ne, t.im[i - 1]);
+            fx_mac(yi, er, t.im[i - 1]);
+            fx_mac(yi, ei, t.re[i - 1]);
+        }
+        if (i < 4) {  // conj(e) t_{i+1}
+            const bool s = i == 0 || i == 3;
+            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i, ne = s ? W.ne0i : W.ne1i;
+            fx_mac(yr, er, t.re[i + 1]);
+            fx_mac(yr, ei, t.im[i + 1]);
+            fx_mac(yi, er, t.im[i + 1]);
+            fx_mac(yi, ne, t.re[i + 1]);
+        }
+        ore[i] = fx_sum<61>(yi);
+        oim[i] = -fx_sum<61>(yr);
+    }
+}
+
+// 1/k, k = 1..kFxDegree, without a division
+constexpr int kFxDegree = 24;
+struct FxInv {
+    float v[kFxDegree + 1];
+};
+constexpr FxInv make_fx_inv() {
+    FxInv t{};
+    for (int k = 1; k <= kFxDegree; ++k) t.v[k] = float(1.0 / k);
+    return t;
+}
+static constexpr FxInv kFxInvHost = make_fx_inv();
+__constant__ FxInv c_fx_inv = make_fx_inv();
+QLGA_HD float fx_inv(int k) {
+#ifdef __CUDA_ARCH__
+    return c_fx_inv.v[k];
+#else
+    return kFxInvHost.v[k];
+#endif
+}
+
+// Smallest K with beta^(K+1)/(K+1)! <= tol (beta <= 1: at most 18 for 2^-53)
+QLGA_HD int fx_degree(float beta, float tol) {
+    int K = 0;
+    float term = beta;
+    while (term > tol && K < kFxDegree - 1) {
+        ++K;
+        term *= beta * fx_inv(K + 1);
+    }
+    return K;
+}
+
+// t <- (-i / k) delta W t in FP32
+QLGA_HD void fx_apply_f(const FxW& W, const FxCpxF u[5], const FxCpxF t[5], FxCpxF o[5], float ik) {
+    float ar = 0.f, ai = 0.f;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        ar = fmaf(u[j].re, t[j].re, fmaf(-u[j].im, t[j].im, ar));
+        ai = fmaf(u[j].re, t[j].im, fmaf(u[j].im, t[j].re, ai));
+    }
+    const float gr = W.Rf * ar, gi = W.Rf * ai;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        float yr = fmaf(W.Df[i], t[i].re, fmaf(u[i].re, gr, u[i].im * gi));
+        float yi = fmaf(W.Df[i], t[i].im, fmaf(u[i].re, gi, -u[i].im * gr));
+        if (i > 0) {
+            const bool s = i == 1 || i == 4;
+            const float er = s ? W.e0rf : W.e1rf, ei = s ? W.e0if : W.e1if;
+            yr = fmaf(er, t[i - 1].re, fmaf(-ei, t[i - 1].im, yr));
+            yi = fmaf(er, t[i - 1].im, fmaf(ei, t[i - 1].re, yi));
+        }
+        if (i < 4) {
+            const bool s = i == 0 || i == 3;
+            const float er = s ? W.e0rf : W.e1rf, ei = s ? W.e0if : W.e1if;
+            yr = fmaf(er, t[i + 1].re, fmaf(ei, t[i + 1].im, yr));
+            yi = fmaf(er, t[i + 1].im, fmaf(-ei, t[i + 1].re, yi));
+        }
+        o[i] = {ik * yi, -ik * yr};
+    }
+}
+
+// The quadratic forms of psi (unit 2^(2 e + 60) for components of unit 2^e)
+struct FxForms {
+    i64 rho, Fz, Fpr, Fpi;  // F_+ = 2 (Fpr + i Fpi)
+};
+
+QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
+    i64 n[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const i64 hh = fx_mad(p.re[i].h, p.re[i].h, fx_mad(p.im[i].h, p.im[i].h, 0));
+        const i64 hl = fx_mad(p.re[i].h, p.re[i].l, fx_mad(p.im[i].h, p.im[i].l, 0));
+        n[i] = fx_sum<60>({hh, 2 * hl + (i64(1) << 27)});
+    }
+    f.rho = (n[0] + n[1]) + (n[2] + n[3]) + n[4];
+    f.Fz = 2 * (n[0] - n[4]) + (n[1] - n[3]);
+    i64 fr[2], fi[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {  // conj(p0) p1 + conj(p3) p4, then conj(p1) p2 + conj(p2) p3
+        const int a = q, b = q == 0 ? 3 : 2;
+        FxAcc r = fx_zero<60>(), ip = fx_zero<60>(), in = {0, 0};
+        fx_mac(r, p.re[a], p.re[a + 1]);
+        fx_mac(r, p.im[a], p.im[a + 1]);
+        fx_mac(r, p.re[b], p.re[b + 1]);
+        fx_mac(r, p.im[b], p.im[b + 1]);
+        fx_mac(ip, p.re[a], p.im[a + 1]);
+        fx_mac(in, p.im[a], p.re[a + 1]);
+        fx_mac(ip, p.re[b], p.im[b + 1]);
+        fx_mac(in, p.im[b], p.re[b + 1]);
+        fr[q] = fx_sum<60>(r);
+        fi[q] = fx_sum<60>({ip.hh - in.hh, ip.mid - in.mid});
+    }
+    const Limb r = fx_split(kFxR32m1);
+    f.Fpr = fr[0] + fr[1] + fx_mul(r, fx_split(fr[1]));
+    f.Fpi = fi[0] + fi[1] + fx_mul(r, fx_split(fi[1]));
+}
+
+// float of a fixed-point value times the float c
+QLGA_HD float fx_float(Limb v, float c) { return fmaf(float(v.h), 4294967296.f * c, float(v.l) * c); }
+QLGA_HD float fx_pow2f(int n) {  // 2^n, clamped to the normal range
+    n = n < -126 ? -126 : (n > 127 ? 127 : n);
+    union {
+        unsigned u;
+        float f;
+    } p;
+    p.u = unsigned(n + 127) << 23;
+    return p.f;
+}
+
+// e^{-i theta} - 1 = (-c, -s), theta and the results in 2^61 = 1, |theta| <= 1/4: the Taylor series of
+// sin and cos, the terms that FP32 carries to 2^-57 evaluated in it.
+QLGA_HD void fx_phase(i64 theta, i64& c, i64& s) {
+    const Limb t = fx_split(theta);
+    const Limb q = fx_split(fx_mul(t, t));
+    const float qf = fx_float(q, 4.3368087e-19f);  // 2^-61
+    const i64 s3 = fx_ratio(1, 5040) - (i64(int(9007199254740992.f * qf * (2.7557319e-6f - qf * 2.5052108e-8f))) << 8);
+    const i64 s2 = fx_ratio(1, 120) - fx_mul(q, fx_split(s3));
+    const i64 s1 = fx_ratio(1, 6) - fx_mul(q, fx_split(s2));
+    s = theta - fx_mul(t, fx_split(fx_mul(q, fx_split(s1))));
+    const i64 c3 = fx_ratio(1, 720) - (i64(int(1125899906842624.f * qf * (2.4801587e-5f - qf * (2.7557319e-7f - qf * 2.0876757e-9f)))) << 11);
+    const i64 c2 = fx_ratio(1, 24) - fx_mul(q, fx_split(c3));
+    const i64 c1 = (i64(1) << 60) - fx_mul(q, fx_split(c2));
+    c = fx_mul(q, fx_split(c1));
+}
+
+// What the warp decides from: beta and theta of a lane (as upper bounds)
+struct FxBounds {
+    float beta, theta;
+};
+QLGA_HD FxBounds fx_bounds(const FxForms& f, int e, const FixPot& C) {
+    // the forms in 2^61 = 1, times 2^(2 e + 121)
+    const float c = 4.3368087e-19f;
+    const float rho = fx_float(fx_split(f.rho), c), fz = fx_float(fx_split(f.Fz), c);
+    const float fr = 2.f * fx_float(fx_split(f.Fpr), c), fi = 2.f * fx_float(fx_split(f.Fpi), c);
+    const float F = sqrtf(fmaf(fz, fz, fmaf(fr, fr, fi * fi)));
+    const float u = 1.00001f * fx_pow2f(2 * e + 121);
+    FxBounds b;
+    b.beta = u * fmaf(C.b1, F, C.b2 * rho);
+    b.theta = u * fabsf(C.cphase_f) * rho;
+    return b;
+}
+
+// c q 2^(2 e + 60) in 2^61 = 1, twice that for more = 1 (below 2^62)
+QLGA_HD i64 fx_coupled(const FxConst& c, i64 q, int e, int more) {
+    FxAcc s = fx_zero<60>();
+    fx_mac(s, c.m, fx_split(q));
+    int n = c.ex + 2 * e + 121 + more;
+    n = n < -63 ? -63 : (n > 30 ? 30 : n);
+    return fx_scale(fx_sum<60>(s), n);
+}
+
+QLGA_HD void fx_build_w(const FxVec& p, const FxForms& f, int e, const FixPot& C, FxW& W) {
+    const i64 gz = fx_coupled(C.dz, f.Fz, e, 0), g2r = fx_coupled(C.dr, f.rho, e, 0);
+    const float s61 = 4.3368087e-19f;  // 2^-61
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        W.D[i] = fx_split((2 - i) * gz - g2r);
+        W.Df[i] = fx_float(W.D[i], s61);
+    }
+    const Limb r = fx_split(kFxR32m1);
+    const i64 er = fx_coupled(C.e0, f.Fpr, e, 1), ei = fx_coupled(C.e0, f.Fpi, e, 1);
+    W.e0r = fx_split(er);
+    W.e0i = fx_split(ei);
+    W.e1r = fx_split(er + fx_mul(r, W.e0r));
+    W.e1i = fx_split(ei + fx_mul(r, W.e0i));
+    W.ne0i = fx_neg(W.e0i);
+    W.ne1i = fx_neg(W.e1i);
+    W.e0rf = fx_float(W.e0r, s61);
+    W.e0if = fx_float(W.e0i, s61);
+    W.e1rf = fx_float(W.e1r, s61);
+    W.e1if = fx_float(W.e1i, s61);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        W.u.re[j] = (j & 1) ? fx_neg(p.re[4 - j]) : p.re[4 - j];
+        W.u.im[j] = (j & 1) ? fx_neg(p.im[4 - j]) : p.im[4 - j];
+    }
+    // R 2^(2 e) = m 2^(ex - 60 + 2 e); G conj(u) / 2^61 = R 2^(2 e) dot 2^60 conj(u) and G = W.R dot / 2^55.
+    // |psi|^2 >= 2^114 and beta <= 0.3 bound W.R by 2^62
+    int n = C.R.ex + 2 * e + 116;
+    n = n < -63 ? -63 : (n > 30 ? 30 : n);
+    W.R = fx_split(fx_scale((i64(C.R.m.h) << 32) + C.R.m.l, n));
+    W.Rf = C.R_f * fx_pow2f(2 * e + 116);  // for u in 2^58 = 1
+}
+
+// x <- exp(-i delta W) x for one vector: orders 1..kA in fixed point, kA + 1..K in FP32
+QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
+    FxVec t;
+    i64 tr[5], ti[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        tr[i] = re[i];
+        ti[i] = im[i];
+    }
+#pragma unroll 1
+    for (int k = 1; k <= kA; ++k) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            t.re[i] = fx_split(tr[i]);
+            t.im[i] = fx_split(ti[i]);
+        }
+        fx_apply(W, t, tr, ti);
+        if (k <= 2) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                re[i] += k == 1 ? tr[i] : (tr[i] + 1) >> 1;
+                im[i] += k == 1 ? ti[i] : (ti[i] + 1) >> 1;
+            }
+        } else {
+            const Limb f = fx_inv_fact(k);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                re[i] += fx_mul(f, fx_split(tr[i]));
+                im[i] += fx_mul(f, fx_split(ti[i]));
+            }
+        }
+    }
+    if (K > kA) {
+        FxCpxF tf[5], sf[5], uf[5], of[5];
+        const float s58 = 3.4694470e-18f;  // 2^-58
+        const float fact = s58 * fx_float(fx_inv_fact(kA), 4.3368087e-19f);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            tf[i] = {fx_float(fx_split(tr[i]), fact), fx_float(fx_split(ti[i]), fact)};
+            uf[i] = {fx_float(W.u.re[i], s58), fx_float(W.u.im[i], s58)};
+            sf[i] = {0.f, 0.f};
+        }
+#pragma unroll 1
+        for (int k = kA + 1; k <= K; ++k) {
+            fx_apply_f(W, uf, tf, of, fx_inv(k));
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                tf[i] = of[i];
+                sf[i] = {sf[i].re + of[i].re, sf[i].im + of[i].im};
+            }
+        }
+        const float one = 288230376151711744.f;  // 2^58
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            re[i] += int(rintf(sf[i].re * one));
+            im[i] += int(rintf(sf[i].im * one));
+        }
+    }
+}
+
+// x <- x + (e^{-i theta} - 1) x
+QLGA_HD void fx_rotate(i64 c, i64 s, i64 re[5], i64 im[5]) {
+    const Limb nc = fx_split(-c), sp = fx_split(s), sn = fx_neg(sp);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const Limb r = fx_split(re[i]), m = fx_split(im[i]);
+        FxAcc a = fx_zero<61>(), b = fx_zero<61>();
+        fx_mac(a, nc, r);
+        fx_mac(a, sp, m);
+        fx_mac(b, nc, m);
+        fx_mac(b, sn, r);
+        re[i] += fx_sum<61>(a);
+        im[i] += fx_sum<61>(b);
+    }
+}
+
+#ifdef __CUDACC__
+// e^{-i theta} - 1 = (-c, -s) for a theta of any size (fields denser than |theta| = 1/4 are rare)
+__device__ __noinline__ void fx_phase_large(double theta, i64* c, i64* s) {
+    double sn, cs;
+    sincos(theta, &sn, &cs);
+    *c = __double2ll_rn((1.0 - cs) * 2305843009213693952.0);
+    *s = __double2ll_rn(sn * 2305843009213693952.0);
+}
+
+// U on one site of a warp.  In: psi and d as integers below 2^62 of unit 2^e, `true` amplitudes
+// 2^in_log2 times that; ok = false: a lane whose input has no such form.  Out: (psi', d') =
+// (U psi, U d) as integers of the unit 2^(returned exponent), below 2^60.  Returns false, with
+// nothing changed, if a lane of the warp lies outside the domain.  All 32 lanes take part: the
+// orders of the Taylor sums are those of the warp's largest beta.
+__device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int in_log2, bool ok,
+                                           const FixPot& C) {
+    const int np = fx_headroom(pr, pi), nd0 = fx_headroom(dr, di);
+    // d goes with psi's unit or, where it is larger, its own, below 2^57 there, so that G of its sums
+    // stays below 2^62; psi's sum takes the same unit (its limbs in W have psi's own)
+    const int nd = nd0 + 1 > np ? nd0 + 1 : np;
+    FxVec p;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        p.re[i] = fx_split(fx_shift(pr[i], np));
+        p.im[i] = fx_split(fx_shift(pi[i], np));
+    }
+    FxForms f;
+    fx_forms(p, f);
+    const int et = e + np + in_log2;  // exponent of the true psi
+    const FxBounds bd = fx_bounds(f, et, C);
+    ok = ok && bd.beta <= 0.3f;
+    if (!__all_sync(0xffffffffu, ok)) return false;
+    const float beta = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(bd.beta)));
+    const int K = fx_degree(beta, 1.1102230e-16f);  // 2^-53
+    const int kA = min(K, fx_degree(beta, 4.6566129e-10f));  // 2^-31
+    FxW W;
+    fx_build_w(p, f, et, C, W);
+    i64 pc, ps;
+    if (__any_sync(0xffffffffu, bd.theta > 0.25f)) {
+        const double rho = double(f.rho);
+        const int n = 2 * et < -900 ? -900 : 2 * et;
+        const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * rho;
+        fx_phase_large(th, &pc, &ps);
+    } else {
+        fx_phase(fx_coupled(C.cphase, f.rho, et, 0), pc, ps);
+    }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        pr[i] = fx_shift(pr[i], nd);
+        pi[i] = fx_shift(pi[i], nd);
+        dr[i] = fx_shift(dr[i], nd);
+        di[i] = fx_shift(di[i], nd);
+    }
+#pragma unroll 1
+    for (int v = 0; v < 2; ++v) {  // one copy of the code for both vectors
+        fx_taylor(W, pr, pi, kA, K);
+        fx_rotate(pc, ps, pr, pi);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            const i64 tr = pr[i], ti = pi[i];
+            pr[i] = dr[i];
+            pi[i] = di[i];
+            dr[i] = tr;
+            di[i] = ti;
+        }
+    }
+    e += nd;
+    return true;
+}
+
+// U on the pair (a, b) of one site of a warp in FP64, by fx_unitary; the arguments are those of
+// potential_site, with in_log2 = -log2 sigma and out_log2 = log2 out_scale.  PQ: (a, b) become
+// (P, Q) = (a + i b, a - i b) of the result, summed before the conversion.  Returns false, with nothing changed, outside the domain.
+template <bool PQ>
+__device__ __forceinline__ bool fx_potential(double ar[5], double ai[5], double br[5], double bi[5], int in_log2,
+                                             int out_log2, const FixPot& C) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        m = max(m, max(fx_hi(ar[i]) & 0x7fffffffu, fx_hi(ai[i]) & 0x7fffffffu));
+        m = max(m, max(fx_hi(br[i]) & 0x7fffffffu, fx_hi(bi[i]) & 0x7fffffffu));
+    }
+    const bool ok = m < (unsigned(1023 + 60) << 20);  // finite, below 2^60
+    const int E = fx_exponent(m);
+    int e = E - 1022 - 60;
+    i64 pr[5], pi[5], dr[5], di[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const i64 a0 = fx_from_double<60>(ar[i], E), a1 = fx_from_double<60>(ai[i], E);
+        const i64 b0 = fx_from_double<60>(br[i], E), b1 = fx_from_double<60>(bi[i], E);
+        pr[i] = a0 + b0;
+        pi[i] = a1 + b1;
+        dr[i] = a0 - b0;
+        di[i] = a1 - b1;
+    }
+    if (!fx_unitary(pr, pi, dr, di, e, in_log2, ok, C)) return false;
+    const FxToDouble to(e + out_log2);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const i64 a0 = pr[i] + dr[i], a1 = pi[i] + di[i], b0 = pr[i] - dr[i], b1 = pi[i] - di[i];
+        ar[i] = to(PQ ? a0 - b1 : a0);
+        ai[i] = to(PQ ? a1 + b0 : a1);
+        br[i] = to(PQ ? a0 + b1 : b0);
+        bi[i] = to(PQ ? a1 - b0 : b1);
+    }
+    return true;
+}
+#endif
+
+}  // namespace qlga

@@ -1,21 +1,28 @@
-// qlga_step2d_f64.cuh -- fused 2D FP64 QLGA step: one pass over the state per step.
+// qlga_step2d_f64.cuh -- the 2D FP64 kinetic operator in integer fixed point.
 //
-// The FP64 form of the warp-strip step of qlga_step2d.cuh: a warp owns 32 columns and a row
-// range, stages rows (plus the 4-column periodic halo) in its own cp.async ring, applies the
-// nine-point x stencil from shared memory, runs the four y blocks as a register pipeline, then
-// the potential unitary, and stores the site.  In FP64 every arithmetic instruction occupies the
-// FP64 pipe (2 FMA per SM per cycle on GB300), so the y pipeline -- 8 collides of 4 additions per
-// level instead of a second nine-point stencil -- and the single pass are what matter, and so
-// does the held form: states pending K are stored as (P, Q) = (a + bt, a - bt) as in FP32, whose
-// x stencil has 24 nonzero integer taps per level against 32 in (a, bt); zero taps are skipped at
-// compile time and +-1 taps are additions.
+// K along x and y in one pass, by the y-marching warp strips of qlga_step2d.cuh: a warp owns 32 columns
+// and a row range, stages rows (with the 4-column periodic halo) in its own cp.async ring, applies
+// the nine-point x stencil from shared memory and runs the four y blocks as a register pipeline.  All
+// of K's coefficients are small integers, so on integers K is exact up to one rounding between the
+// axes, and an addition costs 2 cycles per sub-partition where FP64 takes 76 (qlga_fixed.cuh): at 1024^2 the
+// pass takes 0.25 ms, against 1.36 ms for K in FP64.  The potential is a pass of its own
+// (k_potential): it needs the registers that hold the pipeline here, and FP64 state traffic is far
+// from the bound (the step 0.66 ms; both in one kernel, K in FP64, 1.83 ms with 1 KB of spills a
+// thread; all in FP64, 3.05 ms).
+//
+// Numbers.  A row is converted once, in place in the ring, each lane its column and an equal share of
+// the eight halo columns, to int64 with one exponent per warp: components below 2^58, the largest of
+// the last 8 to 16 rows in [2^57, 2^58) when its row was read.  The stencil's taps sum to at most 30
+// in magnitude, so its sums fit; they are rounded to 2^-8 of their unit, and the y blocks (taps at
+// most 44) then end below 2^61 and hold the true K X.  Where a row is larger than all before it the
+// pipeline is shifted down, where the last 16 rows are smaller it is shifted up.  The resolution is
+// thus 2^-54 of the largest component in a strip of 40 columns and 8 to 16 rows.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "qlga_device.cuh"
-#include "qlga_interleave.cuh"  // ilv_stream / ilv_collide (streaming blocks on cpx<T>)
-#include "qlga_step2d.cuh"      // cp.async helpers, strip geometry
+#include "qlga_step2d.cuh"  // cp.async helpers, strip geometry
 
 namespace qlga {
 
@@ -27,36 +34,75 @@ __device__ __forceinline__ void put_pq(double* X, int64_t pair, cpx<double> a, c
     p[1] = make_double2(a.re + b.im, a.im - b.re);
 }
 
-// acc + c x for a compile-time integer c (0: nothing, +-1: an addition)
+// acc + c x for a compile-time integer c, by shifts and additions
 template <int C>
-__device__ __forceinline__ double tap64(double x, double acc) {
+__device__ __forceinline__ i64 tap_int(i64 x, i64 acc) {
     if constexpr (C == 0) return acc;
-    else if constexpr (C == 1) return acc + x;
-    else if constexpr (C == -1) return acc - x;
-    else return fma(double(C), x, acc);
+    else if constexpr (C < 0) {
+        if constexpr (C == -1) return acc - x;
+        else if constexpr (C == -3) return acc - x - (x << 1);
+        else if constexpr (C == -5) return acc - x - (x << 2);
+        else return acc - i64(-C) * x;
+    } else {
+        if constexpr (C == 1) return acc + x;
+        else if constexpr (C == 3) return acc + x + (x << 1);
+        else if constexpr (C == 5) return acc + x + (x << 2);
+        else return acc + i64(C) * x;
+    }
 }
+
+struct cpi {
+    i64 re, im;
+};
 
 // One tap of the x stencil on a staged (P, Q) pair (re and im of each).
 template <int VARIANT, int K>
-__device__ __forceinline__ void stencil_tap64(const double2 P, const double2 Q, cpx<double>& xa, cpx<double>& xbt) {
+__device__ __forceinline__ void stencil_tap_int(const longlong2 P, const longlong2 Q, cpi& xa, cpi& xbt) {
     constexpr KinStencil S = kStencilPQ[VARIANT];
-    xa.re = tap64<S.g[0][1][K]>(Q.x, tap64<S.g[0][0][K]>(P.x, xa.re));
-    xa.im = tap64<S.g[0][1][K]>(Q.y, tap64<S.g[0][0][K]>(P.y, xa.im));
-    xbt.re = tap64<S.g[1][1][K]>(Q.x, tap64<S.g[1][0][K]>(P.x, xbt.re));
-    xbt.im = tap64<S.g[1][1][K]>(Q.y, tap64<S.g[1][0][K]>(P.y, xbt.im));
+    xa.re = tap_int<S.g[0][1][K]>(Q.x, tap_int<S.g[0][0][K]>(P.x, xa.re));
+    xa.im = tap_int<S.g[0][1][K]>(Q.y, tap_int<S.g[0][0][K]>(P.y, xa.im));
+    xbt.re = tap_int<S.g[1][1][K]>(Q.x, tap_int<S.g[1][0][K]>(P.x, xbt.re));
+    xbt.im = tap_int<S.g[1][1][K]>(Q.y, tap_int<S.g[1][0][K]>(P.y, xbt.im));
+}
+
+// One streaming block along y for one component of one level (stream_block, qlga_step2d.cuh).
+template <int C, int FIRST>
+__device__ __forceinline__ void stream_int(i64& a, i64& bt, i64& yo, i64& wc) {
+    const i64 ia = a, ibt = bt;
+    if (C == 1) {
+        const i64 ybt = FIRST == 0 ? ibt - ia : ia + ibt;
+        const i64 wa = yo + ybt, wbt = ybt - yo;
+        yo = FIRST == 0 ? ia + ibt : ia - ibt;
+        a = wa;
+        bt = wc;
+        wc = wbt;
+    } else {
+        const i64 ya = FIRST == 0 ? ia + ibt : ia - ibt;
+        const i64 wa = ya + yo, wbt = yo - ya;
+        yo = FIRST == 0 ? ibt - ia : ia + ibt;
+        a = wc;
+        bt = wbt;
+        wc = wa;
+    }
 }
 
 constexpr int kStep2d64WarpsPerCta = 2;
+constexpr int kStep2d64Stages = 3;
 constexpr int kStep2d64SmemBytes =
-    kStep2d64WarpsPerCta * kStep2dStages * 5 * kStep2dWarpRowSites * 32;  // double pairs
+    kStep2d64WarpsPerCta * kStep2d64Stages * 5 * kStep2dWarpRowSites * 32;  // double pairs
+constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
 
-template <int VARIANT, bool POT>
+// out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt).  nx >= 32
+// of any remainder: the lanes of the last strip that lie past the row's end work on its periodic
+// image and store nothing.  A row holding a value that is not finite gives NaN wherever the strip
+// depends on it.
+template <int VARIANT>
 __global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
-    k_step2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks,
-                 PotConst<double> PC, unsigned* status) {
-    extern __shared__ double2 dring[];  // [warp][kStages][5][kStep2dWarpRowSites][2]
+    k_kinetic2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks) {
+    extern __shared__ double2 dring[];  // [warp][kStep2d64Stages][5][kStep2dWarpRowSites][2]
+    constexpr int kRow = 5 * kStep2dWarpRowSites * 2;  // double2 of a row
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int strips = nx / kStep2dWarpCols;
+    const int strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
     const int gw = blockIdx.x * kStep2d64WarpsPerCta + w;
     if (gw >= strips * chunks) return;  // whole warp: no block-wide barrier follows
     const int strip = gw % strips;
@@ -67,18 +113,20 @@ __global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
     const int64_t nsites = int64_t(nx) * ny;
     const double2* in2 = reinterpret_cast<const double2*>(in);
     double2* out2 = reinterpret_cast<double2*>(out);
-    double2* ring = dring + w * (kStep2dStages * 5 * kStep2dWarpRowSites * 2);
+    double2* ring = dring + w * (kStep2d64Stages * kRow);
 
     const int nrows = (y_end - y_begin) + 8;
-    int xm = x0 - kStep2dHalo + lane;
-    xm = xm < 0 ? xm + nx : xm;
-    int xh = x0 + kStep2dWarpCols - kStep2dHalo + lane;
-    xh = xh >= nx ? xh - nx : xh;
-    xh = xh >= nx ? xh - nx : xh;
+    auto wrap_x = [&](int x) {  // x < nx + 36 < 3 nx
+        x = x < 0 ? x + nx : x;
+        x = x >= nx ? x - nx : x;
+        return x >= nx ? x - nx : x;
+    };
+    const int xm = wrap_x(x0 - kStep2dHalo + lane);
+    const int xh = wrap_x(x0 + kStep2dWarpCols - kStep2dHalo + lane);
     auto issue_row = [&](int r) {
         int y = y_begin - kStep2dHalo + r;
         y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-        double2* dst = ring + (r % kStep2dStages) * (5 * kStep2dWarpRowSites * 2);
+        double2* dst = ring + (r % kStep2d64Stages) * kRow;
         const double2* src = in2 + 2 * int64_t(y) * nx;
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
@@ -99,66 +147,114 @@ __global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
     };
 
 #pragma unroll
-    for (int r = 0; r < kStep2dStages - 1; ++r) {
+    for (int r = 0; r < kStep2d64Stages - 1; ++r) {
         if (r < nrows) issue_row(r);
         cp_async_commit();
     }
 
-    cpx<double> yo[4][5], wc[4][5];
+    cpi yo[4][5], wc[4][5];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int m = 0; m < 5; ++m) yo[k][m] = wc[k][m] = {0.0, 0.0};
+        for (int m = 0; m < 5; ++m) yo[k][m] = wc[k][m] = {0, 0};
+    int E = kFxMinExp;                              // the pipeline's exponent
+    int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
+    int bad_until = -1;                             // rows up to here depend on one that is not finite
 
     for (int r = 0; r < nrows; ++r) {
-        cp_async_wait<kStep2dStages - 2>();
+        cp_async_wait<kStep2d64Stages - 2>();
         __syncwarp();
-        if (r + kStep2dStages - 1 < nrows) issue_row(r + kStep2dStages - 1);
+        if (r + kStep2d64Stages - 1 < nrows) issue_row(r + kStep2d64Stages - 1);
         cp_async_commit();
 
-        const double2* row = ring + (r % kStep2dStages) * (5 * kStep2dWarpRowSites * 2);
-        cpx<double> oa[5], ob[5];
+        double2* row = ring + (r % kStep2d64Stages) * kRow;
+        // convert the row in place: column `lane` of the ring and, of columns 32..39, the lane's
+        // component of each level
+        double halo[5];
+        double2 own[10];
+        unsigned top = 0;
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
-            // x axis: nine-point stencil (x16, unnormalised) from the held (P, Q) pairs to (a, bt)
-            cpx<double> xa = {0.0, 0.0}, xbt = {0.0, 0.0};
             const double2* p = row + 2 * (m * kStep2dWarpRowSites + lane);
-            stencil_tap64<VARIANT, 0>(p[0], p[1], xa, xbt);
-            stencil_tap64<VARIANT, 1>(p[2], p[3], xa, xbt);
-            stencil_tap64<VARIANT, 2>(p[4], p[5], xa, xbt);
-            stencil_tap64<VARIANT, 3>(p[6], p[7], xa, xbt);
-            stencil_tap64<VARIANT, 4>(p[8], p[9], xa, xbt);
-            stencil_tap64<VARIANT, 5>(p[10], p[11], xa, xbt);
-            stencil_tap64<VARIANT, 6>(p[12], p[13], xa, xbt);
-            stencil_tap64<VARIANT, 7>(p[14], p[15], xa, xbt);
-            stencil_tap64<VARIANT, 8>(p[16], p[17], xa, xbt);
-            // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16, unnormalised)
-            ilv_stream<double, VARIANT>(1, xa, xbt, yo[0][m], wc[0][m]);
-            ilv_stream<double, VARIANT>(1, xa, xbt, yo[1][m], wc[1][m]);
-            ilv_stream<double, VARIANT>(0, xa, xbt, yo[2][m], wc[2][m]);
-            ilv_stream<double, VARIANT>(0, xa, xbt, yo[3][m], wc[3][m]);
-            oa[m] = xa;
-            ob[m] = {xbt.im, -xbt.re};  // b = -i bt
+            own[2 * m] = p[0];
+            own[2 * m + 1] = p[1];
+            halo[m] = reinterpret_cast<const double*>(row + 2 * (m * kStep2dWarpRowSites + kStep2dWarpCols))[lane];
+            top = max(top, fx_hi(halo[m]) & 0x7fffffffu);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                top = max(top, max(fx_hi(own[2 * m + q].x) & 0x7fffffffu, fx_hi(own[2 * m + q].y) & 0x7fffffffu));
         }
-        if (r >= 8) {  // pipeline full: this is output row y_begin + r - 8
-            if (POT) {
-                potential_site<double, false, kZframe64<double>>(oa, ob, PC, 1.0 / 65536.0, 0.5 / 256.0, status);
-            } else {
+        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, top));
+        const bool bad = Er > kKin64MaxExp;
+        if (bad) {
+            Er = kFxMinExp;
+            bad_until = r + 8;
+        }
+        if ((r & 7) == 0) {
+            seen_before = seen;
+            seen = kFxMinExp;
+        }
+        seen = max(seen, Er);
+        const int En = max(seen, seen_before);
+        if (En != E) {  // warp-uniform, rare on smooth fields
+            const int n = max(E - En, -63);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
 #pragma unroll
                 for (int m = 0; m < 5; ++m) {
-                    oa[m] = (1.0 / 256.0) * oa[m];
-                    ob[m] = (1.0 / 256.0) * ob[m];
+                    yo[k][m] = {fx_scale(yo[k][m].re, n), fx_scale(yo[k][m].im, n)};
+                    wc[k][m] = {fx_scale(wc[k][m].re, n), fx_scale(wc[k][m].im, n)};
                 }
-            }
-            const int64_t site = int64_t(y_begin + r - 8) * nx + x0 + lane;
+            E = En;
+        }
 #pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                if (POT) {  // held pending K again, as (P, Q)
-                    put_pq(out, int64_t(m) * nsites + site, oa[m], ob[m]);
-                } else {  // the true state, in the resident layout (a, bt = i b)
-                    double2* p = out2 + 2 * (int64_t(m) * nsites + site);
-                    p[0] = make_double2(oa[m].re, oa[m].im);
-                    p[1] = make_double2(-ob[m].im, ob[m].re);
+        for (int m = 0; m < 5; ++m) {
+            longlong2* p = reinterpret_cast<longlong2*>(row + 2 * (m * kStep2dWarpRowSites + lane));
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                p[q] = bad ? make_longlong2(0, 0)
+                           : make_longlong2(fx_from_double<58>(own[2 * m + q].x, E), fx_from_double<58>(own[2 * m + q].y, E));
+            reinterpret_cast<i64*>(row + 2 * (m * kStep2dWarpRowSites + kStep2dWarpCols))[lane] =
+                bad ? 0 : fx_from_double<58>(halo[m], E);
+        }
+        __syncwarp();
+
+        const bool store = r >= 8 && x0 + lane < nx;  // pipeline full: this is output row y_begin + r - 8
+        const int64_t site = int64_t(y_begin + r - 8) * nx + x0 + lane;
+        const FxToDouble to(E - 1022 - 58);
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+            // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-8
+            cpi xa = {128, 128}, xbt = {128, 128};
+            const longlong2* p = reinterpret_cast<const longlong2*>(row + 2 * (m * kStep2dWarpRowSites + lane));
+            stencil_tap_int<VARIANT, 0>(p[0], p[1], xa, xbt);
+            stencil_tap_int<VARIANT, 1>(p[2], p[3], xa, xbt);
+            stencil_tap_int<VARIANT, 2>(p[4], p[5], xa, xbt);
+            stencil_tap_int<VARIANT, 3>(p[6], p[7], xa, xbt);
+            stencil_tap_int<VARIANT, 4>(p[8], p[9], xa, xbt);
+            stencil_tap_int<VARIANT, 5>(p[10], p[11], xa, xbt);
+            stencil_tap_int<VARIANT, 6>(p[12], p[13], xa, xbt);
+            stencil_tap_int<VARIANT, 7>(p[14], p[15], xa, xbt);
+            stencil_tap_int<VARIANT, 8>(p[16], p[17], xa, xbt);
+            xa = {xa.re >> 8, xa.im >> 8};
+            xbt = {xbt.re >> 8, xbt.im >> 8};
+            // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16: the true K X)
+            stream_int<1, VARIANT>(xa.re, xbt.re, yo[0][m].re, wc[0][m].re);
+            stream_int<1, VARIANT>(xa.im, xbt.im, yo[0][m].im, wc[0][m].im);
+            stream_int<1, VARIANT>(xa.re, xbt.re, yo[1][m].re, wc[1][m].re);
+            stream_int<1, VARIANT>(xa.im, xbt.im, yo[1][m].im, wc[1][m].im);
+            stream_int<0, VARIANT>(xa.re, xbt.re, yo[2][m].re, wc[2][m].re);
+            stream_int<0, VARIANT>(xa.im, xbt.im, yo[2][m].im, wc[2][m].im);
+            stream_int<0, VARIANT>(xa.re, xbt.re, yo[3][m].re, wc[3][m].re);
+            stream_int<0, VARIANT>(xa.im, xbt.im, yo[3][m].im, wc[3][m].im);
+            if (store) {
+                double2* p2 = out2 + 2 * (int64_t(m) * nsites + site);
+                if (r <= bad_until) {  // warp-uniform
+                    const double nan = fx_bits(0x7ff80000u, 0u);
+                    p2[0] = p2[1] = make_double2(nan, nan);
+                } else {
+                    p2[0] = make_double2(to(xa.re), to(xa.im));
+                    p2[1] = make_double2(to(xbt.re), to(xbt.im));
                 }
             }
         }
