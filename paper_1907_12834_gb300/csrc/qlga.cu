@@ -132,7 +132,7 @@ __device__ __forceinline__ void put_pq(float* X, int64_t pair, cpx<float> a, cpx
 template <class T, bool SPLIT, bool HELD_PQ = false>
 // FP64: 128 registers, so that 16 warps per SM cover the latency of the integer sums (0.41 ms at 1024^2
 // against 0.48 at 250 registers and 8 warps).
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 1) k_potential(T* X, int64_t nsites, PotConst<T> PC,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 0) k_potential(T* X, int64_t nsites, PotConst<T> PC,
                                                         unsigned* status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t base = int64_t(blockIdx.x) * blockDim.x; base < nsites; base += stride) {
@@ -617,10 +617,14 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const double
 
 namespace qlga {
 
-inline bool step2d_f32_supported(int64_t nx, int64_t ny) {
-    return nx % kStep2dWarpCols == 0 && nx >= kStep2dWarpCols && ny >= 1 && nx <= (int64_t(1) << 30) &&
-           ny <= (int64_t(1) << 30);
+// The warp-strip kernels take every width from one strip on; the mode QLGA_STEP2D_FUSED only multiples of 32.
+inline bool step2d_strips_supported(int64_t nx, int64_t ny) {
+    return nx >= kStep2dWarpCols && ny >= 1 && nx <= (int64_t(1) << 30) && ny <= (int64_t(1) << 30);
 }
+inline bool step2d_f32_supported(int64_t nx, int64_t ny) {
+    return nx % kStep2dWarpCols == 0 && step2d_strips_supported(nx, ny);
+}
+inline int64_t step2d_strips(int64_t nx) { return (nx + kStep2dWarpCols - 1) / kStep2dWarpCols; }
 
 // Relative throughput of an SM sub-partition that holds k warps of a fused strip kernel.  FP32:
 // the FMA pipe needs about three warps to stay busy (fitted to the 2D step timed at 256^2 ..
@@ -679,15 +683,19 @@ inline int step2d_device(Step2dDevice* out) {
         int sms = 0, ctas = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
         const int smem = kStep2dWarpSmemBytes;
-        if (cudaFuncSetAttribute(k_step2d_f32<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f32<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f32<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_step2d_f32<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_batch_step2d_f32<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_batch_step2d_f32<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_batch_step2d_f32<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_batch_step2d_f32<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_step2d_f32<0, true>, kStep2dWarpsPerCta * 32, smem) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_step2d_f32<0, true, true>, kStep2dWarpsPerCta * 32, smem) != cudaSuccess)
             return 1;
         d.per_sm = ctas > 0 ? ctas * kStep2dWarpsPerCta : 1;
         const int s64 = kStep2d64SmemBytes;
@@ -697,12 +705,16 @@ inline int step2d_device(Step2dDevice* out) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas64, k_kinetic2d_f64<0>, kStep2d64WarpsPerCta * 32, s64) != cudaSuccess)
             return 1;
         d.per_sm64 = ctas64 > 0 ? ctas64 * kStep2d64WarpsPerCta : 1;
-        if (cudaFuncSetAttribute(k_obs2d_f32<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_obs2d_f32<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_obs2d_f32<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_obs2d_f32<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_obs2d_f32<1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         int ctas_obs = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_obs, k_obs2d_f32<0, true>, kStep2dWarpsPerCta * 32, smem) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_obs, k_obs2d_f32<0, true, true>, kStep2dWarpsPerCta * 32, smem) != cudaSuccess)
             return 1;
         d.per_sm_obs = ctas_obs > 0 ? ctas_obs * kStep2dWarpsPerCta : 1;
         d.sms = sms;
@@ -716,7 +728,7 @@ inline int step2d_device(Step2dDevice* out) {
 inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64_t ny, int variant, cudaStream_t stream) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
-    const int64_t strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
+    const int64_t strips = step2d_strips(nx);
     const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm64, true, 70);  // a warm-up row costs 0.9 of a row
     const int grid = int((strips * chunks + kStep2d64WarpsPerCta - 1) / kStep2d64WarpsPerCta);
     const dim3 b(kStep2d64WarpsPerCta * 32);
@@ -731,17 +743,18 @@ inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny
                              PotConst<float> PC, unsigned* status, cudaStream_t stream) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
-    const int64_t strips = nx / kStep2dWarpCols;
+    const int64_t strips = step2d_strips(nx);
     const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm, true, 32);
     const int grid = int((strips * chunks + kStep2dWarpsPerCta - 1) / kStep2dWarpsPerCta);
-    const dim3 b(kStep2dWarpsPerCta * 32);
-    const int smem = kStep2dWarpSmemBytes;
-    if (variant == 0) {
-        if (pot) k_step2d_f32<0, true><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-        else k_step2d_f32<0, false><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, kStep2dWarpsPerCta * 32, kStep2dWarpSmemBytes, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
+    };
+    if (nx % kStep2dWarpCols == 0) {
+        if (variant == 0) pot ? launch(k_step2d_f32<0, true, false>) : launch(k_step2d_f32<0, false, false>);
+        else pot ? launch(k_step2d_f32<1, true, false>) : launch(k_step2d_f32<1, false, false>);
     } else {
-        if (pot) k_step2d_f32<1, true><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
-        else k_step2d_f32<1, false><<<grid, b, smem, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
+        if (variant == 0) pot ? launch(k_step2d_f32<0, true, true>) : launch(k_step2d_f32<0, false, true>);
+        else pot ? launch(k_step2d_f32<1, true, true>) : launch(k_step2d_f32<1, false, true>);
     }
     return cudaPeekAtLastError() != cudaSuccess;
 }
@@ -756,12 +769,12 @@ inline int obs2d_edge_blocks(int64_t strips, int64_t ny) {
 }
 
 inline size_t obs2d_edge_bytes(int64_t nx, int64_t ny) {
-    return (size_t(nx / kStep2dWarpCols) * size_t(ny) * 5 * sizeof(float2) + 255) & ~size_t(255);
+    return (size_t(step2d_strips(nx)) * size_t(ny) * 5 * sizeof(float2) + 255) & ~size_t(255);
 }
 
 inline size_t obs2d_scratch_bytes(int64_t nx, int64_t ny, int warps) {
     return 2 * obs2d_edge_bytes(nx, ny) +
-           sizeof(double) * OBS_COUNT * size_t(warps + obs2d_edge_blocks(nx / kStep2dWarpCols, ny));
+           sizeof(double) * OBS_COUNT * size_t(warps + obs2d_edge_blocks(step2d_strips(nx), ny));
 }
 
 // Launches the read-out; on return partials (inside scratch) holds *rows rows of OBS_COUNT sums.
@@ -771,7 +784,7 @@ inline int obs2d_f32_launch(const float* in, const float* ref, int64_t nx, int64
                             double** partials, int* rows) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
-    const int64_t strips = nx / kStep2dWarpCols;
+    const int64_t strips = step2d_strips(nx);
     const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm_obs, true, 32);
     const int warps = int(strips * chunks);
     if (obs2d_scratch_bytes(nx, ny, warps) > scratch_bytes) return 2;
@@ -781,14 +794,16 @@ inline int obs2d_f32_launch(const float* in, const float* ref, int64_t nx, int64
     double* part = reinterpret_cast<double*>(p + 2 * obs2d_edge_bytes(nx, ny));
     const int grid = (warps + kStep2dWarpsPerCta - 1) / kStep2dWarpsPerCta;
     const float hg0 = float(0.5 * g0), hg1 = float(0.5 * g1), tg2 = float(0.1 * g2);
-    const dim3 b(kStep2dWarpsPerCta * 32);
-    const int sm = kStep2dWarpSmemBytes;
-    if (variant == 0) {
-        if (ref) k_obs2d_f32<0, true><<<grid, b, sm, stream>>>(in, ref, int(nx), int(ny), chunks, hg0, hg1, tg2, edge_l, edge_r, part);
-        else k_obs2d_f32<0, false><<<grid, b, sm, stream>>>(in, ref, int(nx), int(ny), chunks, hg0, hg1, tg2, edge_l, edge_r, part);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, kStep2dWarpsPerCta * 32, kStep2dWarpSmemBytes, stream>>>(in, ref, int(nx), int(ny), chunks, hg0,
+                                                                               hg1, tg2, edge_l, edge_r, part);
+    };
+    if (nx % kStep2dWarpCols == 0) {
+        if (variant == 0) ref ? launch(k_obs2d_f32<0, true, false>) : launch(k_obs2d_f32<0, false, false>);
+        else ref ? launch(k_obs2d_f32<1, true, false>) : launch(k_obs2d_f32<1, false, false>);
     } else {
-        if (ref) k_obs2d_f32<1, true><<<grid, b, sm, stream>>>(in, ref, int(nx), int(ny), chunks, hg0, hg1, tg2, edge_l, edge_r, part);
-        else k_obs2d_f32<1, false><<<grid, b, sm, stream>>>(in, ref, int(nx), int(ny), chunks, hg0, hg1, tg2, edge_l, edge_r, part);
+        if (variant == 0) ref ? launch(k_obs2d_f32<0, true, true>) : launch(k_obs2d_f32<0, false, true>);
+        else ref ? launch(k_obs2d_f32<1, true, true>) : launch(k_obs2d_f32<1, false, true>);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return 1;
     const int eb = obs2d_edge_blocks(strips, ny);
@@ -1020,15 +1035,11 @@ qlga_status launch_pot(qlga_handle* h, void* buf, double delta) {
     return h->cfg.precision == 32 ? launch_potential<float>(h, buf, delta) : launch_potential<double>(h, buf, delta);
 }
 
-bool step2d_uses_fused(const qlga_handle* h);
-
-// Whether K of this 2D lattice runs in the warp-strip kernels: the fused FP32 step, and FP64 from 32
-// columns on, where K is one pass and U the other whatever the mode.
+// Whether K of this 2D lattice runs in the warp-strip kernels, from 32 columns on: the FP32 step unless
+// two passes are asked for, and FP64, where K is one pass and U the other, whatever the mode.
 bool step2d_uses_strips(const qlga_handle* h) {
-    if (h->cfg.ndim != 2) return false;
-    if (h->cfg.precision == 64)
-        return h->cfg.nx >= kStep2dWarpCols && h->cfg.nx <= (int64_t(1) << 30) && h->cfg.ny <= (int64_t(1) << 30);
-    return step2d_uses_fused(h);
+    if (h->cfg.ndim != 2 || !step2d_strips_supported(h->cfg.nx, h->cfg.ny)) return false;
+    return h->cfg.precision == 64 || h->step2d_mode != QLGA_STEP2D_TWO_PASS;
 }
 
 // Whether this handle holds its states pending K in the (P, Q) form: 1D lattices and the strip
@@ -1792,7 +1803,7 @@ static void fill_obs(const double* o, int64_t step, qlga_obs* out) {
 // Partial rows of the observable sums of the handle's true state (with the optional reference
 // state for the overlap): *partials, *rows.
 qlga_status observables_partials(qlga_handle* h, const void* ref_state_device, double** partials, int* rows) {
-    if (h->pending_k && h->cfg.precision == 32 && step2d_uses_fused(h)) {
+    if (h->pending_k && h->cfg.precision == 32 && step2d_uses_strips(h)) {
         // one read of the state: K on the fly in the warp strips, the sums in the same pass; the
         // work buffer is free between steps and holds the edge fields and partial rows
         const int err = obs2d_f32_launch(static_cast<const float*>(h->X[h->cur]),

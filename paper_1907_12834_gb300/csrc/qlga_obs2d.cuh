@@ -37,14 +37,16 @@ __device__ __forceinline__ int64_t obs2d_edge_index(int strip, int y, int ny, in
 // the unnormalised K X (256 times the true field, so the field psi = a + b is 256 psi_true) and
 // each sum is scaled once at the end by the power of 1/256 of its degree (exact in binary); the
 // qubit norm is the sum of the populations.
-template <int VARIANT, bool REF, int STYLE = QLGA_STEP2D_STYLE>
+// RAGGED: for nx of any remainder; the last strip has fewer than 32 columns, and its lanes past the
+// row's end add nothing.
+template <int VARIANT, bool REF, bool RAGGED, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     k_obs2d_f32(const float* __restrict__ in, const float* __restrict__ ref, int nx, int ny, int chunks,
                 float hg0, float hg1, float tg2, float2* __restrict__ edge_l, float2* __restrict__ edge_r,
                 double* __restrict__ partials) {
     extern __shared__ float4 wring[];  // [warp][kStages][5][kStep2dWarpRowSites]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int strips = nx / kStep2dWarpCols;
+    const int strips = RAGGED ? (nx + kStep2dWarpCols - 1) / kStep2dWarpCols : nx / kStep2dWarpCols;
     const int gw = blockIdx.x * kStep2dWarpsPerCta + w;
     if (gw >= strips * chunks) return;  // whole warp: no block-wide barrier follows
     const int strip = gw % strips;
@@ -52,12 +54,13 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     const int y_begin = int((int64_t(chunk) * ny) / chunks);
     const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
     const int x0 = strip * kStep2dWarpCols;
+    const int cols = RAGGED && nx - x0 < kStep2dWarpCols ? nx - x0 : kStep2dWarpCols;
     const int64_t nsites = int64_t(nx) * ny;
     const float s2 = 1.0f / 65536.0f;  // (1/256)^2: quartic terms to the quadratic scale
 
     ThreadSum<float> acc[OBS_COUNT];  // OBS_NORM_QUBIT unused (sum of the populations)
     cpx<float> prev[5];               // the field of the previous output row at this lane's column
-    strip_kinetic_rows<VARIANT, STYLE>(
+    strip_kinetic_rows<VARIANT, STYLE, RAGGED>(
         in, nx, ny, x0, y_begin - 1, y_end, wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane,
         [&](int y, cpx<float>(&oa)[5], cpx<float>(&ob)[5]) {
             cpx<float> psi[5];
@@ -65,6 +68,10 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
             for (int m = 0; m < 5; ++m) psi[m] = oa[m] + ob[m];
             if (y >= y_begin) {  // warp-uniform; row y_begin - 1 only seeds prev
                 float rho = 0.f, grad = 0.f;
+                if (RAGGED && lane >= cols) {
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) psi[m] = oa[m] = ob[m] = {0.f, 0.f};
+                }
 #pragma unroll
                 for (int m = 0; m < 5; ++m) {
                     acc[OBS_POP0 + m].add(norm2(oa[m]) + norm2(ob[m]));
@@ -72,9 +79,9 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
                     // +x pair inside the strip: (x, x + 1) from the next lane
                     const cpx<float> nb = {__shfl_down_sync(0xffffffffu, psi[m].re, 1),
                                            __shfl_down_sync(0xffffffffu, psi[m].im, 1)};
-                    if (lane < kStep2dWarpCols - 1) grad += norm2(nb - psi[m]);
+                    if (lane < cols - 1) grad += norm2(nb - psi[m]);
                     // +y pair (y - 1, y)
-                    grad += norm2(psi[m] - prev[m]);
+                    if (!RAGGED || lane < cols) grad += norm2(psi[m] - prev[m]);
                 }
                 acc[OBS_NORM_BOSON].add(rho);
                 float F2;
@@ -86,7 +93,7 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
                 acc[OBS_SINGLET_IM].add(th.im);
                 acc[OBS_THETA2].add(th2);
                 acc[OBS_RHO2].add(rho * rho);
-                if (REF) {
+                if (REF && lane < cols) {
                     const int64_t site = int64_t(y) * nx + x0 + lane;
                     cpx<float> ov = {0.f, 0.f};
 #pragma unroll
@@ -98,11 +105,16 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
                     acc[OBS_OVERLAP_RE].add(ov.re);
                     acc[OBS_OVERLAP_IM].add(ov.im);
                 }
-                if (lane == 0 || lane == kStep2dWarpCols - 1) {
-                    float2* e = lane == 0 ? edge_l : edge_r;
+                auto edge = [&](float2* e) {
 #pragma unroll
                     for (int m = 0; m < 5; ++m)
                         e[obs2d_edge_index(strip, y, ny, m)] = make_float2(psi[m].re, psi[m].im);
+                };
+                if (RAGGED) {  // a strip of one column has both edges in lane 0
+                    if (lane == 0) edge(edge_l);
+                    if (lane == cols - 1) edge(edge_r);
+                } else if (lane == 0 || lane == kStep2dWarpCols - 1) {
+                    edge(lane == 0 ? edge_l : edge_r);
                 }
             }
 #pragma unroll
@@ -132,7 +144,7 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     }
 }
 
-// The x pairs across strip edges: (column 32 s + 31, column 32 (s + 1)), the last strip's pair
+// The x pairs across strip edges: (the last column of strip s, column 32 (s + 1)), the last strip's pair
 // wrapping to column 0.  Each block writes one partial row (energy only).
 __global__ void __launch_bounds__(kObs2dEdgeThreads)
     k_obs2d_edges(const float2* __restrict__ edge_l, const float2* __restrict__ edge_r, int strips, int ny,

@@ -177,7 +177,9 @@ constexpr int kStep2dWarpSmemBytes =
 // periodically); `ring` is the warp's shared-memory ring.  For each output row y it calls
 // row_out(y, a, b) with the lane's site of K X as (a, b) pairs, unnormalised: 256 times the true
 // value (the eight collides of the two axes drop their factor 1/2 each).
-template <int VARIANT, int STYLE, class RowOut>
+// RAGGED: nx is no multiple of 32; the lanes of the last strip that lie past the row's end work on its
+// periodic image.
+template <int VARIANT, int STYLE, bool RAGGED, class RowOut>
 __device__ __forceinline__ void strip_kinetic_rows(const float* __restrict__ in, int nx, int ny, int x0,
                                                    int y_begin, int y_end, float4* ring, int lane,
                                                    RowOut&& row_out) {
@@ -189,6 +191,7 @@ __device__ __forceinline__ void strip_kinetic_rows(const float* __restrict__ in,
     // l < 8, r = 32 + l
     int xm = x0 - kStep2dHalo + lane;
     xm = xm < 0 ? xm + nx : xm;
+    if (RAGGED) xm = xm >= nx ? xm - nx : xm;
     int xh = x0 + kStep2dWarpCols - kStep2dHalo + lane;
     xh = xh >= nx ? xh - nx : xh;
     xh = xh >= nx ? xh - nx : xh;  // nx = 32: the right halo wraps onto the strip itself
@@ -257,18 +260,19 @@ __device__ __forceinline__ void strip_kinetic_rows(const float* __restrict__ in,
 // One warp's share of a step: K on the strip (input held pending K as (P, Q)), then (POT) the
 // potential unitary and the store of rows [y_begin, y_end) as (P, Q) again.  POT = false stores
 // K X alone, the true state, in the resident layout (a, bt).
-template <int VARIANT, bool POT, int STYLE>
+// With RAGGED the lanes past the row's end store nothing.
+template <int VARIANT, bool POT, int STYLE, bool RAGGED = false>
 __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float* __restrict__ out, int nx,
                                              int ny, int x0, int y_begin, int y_end, const PotConst<float>& PC,
                                              unsigned* status, float4* ring, int lane) {
     const int64_t nsites = int64_t(nx) * ny;
     float4* out4 = reinterpret_cast<float4*>(out);
-    strip_kinetic_rows<VARIANT, STYLE>(
+    strip_kinetic_rows<VARIANT, STYLE, RAGGED>(
         in, nx, ny, x0, y_begin, y_end, ring, lane, [&](int y, cpx<float>(&oa)[5], cpx<float>(&ob)[5]) {
             if (POT) {
                 // d = a - b takes the degree of psi: one warp-uniform Horner loop over both vectors
                 // runs faster here than a separate, per-lane degree for d (fewer branches)
-                potential_site<float, false, true>(oa, ob, PC, 1.0f / 65536.0f, 0.5f / 256.0f, status);
+                potential_site<float, false, !RAGGED>(oa, ob, PC, 1.0f / 65536.0f, 0.5f / 256.0f, status);
             } else {
                 const float s = 1.0f / 256.0f;
 #pragma unroll
@@ -278,6 +282,7 @@ __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float
                 }
             }
             const int64_t site = int64_t(y) * nx + x0 + lane;
+            if (RAGGED && x0 + lane >= nx) return;
 #pragma unroll
             for (int m = 0; m < 5; ++m)  // POT: held pending K again, as (P, Q); else the true state
                 out4[int64_t(m) * nsites + site] =
@@ -287,21 +292,25 @@ __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float
 
 // The kernel.  POT = false applies the kinetic operator alone (out = K X), used to read out a
 // state held pending K.  Warp gw of the grid takes strip gw % strips of row chunk gw / strips.
-// The input is always a state held pending K, stored as (P, Q).
-template <int VARIANT, bool POT = true, int STYLE = QLGA_STEP2D_STYLE>
+// The input is always a state held pending K, stored as (P, Q).  RAGGED: for nx of any remainder
+// (1000 x 701, 20 steps with load and read-out: 1.89 ms as two passes, 1.14 ms in the strips); a form of
+// its own, since the masked store costs the others registers.  Its U takes no z frame: rsqrtf and
+// the frame's products leave a site's norm up to 4e-7 off a step, and the two passes that it
+// replaces had none (error after the 20 steps 5.5e-7 before, 5.1e-7 now; with the frame 1.0e-6 in 1.10 ms).
+template <int VARIANT, bool POT, bool RAGGED, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     k_step2d_f32(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int chunks,
                  PotConst<float> PC, unsigned* status) {
     extern __shared__ float4 wring[];  // [warp][kStages][5][kStep2dWarpRowSites]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int strips = nx / kStep2dWarpCols;
+    const int strips = RAGGED ? (nx + kStep2dWarpCols - 1) / kStep2dWarpCols : nx / kStep2dWarpCols;
     const int gw = blockIdx.x * kStep2dWarpsPerCta + w;
     if (gw >= strips * chunks) return;  // whole warp: no block-wide barrier follows
     const int strip = gw % strips;
     const int chunk = gw / strips;
     const int y_begin = int((int64_t(chunk) * ny) / chunks);
     const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
-    step2d_strip<VARIANT, POT, STYLE>(in, out, nx, ny, strip * kStep2dWarpCols, y_begin, y_end, PC, status,
+    step2d_strip<VARIANT, POT, STYLE, RAGGED>(in, out, nx, ny, strip * kStep2dWarpCols, y_begin, y_end, PC, status,
                                       wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane);
 }
 
