@@ -279,11 +279,11 @@ qlga_status qlga_get_step2d_kernel(qlga_handle* h, int32_t* kernel);
  * block index), or the lane-parallel kernel for small lattices whose one-site-per-thread launches
  * leave most of the GPU idle: shape (5, 0, 1), a site's five levels on five lanes, six sites per
  * warp; or (10, 0, 1), the psi and d = a - b recursions of U on separate lanes, three sites per
- * warp.  The first fused step times the candidates on the live state and keeps the fastest per
- * step: a one-step shape, in FP32 plain steps a two-step shape (temporal blocking, see the
- * batches; qlga_step then takes fused steps two per launch), or, in FP64, a lane-parallel kernel
- * (in FP32 it can be forced: its Taylor degree, a maximum over 3 or 6 sites instead of 32,
- * truncates closer to the tolerance).
+ * warp.  In FP32 the first fused step times the candidates on the live state and keeps the fastest per
+ * step: a one-step shape or, in plain steps, a two-step shape (temporal blocking, see the
+ * batches; qlga_step then takes fused steps two per launch).  FP64 steps run in fixed point, the
+ * lanes per site chosen by the length, and report the shape (32, 1, 1); a forced shape takes the FP64
+ * arithmetic of the tiled and lane-parallel kernels.
  * qlga_set_1d_shape forces a shape (the list of qlga_batch_set_shape, (5, 0, 1), (10, 0, 1), or
  * the (0, 0, 0) reset); qlga_get_1d_shape reports the one fused steps use (zeros before tuning).  Setting waits for the
  * handle's stream and drops captured step graphs.  Errors: QLGA_ERR_UNSUPPORTED on a 2D lattice,

@@ -35,6 +35,7 @@
 #include "qlga_adjoint.cuh"
 #include "qlga_interleave.cuh"
 #include "qlga_step2d_f64.cuh"
+#include "qlga_step1d_f64.cuh"
 #include "qlga_obs2d.cuh"
 #include "qlga_objective.cuh"
 
@@ -837,6 +838,7 @@ constexpr int kBatchNumCands = 11;
 constexpr BatchCand kBatchCands[kBatchNumCands] = {
     {0, 32, 1, 1},  {1, 64, 1, 1},  {2, 128, 1, 1}, {3, 256, 1, 1}, {2, 64, 2, 1},  {3, 128, 2, 1},
     {3, 64, 4, 1},  {5, 64, 4, 2},  {5, 128, 2, 2}, {4, 64, 2, 2},  {5, 256, 1, 2}};
+constexpr int kFixed1dCand = 0;       // the shape of the FP64 fixed-point kernel: 32 threads, one site each, one step
 constexpr int kBatchDefaultCand = 1;  // before tuning: 64 threads, one site each
 
 // Candidate index of a shape (threads, sites per thread, steps), -1 if there is none.
@@ -932,6 +934,7 @@ struct qlga_handle {
     int tile_cand;  // 1D: launch shape of the tiled step (index into kBatchCands), -1 untuned
     int tile_cand2;  // 1D: two-step shape when it beats tile_cand per step, else -1
     int tile_lanes;   // 1D: fused steps by the lane-parallel kernel with 5 or 10 lanes per site, 0: not
+    bool tile_fixed;  // 1D FP64: no forced shape, steps by the fixed-point kernel (reported as kFixed1dCand's shape)
     int step2d_mode;  // QLGA_STEP2D_AUTO / _FUSED / _TWO_PASS
     // CUDA graphs of graph_steps fused steps starting (and ending) on buffer 0 or 1
     int graph_steps;
@@ -1154,8 +1157,7 @@ cudaError_t time_per_step(cudaStream_t stream, cudaStream_t cs, bool graphed, in
 // shapes and keeps its best time, so that one disturbed timing does not decide the choice (single
 // rounds picked shapes 7% apart on the same 16384-site lattice from run to run).
 template <class Launch>
-cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch&& launch, int* best1, int* best2,
-                        float* t1_out = nullptr, float* t2_out = nullptr) {
+cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch&& launch, int* best1, int* best2) {
     EventPair ev;
     cudaError_t e = ev.create();
     cudaStream_t cs = nullptr;
@@ -1187,8 +1189,6 @@ cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch
     }
     if (cs) cudaStreamDestroy(cs);
     if (*best2 >= 0 && !(t2 < t1)) *best2 = -1;
-    if (t1_out) *t1_out = t1;
-    if (t2_out) *t2_out = t2;
     return e;
 }
 
@@ -1201,6 +1201,24 @@ inline int tune_launches(bool two_step, bool graphed) {
         n += graphed ? 4 * (kTuneGraphSteps / steps) : 3;
     }
     return kTuneRounds * n;
+}
+
+// One FP64 step of a single 1D lattice, or K alone, in integer fixed point (qlga_step1d_f64.cuh).
+void step1d_f64_launch(const TileArgs& a) {
+    const PotConst<double> pc(a.single_params);
+    const int L = int(a.single_L);
+    auto launch = [&](auto kernel) {
+        kernel<<<(L + 31) / 32, 32, 0, a.stream>>>(static_cast<const double*>(a.in), static_cast<double*>(a.out), L, pc, a.status);
+    };
+    auto launch_lanes = [&](auto kernel, int sites) {
+        kernel<<<(L + sites - 1) / sites, 32, 0, a.stream>>>(static_cast<const double*>(a.in), static_cast<double*>(a.out), L, pc, a.status);
+    };
+    // us a step (two solitons, g = (1, 0.8, -0.6)) with 10 / 5 / 1 lanes per site: 1024 sites 4.7 / 6.0 / 11.4,
+    // 4096 5.6 / 5.7 / 12.2, 6000 6.9 / 6.3 / 12.0, 16384 13.0 / 9.9 / 12.1, 24000 17.6 / 11.8 / 12.1, 32768 22.6 / 14.8 / 13.0
+    if (a.pot && L <= 4096) a.variant == 0 ? launch_lanes(k_step1d_f64_lanes<0, 10>, 3) : launch_lanes(k_step1d_f64_lanes<1, 10>, 3);
+    else if (a.pot && L <= 24000) a.variant == 0 ? launch_lanes(k_step1d_f64_lanes<0, 5>, 6) : launch_lanes(k_step1d_f64_lanes<1, 5>, 6);
+    else if (a.variant == 0) a.pot ? launch(k_step1d_f64<0, true>) : launch(k_step1d_f64<0, false>);
+    else a.pot ? launch(k_step1d_f64<1, true>) : launch(k_step1d_f64<1, false>);
 }
 
 // One fused step of a single 1D lattice by the lane-parallel kernel (qlga_lanes1d.cuh) with lps
@@ -1227,17 +1245,27 @@ inline void lanes_1d_launch(const TileArgs& a, int lps) {
 
 // 1D: one fused step (or the kinetic operator alone) of the whole lattice, in -> out; `steps`
 // fused steps (2: the two-step shape of the tiled kernel, which the handle has only in FP32 and
-// when it is faster).  The first fused step times, on the live state and writing only `out`, the
-// tiled kernel's launch shapes (shared with the batches) and the lane-parallel kernel, and keeps
+// when it is faster).  FP64 runs the fixed-point kernels.  In FP32 the first fused step times, on the live
+// state and writing only `out`, the tiled kernel's launch shapes (shared with the batches) and keeps
 // the fastest per step; read-outs (pot = false) take the fastest one-step shape of the tiled
-// kernel.
+// kernel.  qlga_set_1d_shape forces a shape of the tiled or the lane-parallel kernel in either precision.
 qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int steps = 1) {
     TileArgs a{h->stream, h->cfg.precision, h->cfg.kinetic_variant, pot, in, out, nullptr, 0, nullptr,
                nullptr, h->status, h->cfg.nx, pot_params(h->cfg, 1.0)};
+    // FP64 without a forced shape: the fixed-point kernel at any size
+    if (h->cfg.precision == 64 && (h->tile_cand < 0 || h->tile_fixed)) {
+        if (pot) {
+            h->tile_fixed = true;
+            h->tile_cand = kFixed1dCand;
+        }
+        step1d_f64_launch(a);
+        QLGA_CUDA(cudaGetLastError(), "k_step1d_f64 launch");
+        h->launches += 1;
+        return QLGA_OK;
+    }
     if (pot && h->tile_cand < 0) {
-        const bool two = h->cfg.precision == 32 && !h->cfg.interleave;
+        const bool two = !h->cfg.interleave;
         const bool graphed = h->graph_steps > 0;
-        float t1 = 0.f, t2 = 0.f, tl = 0.f;
         // the candidates step a copy of the state back and forth between the work buffer and this
         // step's output buffer, both free until the step itself runs
         QLGA_CUDA(cudaMemcpyAsync(h->tmp, in, state_bytes_of(h->cfg), cudaMemcpyDeviceToDevice, h->stream),
@@ -1253,36 +1281,9 @@ qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int ste
                                         alternate(b, st, k);
                                         tile_step_launch(b, ci);
                                     },
-                                    &h->tile_cand, &h->tile_cand2, &t1, &t2);
-        int lanes = 0;
-        // the lane-parallel kernel, 5 and 10 lanes per site, in FP64 (in FP32 it is no faster, and
-        // its warp-maximum Taylor degree over 3 or 6 sites instead of 32 lets the FP32 truncation,
-        // which accumulates, grow: config 0 after 2000 steps 1.1e-4 against ~1e-5)
-        if (e == cudaSuccess && h->cfg.precision == 64) {
-            EventPair ev;
-            cudaStream_t cs = nullptr;
-            e = ev.create();
-            if (e == cudaSuccess && graphed) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-            for (int lps = 5; lps <= 10 && e == cudaSuccess; lps += 5) {
-                e = time_per_step(h->stream, cs, graphed, 1, ev,
-                                  [&](cudaStream_t st, int k) {
-                                      TileArgs b = a;
-                                      alternate(b, st, k);
-                                      lanes_1d_launch(b, lps);
-                                  },
-                                  &tl);
-                if (e == cudaSuccess && tl < t1 && (h->tile_cand2 < 0 || tl < t2)) {
-                    lanes = lps;
-                    t1 = tl;
-                    t2 = tl;
-                }
-            }
-            if (cs) cudaStreamDestroy(cs);
-        }
+                                    &h->tile_cand, &h->tile_cand2);
         if (e != cudaSuccess) return cuda_fail(e, "1D step tuning");
-        h->tile_lanes = lanes;
-        if (lanes) h->tile_cand2 = -1;
-        h->launches += tune_launches(two, graphed) + (h->cfg.precision == 64 ? 2 * (graphed ? 4 * kTuneGraphSteps : 3) : 0);
+        h->launches += tune_launches(two, graphed);
     }
     if (pot && steps == 1 && h->tile_lanes) {
         lanes_1d_launch(a, h->tile_lanes);
@@ -1581,6 +1582,7 @@ static qlga_status init_handle(qlga_handle* h, const qlga_config* cfg, void* str
     h->tile_cand = -1;
     h->tile_cand2 = -1;
     h->tile_lanes = 0;
+    h->tile_fixed = false;
     h->step2d_mode = QLGA_STEP2D_AUTO;
     QLGA_CUDA(cudaMemsetAsync(h->X[0], 0, state_bytes_of(*cfg), h->stream), "state clear");
     QLGA_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream), "status clear");
@@ -2062,6 +2064,7 @@ qlga_status qlga_set_1d_shape(qlga_handle* h, int32_t threads, int32_t sites_per
     h->tile_cand = c1;
     h->tile_cand2 = c2;
     h->tile_lanes = lanes;
+    h->tile_fixed = false;
     return QLGA_OK;
 }
 

@@ -1,25 +1,27 @@
 // qlga_fixed.cuh -- the FP64 potential unitary in 64-bit integer fixed point.
 //
 // GB300 issues one FP64 instruction per SM sub-partition every 64-76 cycles (measured: DFMA 64, DADD and
-// DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4 and a
-// 64-bit addition every 2.4.  A
-// product of two fixed-point numbers takes three of the former, so U on a site costs a quarter of
-// its FP64 form (1024^2 sites of a vortex lattice: 0.41 ms, against about 1.7), at a finer
+// DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4, a
+// 64-bit addition every 2.4 and an FP32 multiply-add every cycle.  A product of two fixed-point numbers
+// takes one of the first and two of the last, so U on a site costs a fifth of
+// its FP64 form (1024^2 sites of a vortex lattice: 0.39 ms, against about 1.7), at a finer
 // resolution: relative to the site's largest component the operands carry 2^-58, where FP64 rounds
 // every operation at 2^-53 of its own result.
 //
 // Numbers.  A site's psi = a + b and d = a - b are int64 with one exponent per vector, psi's largest
 // component in [2^57, 2^58).  An operand of a product is split as v = h 2^32 + l, l the low word
-// taken as signed; h h' and h l' + l h' are summed in two 64-bit accumulators and l l' (zero mean,
-// below 2^62) is dropped.  The entries of delta W and the phase are fixed point with 2^61 = 1, so a
-// dropped product is below 2 units of the vector.
+// taken as signed; h h' is summed in a 64-bit accumulator, h l' + l h' in an FP32 one, and l l' (zero mean,
+// below 2^62) is dropped.  The entries of delta W and the phase are fixed point with 2^61 = 1.  FP32 leaves
+// 2^-24 of the cross terms, 2^-52 of an entry of W times the vector: with beta <= 1/4 below 2^-54, and in a field of
+// the lattice scaling (beta 0.005 to 0.06) below 2^-56.  (All three products in integers: 2D step 3% and
+// 1D step 20% slower, the same errors against 64-bit references.)
 //
 // U = e^{-i delta c} exp(-i delta W) as in potential_site, by the plain Taylor sum: the terms
 // T_k = (-i delta W)^k x are formed in fixed point up to the order k0 - 1 whose successor is bounded
 // by beta^k0 / k0! <= 2^-31 and added as T_k / k!; the terms from k0 on, so small that FP32 carries
-// them to 2^-54 of the site, continue in FP32.  The phase is applied as v + (e^{-i delta c} - 1) v.
+// them to 2^-54 of the site, continue in FP32 to a bound of 2^-57.  The phase is applied as v + (e^{-i delta c} - 1) v.
 //
-// Domain.  beta <= 0.3 and finite components below 2^60; a warp with a lane outside it (among them
+// Domain.  beta <= 0.25 and finite components below 2^60; a warp with a lane outside it (among them
 // every site that the status word reports) takes the FP64 code.  Components below 2^-59 of the
 // site's largest one, and sites below 2^-850, round to zero.
 #pragma once
@@ -102,6 +104,39 @@ QLGA_HD int fx_clz(T v) {  // v != 0
 }
 
 // ------------------------------------------------------------------ constants
+
+// An operand of the products with FP32 cross terms: the high limb, and both limbs in FP32
+struct FxOp {
+    int h;
+    float hf, lf;
+};
+QLGA_HD FxOp fx_op(Limb a) { return {a.h, float(a.h), float(a.l)}; }
+QLGA_HD FxOp fx_op(i64 v) { return fx_op(fx_split(v)); }
+QLGA_HD FxOp fx_neg(FxOp a) { return {-a.h, -a.hf, -a.lf}; }
+QLGA_HD float fx_float(FxOp a, float c) { return fmaf(a.hf, 4294967296.f * c, a.lf * c); }
+
+// The running sum of such products: hh 2^64 + x 2^32
+struct FxAccF {
+    i64 hh;
+    float x;
+};
+QLGA_HD void fx_mac(FxAccF& s, FxOp a, FxOp b) {
+    s.hh = fx_mad(a.h, b.h, s.hh);
+    s.x = fmaf(a.lf, b.hf, fmaf(a.hf, b.lf, s.x));
+}
+QLGA_HD int fx_rint(float x) {
+#ifdef __CUDA_ARCH__
+    return __float2int_rn(x);
+#else
+    return int(rintf(x));
+#endif
+}
+// sum / 2^N in steps of 2^Q (|x| < 2^(N - 1 + Q)), rounded to nearest
+template <int N, int Q>
+QLGA_HD i64 fx_sum(FxAccF s) {
+    constexpr float kUnit = 1.f / float(1LL << (N - 32 + Q));
+    return (s.hh << (64 - N)) + (i64(fx_rint(s.x * kUnit)) << Q);
+}
 
 // A coupling c = m 2^(ex - 60), m in [2^59, 2^60) (0: all zero)
 struct FxConst {
@@ -214,6 +249,18 @@ QLGA_HD i64 fx_from_double(double x, int E) {
     return (v ^ s) - s;
 }
 
+// v 2^e, rounded to nearest, on integers: where the FP64 pair of FxToDouble would be on a warp's
+// critical path.  The result is a normal number (e >= -1022) or zero.
+QLGA_HD double fx_pack(i64 v, int e) {
+    unsigned long long m = static_cast<unsigned long long>(v < 0 ? -v : v);
+    if (m == 0) return 0.0;
+    const int lz = fx_clz(m);
+    m <<= lz;
+    const unsigned long long r = (m >> 11) + ((m >> 10) & 1);  // [2^52, 2^53]: its top bit counts one exponent
+    const unsigned long long u = (static_cast<unsigned long long>(e + 63 - lz + 1022) << 52) + r;
+    return fx_bits(unsigned(u >> 32) | (unsigned(v >> 63) & 0x80000000u), unsigned(u));
+}
+
 // v 2^e (|v| < 2^62, -1022 <= e): one rounding.  scale_hi = 2^(e + 32), scale_lo = 2^e,
 // off = -(2^52 + 2^31) 2^(e + 32) - 2^(e + 52).  Two FP64 instructions: they run beside the integer work.
 struct FxToDouble {
@@ -232,7 +279,7 @@ struct FxToDouble {
 // ------------------------------------------------------------------ the site
 
 struct FxVec {
-    Limb re[5], im[5];
+    FxOp re[5], im[5];
 };
 
 // Shift that brings the largest of the ten components of (re, im) to [2^57, 2^58): v -> v 2^(-n).
@@ -247,32 +294,36 @@ QLGA_HD i64 fx_shift(i64 v, int n) {  // v 2^(-n), n in [-57, 5], rounded to nea
     return ((v << (5 - n)) + 16) >> 5;
 }
 
-// delta W of a site in fixed point (2^61 = 1) and in FP32
+// delta W of a site in fixed point (2^61 = 1)
 struct FxW {
-    Limb D[5];
-    Limb e0r, e0i, e1r, e1i, ne0i, ne1i;  // delta g1 F_+ times 1 and sqrt(3/2); n*: negated imaginary part
-    FxVec u;                              // u_j = (-1)^j psi_{4-j}
-    Limb R;                               // delta g2 / 5: G = R dot / 2^55
-    float Df[5], e0rf, e0if, e1rf, e1if, Rf;
+    FxOp D[5];
+    FxOp e0r, e0i, e1r, e1i;  // delta g1 F_+ times 1 and sqrt(3/2)
+    int ne0i, ne1i;           // the high limbs of their negated imaginary parts
+    FxVec u;                  // u_j = (-1)^j psi_{4-j}
+    Limb R;                   // delta g2 / 5: G = R dot / 2^55
+    float Rf;
 };
 
 // t <- -i delta W t
 QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
-    FxAcc tp = fx_zero<60>(), tn = {0, 0}, ti = fx_zero<60>();
+    FxAccF tp = {0, 0.f}, ti = {0, 0.f};
+    i64 tn = 0;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         fx_mac(tp, W.u.re[j], t.re[j]);
-        fx_mac(tn, W.u.im[j], t.im[j]);
+        tn = fx_mad(W.u.im[j].h, t.im[j].h, tn);
+        tp.x = fmaf(-W.u.im[j].lf, t.im[j].hf, fmaf(-W.u.im[j].hf, t.im[j].lf, tp.x));
         fx_mac(ti, W.u.re[j], t.im[j]);
         fx_mac(ti, W.u.im[j], t.re[j]);
     }
-    const Limb Gr = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>({tp.hh - tn.hh, tp.mid - tn.mid}))));
-    const Limb Gi = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(ti))));
-    const Limb nGr = fx_neg(Gr);
+    tp.hh -= tn;
+    const FxOp Gr = fx_op(fx_mul_full<55>(W.R, fx_split(fx_sum<60, 3>(tp))));
+    const FxOp Gi = fx_op(fx_mul_full<55>(W.R, fx_split(fx_sum<60, 3>(ti))));
+    const FxOp nGr = fx_neg(Gr);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         // y = (W t)_i; o = -i y: o.re = y.im, o.im = -y.re
-        FxAcc yr = fx_zero<61>(), yi = fx_zero<61>();
+        FxAccF yr = {0, 0.f}, yi = {0, 0.f};
         fx_mac(yr, W.D[i], t.re[i]);
         fx_mac(yi, W.D[i], t.im[i]);
         fx_mac(yr, W.u.re[i], Gr);  // conj(u) G
@@ -281,7 +332,8 @@ QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
         fx_mac(yi, W.u.im[i], nGr);
         if (i > 0) {  // e t_{i-1}
             const bool s = i == 1 || i == 4;
-            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i, ne = s ? W.ne0i : W.ne1i;
+            const FxOp er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
+            const FxOp ne = {s ? W.ne0i : W.ne1i, -ei.hf, -ei.lf};
             fx_mac(yr, er, t.re[i - 1]);
             fx_mac(yr, ne, t.im[i - 1]);
             fx_mac(yi, er, t.im[i - 1]);
@@ -289,14 +341,15 @@ QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
         }
         if (i < 4) {  // conj(e) t_{i+1}
             const bool s = i == 0 || i == 3;
-            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i, ne = s ? W.ne0i : W.ne1i;
+            const FxOp er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
+            const FxOp ne = {s ? W.ne0i : W.ne1i, -ei.hf, -ei.lf};
             fx_mac(yr, er, t.re[i + 1]);
             fx_mac(yr, ei, t.im[i + 1]);
             fx_mac(yi, er, t.im[i + 1]);
             fx_mac(yi, ne, t.re[i + 1]);
         }
-        ore[i] = fx_sum<61>(yi);
-        oim[i] = -fx_sum<61>(yr);
+        ore[i] = fx_sum<61, 2>(yi);
+        oim[i] = -fx_sum<61, 2>(yr);
     }
 }
 
@@ -320,7 +373,14 @@ QLGA_HD float fx_inv(int k) {
 #endif
 }
 
-// Smallest K with beta^(K+1)/(K+1)! <= tol (beta <= 1: at most 18 for 2^-53)
+constexpr float kFxBetaMax = 0.25f;
+// Truncation of the Taylor sums, relative to the site: the same terms are missing from step to step, so
+// the bound is a sixteenth of FP64's 2^-53 (a term of the FP32 part costs 2% of U).  Orders whose bound is
+// above kFxTolF run in fixed point.
+constexpr float kFxTol = 6.9388939e-18f;   // 2^-57
+constexpr float kFxTolF = 4.6566129e-10f;  // 2^-31
+
+// Smallest K with beta^(K+1)/(K+1)! <= tol (beta <= 1: at most 19 for 2^-57)
 QLGA_HD int fx_degree(float beta, float tol) {
     int K = 0;
     float term = beta;
@@ -340,19 +400,23 @@ QLGA_HD void fx_apply_f(const FxW& W, const FxCpxF u[5], const FxCpxF t[5], FxCp
         ai = fmaf(u[j].re, t[j].im, fmaf(u[j].im, t[j].re, ai));
     }
     const float gr = W.Rf * ar, gi = W.Rf * ai;
+    const float s61 = 4.3368087e-19f;  // 2^-61
+    const float e0rf = fx_float(W.e0r, s61), e0if = fx_float(W.e0i, s61);
+    const float e1rf = fx_float(W.e1r, s61), e1if = fx_float(W.e1i, s61);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        float yr = fmaf(W.Df[i], t[i].re, fmaf(u[i].re, gr, u[i].im * gi));
-        float yi = fmaf(W.Df[i], t[i].im, fmaf(u[i].re, gi, -u[i].im * gr));
+        const float Df = fx_float(W.D[i], s61);
+        float yr = fmaf(Df, t[i].re, fmaf(u[i].re, gr, u[i].im * gi));
+        float yi = fmaf(Df, t[i].im, fmaf(u[i].re, gi, -u[i].im * gr));
         if (i > 0) {
             const bool s = i == 1 || i == 4;
-            const float er = s ? W.e0rf : W.e1rf, ei = s ? W.e0if : W.e1if;
+            const float er = s ? e0rf : e1rf, ei = s ? e0if : e1if;
             yr = fmaf(er, t[i - 1].re, fmaf(-ei, t[i - 1].im, yr));
             yi = fmaf(er, t[i - 1].im, fmaf(ei, t[i - 1].re, yi));
         }
         if (i < 4) {
             const bool s = i == 0 || i == 3;
-            const float er = s ? W.e0rf : W.e1rf, ei = s ? W.e0if : W.e1if;
+            const float er = s ? e0rf : e1rf, ei = s ? e0if : e1if;
             yr = fmaf(er, t[i + 1].re, fmaf(ei, t[i + 1].im, yr));
             yi = fmaf(er, t[i + 1].im, fmaf(-ei, t[i + 1].re, yi));
         }
@@ -369,9 +433,9 @@ QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
     i64 n[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const i64 hh = fx_mad(p.re[i].h, p.re[i].h, fx_mad(p.im[i].h, p.im[i].h, 0));
-        const i64 hl = fx_mad(p.re[i].h, p.re[i].l, fx_mad(p.im[i].h, p.im[i].l, 0));
-        n[i] = fx_sum<60>({hh, 2 * hl + (i64(1) << 27)});
+        FxAccF s = {fx_mad(p.re[i].h, p.re[i].h, fx_mad(p.im[i].h, p.im[i].h, 0)),
+                    2.f * fmaf(p.re[i].hf, p.re[i].lf, p.im[i].hf * p.im[i].lf)};
+        n[i] = fx_sum<60, 1>(s);
     }
     f.rho = (n[0] + n[1]) + (n[2] + n[3]) + n[4];
     f.Fz = 2 * (n[0] - n[4]) + (n[1] - n[3]);
@@ -379,7 +443,7 @@ QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {  // conj(p0) p1 + conj(p3) p4, then conj(p1) p2 + conj(p2) p3
         const int a = q, b = q == 0 ? 3 : 2;
-        FxAcc r = fx_zero<60>(), ip = fx_zero<60>(), in = {0, 0};
+        FxAccF r = {0, 0.f}, ip = {0, 0.f}, in = {0, 0.f};
         fx_mac(r, p.re[a], p.re[a + 1]);
         fx_mac(r, p.im[a], p.im[a + 1]);
         fx_mac(r, p.re[b], p.re[b + 1]);
@@ -388,8 +452,8 @@ QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
         fx_mac(in, p.im[a], p.re[a + 1]);
         fx_mac(ip, p.re[b], p.im[b + 1]);
         fx_mac(in, p.im[b], p.re[b + 1]);
-        fr[q] = fx_sum<60>(r);
-        fi[q] = fx_sum<60>({ip.hh - in.hh, ip.mid - in.mid});
+        fr[q] = fx_sum<60, 2>(r);
+        fi[q] = fx_sum<60, 2>(FxAccF{ip.hh - in.hh, ip.x - in.x});
     }
     const Limb r = fx_split(kFxR32m1);
     f.Fpr = fr[0] + fr[1] + fx_mul(r, fx_split(fr[1]));
@@ -450,37 +514,33 @@ QLGA_HD i64 fx_coupled(const FxConst& c, i64 q, int e, int more) {
     return fx_scale(fx_sum<60>(s), n);
 }
 
+QLGA_HD void fx_singlet(const FixPot& C, int e, Limb& R, float& Rf) {
+    // R 2^(2 e) = m 2^(ex - 60 + 2 e); G conj(u) / 2^61 = R 2^(2 e) dot 2^60 conj(u) and G = W.R dot / 2^55.
+    // |psi|^2 >= 2^114 and beta <= 0.25 bound W.R by 2^62
+    int n = C.R.ex + 2 * e + 116;
+    n = n < -63 ? -63 : (n > 30 ? 30 : n);
+    R = fx_split(fx_scale((i64(C.R.m.h) << 32) + C.R.m.l, n));
+    Rf = C.R_f * fx_pow2f(2 * e + 116);  // for u in 2^58 = 1
+}
+
 QLGA_HD void fx_build_w(const FxVec& p, const FxForms& f, int e, const FixPot& C, FxW& W) {
     const i64 gz = fx_coupled(C.dz, f.Fz, e, 0), g2r = fx_coupled(C.dr, f.rho, e, 0);
-    const float s61 = 4.3368087e-19f;  // 2^-61
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        W.D[i] = fx_split((2 - i) * gz - g2r);
-        W.Df[i] = fx_float(W.D[i], s61);
-    }
+    for (int i = 0; i < 5; ++i) W.D[i] = fx_op((2 - i) * gz - g2r);
     const Limb r = fx_split(kFxR32m1);
     const i64 er = fx_coupled(C.e0, f.Fpr, e, 1), ei = fx_coupled(C.e0, f.Fpi, e, 1);
-    W.e0r = fx_split(er);
-    W.e0i = fx_split(ei);
-    W.e1r = fx_split(er + fx_mul(r, W.e0r));
-    W.e1i = fx_split(ei + fx_mul(r, W.e0i));
-    W.ne0i = fx_neg(W.e0i);
-    W.ne1i = fx_neg(W.e1i);
-    W.e0rf = fx_float(W.e0r, s61);
-    W.e0if = fx_float(W.e0i, s61);
-    W.e1rf = fx_float(W.e1r, s61);
-    W.e1if = fx_float(W.e1i, s61);
+    W.e0r = fx_op(er);
+    W.e0i = fx_op(ei);
+    W.e1r = fx_op(er + fx_mul(r, fx_split(er)));
+    W.e1i = fx_op(ei + fx_mul(r, fx_split(ei)));
+    W.ne0i = -W.e0i.h;
+    W.ne1i = -W.e1i.h;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         W.u.re[j] = (j & 1) ? fx_neg(p.re[4 - j]) : p.re[4 - j];
         W.u.im[j] = (j & 1) ? fx_neg(p.im[4 - j]) : p.im[4 - j];
     }
-    // R 2^(2 e) = m 2^(ex - 60 + 2 e); G conj(u) / 2^61 = R 2^(2 e) dot 2^60 conj(u) and G = W.R dot / 2^55.
-    // |psi|^2 >= 2^114 and beta <= 0.3 bound W.R by 2^62
-    int n = C.R.ex + 2 * e + 116;
-    n = n < -63 ? -63 : (n > 30 ? 30 : n);
-    W.R = fx_split(fx_scale((i64(C.R.m.h) << 32) + C.R.m.l, n));
-    W.Rf = C.R_f * fx_pow2f(2 * e + 116);  // for u in 2^58 = 1
+    fx_singlet(C, e, W.R, W.Rf);
 }
 
 // x <- exp(-i delta W) x for one vector: orders 1..kA in fixed point, kA + 1..K in FP32
@@ -492,14 +552,19 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
         tr[i] = re[i];
         ti[i] = im[i];
     }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        t.re[i] = fx_op(tr[i]);
+        t.im[i] = fx_op(ti[i]);
+    }
 #pragma unroll 1
     for (int k = 1; k <= kA; ++k) {
+        fx_apply(W, t, tr, ti);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            t.re[i] = fx_split(tr[i]);
-            t.im[i] = fx_split(ti[i]);
+            t.re[i] = fx_op(tr[i]);
+            t.im[i] = fx_op(ti[i]);
         }
-        fx_apply(W, t, tr, ti);
         if (k <= 2) {
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
@@ -507,11 +572,14 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
                 im[i] += k == 1 ? ti[i] : (ti[i] + 1) >> 1;
             }
         } else {
-            const Limb f = fx_inv_fact(k);
+            const FxOp f = fx_op(fx_inv_fact(k));
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
-                re[i] += fx_mul(f, fx_split(tr[i]));
-                im[i] += fx_mul(f, fx_split(ti[i]));
+                FxAccF a = {0, 0.f}, b = {0, 0.f};
+                fx_mac(a, f, t.re[i]);
+                fx_mac(b, f, t.im[i]);
+                re[i] += fx_sum<61, 0>(a);
+                im[i] += fx_sum<61, 0>(b);
             }
         }
     }
@@ -521,7 +589,7 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
         const float fact = s58 * fx_float(fx_inv_fact(kA), 4.3368087e-19f);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            tf[i] = {fx_float(fx_split(tr[i]), fact), fx_float(fx_split(ti[i]), fact)};
+            tf[i] = {fx_float(t.re[i], fact), fx_float(t.im[i], fact)};
             uf[i] = {fx_float(W.u.re[i], s58), fx_float(W.u.im[i], s58)};
             sf[i] = {0.f, 0.f};
         }
@@ -537,17 +605,34 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
         const float one = 288230376151711744.f;  // 2^58
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            re[i] += int(rintf(sf[i].re * one));
-            im[i] += int(rintf(sf[i].im * one));
+            re[i] += fx_rint(sf[i].re * one);
+            im[i] += fx_rint(sf[i].im * one);
         }
     }
 }
 
-// x <- x + (e^{-i theta} - 1) x
-QLGA_HD void fx_rotate(i64 c, i64 s, i64 re[5], i64 im[5]) {
+// x <- x + (e^{-i theta} - 1) x, for |theta| <= 1/4
+template <int N = 5>
+QLGA_HD void fx_rotate(i64 c, i64 s, i64* re, i64* im) {
+    const FxOp nc = fx_op(-c), sp = fx_op(s), sn = fx_neg(sp);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const FxOp r = fx_op(re[i]), m = fx_op(im[i]);
+        FxAccF a = {0, 0.f}, b = {0, 0.f};
+        fx_mac(a, nc, r);
+        fx_mac(a, sp, m);
+        fx_mac(b, nc, m);
+        fx_mac(b, sn, r);
+        re[i] += fx_sum<61, 2>(a);
+        im[i] += fx_sum<61, 2>(b);
+    }
+}
+// the same for any theta, with integer cross terms
+template <int N = 5>
+QLGA_HD void fx_rotate_large(i64 c, i64 s, i64* re, i64* im) {
     const Limb nc = fx_split(-c), sp = fx_split(s), sn = fx_neg(sp);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < N; ++i) {
         const Limb r = fx_split(re[i]), m = fx_split(im[i]);
         FxAcc a = fx_zero<61>(), b = fx_zero<61>();
         fx_mac(a, nc, r);
@@ -568,6 +653,20 @@ __device__ __noinline__ void fx_phase_large(double theta, i64* c, i64* s) {
     *s = __double2ll_rn(sn * 2305843009213693952.0);
 }
 
+// e^{-i theta} - 1 = (-c, -s) of a site from its density; returns whether a lane of the warp has
+// |theta| > 1/4 (fx_rotate_large)
+__device__ __forceinline__ bool fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
+    const bool large = __any_sync(0xffffffffu, theta > 0.25f);
+    if (large) {
+        const int n = 2 * et < -900 ? -900 : 2 * et;
+        const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * double(rho);
+        fx_phase_large(th, &c, &s);
+    } else {
+        fx_phase(fx_coupled(C.cphase, rho, et, 0), c, s);
+    }
+    return large;
+}
+
 // U on one site of a warp.  In: psi and d as integers below 2^62 of unit 2^e, `true` amplitudes
 // 2^in_log2 times that; ok = false: a lane whose input has no such form.  Out: (psi', d') =
 // (U psi, U d) as integers of the unit 2^(returned exponent), below 2^60.  Returns false, with
@@ -582,29 +681,22 @@ __device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 
     FxVec p;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_split(fx_shift(pr[i], np));
-        p.im[i] = fx_split(fx_shift(pi[i], np));
+        p.re[i] = fx_op(fx_shift(pr[i], np));
+        p.im[i] = fx_op(fx_shift(pi[i], np));
     }
     FxForms f;
     fx_forms(p, f);
     const int et = e + np + in_log2;  // exponent of the true psi
     const FxBounds bd = fx_bounds(f, et, C);
-    ok = ok && bd.beta <= 0.3f;
+    ok = ok && bd.beta <= kFxBetaMax;
     if (!__all_sync(0xffffffffu, ok)) return false;
     const float beta = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(bd.beta)));
-    const int K = fx_degree(beta, 1.1102230e-16f);  // 2^-53
-    const int kA = min(K, fx_degree(beta, 4.6566129e-10f));  // 2^-31
+    const int K = fx_degree(beta, kFxTol);
+    const int kA = min(K, fx_degree(beta, kFxTolF));
     FxW W;
     fx_build_w(p, f, et, C, W);
     i64 pc, ps;
-    if (__any_sync(0xffffffffu, bd.theta > 0.25f)) {
-        const double rho = double(f.rho);
-        const int n = 2 * et < -900 ? -900 : 2 * et;
-        const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * rho;
-        fx_phase_large(th, &pc, &ps);
-    } else {
-        fx_phase(fx_coupled(C.cphase, f.rho, et, 0), pc, ps);
-    }
+    const bool large = fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         pr[i] = fx_shift(pr[i], nd);
@@ -615,7 +707,8 @@ __device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 
 #pragma unroll 1
     for (int v = 0; v < 2; ++v) {  // one copy of the code for both vectors
         fx_taylor(W, pr, pi, kA, K);
-        fx_rotate(pc, ps, pr, pi);
+        if (large) fx_rotate_large(pc, ps, pr, pi);
+        else fx_rotate(pc, ps, pr, pi);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             const i64 tr = pr[i], ti = pi[i];
