@@ -11,22 +11,23 @@
 // Potential step at one site (a' = U a, b' = U b, U = exp(-i delta V(psi)), psi = a + b):
 //   gbar_a = U^dagger gbar_a' + h,   gbar_b = U^dagger gbar_b' + h,
 // with h the gradient through psi.  Writing V = c 1 + W (c = (g0 + g2/10) rho) and B = -i delta W,
-// U = e^{-i delta c} P(B) with P the Taylor polynomial of the forward step.  With
-// M = a gbar_a'^dagger + b gbar_b'^dagger and the Frechet derivative L(B, E) = d/dt P(B + t E):
-//   tau    = Im tr(U M) = Im sum_r gbar_r^dagger U x_r                        (r = a, b)
-//   phi_nu = Im tr(f_nu G),  G = e^{-i delta c} L(B, M),  tr(f_nu G) = e^{-i delta c} sum_r
-//            gbar_r^dagger L(B, f_nu) x_r                                      (nu = x, y, z)
-//   H s    = (G s - G^dagger s) / (2i),  s = J conj(psi),
-//            G s = e^{-i delta c} L(B, M) s,  G^dagger s = e^{i delta c} L(-B, M^dagger) s
-//   h      = delta [2 g0 tau psi + 2 g1 sum_nu phi_nu f_nu psi + (2 g2/5) J conj(H s)]
-// and the coupling gradients dL/dg0 = delta rho tau, dL/dg1 = delta sum_nu F_nu phi_nu,
-// dL/dg2 = (delta/5) Re s^dagger H s.  (The identity direction of dV commutes with B; its
+// U = e^{-i delta c} P(B) with P the degree-K Taylor polynomial of the forward step in Horner form,
+//   v_K = x,  v_{k-1} = x + B v_k / k,  P x = v_0.
+// Its reverse sweep starts from lambda_0 = e^{i delta c} gbar' and runs upwards,
+//   mu_k = lambda_{k-1} / k,  lambda_k = B^dagger mu_k,  P^dagger lambda_0 = sum_k lambda_k,
+// and step k adds Im mu_k^dagger d(delta W) v_k to dL.  Summed over the steps and over x = a, b,
+//   phi_nu = Im sum mu_k^dagger f_nu v_k                                            (nu = x, y, z)
+//   q      = sum conj(u . mu_k) v_k - conj(u . v_k) mu_k,  u_m = (-1)^m psi_{-m} = conj(s_m)
+//   tau    = Im lambda_0^dagger P x
+//   h      = delta [2 g0 tau psi + 2 g1 sum_nu phi_nu f_nu psi + (g2/5) i J conj(q)]
+// and the coupling gradients are dL/dg0 = delta rho tau, dL/dg1 = delta sum_nu F_nu phi_nu,
+// dL/dg2 = (delta/5) Im sum conj(u . mu_k) (u . v_k).  (The identity direction of dV commutes with B; its
 // derivative uses the exact exponential, whose trace form is tau.)
 //
-// Each L(B, E) v is the upper block of P([[B, E], [0, B]]) applied to (0, v): the same Horner
-// recursion as the forward step on a pair of 5-vectors, with the degree the forward step used at
-// that site.  No matrix is formed; everything is matrix-vector work on the tridiagonal-plus-
-// rank-one W.
+// Two applications of W per Taylor term and vector, four in all, where the Frechet derivatives of
+// the same polynomial by augmented Horner recursions, one per spin direction and two for the singlet
+// term, took fourteen (a gradient of 24 steps on 512^2 in FP32 4.03 -> 3.56 ms, of 12 on 256^2 in FP64
+// 17.1 -> 9.4 ms).  The Horner iterates wait for the reverse sweep in thread-local memory.
 #pragma once
 
 #include "qlga_device.cuh"
@@ -84,35 +85,6 @@ __device__ __forceinline__ T spin_c(int i) {
     return (i == 0 || i == 3) ? T(1) : T(1.2247448713915890491);  // 1, sqrt(3/2), sqrt(3/2), 1
 }
 
-template <class T>
-__device__ __forceinline__ void apply_fz(const cpx<T> x[5], cpx<T> y[5]) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) y[i] = T(2 - i) * x[i];
-}
-template <class T>
-__device__ __forceinline__ void apply_fx(const cpx<T> x[5], cpx<T> y[5]) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) y[i] = {T(0), T(0)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const T c = spin_c<T>(i);
-        y[i] = y[i] + c * x[i + 1];
-        y[i + 1] = y[i + 1] + c * x[i];
-    }
-}
-template <class T>
-__device__ __forceinline__ void apply_fy(const cpx<T> x[5], cpx<T> y[5]) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) y[i] = {T(0), T(0)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const T c = spin_c<T>(i);
-        // y_i += -i c x_{i+1};  y_{i+1} += i c x_i
-        y[i] = {y[i].re + c * x[i + 1].im, y[i].im - c * x[i + 1].re};
-        y[i + 1] = {y[i + 1].re - c * x[i].im, y[i + 1].im + c * x[i].re};
-    }
-}
-
 // conj(x) . y
 template <class T>
 __device__ __forceinline__ cpx<T> cdot(const cpx<T> x[5], const cpx<T> y[5]) {
@@ -122,20 +94,11 @@ __device__ __forceinline__ cpx<T> cdot(const cpx<T> x[5], const cpx<T> y[5]) {
     return acc;
 }
 
-// v = x + sgn * (-i) * ik * w   (one Horner step of P(sgn B) with B v = -i W v)
+// v = x - i ik w   (one Horner step of P(B) with B v = -i W v)
 template <class T>
-__device__ __forceinline__ void horner_sgn(const cpx<T> x[5], const cpx<T> w[5], cpx<T> v[5], T ik) {
+__device__ __forceinline__ void horner_down(const cpx<T> x[5], const cpx<T> w[5], cpx<T> v[5], T ik) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) v[i] = {fma(ik, w[i].im, x[i].re), fma(-ik, w[i].re, x[i].im)};
-}
-
-// v = ik * (-i * w + e)  (upper block of the augmented Horner step); sik = sgn * ik
-template <class T>
-__device__ __forceinline__ void horner_upper(const cpx<T> w[5], const cpx<T> e[5], cpx<T> v[5], T sik,
-                                             T ik) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-        v[i] = {fma(sik, w[i].im, ik * e[i].re), fma(-sik, w[i].re, ik * e[i].im)};
 }
 
 // The forward step's W at a site (as potential_site builds it, unscaled input) and its degree.
@@ -179,11 +142,10 @@ __device__ __forceinline__ int build_w(const cpx<T> psi[5], const PotConst<T>& C
     return K;
 }
 
-// FP64 pull-backs run the Horner steps of order above k0 in FP32 (Kin = K - k0 inner steps) and
-// the k0 outer ones in FP64, as the forward step does (zframe_inner_fp32), with k0 the smallest
+// FP64 pull-backs run the steps of order above k0 of both sweeps in FP32 (Kin = K - k0 of them) and
+// the k0 others in FP64, as the forward step does (zframe_inner_fp32), with k0 the smallest
 // order whose bound beta^k0 / k0! is at most kAdjInnerTol: smaller than the forward's 2^-31
-// because an error in the inner iterate of the lower recursion enters the Frechet terms once per
-// outer step, multiplied by the spin or rank-two matrix (a factor up to ~k0 / beta more).
+// because v_k0, good to FP32, meets mu_k0 of order beta^(k0 - 1) / k0!.
 constexpr double kAdjInnerTol = 3.637978807091713e-12;  // 2^-38
 
 template <class U>
@@ -203,114 +165,194 @@ __device__ __forceinline__ WOp<U> wop_to(const WOp<double>& W) {
     return V;
 }
 
-// One Horner step (1/k = ik) of trace_terms' four recursions.
+// u . x
 template <class U>
-__device__ __forceinline__ void trace_step(const WOp<U>& W, const cpx<U> x[5], cpx<U> v2[5], cpx<U> vx[5],
-                                           cpx<U> vy[5], cpx<U> vz[5], U ik) {
-    cpx<U> w[5], e[5];
-    W.apply(vx, w);
-    apply_fx(v2, e);
-    horner_upper(w, e, vx, ik, ik);
-    W.apply(vy, w);
-    apply_fy(v2, e);
-    horner_upper(w, e, vy, ik, ik);
-    W.apply(vz, w);
-    apply_fz(v2, e);
-    horner_upper(w, e, vz, ik, ik);
-    W.apply(v2, w);
-    horner_sgn(x, w, v2, ik);
+__device__ __forceinline__ cpx<U> singlet_dot(const WOp<U>& W, const cpx<U> x[5]) {
+    cpx<U> t0 = cmul(W.u[0], x[0]), t1 = cmul(W.u[1], x[1]);
+    t0 = cfma(W.u[2], x[2], t0);
+    t1 = cfma(W.u[3], x[3], t1);
+    return cfma(W.u[4], x[4], t0) + t1;
 }
-
-// tr terms of one input vector x_r with its output cotangent g_r:
-//   tr_xyz[nu] += g_r^dagger L(B, f_nu) x_r,  tuc += g_r^dagger P(B) x_r
-// Wf: W in FP32, for the Kin inner steps of an FP64 call.
-template <class T>
-__device__ __forceinline__ void trace_terms(const WOp<T>& W, const WOp<float>& Wf, const cpx<T> x[5],
-                                            const cpx<T> g[5], int K, int Kin, cpx<T> tr[3], cpx<T>& tuc) {
-    cpx<T> v2[5], vx[5], vy[5], vz[5];
+// y = W x with u . x given
+template <class U>
+__device__ __forceinline__ void apply_dotted(const WOp<U>& W, const cpx<U> x[5], cpx<U> dot, cpx<U> y[5]) {
+    const cpx<U> t = W.R * dot;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        v2[i] = x[i];
-        vx[i] = vy[i] = vz[i] = {T(0), T(0)};
+        const cpx<U> tu = cmulc(W.u[i], t);
+        y[i] = {fma(W.D[i], x[i].re, tu.re), fma(W.D[i], x[i].im, tu.im)};
     }
-    int k = K;
-    if constexpr (std::is_same<T, double>::value) {
-        if (Kin > 0) {  // warp-uniform
-            cpx<float> xf[5], v2f[5], vxf[5], vyf[5], vzf[5];
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                xf[i] = to_prec<float>(x[i]);
-                v2f[i] = xf[i];
-                vxf[i] = vyf[i] = vzf[i] = {0.f, 0.f};
-            }
-            for (; k > K - Kin; --k) trace_step<float>(Wf, xf, v2f, vxf, vyf, vzf, inv_k(k, 0.f));
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                v2[i] = {double(v2f[i].re), double(v2f[i].im)};
-                vx[i] = {double(vxf[i].re), double(vxf[i].im)};
-                vy[i] = {double(vyf[i].re), double(vyf[i].im)};
-                vz[i] = {double(vzf[i].re), double(vzf[i].im)};
-            }
-        }
+    for (int i = 0; i < 4; ++i) {
+        y[i] = cfmac(W.ep[i], x[i + 1], y[i]);
+        y[i + 1] = cfma(W.ep[i], x[i], y[i + 1]);
     }
-    for (; k >= 1; --k) trace_step<T>(W, x, v2, vx, vy, vz, inv_k(k, T(0)));
-    tr[0] = tr[0] + cdot(g, vx);
-    tr[1] = tr[1] + cdot(g, vy);
-    tr[2] = tr[2] + cdot(g, vz);
-    tuc = tuc + cdot(g, v2);
 }
 
-// One Horner step (1/k = ik) of frechet_rank2's two recursions.
+// A Horner iterate kept for the reverse sweep, with u . v
 template <class U>
-__device__ __forceinline__ void frechet_step(const WOp<U>& W, const cpx<U> s[5], const cpx<U> p0[5],
-                                             const cpx<U> q0[5], const cpx<U> p1[5], const cpx<U> q1[5],
-                                             cpx<U> v2[5], cpx<U> out[5], U sgn, U ik) {
-    cpx<U> w[5], e[5];
-    const cpx<U> c0 = cdot(q0, v2), c1 = cdot(q1, v2);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) e[i] = cfma(c1, p1[i], cmul(c0, p0[i]));
-    W.apply(out, w);
-    horner_upper(w, e, out, sgn * ik, ik);
-    W.apply(v2, w);
-    horner_sgn(s, w, v2, sgn * ik);
+struct HornerSlot {
+    cpx<U> v[5], dot;
+};
+// Iterates kept per thread: k = 1 .. kAdjSlots in the arithmetic of the state, and of an FP64 state's
+// FP32 steps the kAdjSlotsF lowest.  Denser sites, whose degree is higher, form the others again.
+template <class T>
+constexpr int kAdjSlots = std::is_same<T, float>::value ? 4 : 6;
+constexpr int kAdjSlotsF = 4;
+
+template <class U>
+__device__ __noinline__ void horner_again(const WOp<U>* W, const cpx<U>* x, int K, int k, HornerSlot<U>* out) {
+    cpx<U> v[5], w[5];
+    for (int i = 0; i < 5; ++i) v[i] = x[i];
+    for (int n = K; n > k; --n) {
+        W->apply(v, w);
+        horner_down(x, w, v, inv_k(n, U(0)));
+    }
+    for (int i = 0; i < 5; ++i) out->v[i] = v[i];
+    out->dot = singlet_dot(*W, v);
 }
 
-// q = L(sgn B, E) s with E v = sum_r p_r (q_r^dagger v): for G s take (p, q) = (x, g) and
-// sgn = +1; for G^dagger s take (p, q) = (g, x) and sgn = -1.  Wf, Kin as in trace_terms.
-template <class T>
-__device__ __forceinline__ void frechet_rank2(const WOp<T>& W, const WOp<float>& Wf, const cpx<T> s[5],
-                                              const cpx<T> p0[5], const cpx<T> q0[5], const cpx<T> p1[5],
-                                              const cpx<T> q1[5], int K, int Kin, T sgn, cpx<T> out[5]) {
-    cpx<T> v2[5];
+// Sums of the reverse sweep over the steps and vectors
+template <class U>
+struct AdjSweep {
+    cpx<U> up[2], dn[2];  // conj(mu_i) v_{i+1} and conj(mu_{i+1}) v_i, over c_i = 1 and over c_i = sqrt(3/2)
+    U z1, z2;             // Im conj(mu_m) v_m over m = +-1 (signed) and m = +-2
+    cpx<U> q[5];
+    U s;                  // Im conj(u . mu) (u . v)
+    __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        v2[i] = s[i];
-        out[i] = {T(0), T(0)};
+        for (int i = 0; i < 2; ++i) up[i] = dn[i] = {U(0), U(0)};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) q[i] = {U(0), U(0)};
+        z1 = z2 = s = U(0);
     }
-    int k = K;
-    if constexpr (std::is_same<T, double>::value) {
+};
+
+// Step k of the reverse sweep (ik = 1/k): lam = lambda_{k-1} -> lambda_k, v = v_k
+template <class U>
+__device__ __forceinline__ void reverse_step(const WOp<U>& W, cpx<U> lam[5], const HornerSlot<U>& h, U ik, AdjSweep<U>& S) {
+    cpx<U> mu[5], w[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) mu[i] = ik * lam[i];
+    const cpx<U> p = singlet_dot(W, mu), nt = {-h.dot.re, -h.dot.im};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = i == 0 || i == 3 ? 0 : 1;
+        S.up[c] = cfmac(mu[i], h.v[i + 1], S.up[c]);
+        S.dn[c] = cfmac(mu[i + 1], h.v[i], S.dn[c]);
+    }
+    auto im = [&](int i, U acc) { return fma(mu[i].re, h.v[i].im, fma(-mu[i].im, h.v[i].re, acc)); };
+    S.z2 = im(0, S.z2) - im(4, U(0));
+    S.z1 = im(1, S.z1) - im(3, U(0));
+#pragma unroll
+    for (int i = 0; i < 5; ++i) S.q[i] = cfmac(nt, mu[i], cfmac(p, h.v[i], S.q[i]));
+    S.s = fma(p.re, h.dot.im, fma(-p.im, h.dot.re, S.s));
+    apply_dotted(W, mu, p, w);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) lam[i] = {-w[i].im, w[i].re};  // B^dagger = i W
+}
+
+// Both sweeps of one vector x with its cotangent g = lambda_0: g <- P^dagger g, tau += Im g^dagger P x,
+// S += the sums.  Wf: W in FP32, for the Kin inner steps of an FP64 state.
+template <class T>
+__device__ __forceinline__ void pull_back_vector(const WOp<T>& W, const WOp<float>& Wf, const cpx<T> x[5], cpx<T> g[5],
+                                                 int K, int Kin, T& tau, AdjSweep<T>& S) {
+    constexpr bool kMixed = std::is_same<T, double>::value;
+    HornerSlot<T> kept[kAdjSlots<T>];
+    [[maybe_unused]] HornerSlot<float> keptf[kMixed ? kAdjSlotsF : 1];
+    [[maybe_unused]] cpx<float> xf[5];
+    const int k0 = K - Kin;
+    HornerSlot<T> h;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) h.v[i] = x[i];
+    if constexpr (kMixed) {
         if (Kin > 0) {  // warp-uniform
-            cpx<float> sf[5], p0f[5], q0f[5], p1f[5], q1f[5], v2f[5], outf[5];
+            HornerSlot<float> f;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                sf[i] = to_prec<float>(s[i]);
-                p0f[i] = to_prec<float>(p0[i]);
-                q0f[i] = to_prec<float>(q0[i]);
-                p1f[i] = to_prec<float>(p1[i]);
-                q1f[i] = to_prec<float>(q1[i]);
-                v2f[i] = sf[i];
-                outf[i] = {0.f, 0.f};
+            for (int i = 0; i < 5; ++i) f.v[i] = xf[i] = to_prec<float>(x[i]);
+#pragma unroll 1
+            for (int k = K; k > k0; --k) {
+                f.dot = singlet_dot(Wf, f.v);
+                if (k - k0 <= kAdjSlotsF) keptf[k - k0 - 1] = f;
+                cpx<float> w[5];
+                apply_dotted(Wf, f.v, f.dot, w);
+                horner_down(xf, w, f.v, inv_k(k, 0.f));
             }
-            for (; k > K - Kin; --k)
-                frechet_step<float>(Wf, sf, p0f, q0f, p1f, q1f, v2f, outf, float(sgn), inv_k(k, 0.f));
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                v2[i] = {double(v2f[i].re), double(v2f[i].im)};
-                out[i] = {double(outf[i].re), double(outf[i].im)};
-            }
+            for (int i = 0; i < 5; ++i) h.v[i] = {double(f.v[i].re), double(f.v[i].im)};
         }
     }
-    for (; k >= 1; --k) frechet_step<T>(W, s, p0, q0, p1, q1, v2, out, sgn, inv_k(k, T(0)));
+#pragma unroll 1
+    for (int k = k0; k >= 1; --k) {
+        h.dot = singlet_dot(W, h.v);
+        if (k <= kAdjSlots<T>) kept[k - 1] = h;
+        cpx<T> w[5];
+        apply_dotted(W, h.v, h.dot, w);
+        horner_down(x, w, h.v, inv_k(k, T(0)));
+    }
+    tau += cdot(g, h.v).im;
+    cpx<T> lam[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) lam[i] = g[i];
+#pragma unroll 1
+    for (int k = 1; k <= k0; ++k) {
+        if (k <= kAdjSlots<T>) {
+            h = kept[k - 1];
+        } else {  // the iterates of the dense sites
+            WOp<T> Wc = W;
+            cpx<T> xc[5];
+            HornerSlot<T> hc;
+            for (int i = 0; i < 5; ++i) xc[i] = x[i];
+            horner_again<T>(&Wc, xc, K, k, &hc);
+            h = hc;
+        }
+        reverse_step(W, lam, h, inv_k(k, T(0)), S);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) g[i] = g[i] + lam[i];
+    }
+    if constexpr (kMixed) {
+        if (Kin > 0) {
+            AdjSweep<float> F;
+            F.clear();
+            cpx<float> lf[5], gf[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                lf[i] = to_prec<float>(lam[i]);
+                gf[i] = {0.f, 0.f};
+            }
+#pragma unroll 1
+            for (int k = k0 + 1; k <= K; ++k) {
+                HornerSlot<float> f;
+                if (k - k0 <= kAdjSlotsF) {
+                    f = keptf[k - k0 - 1];
+                } else {
+                    WOp<float> Wc = Wf;
+                    cpx<float> xc[5];
+                    HornerSlot<float> fc;
+                    for (int i = 0; i < 5; ++i) xc[i] = xf[i];
+                    horner_again<float>(&Wc, xc, K, k, &fc);
+                    f = fc;
+                }
+                reverse_step(Wf, lf, f, inv_k(k, 0.f), F);
+#pragma unroll
+                for (int i = 0; i < 5; ++i) gf[i] = gf[i] + lf[i];
+            }
+            auto add = [](cpx<double>& d, cpx<float> v) { d = {d.re + double(v.re), d.im + double(v.im)}; };
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                add(g[i], gf[i]);
+                add(S.q[i], F.q[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                add(S.up[i], F.up[i]);
+                add(S.dn[i], F.dn[i]);
+            }
+            S.z1 += double(F.z1);
+            S.z2 += double(F.z2);
+            S.s += double(F.s);
+        }
+    }
 }
 
 // Pull-back through U at one site.  (a, b): the state before U.  (ga, gb): cotangents of the
@@ -335,105 +377,58 @@ __device__ __forceinline__ void potential_vjp_site(const cpx<T> a[5], const cpx<
     }
     T sn, cs;
     sin_cos(A.pc.cphase * rho, &sn, &cs);
-    const cpx<T> ph = {cs, -sn};  // e^{-i delta c}
-
-    // tau and phi_nu
-    cpx<T> tr[3] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}};
-    cpx<T> tuc = {T(0), T(0)};
-    trace_terms(W, Wf, a, ga, K, Kin, tr, tuc);
-    trace_terms(W, Wf, b, gb, K, Kin, tr, tuc);
-    const T tau = cmul(ph, tuc).im;
-    const T phx = cmul(ph, tr[0]).im, phy = cmul(ph, tr[1]).im, phz = cmul(ph, tr[2]).im;
-
-    // H s
-    cpx<T> s[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) s[i] = {W.u[i].re, -W.u[i].im};  // s = conj(u)
-    cpx<T> q1[5], q2[5];
-    frechet_rank2(W, Wf, s, a, ga, b, gb, K, Kin, T(1), q1);
-    frechet_rank2(W, Wf, s, ga, a, gb, b, K, Kin, T(-1), q2);
-    cpx<T> Hs[5];
-    const cpx<T> phc = {cs, sn};
+    const cpx<T> phc = {cs, sn};  // e^{i delta c}
+    AdjSweep<T> S;
+    S.clear();
+    T tau = T(0);
+    cpx<T> x[5], y[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const cpx<T> d = cmul(ph, q1[i]) - cmul(phc, q2[i]);
-        Hs[i] = {T(0.5) * d.im, T(-0.5) * d.re};  // d / (2i)
+        x[i] = a[i];
+        y[i] = b[i];
+        ga[i] = cmul(phc, ga[i]);
+        gb[i] = cmul(phc, gb[i]);
     }
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r) {  // one copy of the code for both vectors
+        pull_back_vector(W, Wf, x, ga, K, Kin, tau, S);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            x[i] = y[i];
+            const cpx<T> t = ga[i];
+            ga[i] = gb[i];
+            gb[i] = t;
+        }
+    }
+    const T r32 = T(1.2247448713915890491);  // sqrt(3/2)
+    const cpx<T> up = S.up[0] + r32 * S.up[1], dn = S.dn[0] + r32 * S.dn[1];
+    const T phx = up.im + dn.im, phy = dn.re - up.re, phz = fma(T(2), S.z2, S.z1);
 
-    // h = 2 dg0 tau psi + 2 dg1 (phi_z f_z + phi_x f_x + phi_y f_y) psi + 2 dg2/5 J conj(H s)
-    cpx<T> h[5], fpsi[5];
-    const T t0 = T(2) * A.dg0 * tau;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) h[i] = t0 * psi[i];
-    const T t1 = T(2) * A.dg1;
-    apply_fz(psi, fpsi);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) h[i] = h[i] + (t1 * phz) * fpsi[i];
-    apply_fx(psi, fpsi);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) h[i] = h[i] + (t1 * phx) * fpsi[i];
-    apply_fy(psi, fpsi);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) h[i] = h[i] + (t1 * phy) * fpsi[i];
-    const T t2 = T(2) * A.dg2_5;
+    // h = 2 dg0 tau psi + 2 dg1 (phi_z f_z + phi_x f_x + phi_y f_y) psi + dg2/5 i J conj(q)
+    const T t0 = T(2) * A.dg0 * tau, t1 = T(2) * A.dg1;
+    const cpx<T> lower = {t1 * phx, t1 * phy};  // entry (i + 1, i) per c_i; (i, i + 1) its conjugate
+    cpx<T> h[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const T sg = (i & 1) ? T(-1) : T(1);  // (-1)^m, m = 2 - i
-        const cpx<T> c = {Hs[4 - i].re, -Hs[4 - i].im};
-        h[i] = h[i] + (sg * t2) * c;
+        const T sg = (i & 1) ? -A.dg2_5 : A.dg2_5;
+        h[i] = fma(T(2 - i), t1 * phz, t0) * psi[i];
+        h[i] = {fma(sg, S.q[4 - i].im, h[i].re), fma(sg, S.q[4 - i].re, h[i].im)};  // i conj(q)
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const cpx<T> l = spin_c<T>(i) * lower;
+        h[i] = cfmac(l, psi[i + 1], h[i]);
+        h[i + 1] = cfma(l, psi[i], h[i + 1]);
     }
 
     // coupling gradients
-    cpx<T> sHs = {T(0), T(0)};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) sHs = cfma(W.u[i], Hs[i], sHs);  // conj(s_i) = u_i
     dc[0] = A.delta * rho * tau;
     dc[1] = A.delta * (Fp.re * phx + Fp.im * phy + Fz * phz);
-    dc[2] = A.delta * sHs.re / T(5);
-
-    // U^dagger on the incoming cotangents, plus h
-    cpx<T> pa[5], pb[5];
+    dc[2] = A.delta * S.s / T(5);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        pa[i] = ga[i];
-        pb[i] = gb[i];
-    }
-    int k = K;
-    if constexpr (std::is_same<T, double>::value) {
-        if (Kin > 0) {  // warp-uniform
-            cpx<float> gaf[5], gbf[5], paf[5], pbf[5];
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                gaf[i] = paf[i] = to_prec<float>(ga[i]);
-                gbf[i] = pbf[i] = to_prec<float>(gb[i]);
-            }
-            for (; k > K - Kin; --k) {
-                const float ik = inv_k(k, 0.f);
-                cpx<float> wa[5], wb[5];
-                Wf.apply(paf, wa);
-                Wf.apply(pbf, wb);
-                horner_sgn(gaf, wa, paf, -ik);
-                horner_sgn(gbf, wb, pbf, -ik);
-            }
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                pa[i] = {double(paf[i].re), double(paf[i].im)};
-                pb[i] = {double(pbf[i].re), double(pbf[i].im)};
-            }
-        }
-    }
-    for (; k >= 1; --k) {
-        const T ik = inv_k(k, T(0));
-        cpx<T> wa[5], wb[5];
-        W.apply(pa, wa);
-        W.apply(pb, wb);
-        horner_sgn(ga, wa, pa, -ik);
-        horner_sgn(gb, wb, pb, -ik);
-    }
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        ga[i] = cmul(phc, pa[i]) + h[i];
-        gb[i] = cmul(phc, pb[i]) + h[i];
+        ga[i] = ga[i] + h[i];
+        gb[i] = gb[i] + h[i];
     }
 }
 

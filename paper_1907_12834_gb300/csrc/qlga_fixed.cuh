@@ -13,8 +13,8 @@
 // taken as signed; h h' is summed in a 64-bit accumulator, h l' + l h' in an FP32 one, and l l' (zero mean,
 // below 2^62) is dropped.  The entries of delta W and the phase are fixed point with 2^61 = 1.  FP32 leaves
 // 2^-24 of the cross terms, 2^-52 of an entry of W times the vector: with beta <= 1/4 below 2^-54, and in a field of
-// the lattice scaling (beta 0.005 to 0.06) below 2^-56.  (All three products in integers: 2D step 3% and
-// 1D step 20% slower, the same errors against 64-bit references.)
+// the lattice scaling (beta 0.005 to 0.06) below 2^-56.  (All three products in integers:
+// ten 1024^2 steps with load and read-out 7.36 ms, so 6.37, the same errors against 64-bit references.)
 //
 // U = e^{-i delta c} exp(-i delta W) as in potential_site, by the plain Taylor sum: the terms
 // T_k = (-i delta W)^k x are formed in fixed point up to the order k0 - 1 whose successor is bounded
