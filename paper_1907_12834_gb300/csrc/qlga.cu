@@ -126,22 +126,22 @@ __device__ __forceinline__ void put_pq(float* X, int64_t pair, cpx<float> a, cpx
     reinterpret_cast<float4*>(X)[pair] = pq_of(a, b);
 }
 
-// U on every site, in place.  All lanes of a warp run the potential (the Taylor degree is a
+// U on every site, in -> out (which may be in).  All lanes of a warp run the potential (the Taylor degree is a
 // warp-wide maximum); lanes past the end work on zeros and store nothing.
 // HELD_PQ: store the result as (P, Q) = (a + bt, a - bt), the form in which 1D lattices and the
 // fused 2D steps hold a state pending K (qlga_step2d.cuh); else in the resident layout (a, bt).
 template <class T, bool SPLIT, bool HELD_PQ = false>
 // FP64: 128 registers, so that 16 warps per SM cover the latency of the integer sums (0.41 ms at 1024^2
 // against 0.48 at 250 registers and 8 warps).
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 0) k_potential(T* X, int64_t nsites, PotConst<T> PC,
-                                                        unsigned* status) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 0) k_potential(const T* in, T* out, int64_t nsites,
+                                                        PotConst<T> PC, unsigned* status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t base = int64_t(blockIdx.x) * blockDim.x; base < nsites; base += stride) {
         const int64_t site = base + threadIdx.x;
         const bool active = site < nsites;
         cpx<T> a[5], b[5];
         if (active) {
-            SiteIO<T>::load(X, nsites, site, a, b);
+            SiteIO<T>::load(in, nsites, site, a, b);
         } else {
 #pragma unroll
             for (int m = 0; m < 5; ++m) a[m] = b[m] = {T(0), T(0)};
@@ -152,15 +152,15 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 0) k_potential(
             if constexpr (HELD_PQ && std::is_same<T, double>::value) {
 #pragma unroll
                 for (int m = 0; m < 5; ++m) {
-                    double2* p = reinterpret_cast<double2*>(X) + 2 * (m * nsites + site);
+                    double2* p = reinterpret_cast<double2*>(out) + 2 * (m * nsites + site);
                     p[0] = make_double2(a[m].re, a[m].im);
                     p[1] = make_double2(b[m].re, b[m].im);
                 }
             } else if constexpr (HELD_PQ) {
 #pragma unroll
-                for (int m = 0; m < 5; ++m) put_pq(X, m * nsites + site, a[m], b[m]);
+                for (int m = 0; m < 5; ++m) put_pq(out, m * nsites + site, a[m], b[m]);
             } else {
-                SiteIO<T>::store(X, nsites, site, a, b);
+                SiteIO<T>::store(out, nsites, site, a, b);
             }
         }
     }
@@ -685,9 +685,13 @@ inline int step2d_device(Step2dDevice* out) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
         const int smem = kStep2dWarpSmemBytes;
         if (cudaFuncSetAttribute(k_step2d_f32<0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<0, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
+        if (cudaFuncSetAttribute(k_step2d_f32<1, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_step2d_f32<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
@@ -739,18 +743,21 @@ inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64
 }
 
 // Returns 0 on success (errors are left in cudaGetLastError()).  pot = false applies the kinetic
-// operator alone.
+// operator alone; true_out (with pot): K X is stored there too.
 inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny, int variant, bool pot,
-                             PotConst<float> PC, unsigned* status, cudaStream_t stream) {
+                             PotConst<float> PC, unsigned* status, cudaStream_t stream, float* true_out = nullptr) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
     const int64_t strips = step2d_strips(nx);
     const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm, true, 32);
     const int grid = int((strips * chunks + kStep2dWarpsPerCta - 1) / kStep2dWarpsPerCta);
     auto launch = [&](auto kernel) {
-        kernel<<<grid, kStep2dWarpsPerCta * 32, kStep2dWarpSmemBytes, stream>>>(in, out, int(nx), int(ny), chunks, PC, status);
+        kernel<<<grid, kStep2dWarpsPerCta * 32, kStep2dWarpSmemBytes, stream>>>(in, out, int(nx), int(ny), chunks, PC, status, true_out);
     };
-    if (nx % kStep2dWarpCols == 0) {
+    if (true_out) {
+        if (nx % kStep2dWarpCols == 0) variant == 0 ? launch(k_step2d_f32<0, true, false, true>) : launch(k_step2d_f32<1, true, false, true>);
+        else variant == 0 ? launch(k_step2d_f32<0, true, true, true>) : launch(k_step2d_f32<1, true, true, true>);
+    } else if (nx % kStep2dWarpCols == 0) {
         if (variant == 0) pot ? launch(k_step2d_f32<0, true, false>) : launch(k_step2d_f32<0, false, false>);
         else pot ? launch(k_step2d_f32<1, true, false>) : launch(k_step2d_f32<1, false, false>);
     } else {
@@ -1001,11 +1008,11 @@ int grid_for(int64_t n, int cap = 0) {
 PotParams pot_params(const qlga_config& c, double delta) { return PotParams{c.g0, c.g1, c.g2, delta}; }
 
 template <class T, bool HELD_PQ = false>
-qlga_status launch_potential(qlga_handle* h, void* buf, double delta) {
+qlga_status launch_potential(qlga_handle* h, const void* in, void* out, double delta) {
     const int64_t n = nsites_of(h->cfg);
     const int nt = block_for(n);
     k_potential<T, std::is_same<T, float>::value, HELD_PQ><<<grid_for_block(n, nt), nt, 0, h->stream>>>(
-        static_cast<T*>(buf), n, PotConst<T>(pot_params(h->cfg, delta)), h->status);
+        static_cast<const T*>(in), static_cast<T*>(out), n, PotConst<T>(pot_params(h->cfg, delta)), h->status);
     QLGA_CUDA(cudaGetLastError(), "k_potential launch");
     h->launches += 1;
     return QLGA_OK;
@@ -1034,8 +1041,8 @@ qlga_status launch_axis(qlga_handle* h, const void* in, void* out, int axis, boo
     return pot ? launch_axis_t<double, 1, true>(h, in, out, axis) : launch_axis_t<double, 1, false>(h, in, out, axis);
 }
 
-qlga_status launch_pot(qlga_handle* h, void* buf, double delta) {
-    return h->cfg.precision == 32 ? launch_potential<float>(h, buf, delta) : launch_potential<double>(h, buf, delta);
+qlga_status launch_pot(qlga_handle* h, const void* in, void* out, double delta) {
+    return h->cfg.precision == 32 ? launch_potential<float>(h, in, out, delta) : launch_potential<double>(h, in, out, delta);
 }
 
 // Whether K of this 2D lattice runs in the warp-strip kernels, from 32 columns on: the FP32 step unless
@@ -1051,10 +1058,10 @@ bool held_pq(const qlga_handle* h) { return h->cfg.ndim == 1 || step2d_uses_stri
 
 // U on a true state, leaving it held pending K (X = U psi, true state K X): the first half of a
 // step, in the form the handle's kinetic pass reads.
-qlga_status launch_pot_held(qlga_handle* h, void* buf) {
+qlga_status launch_pot_held(qlga_handle* h, const void* in, void* out) {
     if (held_pq(h))
-        return h->cfg.precision == 32 ? launch_potential<float, true>(h, buf, 1.0) : launch_potential<double, true>(h, buf, 1.0);
-    return launch_pot(h, buf, 1.0);
+        return h->cfg.precision == 32 ? launch_potential<float, true>(h, in, out, 1.0) : launch_potential<double, true>(h, in, out, 1.0);
+    return launch_pot(h, in, out, 1.0);
 }
 
 // One interleaved axis pass (U^(1/(4 ndim)) before each of the axis's four blocks), in -> out.
@@ -1340,11 +1347,30 @@ qlga_status kinetic_into(qlga_handle* h, const void* in, void* out, void* mid, b
                                    h->cfg.kinetic_variant, h->stream);
         if (err) return cuda_fail(cudaGetLastError(), "step2d launch");
         h->launches += 1;
-        return pot && h->cfg.precision == 64 ? launch_pot_held(h, out) : QLGA_OK;
+        return pot && h->cfg.precision == 64 ? launch_pot_held(h, out, out) : QLGA_OK;
     }
     qlga_status s = launch_axis(h, in, mid, 0, false);
     if (s != QLGA_OK) return s;
     return launch_axis(h, mid, out, 1, pot);
+}
+
+// Two results of a state held pending K: true_out = K in, the true state, and out = U K in, held again.
+// The strip kernels read it once (FP64: U reads the true state), the others twice.
+qlga_status kinetic_and_step(qlga_handle* h, const void* in, void* true_out, void* out, void* mid) {
+    if (step2d_uses_strips(h)) {
+        if (h->cfg.precision == 64) {
+            const qlga_status s = kinetic_into(h, in, true_out, mid, false);
+            return s == QLGA_OK ? launch_pot_held(h, true_out, out) : s;
+        }
+        if (step2d_f32_launch(static_cast<const float*>(in), static_cast<float*>(out), h->cfg.nx, h->cfg.ny,
+                              h->cfg.kinetic_variant, true, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
+                              h->stream, static_cast<float*>(true_out)))
+            return cuda_fail(cudaGetLastError(), "step2d launch");
+        h->launches += 1;
+        return QLGA_OK;
+    }
+    const qlga_status s = kinetic_into(h, in, true_out, mid, false);
+    return s == QLGA_OK ? kinetic_into(h, in, out, mid, true) : s;
 }
 
 // ABI layout <-> resident layout (see qlga_device.cuh); src may equal dst.
@@ -1729,7 +1755,7 @@ qlga_status qlga_step(qlga_handle* h, int64_t n) {
                 h->cur ^= 1;
             }
         } else if (!h->pending_k) {
-            s = launch_pot_held(h, h->X[h->cur]);  // X = U psi, true state K X
+            s = launch_pot_held(h, h->X[h->cur], h->X[h->cur]);  // X = U psi, true state K X
             if (s != QLGA_OK) return s;
             h->pending_k = true;
         } else {
@@ -1747,7 +1773,7 @@ qlga_status qlga_apply_potential(qlga_handle* h, double delta) {
     if (!std::isfinite(delta)) return fail(QLGA_ERR_INVALID_ARG, "delta must be finite%s");
     qlga_status s = materialize(h);
     if (s != QLGA_OK) return s;
-    return launch_pot(h, h->X[h->cur], delta);
+    return launch_pot(h, h->X[h->cur], h->X[h->cur], delta);
 }
 
 qlga_status qlga_apply_kinetic(qlga_handle* h) {
@@ -2276,12 +2302,14 @@ qlga_status qlga_adjoint_forward(qlga_handle* h, const void* x0_device, int64_t 
     if (s != QLGA_OK) return s;
     for (int64_t k = 0; k < nsteps; ++k) {
         if (k % checkpoint_every == 0) {
-            const void* view = nullptr;
-            s = true_state_view(h, &view);
-            if (s != QLGA_OK) return s;
-            QLGA_CUDA(cudaMemcpyAsync(L.ckpt + L.state * size_t(k / checkpoint_every), view,
-                                      state_bytes_of(h->cfg), cudaMemcpyDeviceToDevice, h->stream),
-                      "checkpoint copy");
+            char* ck = L.ckpt + L.state * size_t(k / checkpoint_every);
+            if (h->pending_k) {
+                s = kinetic_into(h, h->X[h->cur], ck, h->tmp, false);
+                if (s != QLGA_OK) return s;
+            } else {
+                QLGA_CUDA(cudaMemcpyAsync(ck, h->X[h->cur], state_bytes_of(h->cfg), cudaMemcpyDeviceToDevice, h->stream),
+                          "checkpoint copy");
+            }
         }
         s = qlga_step(h, 1);
         if (s != QLGA_OK) return s;
@@ -2295,7 +2323,6 @@ qlga_status qlga_adjoint_backward(qlga_handle* h, int64_t nsteps, int64_t checkp
     qlga_status s = adj_check(h, nsteps, checkpoint_every, workspace, workspace_bytes, &L);
     if (s != QLGA_OK) return s;
     if (!cot_device) return fail(QLGA_ERR_INVALID_ARG, "cot is NULL%s");
-    const size_t nb = state_bytes_of(h->cfg);
     s = launch_convert(h, cot_device, L.cot, true);
     if (s != QLGA_OK) return s;
     QLGA_CUDA(cudaMemsetAsync(L.partials, 0, sizeof(double) * 3 * kAdjMaxBlocks, h->stream), "partials clear");
@@ -2303,27 +2330,22 @@ qlga_status qlga_adjoint_backward(qlga_handle* h, int64_t nsteps, int64_t checkp
     for (int64_t j = L.nck - 1; j >= 0; --j) {
         const int64_t start = j * checkpoint_every;
         const int64_t len = std::min(nsteps - start, checkpoint_every);
-        // recompute x_start .. x_{start+len-1} into the slots from the checkpoint:
-        // y = U x (post-potential), x_next = K y, y_next = U K y (one fused launch)
-        char* slot0 = L.slots;
-        QLGA_CUDA(cudaMemcpyAsync(slot0, L.ckpt + L.state * size_t(j), nb, cudaMemcpyDeviceToDevice, h->stream), "slot copy");
+        // recompute x_{start+1} .. x_{start+len-1} into the slots from the checkpoint:
+        // y = U x (post-potential), x_next = K y, y_next = U K y
+        const char* x0 = L.ckpt + L.state * size_t(j);
         if (len > 1) {
             void *y = L.w1, *y2 = L.w2;
-            QLGA_CUDA(cudaMemcpyAsync(y, slot0, nb, cudaMemcpyDeviceToDevice, h->stream), "segment copy");
-            s = launch_pot_held(h, y);
+            s = launch_pot_held(h, x0, y);
             if (s != QLGA_OK) return s;
             for (int64_t i = 1; i < len; ++i) {
-                s = kinetic_into(h, y, L.slots + L.state * size_t(i), tmp, false);
+                void* slot = L.slots + L.state * size_t(i);
+                s = i + 1 < len ? kinetic_and_step(h, y, slot, y2, tmp) : kinetic_into(h, y, slot, tmp, false);
                 if (s != QLGA_OK) return s;
-                if (i + 1 < len) {
-                    s = kinetic_into(h, y, y2, tmp, true);
-                    if (s != QLGA_OK) return s;
-                    std::swap(y, y2);
-                }
+                std::swap(y, y2);
             }
         }
         for (int64_t i = len - 1; i >= 0; --i) {
-            s = adj_pullback(h, &cot, &tmp, L.slots + L.state * size_t(i), L.partials);
+            s = adj_pullback(h, &cot, &tmp, i ? L.slots + L.state * size_t(i) : x0, L.partials);
             if (s != QLGA_OK) return s;
         }
     }

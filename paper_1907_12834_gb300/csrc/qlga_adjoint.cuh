@@ -144,9 +144,10 @@ __device__ __forceinline__ int build_w(const cpx<T> psi[5], const PotConst<T>& C
 
 // FP64 pull-backs run the steps of order above k0 of both sweeps in FP32 (Kin = K - k0 of them) and
 // the k0 others in FP64, as the forward step does (zframe_inner_fp32), with k0 the smallest
-// order whose bound beta^k0 / k0! is at most kAdjInnerTol: smaller than the forward's 2^-31
-// because v_k0, good to FP32, meets mu_k0 of order beta^(k0 - 1) / k0!.
-constexpr double kAdjInnerTol = 3.637978807091713e-12;  // 2^-38
+// order whose bound beta^k0 / k0! is at most kAdjInnerTol.  The last FP32 step adds its increment to the exact
+// x, so v_k0 is good to 2^-24 beta / (k0 + 1); it meets mu_k0, of order beta^(k0 - 1) / k0!, and FP32 sees
+// only mu_k of order beta^k0 / (k0 + 1)! and less: 2^-55 of the sums either way.
+constexpr double kAdjInnerTol = 4.656612873077393e-10;  // 2^-31
 
 template <class U>
 __device__ __forceinline__ cpx<U> to_prec(cpx<double> z) { return {U(z.re), U(z.im)}; }
@@ -271,15 +272,19 @@ __device__ __forceinline__ void pull_back_vector(const WOp<T>& W, const WOp<floa
 #pragma unroll
             for (int i = 0; i < 5; ++i) f.v[i] = xf[i] = to_prec<float>(x[i]);
 #pragma unroll 1
-            for (int k = K; k > k0; --k) {
+            for (int k = K;; --k) {
                 f.dot = singlet_dot(Wf, f.v);
                 if (k - k0 <= kAdjSlotsF) keptf[k - k0 - 1] = f;
                 cpx<float> w[5];
                 apply_dotted(Wf, f.v, f.dot, w);
-                horner_down(xf, w, f.v, inv_k(k, 0.f));
-            }
+                const float ik = inv_k(k, 0.f);
+                if (k == k0 + 1) {  // warp-uniform
 #pragma unroll
-            for (int i = 0; i < 5; ++i) h.v[i] = {double(f.v[i].re), double(f.v[i].im)};
+                    for (int i = 0; i < 5; ++i) h.v[i] = {x[i].re + double(ik * w[i].im), x[i].im - double(ik * w[i].re)};
+                    break;
+                }
+                horner_down(xf, w, f.v, ik);
+            }
         }
     }
 #pragma unroll 1

@@ -260,15 +260,22 @@ __device__ __forceinline__ void strip_kinetic_rows(const float* __restrict__ in,
 // One warp's share of a step: K on the strip (input held pending K as (P, Q)), then (POT) the
 // potential unitary and the store of rows [y_begin, y_end) as (P, Q) again.  POT = false stores
 // K X alone, the true state, in the resident layout (a, bt).
-// With RAGGED the lanes past the row's end store nothing.
-template <int VARIANT, bool POT, int STYLE, bool RAGGED = false>
+// With RAGGED the lanes past the row's end store nothing.  BOTH: K X goes to true_out as well.
+template <int VARIANT, bool POT, int STYLE, bool RAGGED = false, bool BOTH = false>
 __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float* __restrict__ out, int nx,
                                              int ny, int x0, int y_begin, int y_end, const PotConst<float>& PC,
-                                             unsigned* status, float4* ring, int lane) {
+                                             unsigned* status, float4* ring, int lane, float* true_out = nullptr) {
     const int64_t nsites = int64_t(nx) * ny;
     float4* out4 = reinterpret_cast<float4*>(out);
     strip_kinetic_rows<VARIANT, STYLE, RAGGED>(
         in, nx, ny, x0, y_begin, y_end, ring, lane, [&](int y, cpx<float>(&oa)[5], cpx<float>(&ob)[5]) {
+            if (BOTH && !(RAGGED && x0 + lane >= nx)) {
+                const float s = 1.0f / 256.0f;
+                float4* true4 = reinterpret_cast<float4*>(true_out) + (int64_t(y) * nx + x0 + lane);
+#pragma unroll
+                for (int m = 0; m < 5; ++m)
+                    true4[int64_t(m) * nsites] = make_float4(s * oa[m].re, s * oa[m].im, -(s * ob[m].im), s * ob[m].re);
+            }
             if (POT) {
                 // d = a - b takes the degree of psi: one warp-uniform Horner loop over both vectors
                 // runs faster here than a separate, per-lane degree for d (fewer branches)
@@ -297,10 +304,12 @@ __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float
 // its own, since the masked store costs the others registers.  Its U takes no z frame: rsqrtf and
 // the frame's products leave a site's norm up to 4e-7 off a step, and the two passes that it
 // replaces had none (error after the 20 steps 5.5e-7 before, 5.1e-7 now; with the frame 1.0e-6 in 1.10 ms).
-template <int VARIANT, bool POT, bool RAGGED, int STYLE = QLGA_STEP2D_STYLE>
+// BOTH: the step with K X, the true state, stored to true_out as well, for a run whose states are kept (a segment
+// of the adjoint at 512^2: one launch instead of 21 us for the step and 16 for the read-out).
+template <int VARIANT, bool POT, bool RAGGED, bool BOTH = false, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     k_step2d_f32(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int chunks,
-                 PotConst<float> PC, unsigned* status) {
+                 PotConst<float> PC, unsigned* status, float* __restrict__ true_out) {
     extern __shared__ float4 wring[];  // [warp][kStages][5][kStep2dWarpRowSites]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int strips = RAGGED ? (nx + kStep2dWarpCols - 1) / kStep2dWarpCols : nx / kStep2dWarpCols;
@@ -310,8 +319,9 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     const int chunk = gw / strips;
     const int y_begin = int((int64_t(chunk) * ny) / chunks);
     const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
-    step2d_strip<VARIANT, POT, STYLE, RAGGED>(in, out, nx, ny, strip * kStep2dWarpCols, y_begin, y_end, PC, status,
-                                      wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane);
+    step2d_strip<VARIANT, POT, STYLE, RAGGED, BOTH>(in, out, nx, ny, strip * kStep2dWarpCols, y_begin, y_end, PC, status,
+                                                    wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane,
+                                                    true_out);
 }
 
 // A batch of 2D lattices: warp gw takes task gw of the table -- a run (its state at pair offset
