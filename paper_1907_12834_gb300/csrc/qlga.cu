@@ -627,23 +627,19 @@ inline bool step2d_f32_supported(int64_t nx, int64_t ny) {
 }
 inline int64_t step2d_strips(int64_t nx) { return (nx + kStep2dWarpCols - 1) / kStep2dWarpCols; }
 
-// Relative throughput of an SM sub-partition that holds k warps of a fused strip kernel.  FP32:
-// the FMA pipe needs about three warps to stay busy (fitted to the 2D step timed at 256^2 ..
-// 1024^2 with one, two and three warps per sub-partition: 0.67, 0.90, 1); FP64: one warp keeps
-// the FP64 pipe busy (a warp's FP64 FMA holds it for many cycles).
-inline double step2d_pipe_eff(bool fp32, int64_t k) {
-    if (!fp32 || k >= 3) return 1.0;
-    return k == 2 ? 0.90 : 0.67;
-}
+// Relative throughput of an SM sub-partition that holds k warps of a fused strip kernel: the FMA pipe needs
+// about three warps to stay busy (fitted to the 2D step timed at 256^2 ..
+// 1024^2 with one, two and three warps per sub-partition: 0.67, 0.90, 1).
+inline double step2d_pipe_eff(int64_t k) { return k >= 3 ? 1.0 : (k == 2 ? 0.90 : 0.67); }
 
 // Row chunks per strip.  A chunk of r rows costs about r + w row updates: its first 8 rows only
 // fill the y pipeline and run the kinetic part of a row update, w = 8 x that part (warm10 = 10 w:
-// 32 in FP32, where the kinetic part is ~0.4 of a row update; 18 in FP64, where it is ~0.23).
+// 32, the kinetic part being ~0.4 of a row update).
 // With W = strips x chunks warps (at most the resident capacity sms x per_sm) the busiest of the
 // 4 sms sub-partitions holds k = ceil(W / (4 sms)) warps and finishes after about
 // k / eff(k) x (ceil(ny / chunks) + w) row times.  Within one k more chunks are shorter, so the
 // candidates are the largest chunk count of each k; the cheapest is used (the larger on ties).
-inline int step2d_chunks(int64_t strips, int64_t ny, int sms, int per_sm, bool fp32, int warm10) {
+inline int step2d_chunks(int64_t strips, int64_t ny, int sms, int per_sm, int warm10) {
     int64_t cmax = (int64_t(sms) * per_sm) / strips;
     if (cmax > ny) cmax = ny;
     if (cmax <= 1) return 1;
@@ -655,7 +651,7 @@ inline int step2d_chunks(int64_t strips, int64_t ny, int sms, int per_sm, bool f
         if (c > cmax) c = cmax;
         if (c >= 1) {
             const int64_t kk = (strips * c + lanes - 1) / lanes;
-            const double cost = double(kk) / step2d_pipe_eff(fp32, kk) * (double((ny + c - 1) / c) + 0.1 * warm10);
+            const double cost = double(kk) / step2d_pipe_eff(kk) * (double((ny + c - 1) / c) + 0.1 * warm10);
             if (best_cost < 0.0 || cost <= best_cost) {
                 best = c;
                 best_cost = cost;
@@ -666,10 +662,31 @@ inline int step2d_chunks(int64_t strips, int64_t ny, int sms, int per_sm, bool f
     return int(best);
 }
 
+// Row chunks per strip of the kernels that give a strip's levels a warp each: strips x chunks groups of five
+// warps, `resident` of them on an SM at a time; cost(rows) is a group's time on a chunk.  The busiest SM runs
+// ceil(groups / SMs) of them; one, two or three resident groups give it 0.45, 0.70 or 0.90 of its rate
+// (256^2 and 1024^2 in FP64: the chunk counts this picks are the fastest of 8 .. 32 and 5 .. 38).
+template <class Cost>
+inline int step2d_level_chunks(int64_t strips, int64_t ny, int sms, int resident, Cost&& cost) {
+    const double eff[4] = {0.0, 0.45, 0.70, 0.90};
+    int best = 1;
+    double best_cost = -1.0;
+    for (int64_t c = 1; c <= ny && c <= 4096; ++c) {
+        const int64_t per_sm = (strips * c + sms - 1) / sms, full = per_sm / resident, rest = per_sm % resident;
+        const double t = (double(resident * full) + (rest ? rest / eff[rest] : 0.0)) * cost(double((ny + c - 1) / c));
+        if (best_cost < 0.0 || t < best_cost) {
+            best = int(c);
+            best_cost = t;
+        }
+        if (strips * c > 16 * int64_t(sms) * resident) break;
+    }
+    return best;
+}
+
 // Per-device launch facts (SM count, resident warp strips per SM), set up once per device.  The
 // shared-memory opt-in is a per-device function attribute, so it is applied on each device.
 struct Step2dDevice {
-    int sms = 0, per_sm = 0, per_sm64 = 0, per_sm_obs = 0;
+    int sms = 0, per_sm = 0, per_sm_obs = 0;
 };
 
 inline int step2d_device(Step2dDevice* out) {
@@ -703,13 +720,6 @@ inline int step2d_device(Step2dDevice* out) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_step2d_f32<0, true, true>, kStep2dWarpsPerCta * 32, smem) != cudaSuccess)
             return 1;
         d.per_sm = ctas > 0 ? ctas * kStep2dWarpsPerCta : 1;
-        const int s64 = kStep2d64SmemBytes;
-        if (cudaFuncSetAttribute(k_kinetic2d_f64<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
-        if (cudaFuncSetAttribute(k_kinetic2d_f64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64) != cudaSuccess) return 1;
-        int ctas64 = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas64, k_kinetic2d_f64<0>, kStep2d64WarpsPerCta * 32, s64) != cudaSuccess)
-            return 1;
-        d.per_sm64 = ctas64 > 0 ? ctas64 * kStep2d64WarpsPerCta : 1;
         if (cudaFuncSetAttribute(k_obs2d_f32<0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_obs2d_f32<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
         if (cudaFuncSetAttribute(k_obs2d_f32<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
@@ -734,11 +744,13 @@ inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
     const int64_t strips = step2d_strips(nx);
-    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm64, true, 70);  // a warm-up row costs 0.9 of a row
-    const int grid = int((strips * chunks + kStep2d64WarpsPerCta - 1) / kStep2d64WarpsPerCta);
-    const dim3 b(kStep2d64WarpsPerCta * 32);
-    if (variant == 0) k_kinetic2d_f64<0><<<grid, b, kStep2d64SmemBytes, stream>>>(in, out, int(nx), int(ny), chunks);
-    else k_kinetic2d_f64<1><<<grid, b, kStep2d64SmemBytes, stream>>>(in, out, int(nx), int(ny), chunks);
+    // a warm-up row costs 0.9 of a row
+    const int chunks = step2d_level_chunks(strips, ny, dv.sms, kKin64Ctas * kKin64Warps / 5, [](double rows) { return rows + 7.0; });
+    auto launch = [&](auto kernel) {
+        kernel<<<int((5 * strips * chunks + kKin64Warps - 1) / kKin64Warps), 32 * kKin64Warps, 0, stream>>>(in, out, int(nx), int(ny), chunks);
+    };
+    if (variant == 0) launch(k_kinetic2d_f64<0>);
+    else launch(k_kinetic2d_f64<1>);
     return cudaPeekAtLastError() != cudaSuccess;
 }
 
@@ -749,7 +761,7 @@ inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
     const int64_t strips = step2d_strips(nx);
-    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm, true, 32);
+    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm, 32);
     const int grid = int((strips * chunks + kStep2dWarpsPerCta - 1) / kStep2dWarpsPerCta);
     auto launch = [&](auto kernel) {
         kernel<<<grid, kStep2dWarpsPerCta * 32, kStep2dWarpSmemBytes, stream>>>(in, out, int(nx), int(ny), chunks, PC, status, true_out);
@@ -793,7 +805,7 @@ inline int obs2d_f32_launch(const float* in, const float* ref, int64_t nx, int64
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
     const int64_t strips = step2d_strips(nx);
-    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm_obs, true, 32);
+    const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm_obs, 32);
     const int warps = int(strips * chunks);
     if (obs2d_scratch_bytes(nx, ny, warps) > scratch_bytes) return 2;
     char* p = static_cast<char*>(scratch);

@@ -1,14 +1,14 @@
 // qlga_step2d_f64.cuh -- the 2D FP64 kinetic operator in integer fixed point.
 //
-// K along x and y in one pass, by the y-marching warp strips of qlga_step2d.cuh: a warp owns 32 columns
-// and a row range, stages rows (with the 4-column periodic halo) in its own cp.async ring, applies
-// the nine-point x stencil from shared memory and runs the four y blocks as a register pipeline.  All
+// K along x and y in one pass, by the y-marching warp strips of qlga_step2d.cuh, a level to a warp: a warp owns
+// 32 columns of one level and a row range, stages rows (with the 4-column periodic halo) in its own cp.async ring,
+// applies the nine-point x stencil from shared memory and runs the four y blocks as a register pipeline.  All
 // of K's coefficients are small integers, so on integers K is exact up to one rounding between the
 // axes, and an addition costs 2 cycles per sub-partition where FP64 takes 76 (qlga_fixed.cuh): at 1024^2 the
-// pass takes 0.25 ms, against 1.36 ms for K in FP64.  The potential is a pass of its own
-// (k_potential): it needs the registers that hold the pipeline here, and FP64 state traffic is far
-// from the bound (the step 0.66 ms; both in one kernel, K in FP64, 1.83 ms with 1 KB of spills a
-// thread; all in FP64, 3.05 ms).
+// pass takes 0.13 ms (K in FP64 1.36; all levels of a strip in one warp, with 255 registers and 8 warps per SM, 0.187),
+// a step of 256^2 52 us (72).
+// The potential is a pass of its own (k_potential): FP64 state traffic is far
+// from the bound.
 //
 // Numbers.  A row is converted once, in place in the ring, each lane its column and an equal share of
 // the eight halo columns, to int64 with one exponent per warp: components below 2^58, the largest of
@@ -16,7 +16,7 @@
 // in magnitude, so its sums fit; they are rounded to 2^-8 of their unit, and the y blocks (taps at
 // most 44) then end below 2^61 and hold the true K X.  Where a row is larger than all before it the
 // pipeline is shifted down, where the last 16 rows are smaller it is shifted up.  The resolution is
-// thus 2^-54 of the largest component in a strip of 40 columns and 8 to 16 rows.
+// thus 2^-54 of the largest component of the level in a strip of 40 columns and 8 to 16 rows.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -86,10 +86,9 @@ __device__ __forceinline__ void stream_int(i64& a, i64& bt, i64& yo, i64& wc) {
     }
 }
 
-constexpr int kStep2d64WarpsPerCta = 2;
-constexpr int kStep2d64Stages = 3;
-constexpr int kStep2d64SmemBytes =
-    kStep2d64WarpsPerCta * kStep2d64Stages * 5 * kStep2dWarpRowSites * 32;  // double pairs
+constexpr int kKin64Warps = 4;  // of a CTA: one to a sub-partition
+constexpr int kKin64Ctas = 5;   // resident per SM
+constexpr int kKin64Stages = 3;
 constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
 
 // out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt).  nx >= 32
@@ -97,23 +96,23 @@ constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no
 // image and store nothing.  A row holding a value that is not finite gives NaN wherever the strip
 // depends on it.
 template <int VARIANT>
-__global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
+__global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
     k_kinetic2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks) {
-    extern __shared__ double2 dring[];  // [warp][kStep2d64Stages][5][kStep2dWarpRowSites][2]
-    constexpr int kRow = 5 * kStep2dWarpRowSites * 2;  // double2 of a row
+    constexpr int kRow = kStep2dWarpRowSites * 2;  // double2 of a row
+    __shared__ double2 ring_all[kKin64Warps][kKin64Stages][kRow];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
-    const int gw = blockIdx.x * kStep2d64WarpsPerCta + w;
-    if (gw >= strips * chunks) return;  // whole warp: no block-wide barrier follows
-    const int strip = gw % strips;
-    const int chunk = gw / strips;
+    const int64_t gw = int64_t(blockIdx.x) * kKin64Warps + w;
+    if (gw >= 5 * int64_t(strips) * chunks) return;  // whole warp: no block-wide barrier follows
+    const int m = int(gw % 5);
+    const int strip = int(gw / 5) % strips, chunk = int(gw / 5) / strips;
     const int x0 = strip * kStep2dWarpCols;
     const int y_begin = int((int64_t(chunk) * ny) / chunks);
     const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
     const int64_t nsites = int64_t(nx) * ny;
-    const double2* in2 = reinterpret_cast<const double2*>(in);
-    double2* out2 = reinterpret_cast<double2*>(out);
-    double2* ring = dring + w * (kStep2d64Stages * kRow);
+    const double2* level = reinterpret_cast<const double2*>(in) + 2 * (m * nsites);
+    double2* out2 = reinterpret_cast<double2*>(out) + 2 * (m * nsites);
+    double2(*ring)[kRow] = ring_all[w];
 
     const int nrows = (y_end - y_begin) + 8;
     auto wrap_x = [&](int x) {  // x < nx + 36 < 3 nx
@@ -123,67 +122,46 @@ __global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
     };
     const int xm = wrap_x(x0 - kStep2dHalo + lane);
     const int xh = wrap_x(x0 + kStep2dWarpCols - kStep2dHalo + lane);
-    auto issue_row = [&](int r) {
-        int y = y_begin - kStep2dHalo + r;
-        y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-        double2* dst = ring + (r % kStep2d64Stages) * kRow;
-        const double2* src = in2 + 2 * int64_t(y) * nx;
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            double2* d = dst + 2 * (m * kStep2dWarpRowSites + lane);
-            const double2* g = src + 2 * (m * nsites + xm);
+    int y_in = y_begin - kStep2dHalo, issued = 0;
+    y_in = y_in < 0 ? y_in + ny : y_in;
+    auto issue_row = [&]() {  // the next row, if there is one
+        if (issued < nrows) {
+            double2* d = ring[issued % kKin64Stages] + 2 * lane;
+            const double2* g = level + 2 * (int64_t(y_in) * nx + xm);
             cp_async_16(d, g);
             cp_async_16(d + 1, g + 1);
-        }
-        if (lane < 2 * kStep2dHalo) {
-#pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                double2* d = dst + 2 * (m * kStep2dWarpRowSites + kStep2dWarpCols + lane);
-                const double2* g = src + 2 * (m * nsites + xh);
-                cp_async_16(d, g);
-                cp_async_16(d + 1, g + 1);
+            if (lane < 2 * kStep2dHalo) {
+                const double2* h = level + 2 * (int64_t(y_in) * nx + xh);
+                cp_async_16(d + 2 * kStep2dWarpCols, h);
+                cp_async_16(d + 2 * kStep2dWarpCols + 1, h + 1);
             }
+            y_in = y_in + 1 == ny ? 0 : y_in + 1;
+            ++issued;
         }
-    };
-
-#pragma unroll
-    for (int r = 0; r < kStep2d64Stages - 1; ++r) {
-        if (r < nrows) issue_row(r);
         cp_async_commit();
-    }
+    };
+#pragma unroll
+    for (int r = 0; r < kKin64Stages - 1; ++r) issue_row();
 
-    cpi yo[4][5], wc[4][5];
+    cpi yo[4], wc[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int m = 0; m < 5; ++m) yo[k][m] = wc[k][m] = {0, 0};
+    for (int k = 0; k < 4; ++k) yo[k] = wc[k] = {0, 0};
     int E = kFxMinExp;                              // the pipeline's exponent
     int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
     int bad_until = -1;                             // rows up to here depend on one that is not finite
 
+#pragma unroll 1
     for (int r = 0; r < nrows; ++r) {
-        cp_async_wait<kStep2d64Stages - 2>();
+        cp_async_wait<kKin64Stages - 2>();
         __syncwarp();
-        if (r + kStep2d64Stages - 1 < nrows) issue_row(r + kStep2d64Stages - 1);
-        cp_async_commit();
+        issue_row();
 
-        double2* row = ring + (r % kStep2d64Stages) * kRow;
-        // convert the row in place: column `lane` of the ring and, of columns 32..39, the lane's
-        // component of each level
-        double halo[5];
-        double2 own[10];
-        unsigned top = 0;
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            const double2* p = row + 2 * (m * kStep2dWarpRowSites + lane);
-            own[2 * m] = p[0];
-            own[2 * m + 1] = p[1];
-            halo[m] = reinterpret_cast<const double*>(row + 2 * (m * kStep2dWarpRowSites + kStep2dWarpCols))[lane];
-            top = max(top, fx_hi(halo[m]) & 0x7fffffffu);
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-                top = max(top, max(fx_hi(own[2 * m + q].x) & 0x7fffffffu, fx_hi(own[2 * m + q].y) & 0x7fffffffu));
-        }
+        double2* row = ring[r % kKin64Stages];
+        // convert the row in place: column `lane` of the ring and the lane's component of columns 32..39
+        const double2 own0 = row[2 * lane], own1 = row[2 * lane + 1];
+        const double halo = reinterpret_cast<const double*>(row + 2 * kStep2dWarpCols)[lane];
+        auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
+        const unsigned top = max(max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y))), hi(halo));
         int Er = fx_exponent(__reduce_max_sync(0xffffffffu, top));
         const bool bad = Er > kKin64MaxExp;
         if (bad) {
@@ -199,63 +177,41 @@ __global__ void __launch_bounds__(kStep2d64WarpsPerCta * 32)
         if (En != E) {  // warp-uniform, rare on smooth fields
             const int n = max(E - En, -63);
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int m = 0; m < 5; ++m) {
-                    yo[k][m] = {fx_scale(yo[k][m].re, n), fx_scale(yo[k][m].im, n)};
-                    wc[k][m] = {fx_scale(wc[k][m].re, n), fx_scale(wc[k][m].im, n)};
-                }
+            for (int k = 0; k < 4; ++k) {
+                yo[k] = {fx_scale(yo[k].re, n), fx_scale(yo[k].im, n)};
+                wc[k] = {fx_scale(wc[k].re, n), fx_scale(wc[k].im, n)};
+            }
             E = En;
         }
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            longlong2* p = reinterpret_cast<longlong2*>(row + 2 * (m * kStep2dWarpRowSites + lane));
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-                p[q] = bad ? make_longlong2(0, 0)
-                           : make_longlong2(fx_from_double<58>(own[2 * m + q].x, E), fx_from_double<58>(own[2 * m + q].y, E));
-            reinterpret_cast<i64*>(row + 2 * (m * kStep2dWarpRowSites + kStep2dWarpCols))[lane] =
-                bad ? 0 : fx_from_double<58>(halo[m], E);
-        }
+        longlong2* p = reinterpret_cast<longlong2*>(row + 2 * lane);
+        p[0] = bad ? make_longlong2(0, 0) : make_longlong2(fx_from_double<58>(own0.x, E), fx_from_double<58>(own0.y, E));
+        p[1] = bad ? make_longlong2(0, 0) : make_longlong2(fx_from_double<58>(own1.x, E), fx_from_double<58>(own1.y, E));
+        reinterpret_cast<i64*>(row + 2 * kStep2dWarpCols)[lane] = bad ? 0 : fx_from_double<58>(halo, E);
         __syncwarp();
 
-        const bool store = r >= 8 && x0 + lane < nx;  // pipeline full: this is output row y_begin + r - 8
-        const int64_t site = int64_t(y_begin + r - 8) * nx + x0 + lane;
-        const FxToDouble to(E - 1022 - 58);
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-8
-            cpi xa = {128, 128}, xbt = {128, 128};
-            const longlong2* p = reinterpret_cast<const longlong2*>(row + 2 * (m * kStep2dWarpRowSites + lane));
-            stencil_tap_int<VARIANT, 0>(p[0], p[1], xa, xbt);
-            stencil_tap_int<VARIANT, 1>(p[2], p[3], xa, xbt);
-            stencil_tap_int<VARIANT, 2>(p[4], p[5], xa, xbt);
-            stencil_tap_int<VARIANT, 3>(p[6], p[7], xa, xbt);
-            stencil_tap_int<VARIANT, 4>(p[8], p[9], xa, xbt);
-            stencil_tap_int<VARIANT, 5>(p[10], p[11], xa, xbt);
-            stencil_tap_int<VARIANT, 6>(p[12], p[13], xa, xbt);
-            stencil_tap_int<VARIANT, 7>(p[14], p[15], xa, xbt);
-            stencil_tap_int<VARIANT, 8>(p[16], p[17], xa, xbt);
-            xa = {xa.re >> 8, xa.im >> 8};
-            xbt = {xbt.re >> 8, xbt.im >> 8};
-            // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16: the true K X)
-            stream_int<1, VARIANT>(xa.re, xbt.re, yo[0][m].re, wc[0][m].re);
-            stream_int<1, VARIANT>(xa.im, xbt.im, yo[0][m].im, wc[0][m].im);
-            stream_int<1, VARIANT>(xa.re, xbt.re, yo[1][m].re, wc[1][m].re);
-            stream_int<1, VARIANT>(xa.im, xbt.im, yo[1][m].im, wc[1][m].im);
-            stream_int<0, VARIANT>(xa.re, xbt.re, yo[2][m].re, wc[2][m].re);
-            stream_int<0, VARIANT>(xa.im, xbt.im, yo[2][m].im, wc[2][m].im);
-            stream_int<0, VARIANT>(xa.re, xbt.re, yo[3][m].re, wc[3][m].re);
-            stream_int<0, VARIANT>(xa.im, xbt.im, yo[3][m].im, wc[3][m].im);
-            if (store) {
-                double2* p2 = out2 + 2 * (int64_t(m) * nsites + site);
-                if (r <= bad_until) {  // warp-uniform
-                    const double nan = fx_bits(0x7ff80000u, 0u);
-                    p2[0] = p2[1] = make_double2(nan, nan);
-                } else {
-                    p2[0] = make_double2(to(xa.re), to(xa.im));
-                    p2[1] = make_double2(to(xbt.re), to(xbt.im));
-                }
+        // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-8
+        cpi xa = {128, 128}, xbt = {128, 128};
+        static_for<9>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value;
+            stencil_tap_int<VARIANT, kk>(p[2 * kk], p[2 * kk + 1], xa, xbt);
+        });
+        xa = {xa.re >> 8, xa.im >> 8};
+        xbt = {xbt.re >> 8, xbt.im >> 8};
+        // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16: the true K X)
+        static_for<4>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value;
+            stream_int<kk < 2 ? 1 : 0, VARIANT>(xa.re, xbt.re, yo[kk].re, wc[kk].re);
+            stream_int<kk < 2 ? 1 : 0, VARIANT>(xa.im, xbt.im, yo[kk].im, wc[kk].im);
+        });
+        if (r >= 8 && x0 + lane < nx) {  // pipeline full: this is output row y_begin + r - 8
+            double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
+            if (r <= bad_until) {  // warp-uniform
+                const double nan = fx_bits(0x7ff80000u, 0u);
+                p2[0] = p2[1] = make_double2(nan, nan);
+            } else {
+                const FxToDouble to(E - 1022 - 58);
+                p2[0] = make_double2(to(xa.re), to(xa.im));
+                p2[1] = make_double2(to(xbt.re), to(xbt.im));
             }
         }
     }
