@@ -8,15 +8,17 @@
 // stages with a dependency cone of +-4 sites.  Two kernels do one axis each in a single pass over
 // the state:
 //
-//   k_interleave_x: a CTA of 128 threads owns a tile of up to 120 consecutive sites of one row
+//   along x: a CTA of 128 threads owns a tile of up to 120 consecutive sites of one row
 //     plus 4 halo sites on each side (periodic); every thread holds one site's 10 amplitudes in
 //     registers.  Per stage: U on the site, then the block, whose two streams exchange the shifted
 //     qubit with the neighbouring thread through shared memory.  The valid part of the tile
 //     shrinks by one site per side per stage; after four stages the 120 interior sites are done.
+//     k_interleave_tile is the kernel for either axis: along y a CTA of 256 threads owns 4 columns
+//     (64-byte segments) of 64 rows, 56 of them its output.
 //   k_interleave_y: a thread owns one column of a row chunk and marches down it; the four stages
 //     form a register pipeline (as in the fused plain step): after each input row, U acts on the
 //     row leaving stage k and the streaming block k consumes it, so stage k lags by k rows.  The
-//     first 8 rows of a chunk only fill the pipeline.
+//     first 8 rows of a chunk only fill the pipeline, which is what lattices of short chunks cannot afford.
 //
 // The kinetic arithmetic is unnormalised in the (a, bt = i b) basis: every block multiplies the
 // true state by a factor of modulus 2 (2i for K1, 2 for K2).  U is invariant under a global
@@ -32,9 +34,14 @@
 
 namespace qlga {
 
-constexpr int kIlvXThreads = 128;
-constexpr int kIlvXHalo = 4;
-constexpr int kIlvXTile = kIlvXThreads - 2 * kIlvXHalo;  // 120 output sites per tile
+constexpr int kIlvHalo = 4;
+// Tiles of the two axes: threads, and columns side by side (along y)
+template <int AXIS>
+struct IlvTile {
+    static constexpr int kThreads = AXIS == 0 ? 128 : 256;
+    static constexpr int kCols = AXIS == 0 ? 1 : 4;
+    static constexpr int kOut = kThreads / kCols - 2 * kIlvHalo;  // output sites along the axis: 120, 56
+};
 constexpr int kIlvYThreads = 64;
 
 // Block qubit of stage k: qubit 2 (bt, index 1) twice, then qubit 1 (a, index 0) twice.
@@ -99,29 +106,34 @@ __device__ __forceinline__ void ilv_store(T* X, int64_t nsites, int64_t site, co
     }
 }
 
-// ------------------------------------------------------------------ x axis
+// ------------------------------------------------------------------ one axis by tiles
 
-template <class T, int VARIANT>
-__global__ void __launch_bounds__(kIlvXThreads) k_interleave_x(const T* __restrict__ in, T* __restrict__ out,
-                                                               int64_t nx, int64_t ny, PotConst<T> PC,
-                                                               unsigned* status) {
-    __shared__ cpx<T> s1[5][kIlvXThreads];
-    __shared__ cpx<T> s2[5][kIlvXThreads];
+template <class T, int VARIANT, int AXIS>
+__global__ void __launch_bounds__(IlvTile<AXIS>::kThreads, AXIS == 1 && sizeof(T) == 8 ? 1 : 0)
+    k_interleave_tile(const T* __restrict__ in, T* __restrict__ out, int64_t nx, int64_t ny, PotConst<T> PC, unsigned* status) {
+    constexpr int kThreads = IlvTile<AXIS>::kThreads, kCols = IlvTile<AXIS>::kCols, kOut = IlvTile<AXIS>::kOut;
+    __shared__ cpx<T> s1[5][kThreads];
+    __shared__ cpx<T> s2[5][kThreads];
     const int t = threadIdx.x;
-    const int64_t tiles_per_row = (nx + kIlvXTile - 1) / kIlvXTile;
-    const int64_t ntiles = tiles_per_row * ny;
+    const int p = t / kCols;  // place along the axis
+    const int64_t n = AXIS == 0 ? nx : ny;
+    const int64_t tiles_along = (n + kOut - 1) / kOut;
+    const int64_t ntiles = tiles_along * (AXIS == 0 ? ny : (nx + kCols - 1) / kCols);
     const int64_t nsites = nx * ny;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t y = tile / tiles_per_row;
-        const int64_t x0 = (tile - y * tiles_per_row) * kIlvXTile;
-        const int w = int(nx - x0 < kIlvXTile ? nx - x0 : kIlvXTile);  // output sites of this tile
-        // thread t holds column x0 - 4 + t (periodic); the tile needs t in [0, w + 8)
-        int64_t col = (x0 - kIlvXHalo + t) % nx;
-        col = col < 0 ? col + nx : col;
-        const int64_t site = y * nx + col;
+        // along y, consecutive CTAs take neighbouring columns
+        const int64_t across = AXIS == 0 ? tile / tiles_along : tile % ((nx + kCols - 1) / kCols);
+        const int64_t first = (AXIS == 0 ? tile - across * tiles_along : tile / ((nx + kCols - 1) / kCols)) * kOut;
+        const int w = int(n - first < kOut ? n - first : kOut);  // output sites of this tile along the axis
+        // place p holds site first - 4 + p (periodic); the tile needs p in [0, w + 8)
+        int64_t along = (first - kIlvHalo + p) % n;
+        along = along < 0 ? along + n : along;
+        const int64_t other = across * kCols + t % kCols;
+        const bool inside = AXIS == 0 || other < nx;
+        const int64_t site = AXIS == 0 ? other * nx + along : along * nx + (inside ? other : nx - 1);
         cpx<T> a[5], bt[5];
         ilv_load(in, nsites, site, a, bt);
-        if (t >= w + 2 * kIlvXHalo) {
+        if (p >= w + 2 * kIlvHalo) {
 #pragma unroll
             for (int m = 0; m < 5; ++m) a[m] = bt[m] = {T(0), T(0)};
         }
@@ -140,7 +152,7 @@ __global__ void __launch_bounds__(kIlvXThreads) k_interleave_x(const T* __restri
             __syncthreads();
 #pragma unroll
             for (int m = 0; m < 5; ++m) {
-                const cpx<T> z = t + 1 < kIlvXThreads ? s1[m][t + 1] : cpx<T>{T(0), T(0)};
+                const cpx<T> z = t + kCols < kThreads ? s1[m][t + kCols] : cpx<T>{T(0), T(0)};
                 if (c == 0) a[m] = z;
                 else bt[m] = z;
                 ilv_collide<T, 0>(a[m], bt[m]);  // C'
@@ -148,21 +160,21 @@ __global__ void __launch_bounds__(kIlvXThreads) k_interleave_x(const T* __restri
             }
             __syncthreads();
             // S_c: qubit c of site j takes qubit c of site j - 1
-            const bool valid = t >= k + 1 && t < w + 2 * kIlvXHalo - k - 1;
+            const bool valid = p >= k + 1 && p < w + 2 * kIlvHalo - k - 1;
 #pragma unroll
             for (int m = 0; m < 5; ++m) {
-                const cpx<T> z = t >= 1 ? s2[m][t - 1] : cpx<T>{T(0), T(0)};
+                const cpx<T> z = t >= kCols ? s2[m][t - kCols] : cpx<T>{T(0), T(0)};
                 if (c == 0) a[m] = z;
                 else bt[m] = z;
                 if (!valid) a[m] = bt[m] = {T(0), T(0)};
             }
         }
-        if (t >= kIlvXHalo && t < kIlvXHalo + w) ilv_store(out, nsites, site, a, bt, T(0.5));
+        if (p >= kIlvHalo && p < kIlvHalo + w && inside) ilv_store(out, nsites, site, a, bt, T(0.5));
         __syncthreads();  // the next tile reuses s1 / s2
     }
 }
 
-// ------------------------------------------------------------------ y axis
+// ------------------------------------------------------------------ y axis by marching
 
 // One streaming block along y for one level (input row n -> output row n - 1, in place); the
 // state keeps the unshifted qubit after the first collide (yo) and the shifted qubit after the
