@@ -320,6 +320,105 @@ __global__ void __launch_bounds__(kThreads) k_observables(const T* __restrict__ 
     }
 }
 
+// The same sums of a 2D FP32 state in the resident layout, over the rows [y0, y1): a warp owns 32 columns
+// and marches down a chunk of rows, so that a site is read once (and the first row of the next chunk again):
+// its +y neighbour is the next row's site, its +x neighbour the next lane's.  One site per thread read every
+// site three times, with a 64-bit division each: 4096^2 0.59 ms, 0.42
+// here; 1024^2 88 us, 40.  (FP64 is bound by its pipe: 410 us at 1024^2 either way.)
+__global__ void __launch_bounds__(kThreads) k_observables2d(const float* __restrict__ X, const float* __restrict__ ref, int nx,
+                                                            int ny, double g0, double g1, double g2,
+                                                            double* __restrict__ partials, int y0, int y1, int chunks) {
+    const int64_t nsites = int64_t(nx) * ny;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int strips = (nx + 31) / 32;
+    const int64_t task = int64_t(blockIdx.x) * (kThreads / 32) + warp;
+    ThreadSum<float> acc[OBS_COUNT];  // OBS_NORM_QUBIT: the sum of the populations
+    const float hg0 = float(0.5 * g0), hg1 = float(0.5 * g1), tg2 = float(0.1 * g2);
+    if (task < int64_t(strips) * chunks) {  // warp-uniform
+        const int strip = int(task % strips), chunk = int(task / strips);
+        const int rows = y1 - y0;
+        const int ya = y0 + int((int64_t(chunk) * rows) / chunks), yb = y0 + int((int64_t(chunk + 1) * rows) / chunks);
+        const int x = strip * 32 + lane;
+        const bool inside = x < nx;
+        const int xs = inside ? x : nx - 1;
+        const bool last = inside && (lane == 31 || x == nx - 1);  // the +x neighbour is not in the next lane
+        const int xn = x + 1 >= nx ? 0 : x + 1;
+        cpx<float> na[5], nb[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) load_pair<float>(X, nsites, m, int64_t(ya) * nx + xs, na[m], nb[m]);
+        for (int y = ya; y < yb; ++y) {
+            cpx<float> psi[5], right[5];
+            float pops[5], rho = float(0);
+            const int64_t row = int64_t(y) * nx;
+#pragma unroll
+            for (int m = 0; m < 5; ++m) {
+                pops[m] = norm2(na[m]) + norm2(nb[m]);
+                psi[m] = na[m] + nb[m];
+                rho += norm2(psi[m]);
+            }
+            const int64_t below = int64_t(y + 1 == ny ? 0 : y + 1) * nx + xs;
+#pragma unroll
+            for (int m = 0; m < 5; ++m) load_pair<float>(X, nsites, m, below, na[m], nb[m]);
+#pragma unroll
+            for (int m = 0; m < 5; ++m)
+                right[m] = {__shfl_down_sync(0xffffffffu, psi[m].re, 1), __shfl_down_sync(0xffffffffu, psi[m].im, 1)};
+            if (last) {
+#pragma unroll
+                for (int m = 0; m < 5; ++m) {
+                    cpx<float> a, b;
+                    load_pair<float>(X, nsites, m, row + xn, a, b);
+                    right[m] = a + b;
+                }
+            }
+            if (inside) {
+                float F2, grad = float(0);
+                cpx<float> th;
+                obs_local(psi, F2, th);
+                const float th2 = norm2(th);
+#pragma unroll
+                for (int m = 0; m < 5; ++m) {
+                    acc[OBS_POP0 + m].add(pops[m]);
+                    grad += norm2(right[m] - psi[m]);
+                    grad += norm2((na[m] + nb[m]) - psi[m]);
+                }
+                acc[OBS_NORM_BOSON].add(rho);
+                acc[OBS_ENERGY].add(grad + hg0 * rho * rho + hg1 * F2 + tg2 * th2);
+                acc[OBS_SINGLET_RE].add(th.re * float(0.44721359549995793928));  // 1/sqrt(5)
+                acc[OBS_SINGLET_IM].add(th.im * float(0.44721359549995793928));
+                acc[OBS_THETA2].add(th2);
+                acc[OBS_RHO2].add(rho * rho);
+                if (ref) {
+                    cpx<float> ov = {float(0), float(0)};
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) {
+                        cpx<float> a, b;
+                        load_pair_abi<float>(ref, nsites, m, row + x, a, b);
+                        ov = cfmac(psi[m], a + b, ov);
+                    }
+                    acc[OBS_OVERLAP_RE].add(ov.re);
+                    acc[OBS_OVERLAP_IM].add(ov.im);
+                }
+            }
+        }
+    }
+    __shared__ double sh[kThreads / 32][OBS_COUNT];
+    double total = 0.0;
+#pragma unroll
+    for (int k = 0; k < OBS_COUNT; ++k) {
+        if (k == OBS_NORM_QUBIT) continue;
+        const double v = warp_sum(acc[k].value());
+        if (k >= OBS_POP0 && k < OBS_POP0 + 5) total += v;
+        if (lane == 0) sh[warp][k] = v;
+    }
+    if (lane == 0) sh[warp][OBS_NORM_QUBIT] = total;
+    __syncthreads();
+    if (threadIdx.x < OBS_COUNT) {
+        double v = 0.0;
+        for (int w = 0; w < kThreads / 32; ++w) v += sh[w][threadIdx.x];
+        partials[int64_t(blockIdx.x) * OBS_COUNT + threadIdx.x] = v;
+    }
+}
+
 // Per-run observables of a batch: one CTA per run; terms in the state's precision (compensated
 // per-thread sums for FP32), FP64 block sums in a fixed order; out[run][OBS_COUNT].
 template <class T>
@@ -447,123 +546,111 @@ __global__ void __launch_bounds__(kThreads) k_fields(const T* __restrict__ X, T*
 }
 
 
-// The same fields on a 2D lattice, by tiles of kFieldsTx x kFieldsTy sites: the phases of the
-// tile and its one-site periodic halo are computed once into shared memory (each site's phase
-// serves the four sites whose diagonal neighbour it is: 1.3 phases per site and level instead of
-// 4), with the FP32 atan2 of psi = a + b formed in FP64 and rounded once (within a few 1e-7 rad;
-// the FP64 atan2 costs 60 times more on GB300).  Each thread reads its own site once: its phases
-// fill the tile's interior and its local fields are written before the block's barrier; the first
-// kFieldsRing threads read the ring of halo sites.  The kernel waits mostly on its loads, so it
-// runs five blocks per SM (48 registers, a few bytes spilled) rather than the four that the 60
-// registers the compiler picks alone allow; consecutive tiles fill alternate phase buffers, so one
-// barrier per tile suffices.  The four phase differences of the vorticity
+// The same fields on a 2D lattice.  A warp marches down a chunk of rows with 32 columns, the outer two of them its
+// halo: it reads a site once, writes the local fields, and keeps the FP32 phases of three rows in
+// registers, where the diagonal neighbours of the vorticity are the next lanes' (a site's phase serves the
+// four sites whose diagonal neighbour it is).  No shared memory and no barrier; 30 of 32 lanes
+// write.  4096^2 FP32 0.465 ms, the DRAM floor 0.31;
+// tiles of 32 x 8 sites with a halo ring in shared memory and a barrier each took 0.71.
+// The phases are the FP32 atan2 of psi = a + b rounded once (within a few 1e-7 rad; the FP64 atan2 costs 60 times
+// more on GB300).  The four phase differences of the vorticity
 // cancel but for their wraps, so it is pi/2 times an integer, the sum of the wrap counts; a count
 // is the one place where the phase error could change a result, and a site and level where one of
 // its four differences lies within 1e-4 of +-pi takes its four phases again in FP64, so every
 // count is the FP64 one and the vorticity is (pi/2) N exactly in either precision.
-constexpr int kFieldsTx = 32, kFieldsTy = 8;
-constexpr int kFieldsRing = 2 * (kFieldsTx + 2) + 2 * kFieldsTy;  // halo sites around a tile: 84
-static_assert(kFieldsRing <= kFieldsTx * kFieldsTy, "one ring site per thread at most");
+constexpr int kFieldsThreads = 128;
+constexpr int kFieldsCols = 30;  // output columns of a warp
+
+// Sum of the wrap counts n01 - n23 - n02 + n13 of a site and level from FP64 phases.
 template <class T>
-__global__ void __launch_bounds__(kFieldsTx * kFieldsTy, 5) k_fields2d(const T* __restrict__ X, T* __restrict__ out,
-                                                                    int64_t nx, int64_t ny) {
-    __shared__ float phb[2][5][kFieldsTy + 2][kFieldsTx + 2];
-    int parity = 0;
-    const int64_t nsites = nx * ny;
+__device__ __noinline__ int wrap_counts_f64(const T* X, int64_t nsites, int m, int64_t s0, int64_t s1, int64_t s2, int64_t s3) {
+    const int64_t nb[4] = {s0, s1, s2, s3};
+    double S[4];
+    for (int k = 0; k < 4; ++k) {
+        cpx<T> a, b;
+        load_pair<T>(X, nsites, m, nb[k], a, b);
+        S[k] = atan2(double(a.im) + double(b.im), double(a.re) + double(b.re));
+    }
+    const double pd = 3.14159265358979323846;
+    auto count = [&](double d) { return d > pd ? -1 : (d <= -pd ? 1 : 0); };
+    return count(S[0] - S[1]) - count(S[2] - S[3]) - count(S[0] - S[2]) + count(S[1] - S[3]);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kFieldsThreads) k_fields2d(const T* __restrict__ X, T* __restrict__ out, int nx, int ny,
+                                                             int chunks) {
+    const int lane = threadIdx.x & 31;
+    const int64_t task = int64_t(blockIdx.x) * (kFieldsThreads / 32) + (threadIdx.x >> 5);
+    const int strips = (nx + kFieldsCols - 1) / kFieldsCols;
+    if (task >= int64_t(strips) * chunks) return;  // whole warp: no barrier follows
+    const int strip = int(task % strips), chunk = int(task / strips);
+    const int ya = int((int64_t(chunk) * ny) / chunks), yb = int((int64_t(chunk + 1) * ny) / chunks);
+    const int64_t nsites = int64_t(nx) * ny;
+    const int x = strip * kFieldsCols - 1 + lane;  // -1 .. nx + 30
+    auto column = [&](int v) { return v < 0 ? v + nx : (v < nx ? v : v % nx); };
+    const int xc = column(x);
+    const bool mine = lane >= 1 && lane <= kFieldsCols && x < nx;
     const T r32 = T(1.2247448713915890491);
-    const int64_t tiles_x = (nx + kFieldsTx - 1) / kFieldsTx, tiles_y = (ny + kFieldsTy - 1) / kFieldsTy;
-    const int tx = threadIdx.x % kFieldsTx, ty = threadIdx.x / kFieldsTx;
-    // the ring entry (hy, hx) of this thread's halo site, for threads below kFieldsRing: the top
-    // and bottom rows of the halo box, then its left and right columns
-    const int r = threadIdx.x;
-    const int ring_hy = r < kFieldsTx + 2 ? 0
-                        : r < 2 * (kFieldsTx + 2) ? kFieldsTy + 1
-                        : 1 + (r - 2 * (kFieldsTx + 2)) % kFieldsTy;
-    const int ring_hx = r < kFieldsTx + 2 ? r
-                        : r < 2 * (kFieldsTx + 2) ? r - (kFieldsTx + 2)
-                        : (r < 2 * (kFieldsTx + 2) + kFieldsTy ? 0 : kFieldsTx + 1);
-    for (int64_t tile = blockIdx.x; tile < tiles_x * tiles_y; tile += gridDim.x) {
-        float (*ph)[kFieldsTy + 2][kFieldsTx + 2] = phb[parity];
-        const int64_t x0 = (tile % tiles_x) * kFieldsTx, y0 = (tile / tiles_x) * kFieldsTy;
-        const int64_t x = x0 + tx, y = y0 + ty;
-        const bool inside = x < nx && y < ny;
-        {
-            // this thread's site, or its periodic image where the tile passes the lattice's edge
-            const int64_t site = (y % ny) * nx + (x % nx);
-            cpx<T> psi[5];
+    float above[5], here[5], below[5];  // phases of the rows y - 1, y, y + 1
+    // row yy (-1 .. ny): its phases to ph and, for a row of the chunk, its local fields
+    auto read_row = [&](int yy, float (&ph)[5], bool own) {
+        const int64_t site = int64_t(yy < 0 ? ny - 1 : (yy >= ny ? 0 : yy)) * nx + xc;
+        cpx<T> psi[5];
 #pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                cpx<T> a, b;
-                load_pair<T>(X, nsites, m, site, a, b);
-                psi[m] = a + b;
-                const double re = double(a.re) + double(b.re), im = double(a.im) + double(b.im);
-                ph[m][ty + 1][tx + 1] = atan2f(float(im), float(re));
-            }
-            if (inside) {
-                const T Fz = T(2) * (norm2(psi[0]) - norm2(psi[4])) + (norm2(psi[1]) - norm2(psi[3]));
-                cpx<T> Fp = cmulc(psi[0], psi[1]) + cmulc(psi[3], psi[4]);
-                const cpx<T> mid = cmulc(psi[1], psi[2]) + cmulc(psi[2], psi[3]);
-                Fp = {T(2) * (Fp.re + r32 * mid.re), T(2) * (Fp.im + r32 * mid.im)};
-                const T fperp = sqrt(norm2(Fp));
-                const cpx<T> t1 = cmul(psi[0], psi[4]), t2 = cmul(psi[1], psi[3]), t3 = cmul(psi[2], psi[2]);
-                const cpx<T> th = {T(2) * (t1.re - t2.re) + t3.re, T(2) * (t1.im - t2.im) + t3.im};
-                const T a00 = sqrt(norm2(th)) * T(0.44721359549995793928);
-                const T nrm = sqrt(Fz * Fz + fperp * fperp + a00 * a00);
-                out[0 * nsites + site] = Fz;
-                out[1 * nsites + site] = fperp;
-                out[2 * nsites + site] = a00;
-                out[3 * nsites + site] = nrm > T(0) ? fabs(Fz) / nrm : T(0);
-                out[4 * nsites + site] = nrm > T(0) ? fperp / nrm : T(0);
-                out[5 * nsites + site] = nrm > T(0) ? a00 / nrm : T(0);
-            }
+        for (int m = 0; m < 5; ++m) {
+            cpx<T> a, b;
+            load_pair<T>(X, nsites, m, site, a, b);
+            psi[m] = a + b;
         }
-        if (r < kFieldsRing) {
-            int64_t xx = (x0 - 1 + ring_hx) % nx, yy = (y0 - 1 + ring_hy) % ny;
-            xx = xx < 0 ? xx + nx : xx;
-            yy = yy < 0 ? yy + ny : yy;
 #pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                cpx<T> a, b;
-                load_pair<T>(X, nsites, m, yy * nx + xx, a, b);
-                const double re = double(a.re) + double(b.re), im = double(a.im) + double(b.im);
-                ph[m][ring_hy][ring_hx] = atan2f(float(im), float(re));
-            }
+        for (int m = 0; m < 5; ++m) ph[m] = atan2f(float(psi[m].im), float(psi[m].re));
+        if (own && mine) {
+            const T Fz = T(2) * (norm2(psi[0]) - norm2(psi[4])) + (norm2(psi[1]) - norm2(psi[3]));
+            cpx<T> Fp = cmulc(psi[0], psi[1]) + cmulc(psi[3], psi[4]);
+            const cpx<T> mid = cmulc(psi[1], psi[2]) + cmulc(psi[2], psi[3]);
+            Fp = {T(2) * (Fp.re + r32 * mid.re), T(2) * (Fp.im + r32 * mid.im)};
+            const T fperp = sqrt(norm2(Fp));
+            const cpx<T> t1 = cmul(psi[0], psi[4]), t2 = cmul(psi[1], psi[3]), t3 = cmul(psi[2], psi[2]);
+            const cpx<T> th = {T(2) * (t1.re - t2.re) + t3.re, T(2) * (t1.im - t2.im) + t3.im};
+            const T a00 = sqrt(norm2(th)) * T(0.44721359549995793928);
+            const T nrm = sqrt(Fz * Fz + fperp * fperp + a00 * a00);
+            out[0 * nsites + site] = Fz;
+            out[1 * nsites + site] = fperp;
+            out[2 * nsites + site] = a00;
+            out[3 * nsites + site] = nrm > T(0) ? fabs(Fz) / nrm : T(0);
+            out[4 * nsites + site] = nrm > T(0) ? fperp / nrm : T(0);
+            out[5 * nsites + site] = nrm > T(0) ? a00 / nrm : T(0);
         }
-        __syncthreads();
-        if (inside) {
-            const int64_t site = y * nx + x;
-            const int64_t xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
-            const int64_t yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
+    };
+    read_row(ya - 1, above, false);
+    read_row(ya, here, true);
+#pragma unroll 1
+    for (int y = ya; y < yb; ++y) {
+        read_row(y + 1, below, y + 1 < yb);
 #pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                // phases at (x+1,y+1), (x+1,y-1), (x-1,y+1), (x-1,y-1): halo index = tile index + 1
-                // the four differences cancel but for their wraps, so the vorticity is
-                // (pi/2)(n01 - n23 - n02 + n13) with n the wrap count of each difference
-                auto count = [](auto d, auto pi) { return d > pi ? -1 : (d <= -pi ? 1 : 0); };
-                const float pf = 3.14159265f;
-                const float S0 = ph[m][ty + 2][tx + 2], S1 = ph[m][ty][tx + 2];
-                const float S2 = ph[m][ty + 2][tx], S3 = ph[m][ty][tx];
-                const float d01 = S0 - S1, d23 = S2 - S3, d02 = S0 - S2, d13 = S1 - S3;
-                auto near = [&](float d) { return fabsf(fabsf(d) - pf) < 1e-4f; };
-                int N = count(d01, pf) - count(d23, pf) - count(d02, pf) + count(d13, pf);
+        for (int m = 0; m < 5; ++m) {
+            // phases at (x+1,y+1), (x+1,y-1), (x-1,y+1), (x-1,y-1); the four differences cancel but for
+            // their wraps, so the vorticity is (pi/2)(n01 - n23 - n02 + n13) with n the wrap count of each
+            const float S0 = __shfl_down_sync(0xffffffffu, below[m], 1), S1 = __shfl_down_sync(0xffffffffu, above[m], 1);
+            const float S2 = __shfl_up_sync(0xffffffffu, below[m], 1), S3 = __shfl_up_sync(0xffffffffu, above[m], 1);
+            const float pf = 3.14159265f;
+            auto count = [&](float d) { return d > pf ? -1 : (d <= -pf ? 1 : 0); };
+            const float d01 = S0 - S1, d23 = S2 - S3, d02 = S0 - S2, d13 = S1 - S3;
+            auto near = [&](float d) { return fabsf(fabsf(d) - pf) < 1e-4f; };
+            int N = count(d01) - count(d23) - count(d02) + count(d13);
+            if (mine) {
                 if (near(d01) || near(d23) || near(d02) || near(d13)) {
-                    const int64_t nb[4] = {yp * nx + xp, ym * nx + xp, yp * nx + xm, ym * nx + xm};
-                    double S[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        cpx<T> a, b;
-                        load_pair<T>(X, nsites, m, nb[k], a, b);
-                        S[k] = atan2(double(a.im) + double(b.im), double(a.re) + double(b.re));
-                    }
-                    const double pd = 3.14159265358979323846;
-                    N = count(S[0] - S[1], pd) - count(S[2] - S[3], pd) - count(S[0] - S[2], pd) +
-                        count(S[1] - S[3], pd);
+                    const int64_t yp = int64_t(y + 1 == ny ? 0 : y + 1) * nx, ym = int64_t(y == 0 ? ny - 1 : y - 1) * nx;
+                    const int xp = column(x + 1), xm = column(x - 1);
+                    N = wrap_counts_f64(X, nsites, m, yp + xp, ym + xp, yp + xm, ym + xm);
                 }
+                const int64_t site = int64_t(y) * nx + x;
                 if constexpr (std::is_same<T, float>::value) out[(6 + m) * nsites + site] = 1.57079633f * float(N);
                 else out[(6 + m) * nsites + site] = 1.5707963267948966 * double(N);
             }
+            above[m] = here[m];
+            here[m] = below[m];
         }
-        parity ^= 1;  // the next tile fills the other buffer: one barrier per tile
     }
 }
 
@@ -1816,13 +1903,25 @@ static qlga_status observables_rows_partials(qlga_handle* h, const void* ref_sta
     qlga_status s = true_state_view(h, &view);
     if (s != QLGA_OK) return s;
     const int64_t s0 = y0 * h->cfg.nx, s1 = y1 * h->cfg.nx;
-    const int blocks = grid_for(s1 - s0, obs_blocks_cap());
-    if (h->cfg.precision == 32)
-        k_observables<float, true><<<blocks, kThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<const float*>(ref_state_device),
-                                                                 h->cfg.nx, h->cfg.ny, h->cfg.ndim, h->cfg.g0, h->cfg.g1, h->cfg.g2, h->partials, s0, s1);
-    else
-        k_observables<double, true><<<blocks, kThreads, 0, h->stream>>>(static_cast<const double*>(view), static_cast<const double*>(ref_state_device),
-                                                                  h->cfg.nx, h->cfg.ny, h->cfg.ndim, h->cfg.g0, h->cfg.g1, h->cfg.g2, h->partials, s0, s1);
+    int blocks;
+    if (h->cfg.ndim == 2 && h->cfg.precision == 32 && h->cfg.nx < (int64_t(1) << 30) && h->cfg.ny < (int64_t(1) << 30) &&
+        (h->cfg.nx + 31) / 32 <= 4 * int64_t(obs_blocks_cap())) {
+        // strips x chunks of at least 4 rows (a chunk reads one row more), two blocks per SM: one wave
+        const int64_t strips = (h->cfg.nx + 31) / 32, per_block = kThreads / 32;
+        const int64_t warps = per_block * std::min(obs_blocks_cap(), 2 * device_sms());
+        const int64_t chunks = std::max<int64_t>(1, std::min((y1 - y0) / 4, warps / strips));
+        blocks = int((strips * chunks + per_block - 1) / per_block);
+        k_observables2d<<<blocks, kThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<const float*>(ref_state_device),
+                                                            int(h->cfg.nx), int(h->cfg.ny), h->cfg.g0, h->cfg.g1, h->cfg.g2, h->partials, int(y0), int(y1), int(chunks));
+    } else {
+        blocks = grid_for(s1 - s0, obs_blocks_cap());
+        if (h->cfg.precision == 32)
+            k_observables<float, true><<<blocks, kThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<const float*>(ref_state_device),
+                                                                     h->cfg.nx, h->cfg.ny, h->cfg.ndim, h->cfg.g0, h->cfg.g1, h->cfg.g2, h->partials, s0, s1);
+        else
+            k_observables<double, true><<<blocks, kThreads, 0, h->stream>>>(static_cast<const double*>(view), static_cast<const double*>(ref_state_device),
+                                                                      h->cfg.nx, h->cfg.ny, h->cfg.ndim, h->cfg.g0, h->cfg.g1, h->cfg.g2, h->partials, s0, s1);
+    }
     QLGA_CUDA(cudaGetLastError(), "k_observables launch");
     h->launches += 1;
     *partials = h->partials;
@@ -2027,20 +2126,20 @@ qlga_status qlga_fields(qlga_handle* h, void* dst, int where) {
     void* target = dst;
     if (where == QLGA_HOST) target = (view == h->tmp) ? h->X[1 - h->cur] : h->tmp;
     if (h->cfg.ndim == 2) {
-        const int64_t tiles = ((h->cfg.nx + kFieldsTx - 1) / kFieldsTx) * ((h->cfg.ny + kFieldsTy - 1) / kFieldsTy);
-        // one wave of resident blocks: each block loops over tiles, so blocks beyond the resident
-        // count would start only when the first wave has finished all of its tiles
+        // one wave of resident blocks, each warp a strip of a chunk of at least 8 rows (a chunk reads two rows more)
         int per_sm = 0;
         QLGA_CUDA(h->cfg.precision == 32
-                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fields2d<float>, kFieldsTx * kFieldsTy, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fields2d<double>, kFieldsTx * kFieldsTy, 0),
+                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fields2d<float>, kFieldsThreads, 0)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fields2d<double>, kFieldsThreads, 0),
                   "k_fields2d occupancy");
-        const int64_t cap = int64_t(per_sm > 0 ? per_sm : 1) * device_sms();
-        const int grid = int(tiles < cap ? tiles : cap);
+        const int64_t per_block = kFieldsThreads / 32, strips = (h->cfg.nx + kFieldsCols - 1) / kFieldsCols;
+        const int64_t warps = per_block * (per_sm > 0 ? per_sm : 1) * device_sms();
+        const int64_t chunks = std::max<int64_t>(1, std::min(h->cfg.ny / 8, warps / strips));
+        const int64_t grid = (strips * chunks + per_block - 1) / per_block;
         if (h->cfg.precision == 32)
-            k_fields2d<float><<<grid, kFieldsTx * kFieldsTy, 0, h->stream>>>(static_cast<const float*>(view), static_cast<float*>(target), h->cfg.nx, h->cfg.ny);
+            k_fields2d<float><<<unsigned(grid), kFieldsThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<float*>(target), int(h->cfg.nx), int(h->cfg.ny), int(chunks));
         else
-            k_fields2d<double><<<grid, kFieldsTx * kFieldsTy, 0, h->stream>>>(static_cast<const double*>(view), static_cast<double*>(target), h->cfg.nx, h->cfg.ny);
+            k_fields2d<double><<<unsigned(grid), kFieldsThreads, 0, h->stream>>>(static_cast<const double*>(view), static_cast<double*>(target), int(h->cfg.nx), int(h->cfg.ny), int(chunks));
     } else if (h->cfg.precision == 32) {
         k_fields<float><<<grid_for(n), kThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<float*>(target), h->cfg.nx, h->cfg.ny, h->cfg.ndim);
     } else {
