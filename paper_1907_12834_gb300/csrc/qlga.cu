@@ -848,6 +848,27 @@ inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
     const int64_t strips = step2d_strips(nx);
+    // by levels (qlga_step2d.cuh): us a step, one warp a strip / by levels: 128^2 7.8 / 6.1, 384 x 107 10.5 / 8.0,
+    // 256^2 12.0 / 9.8, 512^2 22.3 / 23.5, 1024^2 61 / 72; K alone, 512^2 27.0 / 24.4, 1024^2 71 / 66, 2048^2 221 / 221
+    if (nx * ny <= (pot ? int64_t(1) << 17 : int64_t(1) << 20)) {
+        const int levels = step2d_level_chunks(strips, ny, dv.sms, kLevelsCtas, [](double rows) {
+            return 0.4 * (rows + 8.0) + 0.6 * (5.0 * std::ceil(rows / 5.0));  // K is 0.4 of a row, U runs by five rows
+        });
+        auto launch = [&](auto kernel) {
+            kernel<<<int(strips * levels), kLevelsThreads, 0, stream>>>(in, out, int(nx), int(ny), levels, PC, status, true_out);
+        };
+        if (true_out) {
+            if (nx % kStep2dWarpCols == 0) variant == 0 ? launch(k_step2d_levels<0, true, false, true>) : launch(k_step2d_levels<1, true, false, true>);
+            else variant == 0 ? launch(k_step2d_levels<0, true, true, true>) : launch(k_step2d_levels<1, true, true, true>);
+        } else if (nx % kStep2dWarpCols == 0) {
+            if (variant == 0) pot ? launch(k_step2d_levels<0, true, false>) : launch(k_step2d_levels<0, false, false>);
+            else pot ? launch(k_step2d_levels<1, true, false>) : launch(k_step2d_levels<1, false, false>);
+        } else {
+            if (variant == 0) pot ? launch(k_step2d_levels<0, true, true>) : launch(k_step2d_levels<0, false, true>);
+            else pot ? launch(k_step2d_levels<1, true, true>) : launch(k_step2d_levels<1, false, true>);
+        }
+        return cudaPeekAtLastError() != cudaSuccess;
+    }
     const int chunks = step2d_chunks(strips, ny, dv.sms, dv.per_sm, 32);
     const int grid = int((strips * chunks + kStep2dWarpsPerCta - 1) / kStep2dWarpsPerCta);
     auto launch = [&](auto kernel) {

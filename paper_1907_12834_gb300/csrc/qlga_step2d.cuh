@@ -324,6 +324,125 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
                                                     true_out);
 }
 
+// ------------------------------------------------------------------ the step by levels
+//
+// K acts on each level by itself, so here the five levels of a strip go to the five warps of a CTA: a warp
+// holds one level's y pipeline (32 registers instead of 160 a lane) and one level's ring.  Every five output rows
+// the levels meet in shared memory and each warp applies U to one of the rows.  Two exchange buffers in
+// turn, so one barrier per five rows suffices.  Small
+// lattices gain: their chunks are few rows, whose 8 warm-up rows now cost a fifth, and 20 warps share an SM instead of 12
+// (the dispatch in qlga.cu has both sides); on large ones the exchange and a fifth of the work per
+// staged row cost more than the occupancy gives (4096^2 0.98 ms against 0.76).  U takes no z frame: 96
+// registers, and half the error (512^2, 32 steps: 6.6e-7 against 1.5e-6).
+constexpr int kLevelsThreads = 160;
+constexpr int kLevelsCtas = 4;  // resident per SM
+template <int VARIANT, bool POT, bool RAGGED, bool BOTH = false, int STYLE = QLGA_STEP2D_STYLE>
+__global__ void __launch_bounds__(kLevelsThreads, kLevelsCtas)
+    k_step2d_levels(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int chunks,
+                    PotConst<float> PC, unsigned* status, float* __restrict__ true_out) {
+    __shared__ float4 ring_all[5][kStep2dStages][kStep2dWarpRowSites];
+    __shared__ float4 xch[POT ? 2 : 1][POT ? 5 : 1][5][32];  // [buffer][row][level][column]
+    const int lane = threadIdx.x & 31, m = threadIdx.x >> 5;
+    const int strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
+    const int strip = blockIdx.x % strips, chunk = blockIdx.x / strips;
+    const int x0 = strip * kStep2dWarpCols;
+    const int y_begin = int((int64_t(chunk) * ny) / chunks), y_end = int((int64_t(chunk + 1) * ny) / chunks);
+    const int64_t nsites = int64_t(nx) * ny;
+    const bool stored = !RAGGED || x0 + lane < nx;
+    float4* out4 = reinterpret_cast<float4*>(out);
+    float4(*ring)[kStep2dWarpRowSites] = ring_all[m];
+    const float4* level = reinterpret_cast<const float4*>(in) + m * nsites;
+    int xm = x0 - kStep2dHalo + lane;
+    xm = xm < 0 ? xm + nx : xm;
+    if (RAGGED) xm = xm >= nx ? xm - nx : xm;
+    int xh = x0 + kStep2dWarpCols - kStep2dHalo + lane;
+    xh = xh >= nx ? xh - nx : xh;
+    xh = xh >= nx ? xh - nx : xh;
+    const int nrows = (y_end - y_begin) + 8;
+    int y_in = y_begin - kStep2dHalo;
+    y_in = y_in < 0 ? y_in + ny : y_in;
+    int issued = 0;
+    auto issue_row = [&]() {  // the next row, if there is one
+        if (issued < nrows) {
+            float4* dst = ring[issued % kStep2dStages];
+            const float4* src = level + int64_t(y_in) * nx;
+            cp_async_16(dst + lane, src + xm);
+            if (lane < 2 * kStep2dHalo) cp_async_16(dst + kStep2dWarpCols + lane, src + xh);
+            y_in = y_in + 1 == ny ? 0 : y_in + 1;
+            ++issued;
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int r = 0; r < kStep2dStages - 1; ++r) issue_row();
+
+    BlockState st[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) st[k] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    int row = 0, buf = 0;     // of the exchange
+    int y = y_begin;          // the row that goes to place 0
+#pragma unroll 1
+    for (int r = 0; r < nrows; ++r) {
+        cp_async_wait<kStep2dStages - 2>();
+        __syncwarp();
+        issue_row();
+        const float4* p = ring[r % kStep2dStages] + lane;
+        float2 xa = make_float2(0.f, 0.f), xbt = make_float2(0.f, 0.f);
+        float2 ya = make_float2(0.f, 0.f), ybt = make_float2(0.f, 0.f);
+        stencil_tap<VARIANT, 0, STYLE>(p[0], xa, xbt);
+        stencil_tap<VARIANT, 1, STYLE>(p[1], ya, ybt);
+        stencil_tap<VARIANT, 2, STYLE>(p[2], xa, xbt);
+        stencil_tap<VARIANT, 3, STYLE>(p[3], ya, ybt);
+        stencil_tap<VARIANT, 4, STYLE>(p[4], xa, xbt);
+        stencil_tap<VARIANT, 5, STYLE>(p[5], ya, ybt);
+        stencil_tap<VARIANT, 6, STYLE>(p[6], xa, xbt);
+        stencil_tap<VARIANT, 7, STYLE>(p[7], ya, ybt);
+        stencil_tap<VARIANT, 8, STYLE>(p[8], xa, xbt);
+        xa = p_add<STYLE>(xa, ya);
+        xbt = p_add<STYLE>(xbt, ybt);
+        stream_block<1, VARIANT, STYLE>(xa, xbt, st[0]);
+        stream_block<1, VARIANT, STYLE>(xa, xbt, st[1]);
+        stream_block<0, VARIANT, STYLE>(xa, xbt, st[2]);
+        stream_block<0, VARIANT, STYLE>(xa, xbt, st[3]);
+        if (r < 8) continue;
+        if (!POT) {
+            const float s = 1.0f / 256.0f;
+            if (stored)
+                out4[m * nsites + int64_t(y_begin + r - 8) * nx + x0 + lane] = make_float4(s * xa.x, s * xa.y, s * xbt.x, s * xbt.y);
+            continue;
+        }
+        xch[buf][row][m][lane] = make_float4(xa.x, xa.y, xbt.x, xbt.y);
+        if (++row < 5 && r + 1 < nrows) continue;
+        __syncthreads();
+        if (m < row) {  // warp-uniform: this warp's row
+            cpx<float> a[5], b[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const float4 v = xch[buf][m][k][lane];
+                a[k] = {v.x, v.y};
+                b[k] = {v.w, -v.z};  // b = -i bt
+            }
+            const int64_t site = int64_t(y + m) * nx + x0 + lane;
+            if (BOTH && stored) {
+                const float s = 1.0f / 256.0f;
+#pragma unroll
+                for (int k = 0; k < 5; ++k)
+                    reinterpret_cast<float4*>(true_out)[k * nsites + site] =
+                        make_float4(s * a[k].re, s * a[k].im, -(s * b[k].im), s * b[k].re);
+            }
+            potential_site<float, false>(a, b, PC, 1.0f / 65536.0f, 0.5f / 256.0f, status);
+            if (stored) {
+#pragma unroll
+                for (int k = 0; k < 5; ++k) out4[k * nsites + site] = pq_of(a[k], b[k]);
+            }
+        }
+        y += 5;
+        row = 0;
+        buf ^= 1;
+    }
+    cp_async_wait<0>();
+}
+
 // A batch of 2D lattices: warp gw takes task gw of the table -- a run (its state at pair offset
 // base, nx x ny sites, constants consts[run]), a strip and a row range.
 struct WarpTask {
