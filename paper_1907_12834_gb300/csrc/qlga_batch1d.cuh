@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
                                                    const BatchRun* __restrict__ runs,
                                                    const PotConst<T>* __restrict__ consts,
                                                    unsigned* status, int single_L,
-                                                   PotConst<T> single_pc) {
+                                                   PotConst<T> single_pc, bool abi) {
     static_assert(STEPS == 1 || (STEPS == 2 && POT), "two steps per launch are fused steps");
     constexpr int TW = W * SPT;                  // sites per pass
     constexpr int TOUT = TW - 8 * (STEPS - 1);   // output sites of a tile
@@ -191,6 +191,8 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
             for (int m = 0; m < 5; ++m) {
                 if (POT)  // held pending K again, as (P, Q)
                     store_raw_pq(out, run.base + int64_t(m) * L + j, oa[m], ob[m]);
+                else if (abi)  // the true state, straight to a caller's buffer
+                    store_raw_pair(out, run.base + int64_t(m) * L + j, oa[m].re, oa[m].im, ob[m].re, ob[m].im);
                 else  // the true state, (a, bt)
                     store_raw_pair(out, run.base + int64_t(m) * L + j, oa[m].re, oa[m].im, -ob[m].im, ob[m].re);
             }

@@ -109,6 +109,13 @@ struct SiteIO<double> {
     }
 };
 
+// The layout of a true state that a read-out of K writes: the resident pair (a, bt = i b) or, where it goes
+// straight to a caller's buffer, the ABI's (a, b).
+template <class T>
+__device__ __forceinline__ void read_out_pair(cpx<T>& bt, bool abi) {
+    if (abi) bt = {bt.im, -bt.re};  // b = -i bt
+}
+
 // ------------------------------------------------------------------ kinetic stencil
 //
 // One axis of the kinetic operator, I'_1 I'_1 I'_2 I'_2 with I'_c = S_c C' S^T_c C (Sec. VII.B;

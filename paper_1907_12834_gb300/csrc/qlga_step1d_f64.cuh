@@ -35,7 +35,7 @@ constexpr int kFx1dSpread = 7;  // exponents within this of the largest share it
 // K (and U) of site j in FP64, for the warps that the integer form leaves; all lanes take part.
 template <int VARIANT, bool POT>
 __device__ __noinline__ void step1d_site_f64(const double* in, double* out, int L, int j, bool store,
-                                             const PotConstBase<double>* C, unsigned* status) {
+                                             const PotConstBase<double>* C, unsigned* status, bool abi = false) {
     cpx<double> a[5], b[5];
 #pragma unroll 1
     for (int m = 0; m < 5; ++m) {
@@ -52,6 +52,7 @@ __device__ __noinline__ void step1d_site_f64(const double* in, double* out, int 
             b[m] = {xbt.im, -xbt.re};
         } else if (store) {
             const double s = 1.0 / 16.0;
+            read_out_pair(xbt, abi);
             store_raw_pair(out, int64_t(m) * L + j, s * xa.re, s * xa.im, s * xbt.re, s * xbt.im);
         }
     }
@@ -63,10 +64,11 @@ __device__ __noinline__ void step1d_site_f64(const double* in, double* out, int 
 }
 
 // One fused step (K, then U) of a periodic 1D lattice of L sites held pending K as (P, Q), or K alone
-// (POT = false: the true state in the resident layout (a, bt)).
+// (POT = false: the true state in the resident layout (a, bt) or, with abi, the ABI's (a, b)).
 template <int VARIANT, bool POT>
 __global__ void __launch_bounds__(32) k_step1d_f64(const double* __restrict__ in, double* __restrict__ out, int L,
-                                                   const __grid_constant__ PotConst<double> C, unsigned* status) {
+                                                   const __grid_constant__ PotConst<double> C, unsigned* status,
+                                                   bool abi) {
     __shared__ longlong2 sp[5][kFx1dCols], sq[5][kFx1dCols];
     __shared__ int se[kFx1dCols];
     const int lane = threadIdx.x;
@@ -103,7 +105,7 @@ __global__ void __launch_bounds__(32) k_step1d_f64(const double* __restrict__ in
     const unsigned top = __reduce_max_sync(0xffffffffu, max(to, th));
     if (top >= (unsigned(1023 + 50) << 20)) {  // warp-uniform; far outside U's domain, or not finite
         const PotConstBase<double> base = C;
-        step1d_site_f64<VARIANT, POT>(in, out, L, j, store, &base, status);
+        step1d_site_f64<VARIANT, POT>(in, out, L, j, store, &base, status, abi);
         return;
     }
     int Eo = fx_exponent(to), Eh = fx_exponent(th);
@@ -138,8 +140,8 @@ __global__ void __launch_bounds__(32) k_step1d_f64(const double* __restrict__ in
         } else {
             pr[m] = xa.re;
             pi[m] = xa.im;
-            dr[m] = xbt.re;
-            di[m] = xbt.im;
+            dr[m] = abi ? xbt.im : xbt.re;
+            di[m] = abi ? -xbt.re : xbt.im;
         }
     };
     if (shared) {
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(32) k_step1d_f64(const double* __restrict__ in
         int e = E - 1022 - 55;
         if (!fx_unitary(pr, pi, dr, di, e, -4, true, C.fx)) {
             const PotConstBase<double> base = C;
-            step1d_site_f64<VARIANT, POT>(in, out, L, j, store, &base, status);
+            step1d_site_f64<VARIANT, POT>(in, out, L, j, store, &base, status, abi);
             return;
         }
         if (!store) return;

@@ -259,12 +259,12 @@ __device__ __forceinline__ void strip_kinetic_rows(const float* __restrict__ in,
 
 // One warp's share of a step: K on the strip (input held pending K as (P, Q)), then (POT) the
 // potential unitary and the store of rows [y_begin, y_end) as (P, Q) again.  POT = false stores
-// K X alone, the true state, in the resident layout (a, bt).
+// K X alone, the true state, in the resident layout (a, bt) or, with abi, the ABI's (a, b).
 // With RAGGED the lanes past the row's end store nothing.  BOTH: K X goes to true_out as well.
 template <int VARIANT, bool POT, int STYLE, bool RAGGED = false, bool BOTH = false>
 __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float* __restrict__ out, int nx,
                                              int ny, int x0, int y_begin, int y_end, const PotConst<float>& PC,
-                                             unsigned* status, float4* ring, int lane, float* true_out = nullptr) {
+                                             unsigned* status, float4* ring, int lane, float* true_out = nullptr, bool abi = false) {
     const int64_t nsites = int64_t(nx) * ny;
     float4* out4 = reinterpret_cast<float4*>(out);
     strip_kinetic_rows<VARIANT, STYLE, RAGGED>(
@@ -293,7 +293,8 @@ __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float
 #pragma unroll
             for (int m = 0; m < 5; ++m)  // POT: held pending K again, as (P, Q); else the true state
                 out4[int64_t(m) * nsites + site] =
-                    POT ? pq_of(oa[m], ob[m]) : make_float4(oa[m].re, oa[m].im, -ob[m].im, ob[m].re);
+                    POT ? pq_of(oa[m], ob[m])
+                        : (abi ? make_float4(oa[m].re, oa[m].im, ob[m].re, ob[m].im) : make_float4(oa[m].re, oa[m].im, -ob[m].im, ob[m].re));
         });
 }
 
@@ -309,7 +310,7 @@ __device__ __forceinline__ void step2d_strip(const float* __restrict__ in, float
 template <int VARIANT, bool POT, bool RAGGED, bool BOTH = false, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     k_step2d_f32(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int chunks,
-                 PotConst<float> PC, unsigned* status, float* __restrict__ true_out) {
+                 PotConst<float> PC, unsigned* status, float* __restrict__ true_out, bool abi) {
     extern __shared__ float4 wring[];  // [warp][kStages][5][kStep2dWarpRowSites]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int strips = RAGGED ? (nx + kStep2dWarpCols - 1) / kStep2dWarpCols : nx / kStep2dWarpCols;
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
     step2d_strip<VARIANT, POT, STYLE, RAGGED, BOTH>(in, out, nx, ny, strip * kStep2dWarpCols, y_begin, y_end, PC, status,
                                                     wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane,
-                                                    true_out);
+                                                    true_out, abi);
 }
 
 // ------------------------------------------------------------------ the step by levels
@@ -339,7 +340,7 @@ constexpr int kLevelsCtas = 4;  // resident per SM
 template <int VARIANT, bool POT, bool RAGGED, bool BOTH = false, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kLevelsThreads, kLevelsCtas)
     k_step2d_levels(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int chunks,
-                    PotConst<float> PC, unsigned* status, float* __restrict__ true_out) {
+                    PotConst<float> PC, unsigned* status, float* __restrict__ true_out, bool abi) {
     __shared__ float4 ring_all[5][kStep2dStages][kStep2dWarpRowSites];
     __shared__ float4 xch[POT ? 2 : 1][POT ? 5 : 1][5][32];  // [buffer][row][level][column]
     const int lane = threadIdx.x & 31, m = threadIdx.x >> 5;
@@ -407,6 +408,7 @@ __global__ void __launch_bounds__(kLevelsThreads, kLevelsCtas)
         if (r < 8) continue;
         if (!POT) {
             const float s = 1.0f / 256.0f;
+            if (abi) xbt = make_float2(xbt.y, -xbt.x);  // b = -i bt
             if (stored)
                 out4[m * nsites + int64_t(y_begin + r - 8) * nx + x0 + lane] = make_float4(s * xa.x, s * xa.y, s * xbt.x, s * xbt.y);
             continue;
@@ -459,7 +461,7 @@ template <int VARIANT, bool POT = true, int STYLE = QLGA_STEP2D_STYLE>
 __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     k_batch_step2d_f32(const float* __restrict__ in, float* __restrict__ out,
                        const WarpTask* __restrict__ tasks, int ntasks, const Run2d* __restrict__ runs,
-                       const PotConst<float>* __restrict__ consts, unsigned* status) {
+                       const PotConst<float>* __restrict__ consts, unsigned* status, bool abi) {
     extern __shared__ float4 wring[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int gw = blockIdx.x * kStep2dWarpsPerCta + w;
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(kStep2dWarpsPerCta * 32, 3)
     const PotConst<float> PC = consts[task.run];
     step2d_strip<VARIANT, POT, STYLE>(in + 4 * run.base, out + 4 * run.base, run.nx, run.ny, task.x0,
                                       task.y_begin, task.y_end, PC, status,
-                                      wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane);
+                                      wring + w * (kStep2dStages * 5 * kStep2dWarpRowSites), lane, nullptr, abi);
 }
 
 }  // namespace qlga

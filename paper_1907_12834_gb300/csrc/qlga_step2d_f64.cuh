@@ -91,13 +91,14 @@ constexpr int kKin64Ctas = 5;   // resident per SM
 constexpr int kKin64Stages = 3;
 constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
 
-// out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt).  nx >= 32
+// out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt) or,
+// with abi, the ABI's (a, b).  nx >= 32
 // of any remainder: the lanes of the last strip that lie past the row's end work on its periodic
 // image and store nothing.  A row holding a value that is not finite gives NaN wherever the strip
 // depends on it.
 template <int VARIANT>
 __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
-    k_kinetic2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks) {
+    k_kinetic2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks, bool abi) {
     constexpr int kRow = kStep2dWarpRowSites * 2;  // double2 of a row
     __shared__ double2 ring_all[kKin64Warps][kKin64Stages][kRow];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
             } else {
                 const FxToDouble to(E - 1022 - 58);
                 p2[0] = make_double2(to(xa.re), to(xa.im));
-                p2[1] = make_double2(to(xbt.re), to(xbt.im));
+                p2[1] = abi ? make_double2(to(xbt.im), to(-xbt.re)) : make_double2(to(xbt.re), to(xbt.im));
             }
         }
     }
