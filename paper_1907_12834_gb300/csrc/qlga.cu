@@ -962,9 +962,14 @@ struct BatchCand {
     int tile, threads, spt, steps;
 };
 constexpr int kBatchNumCands = 11;
-constexpr BatchCand kBatchCands[kBatchNumCands] = {
+// ... and two that advance a single FP32 lattice four or eight steps per launch, for lattices bound by the launches
+// (16384 sites: 2.57 us a step two at a time, 1.80 now; 1024 sites 1.46; both pick four or eight up to the
+// graphs' 262144 sites); the caller cannot ask for them.
+constexpr int kTileNumCands = kBatchNumCands + 2;
+constexpr BatchCand kBatchCands[kTileNumCands] = {
     {0, 32, 1, 1},  {1, 64, 1, 1},  {2, 128, 1, 1}, {3, 256, 1, 1}, {2, 64, 2, 1},  {3, 128, 2, 1},
-    {3, 64, 4, 1},  {5, 64, 4, 2},  {5, 128, 2, 2}, {4, 64, 2, 2},  {5, 256, 1, 2}};
+    {3, 64, 4, 1},  {5, 64, 4, 2},  {5, 128, 2, 2}, {4, 64, 2, 2},  {5, 256, 1, 2},
+    {-1, 128, 1, 4}, {-1, 128, 1, 8}};
 constexpr int kFixed1dCand = 0;       // the shape of the FP64 fixed-point kernel: 32 threads, one site each, one step
 constexpr int kBatchDefaultCand = 1;  // before tuning: 64 threads, one site each
 
@@ -1020,14 +1025,16 @@ void tile_launch_cand(const TileArgs& a, int ci) {
             case 8: tile_launch_shape<T, V, POT, 128, 2, 2>(a); return;
             case 9: tile_launch_shape<T, V, POT, 64, 2, 2>(a); return;
             case 10: tile_launch_shape<T, V, POT, 256, 1, 2>(a); return;
+            case 11: tile_launch_shape<T, V, POT, 128, 1, 4>(a); return;
+            case 12: tile_launch_shape<T, V, POT, 128, 1, 8>(a); return;
             default: break;
         }
     }
 }
 
-// Whether shape ci runs for this precision and kind of launch (two-step shapes: FP32 fused steps).
+// Whether shape ci runs for this precision and kind of launch (shapes of several steps: FP32 fused steps).
 inline bool tile_cand_ok(int precision, bool pot, int ci) {
-    return ci >= 0 && ci < kBatchNumCands && (kBatchCands[ci].steps == 1 || (precision == 32 && pot));
+    return ci >= 0 && ci < kTileNumCands && (kBatchCands[ci].steps == 1 || (precision == 32 && pot));
 }
 
 // Launch k_batch_step with shape ci (errors left in cudaGetLastError()); ci must pass
@@ -1060,7 +1067,7 @@ struct qlga_handle {
     int64_t step;
     int64_t launches;  // kernels launched by this handle
     int tile_cand;  // 1D: launch shape of the tiled step (index into kBatchCands), -1 untuned
-    int tile_cand2;  // 1D: two-step shape when it beats tile_cand per step, else -1
+    int tile_cand2;  // 1D: shape of several steps per launch when it beats tile_cand per step, else -1
     int tile_lanes;   // 1D: fused steps by the lane-parallel kernel with 5 or 10 lanes per site, 0: not
     bool tile_fixed;  // 1D FP64: no forced shape, steps by the fixed-point kernel (reported as kFixed1dCand's shape)
     int step2d_mode;  // QLGA_STEP2D_AUTO / _FUSED / _TWO_PASS
@@ -1287,14 +1294,14 @@ cudaError_t time_per_step(cudaStream_t stream, cudaStream_t cs, bool graphed, in
     return e;
 }
 
-// Times the launch shapes of the tiled kernel (launch(ci, stream, k): launch k of shape ci) with
+// Times the first `cands` launch shapes of the tiled kernel (launch(ci, stream, k): launch k of shape ci) with
 // time_per_step and compares the time per step.  best1 is the fastest one-step shape (its time
-// in *t1); best2 the fastest two-step shape if `two_step` allows them and it beats best1 per step,
+// in *t1); best2 the fastest shape of several steps if `two_step` allows them and it beats best1 per step,
 // else -1 (*t2 its time, or a large value).  Every shape is timed in kTuneRounds rounds over all
 // shapes and keeps its best time, so that one disturbed timing does not decide the choice (single
 // rounds picked shapes 7% apart on the same 16384-site lattice from run to run).
 template <class Launch>
-cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch&& launch, int* best1, int* best2) {
+cudaError_t tune_shapes(cudaStream_t stream, int cands, bool two_step, bool graphed, Launch&& launch, int* best1, int* best2) {
     EventPair ev;
     cudaError_t e = ev.create();
     cudaStream_t cs = nullptr;
@@ -1302,24 +1309,24 @@ cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch
     float t1 = 1e30f, t2 = 1e30f;
     *best1 = kBatchDefaultCand;
     *best2 = -1;
-    float best_ms[kBatchNumCands];
-    for (int ci = 0; ci < kBatchNumCands; ++ci) best_ms[ci] = 1e30f;
+    float best_ms[kTileNumCands];
+    for (int ci = 0; ci < cands; ++ci) best_ms[ci] = 1e30f;
     for (int round = 0; round < kTuneRounds && e == cudaSuccess; ++round) {
-        for (int ci = 0; ci < kBatchNumCands && e == cudaSuccess; ++ci) {
+        for (int ci = 0; ci < cands && e == cudaSuccess; ++ci) {
             const int steps = kBatchCands[ci].steps;
-            if (steps == 2 && !two_step) continue;
+            if (steps > 1 && !two_step) continue;
             float ms = 0.f;
             e = time_per_step(stream, cs, graphed, steps, ev, [&](cudaStream_t st, int k) { launch(ci, st, k); }, &ms);
             if (e == cudaSuccess && ms < best_ms[ci]) best_ms[ci] = ms;
         }
     }
-    for (int ci = 0; ci < kBatchNumCands && e == cudaSuccess; ++ci) {
+    for (int ci = 0; ci < cands && e == cudaSuccess; ++ci) {
         const int steps = kBatchCands[ci].steps;
-        if (steps == 2 && !two_step) continue;
+        if (steps > 1 && !two_step) continue;
         if (steps == 1 && best_ms[ci] < t1) {
             t1 = best_ms[ci];
             *best1 = ci;
-        } else if (steps == 2 && best_ms[ci] < t2) {
+        } else if (steps > 1 && best_ms[ci] < t2) {
             t2 = best_ms[ci];
             *best2 = ci;
         }
@@ -1330,11 +1337,11 @@ cudaError_t tune_shapes(cudaStream_t stream, bool two_step, bool graphed, Launch
 }
 
 // Number of kernel launches tune_shapes issues.
-inline int tune_launches(bool two_step, bool graphed) {
+inline int tune_launches(int cands, bool two_step, bool graphed) {
     int n = 0;
-    for (int ci = 0; ci < kBatchNumCands; ++ci) {
+    for (int ci = 0; ci < cands; ++ci) {
         const int steps = kBatchCands[ci].steps;
-        if (steps == 2 && !two_step) continue;
+        if (steps > 1 && !two_step) continue;
         n += graphed ? 4 * (kTuneGraphSteps / steps) : 3;
     }
     return kTuneRounds * n;
@@ -1412,7 +1419,9 @@ qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int ste
             b.in = (k & 1) ? out : h->tmp;
             b.out = (k & 1) ? h->tmp : out;
         };
-        cudaError_t e = tune_shapes(h->stream, two, graphed,
+        // lattices stepped without graphs are too large to gain from more than two steps per launch
+        const int cands = graphed ? kTileNumCands : kBatchNumCands;
+        cudaError_t e = tune_shapes(h->stream, cands, two, graphed,
                                     [&](int ci, cudaStream_t st, int k) {
                                         TileArgs b = a;
                                         alternate(b, st, k);
@@ -1420,7 +1429,7 @@ qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int ste
                                     },
                                     &h->tile_cand, &h->tile_cand2);
         if (e != cudaSuccess) return cuda_fail(e, "1D step tuning");
-        h->launches += tune_launches(two, graphed);
+        h->launches += tune_launches(cands, two, graphed);
     }
     if (pot && steps == 1 && h->tile_lanes) {
         lanes_1d_launch(a, h->tile_lanes);
@@ -1428,7 +1437,7 @@ qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int ste
         h->launches += 1;
         return QLGA_OK;
     }
-    const int ci = steps == 2 ? h->tile_cand2 : (h->tile_cand >= 0 ? h->tile_cand : kBatchDefaultCand);
+    const int ci = steps > 1 ? h->tile_cand2 : (h->tile_cand >= 0 ? h->tile_cand : kBatchDefaultCand);
     if (!tile_cand_ok(h->cfg.precision, pot, ci)) return fail(QLGA_ERR_INVALID_ARG, "no launch shape for this 1D step%s");
     tile_step_launch(a, ci);
     QLGA_CUDA(cudaGetLastError(), "k_batch_step launch (1D)");
@@ -1436,9 +1445,9 @@ qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int ste
     return QLGA_OK;
 }
 
-// Whether the next fused steps of this handle can go two per launch (1D FP32, tuned or forced).
-bool two_step_1d(const qlga_handle* h) {
-    return h->cfg.ndim == 1 && !h->cfg.interleave && h->pending_k && h->tile_cand2 >= 0;
+// Steps per launch of this handle's next fused steps (1D FP32, tuned or forced; else 1).
+int steps_per_launch_1d(const qlga_handle* h) {
+    return h->cfg.ndim == 1 && !h->cfg.interleave && h->pending_k && h->tile_cand2 >= 0 ? kBatchCands[h->tile_cand2].steps : 1;
 }
 
 // The 2D kernel form of this handle's steps (see qlga_set_step2d_mode).
@@ -1585,15 +1594,16 @@ qlga_status graph_steps_launch(qlga_handle* h) {
         if (e == cudaSuccess) {
             h->stream = cs;
             int c = h->cur;
-            // two fused steps per launch where the handle has them (1D FP32), with an even number
+            // several fused steps per launch where the handle has them (1D FP32), with an even number
             // of launches so that the graph ends on the buffer it starts from
-            const int gs = h->graph_steps;
-            const int twos = two_step_1d(h) ? (gs % 4 == 0 ? gs / 2 : (gs - 2) / 2) : 0;
-            for (int k = 0; k < twos && s == QLGA_OK; ++k) {
-                s = tile_1d(h, h->X[c], h->X[1 - c], true, 2);
+            const int gs = h->graph_steps, per = steps_per_launch_1d(h);
+            int many = per > 1 ? gs / per : 0;
+            if (many > 0 && (many + gs - per * many) % 2) --many;
+            for (int k = 0; k < many && s == QLGA_OK; ++k) {
+                s = tile_1d(h, h->X[c], h->X[1 - c], true, per);
                 c ^= 1;
             }
-            for (int k = 2 * twos; k < gs && s == QLGA_OK; ++k) {
+            for (int k = per * many; k < gs && s == QLGA_OK; ++k) {
                 s = kinetic_into(h, h->X[c], h->X[1 - c], h->tmp, true);
                 c ^= 1;
             }
@@ -1877,12 +1887,13 @@ qlga_status qlga_step(qlga_handle* h, int64_t n) {
             i += h->graph_steps - 1;
             continue;
         }
-        if (two_step_1d(h) && n - i >= 2) {  // two fused steps in one launch
-            s = tile_1d(h, h->X[h->cur], h->X[1 - h->cur], true, 2);
+        const int per = steps_per_launch_1d(h);
+        if (per > 1 && n - i >= per) {  // several fused steps in one launch
+            s = tile_1d(h, h->X[h->cur], h->X[1 - h->cur], true, per);
             if (s != QLGA_OK) return s;
             h->cur ^= 1;
-            h->step += 2;
-            ++i;
+            h->step += per;
+            i += per - 1;
             continue;
         }
         if (h->cfg.interleave) {
@@ -2662,7 +2673,7 @@ qlga_status batch_tune(qlga_batch* b) {
     void* other = b->X[1 - b->cur];
     QLGA_CUDA(cudaMemcpyAsync(b->tmp, b->X[b->cur], batch_state_bytes_of(b->precision, b->total_sites),
                               cudaMemcpyDeviceToDevice, b->stream), "batch tuning copy");
-    cudaError_t e = tune_shapes(b->stream, two, b->use_graph,
+    cudaError_t e = tune_shapes(b->stream, kBatchNumCands, two, b->use_graph,
                                 [&](int ci, cudaStream_t st, int k) {
                                     cudaStream_t saved = b->stream;
                                     b->stream = st;

@@ -102,9 +102,10 @@ __device__ __forceinline__ void batch_kinetic_at(const Pair4<T>* src, int stride
 // operator alone the true state (a, bt).  A CTA of W threads computes W * SPT consecutive sites of one run per pass
 // (thread t owns sites t, t + W, ...).  The tile and its periodic halo of 4 * STEPS sites on
 // each side are staged in shared memory with 16-byte cp.async copies, all in flight at once.
-// STEPS = 2 (temporal blocking): the first step covers the tile and 4 halo sites per side, into
-// a second shared buffer; the second step reads that buffer.  The tile is then W * SPT - 8
-// sites wide, so both passes fill the threads; the state is read and written once per two
+// STEPS = 2, 4, 8 (temporal blocking): the first step covers the tile and 4 (STEPS - 1) halo sites per side,
+// into a second shared buffer; each further step reads one buffer and covers 4 sites per side
+// less.  The tile is W * SPT - 8 (STEPS - 1)
+// sites wide, so that the first pass fills the threads; the state is read and written once per STEPS
 // steps, each site's arithmetic unchanged.
 // tiles == nullptr: one 1D lattice of single_L sites with constants single_pc; tile b starts at
 // site b * (tile width), and no table is read.
@@ -115,12 +116,12 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
                                                    const PotConst<T>* __restrict__ consts,
                                                    unsigned* status, int single_L,
                                                    PotConst<T> single_pc, bool abi) {
-    static_assert(STEPS == 1 || (STEPS == 2 && POT), "two steps per launch are fused steps");
+    static_assert(STEPS == 1 || POT, "several steps per launch are fused steps");
     constexpr int TW = W * SPT;                  // sites per pass
     constexpr int TOUT = TW - 8 * (STEPS - 1);   // output sites of a tile
     constexpr int H = 4 * STEPS;                 // staged halo per side: TOUT + 2 H = TW + 8
     __shared__ __align__(16) Pair4<T> sm[5][TW + 8];  // 16-byte aligned for cp.async
-    __shared__ __align__(16) Pair4<T> mid[5][STEPS == 2 ? TW : 1];
+    __shared__ __align__(16) Pair4<T> mid[5][STEPS > 1 ? TW : 1];
     const bool single = tiles == nullptr;
     const BatchTile tile = single ? BatchTile{0, int(blockIdx.x) * TOUT} : tiles[blockIdx.x];
     const BatchRun run = single ? BatchRun{0, single_L, 1} : runs[tile.run];
@@ -149,28 +150,42 @@ __global__ void __launch_bounds__(W) k_batch_step(const T* __restrict__ in, T* _
     cp_async_wait<0>();
     __syncthreads();
     const PotConst<T> C = single ? single_pc : consts[tile.run];
-    if constexpr (STEPS == 2) {
-        // first step on columns 0 .. TW - 1 of mid: sites start - 4 .. start + TOUT + 3
+    // steps before the last: step i reads columns 0 .. TW + 7 - 8 i of one buffer and writes 0 .. TW - 1 - 8 i of
+    // the other, the sites start - H + 4 (i + 1) and on
+#pragma unroll 1
+    for (int i = 0; i + 1 < STEPS; ++i) {
+        const bool even = (i & 1) == 0;
+        const Pair4<T>* from = even ? &sm[0][0] : &mid[0][0];
+        Pair4<T>* to = even ? &mid[0][0] : &sm[0][0];
+        const int from_stride = even ? TW + 8 : TW, to_stride = even ? TW : TW + 8;
+        const int width = TW - 8 * i;
 #pragma unroll 1
         for (int k = 0; k < SPT; ++k) {
-            const int p = t + k * W;
+            const int pt = t + k * W;
+            if (STEPS > 2 && (pt & ~31) >= width) break;  // whole warp
+            // lanes past the last column redo it and store nothing
+            const int p = STEPS > 2 && pt >= width ? width - 1 : pt;
             cpx<T> oa[5], ob[5];
-            batch_kinetic_at<T, VARIANT>(&sm[0][0], TW + 8, p, oa, ob);
+            batch_kinetic_at<T, VARIANT>(from, from_stride, p, oa, ob);
             // d takes the degree of psi: one warp-uniform Horner loop (2-3% faster than a per-lane
             // degree for d on the 1D scattering batches and on config 1)
             potential_site<T, false>(oa, ob, C, T(1.0 / 256.0), T(0.5 / 16.0), status);
+            if (STEPS > 2 && pt >= width) continue;
 #pragma unroll
             for (int m = 0; m < 5; ++m)  // held pending K, as (P, Q)
-                mid[m][p] = Pair4<T>{{oa[m].re - ob[m].im, oa[m].im + ob[m].re, oa[m].re + ob[m].im, oa[m].im - ob[m].re}};
+                to[m * to_stride + p] = Pair4<T>{{oa[m].re - ob[m].im, oa[m].im + ob[m].re, oa[m].re + ob[m].im, oa[m].im - ob[m].re}};
         }
         __syncthreads();
     }
-    const Pair4<T>* src = STEPS == 2 ? &mid[0][0] : &sm[0][0];
-    const int stride = STEPS == 2 ? TW : TW + 8;
+    // an even number of steps ends on mid
+    static_assert(STEPS == 1 || STEPS % 2 == 0, "the last step reads mid");
+    const Pair4<T>* src = STEPS > 1 ? &mid[0][0] : &sm[0][0];
+    const int stride = STEPS > 1 ? TW : TW + 8;
 #pragma unroll 1
     for (int k = 0; k < SPT; ++k) {
         const int tt = t + k * W;
-        // positions past the tile's output (STEPS = 2: the last 8) redo a valid site and store nothing
+        // positions past the tile's output (the last 8 (STEPS - 1)) redo a valid site and store nothing
+        if (STEPS > 2 && (tt & ~31) >= TOUT) break;  // whole warp
         const int p = tt < TOUT ? tt : TOUT - 1;
         const int j = tile.start + tt;
         cpx<T> oa[5], ob[5];
