@@ -32,7 +32,7 @@
 #include "qlga_step2d.cuh"
 #include "qlga_batch1d.cuh"
 #include "qlga_lanes1d.cuh"
-#include "qlga_adjoint.cuh"
+#include "qlga_adjoint_kernel.cuh"
 #include "qlga_interleave.cuh"
 #include "qlga_step2d_f64.cuh"
 #include "qlga_step1d_f64.cuh"
