@@ -1294,6 +1294,12 @@ cudaError_t time_per_step(cudaStream_t stream, cudaStream_t cs, bool graphed, in
     return e;
 }
 
+// Whether the tuner times a shape: several steps per launch where they are allowed, and four sites per thread not
+// for a single graphed lattice (`small`), which has too few sites to want them.
+inline bool tuned_shape(int ci, bool two_step, bool small) {
+    return (kBatchCands[ci].steps == 1 || two_step) && !(small && kBatchCands[ci].spt == 4);
+}
+
 // Times the first `cands` launch shapes of the tiled kernel (launch(ci, stream, k): launch k of shape ci) with
 // time_per_step and compares the time per step.  best1 is the fastest one-step shape (its time
 // in *t1); best2 the fastest shape of several steps if `two_step` allows them and it beats best1 per step,
@@ -1314,7 +1320,7 @@ cudaError_t tune_shapes(cudaStream_t stream, int cands, bool two_step, bool grap
     for (int round = 0; round < kTuneRounds && e == cudaSuccess; ++round) {
         for (int ci = 0; ci < cands && e == cudaSuccess; ++ci) {
             const int steps = kBatchCands[ci].steps;
-            if (steps > 1 && !two_step) continue;
+            if (!tuned_shape(ci, two_step, cands > kBatchNumCands)) continue;
             float ms = 0.f;
             e = time_per_step(stream, cs, graphed, steps, ev, [&](cudaStream_t st, int k) { launch(ci, st, k); }, &ms);
             if (e == cudaSuccess && ms < best_ms[ci]) best_ms[ci] = ms;
@@ -1322,7 +1328,7 @@ cudaError_t tune_shapes(cudaStream_t stream, int cands, bool two_step, bool grap
     }
     for (int ci = 0; ci < cands && e == cudaSuccess; ++ci) {
         const int steps = kBatchCands[ci].steps;
-        if (steps > 1 && !two_step) continue;
+        if (!tuned_shape(ci, two_step, cands > kBatchNumCands)) continue;
         if (steps == 1 && best_ms[ci] < t1) {
             t1 = best_ms[ci];
             *best1 = ci;
@@ -1341,7 +1347,7 @@ inline int tune_launches(int cands, bool two_step, bool graphed) {
     int n = 0;
     for (int ci = 0; ci < cands; ++ci) {
         const int steps = kBatchCands[ci].steps;
-        if (steps > 1 && !two_step) continue;
+        if (!tuned_shape(ci, two_step, cands > kBatchNumCands)) continue;
         n += graphed ? 4 * (kTuneGraphSteps / steps) : 3;
     }
     return kTuneRounds * n;
