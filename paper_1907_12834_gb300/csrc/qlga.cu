@@ -1579,16 +1579,32 @@ qlga_status true_state_view(qlga_handle* h, const void** view) {
     return s;
 }
 
-qlga_status check_status_word(qlga_handle* h) {
-    unsigned st = 0;
-    QLGA_CUDA(cudaMemcpyAsync(&st, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream), "status read");
-    QLGA_CUDA(cudaStreamSynchronize(h->stream), "stream sync");
+qlga_status judge_status(qlga_handle* h, unsigned st) {
     if (st & 1u) {
         cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream);
         return fail(QLGA_ERR_NOT_FINITE,
                     "the potential exponent ||delta (V - c)|| exceeded 4 or was not finite: the "
                     "field is too large for the lattice scaling (use a smaller epsilon)%s");
     }
+    return QLGA_OK;
+}
+
+qlga_status check_status_word(qlga_handle* h) {
+    unsigned st = 0;
+    QLGA_CUDA(cudaMemcpyAsync(&st, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream), "status read");
+    QLGA_CUDA(cudaStreamSynchronize(h->stream), "stream sync");
+    return judge_status(h, st);
+}
+
+// The first n results and the status word behind them (init_handle) in one copy and one wait: each of them
+// costs a read-out about 10 us.
+constexpr size_t kResultBytes = (sizeof(double) * OBS_COUNT + 255) & ~size_t(255);  // align256
+qlga_status read_results(qlga_handle* h, double* o, int n, unsigned* st) {
+    unsigned char buf[kResultBytes + sizeof(unsigned)];
+    QLGA_CUDA(cudaMemcpyAsync(buf, h->obs_dev, sizeof(buf), cudaMemcpyDeviceToHost, h->stream), "results copy");
+    QLGA_CUDA(cudaStreamSynchronize(h->stream), "results sync");
+    std::memcpy(o, buf, sizeof(double) * n);
+    std::memcpy(st, buf + kResultBytes, sizeof(unsigned));
     return QLGA_OK;
 }
 
@@ -1760,7 +1776,7 @@ static qlga_status init_handle(qlga_handle* h, const qlga_config* cfg, void* str
     h->partials = reinterpret_cast<double*>(w);
     w += align256(sizeof(double) * kObsMaxBlocks * OBS_COUNT);
     h->obs_dev = reinterpret_cast<double*>(w);
-    w += align256(sizeof(double) * OBS_COUNT);
+    w += kResultBytes;  // read_results copies the results and the status word at once
     h->status = reinterpret_cast<unsigned*>(w);
     h->cur = 0;
     h->pending_k = false;
@@ -2042,10 +2058,11 @@ qlga_status qlga_observables(qlga_handle* h, const void* ref_state_device, qlga_
     QLGA_CUDA(cudaGetLastError(), "k_reduce_partials launch");
     h->launches += 1;
     double o[OBS_COUNT];
-    QLGA_CUDA(cudaMemcpyAsync(o, h->obs_dev, sizeof(o), cudaMemcpyDeviceToHost, h->stream), "observables copy");
-    QLGA_CUDA(cudaStreamSynchronize(h->stream), "observables sync");
+    unsigned st = 0;
+    s = read_results(h, o, OBS_COUNT, &st);
+    if (s != QLGA_OK) return s;
     fill_obs(o, h->step, out);
-    s = check_status_word(h);
+    s = judge_status(h, st);
     if (s != QLGA_OK) return s;
     if (!std::isfinite(out->norm_qubit) || !std::isfinite(out->energy))
         return fail(QLGA_ERR_NOT_FINITE, "the state holds NaN or Inf%s");
@@ -2063,10 +2080,9 @@ qlga_status qlga_observable_sums(qlga_handle* h, int64_t y0, int64_t y1, const v
     k_reduce_partials<<<OBS_COUNT, kReduceThreads, 0, h->stream>>>(partials, rows, OBS_COUNT, h->obs_dev);
     QLGA_CUDA(cudaGetLastError(), "k_reduce_partials launch");
     h->launches += 1;
-    QLGA_CUDA(cudaMemcpyAsync(sums, h->obs_dev, sizeof(double) * OBS_COUNT, cudaMemcpyDeviceToHost, h->stream),
-              "observable sums copy");
-    QLGA_CUDA(cudaStreamSynchronize(h->stream), "observable sums sync");
-    return check_status_word(h);
+    unsigned st = 0;
+    s = read_results(h, sums, OBS_COUNT, &st);
+    return s == QLGA_OK ? judge_status(h, st) : s;
 }
 
 qlga_status qlga_obs_from_sums(const double* sums, int64_t step, qlga_obs* out) {
@@ -2348,7 +2364,6 @@ struct AdjLayout {
     void* w1;
     void* w2;
     double* partials;
-    double* result;
     char* ckpt;
     char* slots;
     size_t state;
@@ -2373,7 +2388,7 @@ AdjLayout adj_layout(const qlga_config& c, int64_t n, int64_t C, void* base) {
     L.w1 = take(L.state);
     L.w2 = take(L.state);
     L.partials = reinterpret_cast<double*>(take(sizeof(double) * 3 * kAdjMaxBlocks));
-    L.result = reinterpret_cast<double*>(take(sizeof(double) * 3));
+    take(sizeof(double) * 3);  // unused: the sums go to the handle's results
     L.ckpt = take(L.state * size_t(L.nck));
     L.slots = take(L.state * size_t(L.nslots));
     L.total = off;
@@ -2433,17 +2448,18 @@ qlga_status adj_pullback(qlga_handle* h, void** cot, void** tmp, const void* xk,
 }
 
 qlga_status adj_finish(qlga_handle* h, const AdjLayout& L, void* cot_res, void* cot_dev, double* dcoup) {
-    k_reduce_partials<<<3, kReduceThreads, 0, h->stream>>>(L.partials, kAdjMaxBlocks, 3, L.result);
+    k_reduce_partials<<<3, kReduceThreads, 0, h->stream>>>(L.partials, kAdjMaxBlocks, 3, h->obs_dev);
     QLGA_CUDA(cudaGetLastError(), "k_reduce_partials launch (adjoint)");
     h->launches += 1;
     qlga_status s = launch_convert(h, cot_res, cot_dev, false);
     if (s != QLGA_OK) return s;
     double d[3];
-    QLGA_CUDA(cudaMemcpyAsync(d, L.result, sizeof(d), cudaMemcpyDeviceToHost, h->stream), "adjoint result copy");
-    QLGA_CUDA(cudaStreamSynchronize(h->stream), "adjoint sync");
+    unsigned st = 0;
+    s = read_results(h, d, 3, &st);
+    if (s != QLGA_OK) return s;
     if (dcoup)
         for (int i = 0; i < 3; ++i) dcoup[i] = d[i];
-    return check_status_word(h);
+    return judge_status(h, st);
 }
 
 }  // namespace
