@@ -32,6 +32,7 @@
 #include "qlga_step2d.cuh"
 #include "qlga_batch1d.cuh"
 #include "qlga_lanes1d.cuh"
+#include "qlga_adjoint2d_f64.cuh"
 #include "qlga_adjoint_kernel.cuh"
 #include "qlga_interleave.cuh"
 #include "qlga_step2d_f64.cuh"
@@ -2432,6 +2433,23 @@ qlga_status adj_axis(qlga_handle* h, const void* gin, void* gout, const void* X,
     return QLGA_OK;
 }
 
+// FP64 on a 2D lattice of at least 32 columns: K^dagger in integer fixed point, then the pull-back through U.
+template <int V>
+qlga_status adj_pullback2d_f64(qlga_handle* h, const double* cot, double* tmp, double* out, const double* xk, double* partials) {
+    Step2dDevice dv;
+    if (step2d_device(&dv)) return cuda_fail(cudaGetLastError(), "2D adjoint set-up");
+    const int64_t nx = h->cfg.nx, ny = h->cfg.ny, strips = step2d_strips(nx);
+    const int chunks = step2d_level_chunks(strips, ny, dv.sms, std::max(1, kAdj64Ctas * kKin64Warps / 5), [](double rows) { return rows + 7.0; });
+    k_adjoint2d_f64<V><<<int((5 * strips * chunks + kKin64Warps - 1) / kKin64Warps), 32 * kKin64Warps, 0, h->stream>>>(cot, tmp, int(nx), int(ny), chunks);
+    QLGA_CUDA(cudaGetLastError(), "k_adjoint2d_f64 launch");
+    const int blocks = grid_for_block(nsites_of(h->cfg), kAdjThreads, std::min(kAdjMaxBlocks, 8 * device_sms()));
+    k_adjoint_axis<double, V, true, true><<<blocks, kAdjThreads, 0, h->stream>>>(tmp, out, xk, nx, ny, 0, AdjConst<double>(pot_params(h->cfg, 1.0)),
+                                                                             partials, h->status);
+    QLGA_CUDA(cudaGetLastError(), "k_adjoint_axis launch");
+    h->launches += 2;
+    return QLGA_OK;
+}
+
 // cot <- (d step / d x at x_k)^T cot.  The cotangent lives in *cot; 1D swaps it with *tmp.
 qlga_status adj_pullback(qlga_handle* h, void** cot, void** tmp, const void* xk, double* partials) {
     qlga_status s;
@@ -2440,6 +2458,11 @@ qlga_status adj_pullback(qlga_handle* h, void** cot, void** tmp, const void* xk,
         if (s != QLGA_OK) return s;
         std::swap(*cot, *tmp);
         return QLGA_OK;
+    }
+    if (h->cfg.precision == 64 && step2d_strips_supported(h->cfg.nx, h->cfg.ny)) {
+        double *c = static_cast<double*>(*cot), *t = static_cast<double*>(*tmp);
+        const double* x = static_cast<const double*>(xk);
+        return h->cfg.kinetic_variant == 0 ? adj_pullback2d_f64<0>(h, c, t, c, x, partials) : adj_pullback2d_f64<1>(h, c, t, c, x, partials);
     }
     // K = K_y K_x, so K^dagger = K_x^dagger K_y^dagger: y first, then x with the pull-back of U
     s = adj_axis(h, *cot, *tmp, xk, 1, false, partials);

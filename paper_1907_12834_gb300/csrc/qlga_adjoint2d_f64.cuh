@@ -1,0 +1,193 @@
+// qlga_adjoint2d_f64.cuh -- K^dagger of a 2D FP64 lattice in integer fixed point, both axes in one pass.
+//
+// The adjoint of k_kinetic2d_f64 (qlga_step2d_f64.cuh): warp strips of one level that march along y.  K = K_y K_x, so
+// y comes first here: each lane runs the four adjoint blocks of y as a register pipeline on its column, lanes 0
+// to 7 also on the eight columns beyond, the row goes to shared memory, and the adjoint nine-point stencil
+// of x reads it there.  The FP64 form was two passes of 320 FP64 instructions a site (66 cycles each): 106 us at 256^2, 27 here.
+//
+// Numbers.  As there, with components below 2^56 after conversion: the y blocks' taps (at most 44 in magnitude) keep
+// below 2^62, are rounded to 2^-6 of that, and the x stencil's sums are 2^58 times the true K^dagger g.
+#pragma once
+
+#include "qlga_adjoint.cuh"
+#include "qlga_step2d_f64.cuh"
+
+namespace qlga {
+
+// One adjoint block C^dagger S_c C'^dagger S_c^T along y for one component (make_stencil_adjoint has the same
+// factors): input row n -> output row n - 1; yo: the other qubit of the previous row, wc: the shifted qubit after the
+// first collide of the previous row.
+template <int C, int FIRST>
+__device__ __forceinline__ void stream_adj_int(i64& a, i64& bt, i64& yo, i64& wc) {
+    const i64 ya = C == 1 ? yo : a, yb = C == 1 ? bt : yo;
+    yo = C == 1 ? a : bt;
+    const i64 wa = ya - yb, wb = ya + yb;
+    const i64 za = C == 1 ? wa : wc, zb = C == 1 ? wc : wb;
+    wc = C == 1 ? wb : wa;
+    a = FIRST == 0 ? za - zb : za + zb;
+    bt = FIRST == 0 ? za + zb : zb - za;
+}
+
+struct AdjColumn {
+    cpi yo[4], wc[4];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) yo[k] = wc[k] = {0, 0};
+    }
+    __device__ __forceinline__ void scale(int n) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            yo[k] = {fx_scale(yo[k].re, n), fx_scale(yo[k].im, n)};
+            wc[k] = {fx_scale(wc[k].re, n), fx_scale(wc[k].im, n)};
+        }
+    }
+    template <int VARIANT>
+    __device__ __forceinline__ void push(longlong2& a, longlong2& bt) {
+        static_for<4>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value, c = kk < 2 ? 0 : 1;  // the blocks of qubit 1 first
+            stream_adj_int<c, VARIANT>(a.x, bt.x, yo[kk].re, wc[kk].re);
+            stream_adj_int<c, VARIANT>(a.y, bt.y, yo[kk].im, wc[kk].im);
+        });
+        auto down = [](i64 v) { return (v + 32) >> 6; };
+        a = make_longlong2(down(a.x), down(a.y));
+        bt = make_longlong2(down(bt.x), down(bt.y));
+    }
+};
+
+constexpr int kAdj64Ctas = 4;  // resident per SM, of kKin64Warps warps
+
+// out = K^dagger in, both in the resident layout (a, bt); strips, chunks and values that are not finite as in
+// k_kinetic2d_f64.
+template <int VARIANT>
+__global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
+    k_adjoint2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks) {
+    constexpr KinStencil S = kStencilAdj[VARIANT];
+    constexpr int kRow = kStep2dWarpRowSites * 2;  // double2 of a row
+    __shared__ double2 ring_all[kKin64Warps][kKin64Stages][kRow];
+    __shared__ longlong2 yrow_all[kKin64Warps][kRow];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int strips = (nx + kStep2dWarpCols - 1) / kStep2dWarpCols;
+    const int64_t gw = int64_t(blockIdx.x) * kKin64Warps + w;
+    if (gw >= 5 * int64_t(strips) * chunks) return;  // whole warp: no block-wide barrier follows
+    const int m = int(gw % 5);
+    const int strip = int(gw / 5) % strips, chunk = int(gw / 5) / strips;
+    const int x0 = strip * kStep2dWarpCols;
+    const int y_begin = int((int64_t(chunk) * ny) / chunks);
+    const int y_end = int((int64_t(chunk + 1) * ny) / chunks);
+    const int64_t nsites = int64_t(nx) * ny;
+    const double2* level = reinterpret_cast<const double2*>(in) + 2 * (m * nsites);
+    double2* out2 = reinterpret_cast<double2*>(out) + 2 * (m * nsites);
+    double2(*ring)[kRow] = ring_all[w];
+    longlong2* yrow = yrow_all[w];
+
+    const int nrows = (y_end - y_begin) + 8;
+    auto wrap_x = [&](int x) {  // x < nx + 36 < 3 nx
+        x = x < 0 ? x + nx : x;
+        x = x >= nx ? x - nx : x;
+        return x >= nx ? x - nx : x;
+    };
+    const int xm = wrap_x(x0 - kStep2dHalo + lane);
+    const int xh = wrap_x(x0 + kStep2dWarpCols - kStep2dHalo + lane);
+    int y_in = y_begin - kStep2dHalo, issued = 0;
+    y_in = y_in < 0 ? y_in + ny : y_in;
+    auto issue_row = [&]() {  // the next row, if there is one
+        if (issued < nrows) {
+            double2* d = ring[issued % kKin64Stages] + 2 * lane;
+            const double2* g = level + 2 * (int64_t(y_in) * nx + xm);
+            cp_async_16(d, g);
+            cp_async_16(d + 1, g + 1);
+            if (lane < 2 * kStep2dHalo) {
+                const double2* h = level + 2 * (int64_t(y_in) * nx + xh);
+                cp_async_16(d + 2 * kStep2dWarpCols, h);
+                cp_async_16(d + 2 * kStep2dWarpCols + 1, h + 1);
+            }
+            y_in = y_in + 1 == ny ? 0 : y_in + 1;
+            ++issued;
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int r = 0; r < kKin64Stages - 1; ++r) issue_row();
+
+    AdjColumn own, beyond;
+    own.clear();
+    beyond.clear();
+    int E = kFxMinExp;                              // the pipelines' exponent
+    int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
+    int bad_until = -1;                             // rows up to here depend on one that is not finite
+
+#pragma unroll 1
+    for (int r = 0; r < nrows; ++r) {
+        cp_async_wait<kKin64Stages - 2>();
+        __syncwarp();
+        issue_row();
+
+        double2* row = ring[r % kKin64Stages];
+        const double2 own0 = row[2 * lane], own1 = row[2 * lane + 1];
+        double2* tail = row + 2 * kStep2dWarpCols;  // columns 32..39: the lane's component
+        const double halo = reinterpret_cast<const double*>(tail)[lane];
+        auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
+        const unsigned top = max(max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y))), hi(halo));
+        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, top));
+        const bool bad = Er > kKin64MaxExp;
+        if (bad) {
+            Er = kFxMinExp;
+            bad_until = r + 8;
+        }
+        if ((r & 7) == 0) {
+            seen_before = seen;
+            seen = kFxMinExp;
+        }
+        seen = max(seen, Er);
+        const int En = max(seen, seen_before);
+        if (En != E) {  // warp-uniform, rare on smooth fields
+            const int n = max(E - En, -63);
+            own.scale(n);
+            beyond.scale(n);
+            E = En;
+        }
+        longlong2 a = make_longlong2(0, 0), bt = a;
+        if (!bad) {
+            a = make_longlong2(fx_from_double<56>(own0.x, E), fx_from_double<56>(own0.y, E));
+            bt = make_longlong2(fx_from_double<56>(own1.x, E), fx_from_double<56>(own1.y, E));
+        }
+        reinterpret_cast<i64*>(tail)[lane] = bad ? 0 : fx_from_double<56>(halo, E);
+        __syncwarp();  // also: the last row's stencil has read yrow
+        own.push<VARIANT>(a, bt);
+        yrow[2 * lane] = a;
+        yrow[2 * lane + 1] = bt;
+        if (lane < 2 * kStep2dHalo) {
+            const longlong2* h = reinterpret_cast<const longlong2*>(tail) + 2 * lane;
+            longlong2 ha = h[0], hb = h[1];
+            beyond.push<VARIANT>(ha, hb);
+            yrow[2 * (kStep2dWarpCols + lane)] = ha;
+            yrow[2 * (kStep2dWarpCols + lane) + 1] = hb;
+        }
+        if (r < 8) continue;  // the pipelines fill
+        __syncwarp();
+        cpi xa = {0, 0}, xbt = {0, 0};
+        const longlong2* p = yrow + 2 * lane;
+        static_for<9>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value;
+            const longlong2 P = p[2 * kk], Q = p[2 * kk + 1];
+            xa.re = tap_int<S.g[0][1][kk]>(Q.x, tap_int<S.g[0][0][kk]>(P.x, xa.re));
+            xa.im = tap_int<S.g[0][1][kk]>(Q.y, tap_int<S.g[0][0][kk]>(P.y, xa.im));
+            xbt.re = tap_int<S.g[1][1][kk]>(Q.x, tap_int<S.g[1][0][kk]>(P.x, xbt.re));
+            xbt.im = tap_int<S.g[1][1][kk]>(Q.y, tap_int<S.g[1][0][kk]>(P.y, xbt.im));
+        });
+        if (x0 + lane < nx) {  // output row y_begin + r - 8
+            double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
+            if (r <= bad_until) {  // warp-uniform
+                const double nan = fx_bits(0x7ff80000u, 0u);
+                p2[0] = p2[1] = make_double2(nan, nan);
+            } else {
+                const FxToDouble to(E - 1022 - 58);
+                p2[0] = make_double2(to(xa.re), to(xa.im));
+                p2[1] = make_double2(to(xbt.re), to(xbt.im));
+            }
+        }
+    }
+    cp_async_wait<0>();
+}
+
+}  // namespace qlga

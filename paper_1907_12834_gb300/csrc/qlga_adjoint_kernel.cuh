@@ -58,7 +58,8 @@ __device__ __noinline__ void potential_vjp_f64(const cpx<double>* a, const cpx<d
 // stencil of one axis, optionally followed by the pull-back through U at the state X (resident,
 // the true state before U).  VJP: dL/dg of this launch is added to partials[block][3] (each block
 // owns its row, so repeated launches with the same grid accumulate deterministically).
-template <class T, int VARIANT, bool VJP>
+// LOCAL (with VJP): gin is K^dagger g already (k_adjoint2d_f64), and only the pull-back through U follows.
+template <class T, int VARIANT, bool VJP, bool LOCAL = false>
 // FP32: 4 resident CTAs per SM (128 registers, a few spilled) beat 3 at 168 registers by 12%.
 __global__ void __launch_bounds__(kAdjThreads, sizeof(T) == 4 ? 4 : 1) k_adjoint_axis(const T* __restrict__ gin, T* __restrict__ gout,
                                                               const T* __restrict__ X, int64_t nx, int64_t ny,
@@ -87,8 +88,9 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(T) == 4 ? 4 : 1) k_adjoint
             }
         }
         cpx<T> ga[5], gb[5];
+        if (LOCAL) SiteIO<T>::load(gin, nsites, s, ga, gb);
 #pragma unroll
-        for (int m = 0; m < 5; ++m) {
+        for (int m = 0; m < (LOCAL ? 0 : 5); ++m) {
             cpx<T> acc_a = {T(0), T(0)}, acc_bt = {T(0), T(0)};
             static_for<9>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;

@@ -50,3 +50,30 @@ def test_pull_back_domain(kind, g, nx, ny):
         got, dg = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
     assert np.linalg.norm(got.cpu().numpy() - ref) <= 1e-11 * np.linalg.norm(ref)
     assert np.abs(dg - dref).max() <= 1e-11 * max(np.abs(dref).max(), np.abs(cot).max() * np.abs(st).max() ** 3)
+
+
+# K^dagger alone (no couplings), at the ends of strips and chunks: 2e-15 of the largest component (one rounding of 2^-54 of the
+# strip's largest between the axes, amplified by at most 44/16, twice, and the conversions)
+@pytest.mark.parametrize("nx,ny,variant", [(32, 8, 0), (33, 9, 1), (63, 21, 0), (64, 8, 1), (95, 40, 0), (256, 67, 1), (31, 12, 0)])
+@pytest.mark.parametrize("rows", ["even", "jumps"])
+def test_kinetic_adjoint_strips(nx, ny, variant, rows):
+    rng = np.random.default_rng(nx + ny)
+    st = I.random_state(rng, nx, ny, scale=0.05)
+    cot = rng.standard_normal(st.shape)
+    if rows == "jumps":
+        cot *= 2.0 ** rng.integers(-40, 1, size=(1, ny, 1, 1, 1))
+    ref = cot.copy()
+    oracle.vjp_step(np.ascontiguousarray(st), ref, oracle.make_cfg(2, nx, ny, 0.0, 0.0, 0.0, kinetic_variant=variant))
+    with qlga.Lattice(2, nx, ny, precision=64, g=(0.0, 0.0, 0.0), kinetic_variant=variant) as lat:
+        got, _ = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
+    assert np.abs(got.cpu().numpy() - ref).max() <= 2e-15 * np.abs(ref).max()
+
+
+def test_nan_cotangent_stays_visible():
+    nx, ny = 70, 20
+    rng = np.random.default_rng(4)
+    st, cot = I.random_state(rng, nx, ny, scale=0.05), rng.standard_normal((5, ny, nx, 2, 2))
+    cot[1, 9, 40, 0, 1] = np.nan
+    with qlga.Lattice(2, nx, ny, precision=64, g=(1.0, 0.1, 1.0)) as lat:
+        got, dg = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
+    assert np.isnan(got[:, 9, 40].cpu().numpy()).any() and np.isnan(dg).any()
