@@ -16,7 +16,9 @@
 // in magnitude, so its sums fit; they are rounded to 2^-8 of their unit, and the y blocks (taps at
 // most 44) then end below 2^61 and hold the true K X.  Where a row is larger than all before it the
 // pipeline is shifted down, where the last 16 rows are smaller it is shifted up.  The resolution is
-// thus 2^-54 of the largest component of the level in a strip of 40 columns and 8 to 16 rows.
+// thus 2^-54 of the largest component of the level in a strip of 40 columns and 8 to 16 rows.  A warp that meets a
+// column more than 2^-kKin64Spread below that (the tail of a localised state) redoes its chunk in FP64, where
+// every component keeps its own digits.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -89,7 +91,59 @@ __device__ __forceinline__ void stream_int(i64& a, i64& bt, i64& yo, i64& wc) {
 constexpr int kKin64Warps = 4;  // of a CTA: one to a sub-partition
 constexpr int kKin64Ctas = 5;   // resident per SM
 constexpr int kKin64Stages = 3;
+constexpr int kKin64Spread = 20;
 constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
+
+// The chunk of one warp in FP64: rows [y_begin, y_end) of its 32 columns of one level, straight from global memory.
+template <int VARIANT>
+__device__ __noinline__ void kinetic_strip_f64(const double2* level, double2* out2, int nx, int ny, int x0, int y_begin,
+                                               int y_end, bool abi) {
+    const int lane = threadIdx.x & 31;
+    const int xc = (x0 + lane) % nx;
+    cpx<double> yo[4], wc[4];
+    for (int k = 0; k < 4; ++k) yo[k] = wc[k] = {0.0, 0.0};
+    const int nrows = (y_end - y_begin) + 8;
+#pragma unroll 1
+    for (int r = 0; r < nrows; ++r) {
+        int y = y_begin - kStep2dHalo + r;
+        y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+        cpx<double> xa = {0.0, 0.0}, xbt = {0.0, 0.0};
+        static_for<9>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value;
+            constexpr KinStencil S = kStencilPQ[VARIANT];
+            int x = xc + kk - 4;
+            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+            const double2* g = level + 2 * (int64_t(y) * nx + x);
+            const double2 P = __ldg(g), Q = __ldg(g + 1);
+            kin_tap4<S.g[0][0][kk], S.g[0][1][kk], S.g[1][0][kk], S.g[1][1][kk]>(cpx<double>{P.x, P.y}, cpx<double>{Q.x, Q.y}, xa, xbt);
+        });
+        static_for<4>([&](auto kc) {  // stream_block, qlga_step2d.cuh
+            constexpr int kk = decltype(kc)::value;
+            const cpx<double> ia = xa, ibt = xbt;
+            if (kk < 2) {
+                const cpx<double> ybt = VARIANT == 0 ? ibt - ia : ia + ibt;
+                const cpx<double> wa = yo[kk] + ybt, wbt = ybt - yo[kk];
+                yo[kk] = VARIANT == 0 ? ia + ibt : ia - ibt;
+                xa = wa;
+                xbt = wc[kk];
+                wc[kk] = wbt;
+            } else {
+                const cpx<double> ya = VARIANT == 0 ? ia + ibt : ia - ibt;
+                const cpx<double> wa = ya + yo[kk], wbt = yo[kk] - ya;
+                yo[kk] = VARIANT == 0 ? ibt - ia : ia + ibt;
+                xa = wc[kk];
+                xbt = wbt;
+                wc[kk] = wa;
+            }
+        });
+        if (r >= 8 && x0 + lane < nx) {
+            const double s = 1.0 / 256.0;
+            double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
+            p2[0] = make_double2(s * xa.re, s * xa.im);
+            p2[1] = abi ? make_double2(s * xbt.im, -(s * xbt.re)) : make_double2(s * xbt.re, s * xbt.im);
+        }
+    }
+}
 
 // out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt) or,
 // with abi, the ABI's (a, b).  nx >= 32
@@ -162,8 +216,10 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         const double2 own0 = row[2 * lane], own1 = row[2 * lane + 1];
         const double halo = reinterpret_cast<const double*>(row + 2 * kStep2dWarpCols)[lane];
         auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
-        const unsigned top = max(max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y))), hi(halo));
-        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, top));
+        const unsigned column = max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y)));
+        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, max(column, hi(halo))));
+        // the smallest column that is not empty (a high word of 0: nothing, or below the normal range)
+        const int low = int(__reduce_min_sync(0xffffffffu, column ? column : 0x7fffffffu) >> 20);
         const bool bad = Er > kKin64MaxExp;
         if (bad) {
             Er = kFxMinExp;
@@ -175,6 +231,11 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         }
         seen = max(seen, Er);
         const int En = max(seen, seen_before);
+        if (En - low > kKin64Spread) {  // warp-uniform
+            cp_async_wait<0>();
+            kinetic_strip_f64<VARIANT>(level, out2, nx, ny, x0, y_begin, y_end, abi);
+            return;
+        }
         if (En != E) {  // warp-uniform, rare on smooth fields
             const int n = max(E - En, -63);
 #pragma unroll

@@ -71,3 +71,27 @@ def test_interleaved_tiles(nx, ny, precision):
         lat.step(4)
         got = lat.get_state()
     assert np.linalg.norm(got - ref) <= (1e-11 if precision == 64 else 1e-5) * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("nx,ny", [(96, 70), (101, 64)])
+@pytest.mark.parametrize("variant", [0, 1])
+def test_tails_of_a_localised_fp64_state(nx, ny, variant):
+    """K of a 2D FP64 state runs on integers with one exponent per strip of 40 columns and 16 rows; strips with a column
+    2^-20 below the largest take FP64.  Every site within 1e-9 of the largest within the 8 rows and columns that two
+    steps reach (2^-54 of a strip's largest is 2^-34 of its smallest column, amplified by at most (44/16)^2 a
+    step)."""
+    rng = np.random.default_rng(nx)
+    x, y = np.arange(nx)[None, :], np.arange(ny)[:, None]
+    env = np.exp(-1.1 * np.sqrt((x - nx / 2.0) ** 2 + (y - ny / 2.0) ** 2))
+    st = I.random_state(rng, nx, ny, scale=0.05) * env[None, :, :, None, None]
+    ref = np.ascontiguousarray(st).copy()
+    oracle.step(ref, oracle.make_cfg(2, nx, ny, *G, kinetic_variant=variant), 2)
+    with qlga.Lattice(2, nx, ny, precision=64, g=G, kinetic_variant=variant) as lat:
+        lat.load_state(st)
+        lat.step(2)
+        got = lat.get_state()
+    err = np.sqrt(((got - ref) ** 2).sum(axis=(0, 3, 4)))
+    near = np.sqrt((st ** 2).sum(axis=(0, 3, 4)))
+    for axis in (0, 1):
+        near = np.max([np.roll(near, k, axis=axis) for k in range(-8, 9)], axis=0)
+    assert np.all(err <= 1e-9 * near), float(np.max(err / near))
