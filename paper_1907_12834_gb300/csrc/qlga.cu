@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(kThreads) k_observables(const T* __restrict__ 
             cpx<T> a, b;
             if (RESIDENT) load_pair<T>(X, nsites, m, site, a, b); else load_pair_abi<T>(X, nsites, m, site, a, b);
             const T pm = norm2(a) + norm2(b);
-            acc[OBS_NORM_QUBIT].add(pm);
             acc[OBS_POP0 + m].add(pm);
             psi[m] = a + b;
             rho += norm2(psi[m]);
@@ -308,11 +307,15 @@ __global__ void __launch_bounds__(kThreads) k_observables(const T* __restrict__ 
     }
     __shared__ double sh[kThreads / 32][OBS_COUNT];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double total = 0.0;  // the qubit norm is the sum of the populations
 #pragma unroll
     for (int k = 0; k < OBS_COUNT; ++k) {
+        if (k == OBS_NORM_QUBIT) continue;
         const double v = warp_sum(acc[k].value());
+        if (k >= OBS_POP0 && k < OBS_POP0 + 5) total += v;
         if (lane == 0) sh[warp][k] = v;
     }
+    if (lane == 0) sh[warp][OBS_NORM_QUBIT] = total;
     __syncthreads();
     if (threadIdx.x < OBS_COUNT) {
         double s = 0.0;
@@ -2197,6 +2200,24 @@ qlga_status qlga_exchange_rows(qlga_handle* src, int64_t ysrc, qlga_handle* dst,
     return QLGA_OK;
 }
 
+// Row chunks of the FP64 fields, which are bound by the sub-partitions' FP64 pipes: a row is about 120 FP64
+// instructions and each of the two halo rows of a chunk 20; the busiest of the `units` sub-partitions has ceil(warps / units)
+// chunks, and one or two warps give its pipe 0.7 or 0.9 of its rate (640^2: 168 us with one warp each, 137 with three).
+static int64_t fields_chunks_f64(int64_t strips, int64_t ny, int64_t units) {
+    int64_t best = 1;
+    double best_cost = -1.0;
+    for (int64_t c = 1; c <= ny && (c == 1 || strips * c <= 16 * units); ++c) {
+        const int64_t k = (strips * c + units - 1) / units;
+        const double eff = k >= 3 ? 1.0 : (k == 2 ? 0.9 : 0.7);
+        const double cost = double(k) / eff * (120.0 * double((ny + c - 1) / c) + 40.0);
+        if (best_cost < 0.0 || cost < best_cost) {
+            best = c;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 qlga_status qlga_fields(qlga_handle* h, void* dst, int where) {
     if (!h || !dst) return fail(QLGA_ERR_INVALID_ARG, "NULL argument%s");
     if (where != QLGA_HOST && where != QLGA_DEVICE) return fail(QLGA_ERR_INVALID_ARG, "where must be QLGA_HOST or QLGA_DEVICE%s");
@@ -2216,7 +2237,8 @@ qlga_status qlga_fields(qlga_handle* h, void* dst, int where) {
                   "k_fields2d occupancy");
         const int64_t per_block = kFieldsThreads / 32, strips = (h->cfg.nx + kFieldsCols - 1) / kFieldsCols;
         const int64_t warps = per_block * (per_sm > 0 ? per_sm : 1) * device_sms();
-        const int64_t chunks = std::max<int64_t>(1, std::min(h->cfg.ny / 8, warps / strips));
+        int64_t chunks = std::max<int64_t>(1, std::min(h->cfg.ny / 8, warps / strips));
+        if (h->cfg.precision == 64) chunks = fields_chunks_f64(strips, h->cfg.ny, 4 * int64_t(device_sms()));
         const int64_t grid = (strips * chunks + per_block - 1) / per_block;
         if (h->cfg.precision == 32)
             k_fields2d<float><<<unsigned(grid), kFieldsThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<float*>(target), int(h->cfg.nx), int(h->cfg.ny), int(chunks));
