@@ -759,7 +759,7 @@ __device__ __forceinline__ void potential_direct(cpx<T> a[5], cpx<T> b[5], const
     }
 }
 
-// The FP64 form of U for the warps that the fixed-point form leaves (a lane with beta > 1 or a
+// The FP64 form of U for the warps that the fixed-point form leaves (a lane with beta > 1/4 or a
 // value that is not finite, so every site that sets the status word): a call, so that the kernels
 // keep the registers and the instruction cache for the other.
 __device__ __noinline__ void potential_direct_f64(cpx<double>* a, cpx<double>* b, const PotConstBase<double>* C,
