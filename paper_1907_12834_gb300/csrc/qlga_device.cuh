@@ -262,7 +262,7 @@ struct PotConstBase {
     T dr;      // delta g2 / 10: diagonal shift of the singlet term per unit rho
     T e0, e1;  // delta g1, delta g1 sqrt(3/2): off-diagonal spin entries per unit F_+
     T R;       // delta g2 / 5: singlet rank-one term
-    T b1, b2;  // 2 |g1| delta, |g2| delta / 10: beta = b1 |F| + b2 rho
+    T b1, b2;  // 2 |g1 delta|, |g2 delta| / 10: beta = b1 |F| + b2 rho (delta < 0 steps back)
     PotConstBase() = default;
     __host__ __device__ explicit PotConstBase(const PotParams& P) {
         cphase = T(P.delta * (P.g0 + P.g2 / 10.0));
@@ -271,8 +271,8 @@ struct PotConstBase {
         e0 = T(P.delta * P.g1);
         e1 = T(P.delta * P.g1 * 1.2247448713915890491);  // sqrt(3/2)
         R = T(P.delta * P.g2 / 5.0);
-        b1 = T(2.0 * fabs(P.g1) * P.delta);
-        b2 = T(0.1 * fabs(P.g2) * P.delta);
+        b1 = T(2.0 * fabs(P.g1 * P.delta));
+        b2 = T(0.1 * fabs(P.g2 * P.delta));
     }
 };
 template <class T>
