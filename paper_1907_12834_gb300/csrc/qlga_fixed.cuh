@@ -216,6 +216,10 @@ QLGA_HD unsigned fx_lo(double x) {
     return unsigned(u);
 #endif
 }
+QLGA_HD unsigned fx_top(unsigned m, double x) {  // the larger of m and x's high word without sign
+    const unsigned h = fx_hi(x) & 0x7fffffffu;
+    return h > m ? h : m;
+}
 QLGA_HD double fx_bits(unsigned hi, unsigned lo) {
 #ifdef __CUDA_ARCH__
     return __hiloint2double(int(hi), int(lo));
@@ -290,9 +294,7 @@ QLGA_HD int fx_headroom(const i64 re[5], const i64 im[5]) {
     for (int i = 0; i < 5; ++i) m |= static_cast<unsigned long long>(re[i] ^ (re[i] >> 63)) | static_cast<unsigned long long>(im[i] ^ (im[i] >> 63));
     return m ? 6 - fx_clz(m) : -57;  // 64 - clz bits now, 58 wanted
 }
-QLGA_HD i64 fx_shift(i64 v, int n) {  // v 2^(-n), n in [-57, 5], rounded to nearest (|v| < 2^(58 + n))
-    return ((v << (5 - n)) + 16) >> 5;
-}
+QLGA_HD i64 fx_shift(i64 v, int n) { return fx_scale(v, -n); }  // v 2^(-n), n in [-57, 5] (|v| < 2^(58 + n) and 2^62)
 
 // delta W of a site in fixed point (2^61 = 1)
 struct FxW {
@@ -644,19 +646,34 @@ QLGA_HD void fx_rotate_large(i64 c, i64 s, i64* re, i64* im) {
     }
 }
 
-#ifdef __CUDACC__
+// Decisions of a warp; on the host every site is a warp of its own
+QLGA_HD bool fx_warp_all(bool v) {
+#ifdef __CUDA_ARCH__
+    return __all_sync(0xffffffffu, v);
+#else
+    return v;
+#endif
+}
+QLGA_HD float fx_warp_max(float v) {  // v >= 0
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+#else
+    return v;
+#endif
+}
+
 // e^{-i theta} - 1 = (-c, -s) for a theta of any size (fields denser than |theta| = 1/4 are rare)
-__device__ __noinline__ void fx_phase_large(double theta, i64* c, i64* s) {
+static __host__ __device__ __noinline__ void fx_phase_large(double theta, i64* c, i64* s) {
     double sn, cs;
     sincos(theta, &sn, &cs);
-    *c = __double2ll_rn((1.0 - cs) * 2305843009213693952.0);
-    *s = __double2ll_rn(sn * 2305843009213693952.0);
+    *c = i64(rint((1.0 - cs) * 2305843009213693952.0));
+    *s = i64(rint(sn * 2305843009213693952.0));
 }
 
 // e^{-i theta} - 1 = (-c, -s) of a site from its density; returns whether a lane of the warp has
 // |theta| > 1/4 (fx_rotate_large)
-__device__ __forceinline__ bool fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
-    const bool large = __any_sync(0xffffffffu, theta > 0.25f);
+QLGA_HD bool fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
+    const bool large = !fx_warp_all(theta <= 0.25f);
     if (large) {
         const int n = 2 * et < -900 ? -900 : 2 * et;
         const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * double(rho);
@@ -672,7 +689,7 @@ __device__ __forceinline__ bool fx_site_phase(i64 rho, int et, float theta, cons
 // (U psi, U d) as integers of the unit 2^(returned exponent), below 2^60.  Returns false, with
 // nothing changed, if a lane of the warp lies outside the domain.  All 32 lanes take part: the
 // orders of the Taylor sums are those of the warp's largest beta.
-__device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int in_log2, bool ok,
+QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int in_log2, bool ok,
                                            const FixPot& C) {
     const int np = fx_headroom(pr, pi), nd0 = fx_headroom(dr, di);
     // d goes with psi's unit or, where it is larger, its own, below 2^57 there, so that G of its sums
@@ -689,10 +706,10 @@ __device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 
     const int et = e + np + in_log2;  // exponent of the true psi
     const FxBounds bd = fx_bounds(f, et, C);
     ok = ok && bd.beta <= kFxBetaMax;
-    if (!__all_sync(0xffffffffu, ok)) return false;
-    const float beta = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(bd.beta)));
-    const int K = fx_degree(beta, kFxTol);
-    const int kA = min(K, fx_degree(beta, kFxTolF));
+    if (!fx_warp_all(ok)) return false;
+    const float beta = fx_warp_max(bd.beta);
+    const int K = fx_degree(beta, kFxTol), k0 = fx_degree(beta, kFxTolF);
+    const int kA = K < k0 ? K : k0;
     FxW W;
     fx_build_w(p, f, et, C, W);
     i64 pc, ps;
@@ -726,13 +743,13 @@ __device__ __forceinline__ bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 
 // potential_site, with in_log2 = -log2 sigma and out_log2 = log2 out_scale.  PQ: (a, b) become
 // (P, Q) = (a + i b, a - i b) of the result, summed before the conversion.  Returns false, with nothing changed, outside the domain.
 template <bool PQ>
-__device__ __forceinline__ bool fx_potential(double ar[5], double ai[5], double br[5], double bi[5], int in_log2,
+QLGA_HD bool fx_potential(double ar[5], double ai[5], double br[5], double bi[5], int in_log2,
                                              int out_log2, const FixPot& C) {
     unsigned m = 0;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        m = max(m, max(fx_hi(ar[i]) & 0x7fffffffu, fx_hi(ai[i]) & 0x7fffffffu));
-        m = max(m, max(fx_hi(br[i]) & 0x7fffffffu, fx_hi(bi[i]) & 0x7fffffffu));
+        m = fx_top(fx_top(m, ar[i]), ai[i]);
+        m = fx_top(fx_top(m, br[i]), bi[i]);
     }
     const bool ok = m < (unsigned(1023 + 60) << 20);  // finite, below 2^60
     const int E = fx_exponent(m);
@@ -759,6 +776,5 @@ __device__ __forceinline__ bool fx_potential(double ar[5], double ai[5], double 
     }
     return true;
 }
-#endif
 
 }  // namespace qlga

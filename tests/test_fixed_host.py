@@ -1,0 +1,108 @@
+"""The integer fixed-point potential unitary on single sites, on the CPU: its functions compiled for the host
+(fixed_host.cu) against the Taylor series of exp(-i delta V) in numpy's long double (at least 64 bits)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1907_12834_gb300 import build as qbuild
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+R = np.sqrt(np.longdouble(1.5))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fixed") / "fixed_host.so")
+    cmd = [qbuild._nvcc(), "-std=c++17", "--expt-relaxed-constexpr", "-gencode", "arch=compute_103a,code=sm_103a",
+           "-Xcompiler", "-fPIC", "-shared", "-I", qbuild.CSRC, "-I", os.path.join(ROOT, "include"), "-o", so,
+           os.path.join(HERE, "fixed_host.cu")]
+    try:
+        subprocess.run(cmd, check=True, capture_output=True, text=True)
+    except FileNotFoundError:
+        pytest.skip("nvcc not found")
+    lib = ctypes.CDLL(so)
+    lib.host_shift.restype = ctypes.c_longlong
+    lib.host_shift.argtypes = [ctypes.c_longlong, ctypes.c_int]
+    lib.host_potential.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double]
+    return lib
+
+
+def potential(lib, x, g, delta=1.0):
+    """x (n, 5, 2) complex: U on every site in fixed point, and which sites are in its domain."""
+    y = np.ascontiguousarray(x, dtype=np.complex128).copy()
+    g = np.array(g, dtype=np.float64)
+    ok = [lib.host_potential(s.ctypes.data, g.ctypes.data, delta) for s in y]
+    return y, np.array(ok, dtype=bool)
+
+
+def forms(p):
+    """rho, F_z, F_+ of fields p (n, 5)."""
+    n = p.real ** 2 + p.imag ** 2
+    fz = 2 * (n[:, 0] - n[:, 4]) + n[:, 1] - n[:, 3]
+    fp = 2 * (p[:, 0].conj() * p[:, 1] + p[:, 3].conj() * p[:, 4] + R * (p[:, 1].conj() * p[:, 2] + p[:, 2].conj() * p[:, 3]))
+    return n.sum(axis=1), fz, fp
+
+
+def reference(x, g, delta=1.0, dtype=np.clongdouble):
+    """U by its Taylor series about V's centre, in the arithmetic of dtype."""
+    real = np.zeros(1, dtype).real.dtype.type
+    x = x.astype(dtype)
+    p = x[:, :, 0] + x[:, :, 1]
+    rho, fz, fp = forms(p)
+    fz, fp = fz.astype(real), fp.astype(dtype)
+    g0, g1, g2 = (real(v) * real(delta) for v in g)
+    u = np.stack([p[:, 4], -p[:, 3], p[:, 2], -p[:, 1], p[:, 0]], axis=1)
+    c = [real(1), real(R), real(R), real(1)]
+
+    def w(v):  # (V - (g0 + g2 / 10) rho) v
+        dot = (u * v).sum(axis=1)
+        y = np.empty_like(v)
+        for m in range(5):
+            y[:, m] = (real(2 - m) * g1 * fz - g2 / 10 * rho) * v[:, m] + (g2 / 5) * u[:, m].conj() * dot
+            if m < 4:
+                y[:, m] += g1 * c[m] * fp.conj() * v[:, m + 1]
+            if m > 0:
+                y[:, m] += g1 * c[m - 1] * fp * v[:, m - 1]
+        return y
+
+    out = np.empty_like(x)
+    theta = (g0 + g2 / 10) * rho
+    phase = np.cos(theta) - 1j * np.sin(theta)
+    for q in range(2):
+        v = x[:, :, q].copy()
+        for k in range(28, 0, -1):
+            v = x[:, :, q] - dtype(1j) / real(k) * w(v)
+        out[:, :, q] = phase[:, None] * v
+    return out
+
+
+def sites(rng, n, scale=0.05):
+    return scale * (rng.standard_normal((n, 5, 2)) + 1j * rng.standard_normal((n, 5, 2)))
+
+
+def test_shift_at_the_ends_of_its_domain(lib):
+    """v 2^-n rounded to nearest for every n and |v| < 2^(58 + n), 2^62: the sum with the rounding bit may not wrap."""
+    for n in range(-57, 6):
+        top = (1 << min(58 + n, 62)) - 1
+        for v in {top, top - 1, top // 2 + 1, 1, 0}:
+            want = v << -n if n <= 0 else (v + (1 << (n - 1))) >> n
+            assert lib.host_shift(v, n) == want, (v, n)
+            assert abs(lib.host_shift(-v, n) + want) <= (n > 0)  # a half rounds up
+
+
+def test_a_component_just_below_a_power_of_two(lib):
+    """a + b = 2^59 - 1 units in the site's largest component: its rounding must not turn psi's sign.  Tolerance 4e-14
+    of the site, as the domain test on the GPU."""
+    g = (0.02, 0.02, 0.02)
+    x = sites(np.random.default_rng(1), 2, 0.2)
+    x[:, 2, 0] = 1.0 + 0.1j
+    x[:, 2, 1] = -2.0 ** -59
+    x[1] = -x[1]
+    got, ok = potential(lib, x, g)
+    ref = reference(x, g)
+    assert ok.all()
+    assert np.abs(got - ref).max() <= 4e-14 * np.abs(ref).max()
