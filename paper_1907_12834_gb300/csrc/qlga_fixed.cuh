@@ -11,7 +11,7 @@
 // Numbers.  A site's psi = a + b and d = a - b are int64 with one exponent per vector, psi's largest
 // component in [2^57, 2^58).  An operand of a product is split as v = h 2^32 + l, l the low word
 // taken as signed; h h' is summed in a 64-bit accumulator, h l' + l h' in an FP32 one, and l l' (zero mean,
-// below 2^62) is dropped.  The entries of delta W and the phase are fixed point with 2^61 = 1.  FP32 leaves
+// below 2^62) is dropped.  The quadratic forms take all four products in integers.  The entries of delta W and the phase are fixed point with 2^61 = 1.  FP32 leaves
 // 2^-24 of the cross terms, 2^-52 of an entry of W times the vector: with beta <= 1/4 below 2^-54, and in a field of
 // the lattice scaling (beta 0.005 to 0.06) below 2^-56.  (All three products in integers:
 // ten 1024^2 steps with load and read-out 7.36 ms, so 6.37, the same errors against 64-bit references.)
@@ -431,13 +431,15 @@ struct FxForms {
     i64 rho, Fz, Fpr, Fpi;  // F_+ = 2 (Fpr + i Fpi)
 };
 
-QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
+QLGA_HD void fx_forms(const Limb re[5], const Limb im[5], FxForms& f) {
     i64 n[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        FxAccF s = {fx_mad(p.re[i].h, p.re[i].h, fx_mad(p.im[i].h, p.im[i].h, 0)),
-                    2.f * fmaf(p.re[i].hf, p.re[i].lf, p.im[i].hf * p.im[i].lf)};
-        n[i] = fx_sum<60, 1>(s);
+    for (int i = 0; i < 5; ++i) {  // with l l': of a square it has no zero mean
+        FxAcc s = fx_zero<60>();
+        fx_mac(s, re[i], re[i]);
+        fx_mac(s, im[i], im[i]);
+        s.mid += (fx_mad(re[i].l, re[i].l, 0) >> 32) + (fx_mad(im[i].l, im[i].l, 0) >> 32);
+        n[i] = fx_sum<60>(s);
     }
     f.rho = (n[0] + n[1]) + (n[2] + n[3]) + n[4];
     f.Fz = 2 * (n[0] - n[4]) + (n[1] - n[3]);
@@ -445,17 +447,17 @@ QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {  // conj(p0) p1 + conj(p3) p4, then conj(p1) p2 + conj(p2) p3
         const int a = q, b = q == 0 ? 3 : 2;
-        FxAccF r = {0, 0.f}, ip = {0, 0.f}, in = {0, 0.f};
-        fx_mac(r, p.re[a], p.re[a + 1]);
-        fx_mac(r, p.im[a], p.im[a + 1]);
-        fx_mac(r, p.re[b], p.re[b + 1]);
-        fx_mac(r, p.im[b], p.im[b + 1]);
-        fx_mac(ip, p.re[a], p.im[a + 1]);
-        fx_mac(in, p.im[a], p.re[a + 1]);
-        fx_mac(ip, p.re[b], p.im[b + 1]);
-        fx_mac(in, p.im[b], p.re[b + 1]);
-        fr[q] = fx_sum<60, 2>(r);
-        fi[q] = fx_sum<60, 2>(FxAccF{ip.hh - in.hh, ip.x - in.x});
+        FxAcc r = fx_zero<60>(), i = fx_zero<60>();
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int j = k ? b : a;
+            fx_mac(r, re[j], re[j + 1]);
+            fx_mac(r, im[j], im[j + 1]);
+            fx_mac(i, re[j], im[j + 1]);
+            fx_mac(i, fx_neg(im[j]), re[j + 1]);
+        }
+        fr[q] = fx_sum<60>(r);
+        fi[q] = fx_sum<60>(i);
     }
     const Limb r = fx_split(kFxR32m1);
     f.Fpr = fr[0] + fr[1] + fx_mul(r, fx_split(fr[1]));
@@ -695,14 +697,20 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
     // d goes with psi's unit or, where it is larger, its own, below 2^57 there, so that G of its sums
     // stays below 2^62; psi's sum takes the same unit (its limbs in W have psi's own)
     const int nd = nd0 + 1 > np ? nd0 + 1 : np;
+    Limb lr[5], li[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        lr[i] = fx_split(fx_shift(pr[i], np));
+        li[i] = fx_split(fx_shift(pi[i], np));
+    }
+    FxForms f;
+    fx_forms(lr, li, f);
     FxVec p;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_op(fx_shift(pr[i], np));
-        p.im[i] = fx_op(fx_shift(pi[i], np));
+        p.re[i] = fx_op(lr[i]);
+        p.im[i] = fx_op(li[i]);
     }
-    FxForms f;
-    fx_forms(p, f);
     const int et = e + np + in_log2;  // exponent of the true psi
     const FxBounds bd = fx_bounds(f, et, C);
     ok = ok && bd.beta <= kFxBetaMax;

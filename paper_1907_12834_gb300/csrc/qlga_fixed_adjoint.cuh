@@ -152,14 +152,17 @@ __device__ __forceinline__ bool fx_vjp_site(const cpx<double> a[5], const cpx<do
     }
     int ex = Ex - 1022 - 60, eg = Eg - 1022 - 60;
     const int np = fx_headroom(xr, xi);
+    Limb lxr[5], lxi[5];
     FxVec p;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_op(fx_shift(xr[i], np));
-        p.im[i] = fx_op(fx_shift(xi[i], np));
+        lxr[i] = fx_split(fx_shift(xr[i], np));
+        lxi[i] = fx_split(fx_shift(xi[i], np));
+        p.re[i] = fx_op(lxr[i]);
+        p.im[i] = fx_op(lxi[i]);
     }
     FxForms f;
-    fx_forms(p, f);
+    fx_forms(lxr, lxi, f);
     const int et = ex + np;
     const FxBounds bd = fx_bounds(f, et, C);
     ok = ok && bd.beta <= kFxBetaMax;

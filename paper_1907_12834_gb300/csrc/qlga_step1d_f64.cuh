@@ -224,6 +224,10 @@ __device__ __forceinline__ FxOp fx_shfl(FxOp v, int src) {
     return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.hf, src), __shfl_sync(0xffffffffu, v.lf, src)};
 }
 
+__device__ __forceinline__ Limb fx_shfl(Limb v, int src) {
+    return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.l, src)};
+}
+
 // The lane's place in its group of five, and the group's sums (exact on integers in any order)
 struct FxGroup {
     int m, base, s1, s2, s4;
@@ -383,20 +387,25 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
     const int np = bp ? bp - 58 : -57, nd0 = bd0 ? bd0 - 58 : -57;
     const int nd = nd0 + 1 > np ? nd0 + 1 : np;
     int e = E - 1022 - 55;
-    const FxOp opr = fx_op(fx_shift(pr, np)), opi = fx_op(fx_shift(pi, np));
+    const Limb lpr = fx_split(fx_shift(pr, np)), lpi = fx_split(fx_shift(pi, np));
+    const FxOp opr = fx_op(lpr), opi = fx_op(lpi);
     FxForms f;
-    const i64 n = fx_sum<60, 1>(FxAccF{fx_mad(opr.h, opr.h, fx_mad(opi.h, opi.h, 0)), 2.f * fmaf(opr.hf, opr.lf, opi.hf * opi.lf)});
+    FxAcc nn = fx_zero<60>();
+    fx_mac(nn, lpr, lpr);
+    fx_mac(nn, lpi, lpi);
+    nn.mid += (fx_mad(lpr.l, lpr.l, 0) >> 32) + (fx_mad(lpi.l, lpi.l, 0) >> 32);
+    const i64 n = fx_sum<60>(nn);
     f.rho = g.sum(n);
     f.Fz = g.sum((2 - g.m) * n);
     const Limb r32m1 = fx_split(kFxR32m1);
     {
-        const FxOp ur = fx_shfl(opr, g.up()), ui = fx_shfl(opi, g.up());
-        FxAccF a = {0, 0.f}, b = {0, 0.f};
-        fx_mac(a, opr, ur);
-        fx_mac(a, opi, ui);
-        fx_mac(b, opr, ui);
-        fx_mac(b, fx_neg(opi), ur);
-        i64 fr = fx_sum<60, 1>(a), fi = fx_sum<60, 1>(b);
+        const Limb ur = fx_shfl(lpr, g.up()), ui = fx_shfl(lpi, g.up());
+        FxAcc a = fx_zero<60>(), b = fx_zero<60>();
+        fx_mac(a, lpr, ur);
+        fx_mac(a, lpi, ui);
+        fx_mac(b, lpr, ui);
+        fx_mac(b, fx_neg(lpi), ur);
+        i64 fr = fx_sum<60>(a), fi = fx_sum<60>(b);
         if (g.m == 1 || g.m == 2) {
             fr += fx_mul(r32m1, fx_split(fr));
             fi += fx_mul(r32m1, fx_split(fi));

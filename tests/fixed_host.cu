@@ -8,6 +8,27 @@ extern "C" {
 
 long long host_shift(long long v, int n) { return fx_shift(v, n); }
 
+// The density of a field psi[level][re, im]
+double host_density(const double* psi) {
+    unsigned m = 0;
+    for (int i = 0; i < 10; ++i) m = fx_top(m, psi[i]);
+    const int E = fx_exponent(m);
+    i64 re[5], im[5];
+    for (int i = 0; i < 5; ++i) {
+        re[i] = fx_from_double<60>(psi[2 * i], E);
+        im[i] = fx_from_double<60>(psi[2 * i + 1], E);
+    }
+    const int n = fx_headroom(re, im);
+    Limb lr[5], li[5];
+    for (int i = 0; i < 5; ++i) {
+        lr[i] = fx_split(fx_shift(re[i], n));
+        li[i] = fx_split(fx_shift(im[i], n));
+    }
+    FxForms f;
+    fx_forms(lr, li, f);
+    return std::ldexp(double(f.rho), 2 * (E - 1022 - 60 + n) + 60);
+}
+
 // U on the pair (a, b) of a site; x[level][qubit][re, im], in place.  Returns whether the site is in the domain.
 int host_potential(double* x, const double* g, double delta) {
     const PotConst<double> C(PotParams{g[0], g[1], g[2], delta});

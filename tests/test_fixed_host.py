@@ -27,6 +27,8 @@ def lib(tmp_path_factory):
     lib = ctypes.CDLL(so)
     lib.host_shift.restype = ctypes.c_longlong
     lib.host_shift.argtypes = [ctypes.c_longlong, ctypes.c_int]
+    lib.host_density.restype = ctypes.c_double
+    lib.host_density.argtypes = [ctypes.c_void_p]
     lib.host_potential.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double]
     return lib
 
@@ -106,3 +108,15 @@ def test_a_component_just_below_a_power_of_two(lib):
     ref = reference(x, g)
     assert ok.all()
     assert np.abs(got - ref).max() <= 4e-14 * np.abs(ref).max()
+
+
+def test_density_is_not_biased(lib):
+    """The mean relative error of rho over random sites: the dropped part of a square always has one sign and shifts
+    every site's phase alike.  Tolerance 2^-55: four means' deviations of a sum rounded at 2^-53 over 4000 sites are
+    below 2^-56, and the conversion to double that the test itself makes has none."""
+    x = sites(np.random.default_rng(5), 4000)
+    p = np.ascontiguousarray(x.sum(axis=2))
+    got = np.array([lib.host_density(s.ctypes.data) for s in p])
+    rho, _, _ = forms(p.astype(np.clongdouble))
+    err = ((got - rho) / rho).astype(np.float64)
+    assert abs(err.mean()) <= 2.0 ** -55, err.mean()
