@@ -3,18 +3,17 @@
 // GB300 issues one FP64 instruction per SM sub-partition every 64-76 cycles (measured: DFMA 64, DADD and
 // DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4, a
 // 64-bit addition every 2.4 and an FP32 multiply-add every cycle.  A product of two fixed-point numbers
-// takes one of the first and two of the last, so U on a site costs a fifth of
-// its FP64 form (1024^2 sites of a vortex lattice: 0.39 ms, against about 1.7), at a finer
+// takes three of the first, so U on a site costs a quarter of its FP64 form, at a finer
 // resolution: relative to the site's largest component the operands carry 2^-58, where FP64 rounds
 // every operation at 2^-53 of its own result.
 //
 // Numbers.  A site's psi = a + b and d = a - b are int64 with one exponent per vector, psi's largest
 // component in [2^57, 2^58).  An operand of a product is split as v = h 2^32 + l, l the low word
-// taken as signed; h h' is summed in a 64-bit accumulator, h l' + l h' in an FP32 one, and l l' (zero mean,
-// below 2^62) is dropped.  The quadratic forms take all four products in integers.  The entries of delta W and the phase are fixed point with 2^61 = 1.  FP32 leaves
-// 2^-24 of the cross terms, 2^-52 of an entry of W times the vector: with beta <= 1/4 below 2^-54, and in a field of
-// the lattice scaling (beta 0.005 to 0.06) below 2^-56.  (All three products in integers:
-// ten 1024^2 steps with load and read-out 7.36 ms, so 6.37, the same errors against 64-bit references.)
+// taken as signed; h h' and h l' + l h' are summed in 64-bit accumulators, and l l' (zero mean,
+// below 2^62) is dropped but in the squares of the density.  The entries of delta W and the phase are fixed point with
+// 2^61 = 1.  (Cross terms in FP32 are 13% of a 1024^2 step, 5.65 against 6.54 ms for ten with load and read-out, but round the
+// low limb of an entry to 24 bits: the phase and W's diagonal, which sites of one density share, were
+// off by up to 2^-55 whatever their size, 7e-17 a step of a run's phase.)
 //
 // U = e^{-i delta c} exp(-i delta W) as in potential_site, by the plain Taylor sum: the terms
 // T_k = (-i delta W)^k x are formed in fixed point up to the order k0 - 1 whose successor is bounded
@@ -46,7 +45,6 @@ struct Limb {
 QLGA_HD Limb fx_split(i64 v) {  // the low limb is the low word as it stands, the high one takes its sign
     return {int(v >> 32) + int(unsigned(v) >> 31), int(unsigned(v))};
 }
-QLGA_HD Limb fx_neg(Limb a) { return {-a.h, -a.l}; }
 
 // s + a b, 32 x 32 bits: one instruction
 QLGA_HD i64 fx_mad(int a, int b, i64 s) {
@@ -70,6 +68,7 @@ QLGA_HD void fx_mac(FxAcc& s, Limb a, Limb b) {
 // Every sum is rounded to nearest, not down: half a unit a step would add up over a run's thousands.
 template <int N>
 QLGA_HD FxAcc fx_zero() { return {0, i64(1) << (N - 33)}; }
+QLGA_HD FxAcc operator-(FxAcc a, FxAcc b) { return {a.hh - b.hh, a.mid - b.mid}; }  // a limb of -2^31 has no negative
 template <int N>
 QLGA_HD i64 fx_sum(FxAcc s) {  // sum / 2^N, 32 < N < 64, of an accumulator that began as fx_zero<N>
     return (s.hh << (64 - N)) + (s.mid >> (N - 32));
@@ -105,37 +104,14 @@ QLGA_HD int fx_clz(T v) {  // v != 0
 
 // ------------------------------------------------------------------ constants
 
-// An operand of the products with FP32 cross terms: the high limb, and both limbs in FP32
-struct FxOp {
-    int h;
-    float hf, lf;
-};
-QLGA_HD FxOp fx_op(Limb a) { return {a.h, float(a.h), float(a.l)}; }
-QLGA_HD FxOp fx_op(i64 v) { return fx_op(fx_split(v)); }
-QLGA_HD FxOp fx_neg(FxOp a) { return {-a.h, -a.hf, -a.lf}; }
-QLGA_HD float fx_float(FxOp a, float c) { return fmaf(a.hf, 4294967296.f * c, a.lf * c); }
-
-// The running sum of such products: hh 2^64 + x 2^32
-struct FxAccF {
-    i64 hh;
-    float x;
-};
-QLGA_HD void fx_mac(FxAccF& s, FxOp a, FxOp b) {
-    s.hh = fx_mad(a.h, b.h, s.hh);
-    s.x = fmaf(a.lf, b.hf, fmaf(a.hf, b.lf, s.x));
-}
+// float of a fixed-point value times the float c
+QLGA_HD float fx_float(Limb v, float c) { return fmaf(float(v.h), 4294967296.f * c, float(v.l) * c); }
 QLGA_HD int fx_rint(float x) {
 #ifdef __CUDA_ARCH__
     return __float2int_rn(x);
 #else
     return int(rintf(x));
 #endif
-}
-// sum / 2^N in steps of 2^Q (|x| < 2^(N - 1 + Q)), rounded to nearest
-template <int N, int Q>
-QLGA_HD i64 fx_sum(FxAccF s) {
-    constexpr float kUnit = 1.f / float(1LL << (N - 32 + Q));
-    return (s.hh << (64 - N)) + (i64(fx_rint(s.x * kUnit)) << Q);
 }
 
 // A coupling c = m 2^(ex - 60), m in [2^59, 2^60) (0: all zero)
@@ -283,7 +259,7 @@ struct FxToDouble {
 // ------------------------------------------------------------------ the site
 
 struct FxVec {
-    FxOp re[5], im[5];
+    Limb re[5], im[5];
 };
 
 // Shift that brings the largest of the ten components of (re, im) to [2^57, 2^58): v -> v 2^(-n).
@@ -298,9 +274,8 @@ QLGA_HD i64 fx_shift(i64 v, int n) { return fx_scale(v, -n); }  // v 2^(-n), n i
 
 // delta W of a site in fixed point (2^61 = 1)
 struct FxW {
-    FxOp D[5];
-    FxOp e0r, e0i, e1r, e1i;  // delta g1 F_+ times 1 and sqrt(3/2)
-    int ne0i, ne1i;           // the high limbs of their negated imaginary parts
+    Limb D[5];
+    Limb e0r, e0i, e1r, e1i;  // delta g1 F_+ times 1 and sqrt(3/2)
     FxVec u;                  // u_j = (-1)^j psi_{4-j}
     Limb R;                   // delta g2 / 5: G = R dot / 2^55
     float Rf;
@@ -308,50 +283,44 @@ struct FxW {
 
 // t <- -i delta W t
 QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
-    FxAccF tp = {0, 0.f}, ti = {0, 0.f};
-    i64 tn = 0;
+    FxAcc tp = fx_zero<60>(), tn = {0, 0}, ti = fx_zero<60>();
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         fx_mac(tp, W.u.re[j], t.re[j]);
-        tn = fx_mad(W.u.im[j].h, t.im[j].h, tn);
-        tp.x = fmaf(-W.u.im[j].lf, t.im[j].hf, fmaf(-W.u.im[j].hf, t.im[j].lf, tp.x));
+        fx_mac(tn, W.u.im[j], t.im[j]);
         fx_mac(ti, W.u.re[j], t.im[j]);
         fx_mac(ti, W.u.im[j], t.re[j]);
     }
-    tp.hh -= tn;
-    const FxOp Gr = fx_op(fx_mul_full<55>(W.R, fx_split(fx_sum<60, 3>(tp))));
-    const FxOp Gi = fx_op(fx_mul_full<55>(W.R, fx_split(fx_sum<60, 3>(ti))));
-    const FxOp nGr = fx_neg(Gr);
+    const Limb Gr = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(tp - tn))));
+    const Limb Gi = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(ti))));
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         // y = (W t)_i; o = -i y: o.re = y.im, o.im = -y.re
-        FxAccF yr = {0, 0.f}, yi = {0, 0.f};
+        FxAcc yr = fx_zero<61>(), yi = fx_zero<61>(), nr = {0, 0}, ni = {0, 0};
         fx_mac(yr, W.D[i], t.re[i]);
         fx_mac(yi, W.D[i], t.im[i]);
         fx_mac(yr, W.u.re[i], Gr);  // conj(u) G
         fx_mac(yr, W.u.im[i], Gi);
         fx_mac(yi, W.u.re[i], Gi);
-        fx_mac(yi, W.u.im[i], nGr);
+        fx_mac(ni, W.u.im[i], Gr);
         if (i > 0) {  // e t_{i-1}
             const bool s = i == 1 || i == 4;
-            const FxOp er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
-            const FxOp ne = {s ? W.ne0i : W.ne1i, -ei.hf, -ei.lf};
+            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
             fx_mac(yr, er, t.re[i - 1]);
-            fx_mac(yr, ne, t.im[i - 1]);
+            fx_mac(nr, ei, t.im[i - 1]);
             fx_mac(yi, er, t.im[i - 1]);
             fx_mac(yi, ei, t.re[i - 1]);
         }
         if (i < 4) {  // conj(e) t_{i+1}
             const bool s = i == 0 || i == 3;
-            const FxOp er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
-            const FxOp ne = {s ? W.ne0i : W.ne1i, -ei.hf, -ei.lf};
+            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
             fx_mac(yr, er, t.re[i + 1]);
             fx_mac(yr, ei, t.im[i + 1]);
             fx_mac(yi, er, t.im[i + 1]);
-            fx_mac(yi, ne, t.re[i + 1]);
+            fx_mac(ni, ei, t.re[i + 1]);
         }
-        ore[i] = fx_sum<61, 2>(yi);
-        oim[i] = -fx_sum<61, 2>(yr);
+        ore[i] = fx_sum<61>(yi - ni);
+        oim[i] = -fx_sum<61>(yr - nr);
     }
 }
 
@@ -431,7 +400,8 @@ struct FxForms {
     i64 rho, Fz, Fpr, Fpi;  // F_+ = 2 (Fpr + i Fpi)
 };
 
-QLGA_HD void fx_forms(const Limb re[5], const Limb im[5], FxForms& f) {
+QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
+    const Limb *re = p.re, *im = p.im;
     i64 n[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {  // with l l': of a square it has no zero mean
@@ -447,25 +417,23 @@ QLGA_HD void fx_forms(const Limb re[5], const Limb im[5], FxForms& f) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {  // conj(p0) p1 + conj(p3) p4, then conj(p1) p2 + conj(p2) p3
         const int a = q, b = q == 0 ? 3 : 2;
-        FxAcc r = fx_zero<60>(), i = fx_zero<60>();
+        FxAcc r = fx_zero<60>(), i = fx_zero<60>(), n = {0, 0};
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int j = k ? b : a;
             fx_mac(r, re[j], re[j + 1]);
             fx_mac(r, im[j], im[j + 1]);
             fx_mac(i, re[j], im[j + 1]);
-            fx_mac(i, fx_neg(im[j]), re[j + 1]);
+            fx_mac(n, im[j], re[j + 1]);
         }
         fr[q] = fx_sum<60>(r);
-        fi[q] = fx_sum<60>(i);
+        fi[q] = fx_sum<60>(i - n);
     }
     const Limb r = fx_split(kFxR32m1);
     f.Fpr = fr[0] + fr[1] + fx_mul(r, fx_split(fr[1]));
     f.Fpi = fi[0] + fi[1] + fx_mul(r, fx_split(fi[1]));
 }
 
-// float of a fixed-point value times the float c
-QLGA_HD float fx_float(Limb v, float c) { return fmaf(float(v.h), 4294967296.f * c, float(v.l) * c); }
 QLGA_HD float fx_pow2f(int n) {  // 2^n, clamped to the normal range
     n = n < -126 ? -126 : (n > 127 ? 127 : n);
     union {
@@ -523,26 +491,25 @@ QLGA_HD void fx_singlet(const FixPot& C, int e, Limb& R, float& Rf) {
     // |psi|^2 >= 2^114 and beta <= 0.25 bound W.R by 2^62
     int n = C.R.ex + 2 * e + 116;
     n = n < -63 ? -63 : (n > 30 ? 30 : n);
-    R = fx_split(fx_scale((i64(C.R.m.h) << 32) + C.R.m.l, n));
+    R = fx_split(fx_scale((i64(C.R.m.h) * (i64(1) << 32)) + C.R.m.l, n));
     Rf = C.R_f * fx_pow2f(2 * e + 116);  // for u in 2^58 = 1
 }
 
 QLGA_HD void fx_build_w(const FxVec& p, const FxForms& f, int e, const FixPot& C, FxW& W) {
     const i64 gz = fx_coupled(C.dz, f.Fz, e, 0), g2r = fx_coupled(C.dr, f.rho, e, 0);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) W.D[i] = fx_op((2 - i) * gz - g2r);
+    for (int i = 0; i < 5; ++i) W.D[i] = fx_split((2 - i) * gz - g2r);
     const Limb r = fx_split(kFxR32m1);
     const i64 er = fx_coupled(C.e0, f.Fpr, e, 1), ei = fx_coupled(C.e0, f.Fpi, e, 1);
-    W.e0r = fx_op(er);
-    W.e0i = fx_op(ei);
-    W.e1r = fx_op(er + fx_mul(r, fx_split(er)));
-    W.e1i = fx_op(ei + fx_mul(r, fx_split(ei)));
-    W.ne0i = -W.e0i.h;
-    W.ne1i = -W.e1i.h;
+    W.e0r = fx_split(er);
+    W.e0i = fx_split(ei);
+    W.e1r = fx_split(er + fx_mul(r, fx_split(er)));
+    W.e1i = fx_split(ei + fx_mul(r, fx_split(ei)));
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-        W.u.re[j] = (j & 1) ? fx_neg(p.re[4 - j]) : p.re[4 - j];
-        W.u.im[j] = (j & 1) ? fx_neg(p.im[4 - j]) : p.im[4 - j];
+        auto turned = [&](Limb v) { return (j & 1) ? fx_split(-(v.h * (i64(1) << 32) + v.l)) : v; };
+        W.u.re[j] = turned(p.re[4 - j]);
+        W.u.im[j] = turned(p.im[4 - j]);
     }
     fx_singlet(C, e, W.R, W.Rf);
 }
@@ -558,16 +525,16 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
     }
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        t.re[i] = fx_op(tr[i]);
-        t.im[i] = fx_op(ti[i]);
+        t.re[i] = fx_split(tr[i]);
+        t.im[i] = fx_split(ti[i]);
     }
 #pragma unroll 1
     for (int k = 1; k <= kA; ++k) {
         fx_apply(W, t, tr, ti);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            t.re[i] = fx_op(tr[i]);
-            t.im[i] = fx_op(ti[i]);
+            t.re[i] = fx_split(tr[i]);
+            t.im[i] = fx_split(ti[i]);
         }
         if (k <= 2) {
 #pragma unroll
@@ -576,14 +543,11 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
                 im[i] += k == 1 ? ti[i] : (ti[i] + 1) >> 1;
             }
         } else {
-            const FxOp f = fx_op(fx_inv_fact(k));
+            const Limb f = fx_inv_fact(k);
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
-                FxAccF a = {0, 0.f}, b = {0, 0.f};
-                fx_mac(a, f, t.re[i]);
-                fx_mac(b, f, t.im[i]);
-                re[i] += fx_sum<61, 0>(a);
-                im[i] += fx_sum<61, 0>(b);
+                re[i] += fx_mul(f, t.re[i]);
+                im[i] += fx_mul(f, t.im[i]);
             }
         }
     }
@@ -615,26 +579,10 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
     }
 }
 
-// x <- x + (e^{-i theta} - 1) x, for |theta| <= 1/4
+// x <- x + (e^{-i theta} - 1) x
 template <int N = 5>
 QLGA_HD void fx_rotate(i64 c, i64 s, i64* re, i64* im) {
-    const FxOp nc = fx_op(-c), sp = fx_op(s), sn = fx_neg(sp);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const FxOp r = fx_op(re[i]), m = fx_op(im[i]);
-        FxAccF a = {0, 0.f}, b = {0, 0.f};
-        fx_mac(a, nc, r);
-        fx_mac(a, sp, m);
-        fx_mac(b, nc, m);
-        fx_mac(b, sn, r);
-        re[i] += fx_sum<61, 2>(a);
-        im[i] += fx_sum<61, 2>(b);
-    }
-}
-// the same for any theta, with integer cross terms
-template <int N = 5>
-QLGA_HD void fx_rotate_large(i64 c, i64 s, i64* re, i64* im) {
-    const Limb nc = fx_split(-c), sp = fx_split(s), sn = fx_neg(sp);
+    const Limb nc = fx_split(-c), sp = fx_split(s), sn = fx_split(-s);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const Limb r = fx_split(re[i]), m = fx_split(im[i]);
@@ -672,18 +620,15 @@ static __host__ __device__ __noinline__ void fx_phase_large(double theta, i64* c
     *s = i64(rint(sn * 2305843009213693952.0));
 }
 
-// e^{-i theta} - 1 = (-c, -s) of a site from its density; returns whether a lane of the warp has
-// |theta| > 1/4 (fx_rotate_large)
-QLGA_HD bool fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
-    const bool large = !fx_warp_all(theta <= 0.25f);
-    if (large) {
+// e^{-i theta} - 1 = (-c, -s) of a site from its density, for a warp with a lane beyond |theta| = 1/4 in FP64
+QLGA_HD void fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
+    if (!fx_warp_all(theta <= 0.25f)) {
         const int n = 2 * et < -900 ? -900 : 2 * et;
         const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * double(rho);
         fx_phase_large(th, &c, &s);
     } else {
         fx_phase(fx_coupled(C.cphase, rho, et, 0), c, s);
     }
-    return large;
 }
 
 // U on one site of a warp.  In: psi and d as integers below 2^62 of unit 2^e, `true` amplitudes
@@ -697,20 +642,14 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
     // d goes with psi's unit or, where it is larger, its own, below 2^57 there, so that G of its sums
     // stays below 2^62; psi's sum takes the same unit (its limbs in W have psi's own)
     const int nd = nd0 + 1 > np ? nd0 + 1 : np;
-    Limb lr[5], li[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        lr[i] = fx_split(fx_shift(pr[i], np));
-        li[i] = fx_split(fx_shift(pi[i], np));
-    }
-    FxForms f;
-    fx_forms(lr, li, f);
     FxVec p;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_op(lr[i]);
-        p.im[i] = fx_op(li[i]);
+        p.re[i] = fx_split(fx_shift(pr[i], np));
+        p.im[i] = fx_split(fx_shift(pi[i], np));
     }
+    FxForms f;
+    fx_forms(p, f);
     const int et = e + np + in_log2;  // exponent of the true psi
     const FxBounds bd = fx_bounds(f, et, C);
     ok = ok && bd.beta <= kFxBetaMax;
@@ -721,7 +660,7 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
     FxW W;
     fx_build_w(p, f, et, C, W);
     i64 pc, ps;
-    const bool large = fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
+    fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         pr[i] = fx_shift(pr[i], nd);
@@ -732,8 +671,7 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
 #pragma unroll 1
     for (int v = 0; v < 2; ++v) {  // one copy of the code for both vectors
         fx_taylor(W, pr, pi, kA, K);
-        if (large) fx_rotate_large(pc, ps, pr, pi);
-        else fx_rotate(pc, ps, pr, pi);
+        fx_rotate(pc, ps, pr, pi);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             const i64 tr = pr[i], ti = pi[i];

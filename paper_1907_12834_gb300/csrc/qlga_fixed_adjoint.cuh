@@ -2,9 +2,8 @@
 //
 // The FP64 pull-back (qlga_adjoint.cuh) is 2250 FP64 instructions a site in its sweeps alone, one every 66 cycles
 // (qlga_fixed.cuh).  Here both sweeps run on the numbers of fx_unitary: W, the phase and the vectors psi = a + b, d = a - b
-// with one exponent; the cotangents ga + gb and ga - gb with another.  W is applied with FP32 cross terms,
-// the contractions of mu_k with v_k take all three products in integers (they are not multiplied by W, so
-// FP32's 2^-52 would be the result's).  Orders whose bound is below 2^-31 run in FP32, as
+// with one exponent; the cotangents ga + gb and ga - gb with another.
+// Orders whose bound is below 2^-31 run in FP32, as
 // there.  256^2 (g = (1, 0.1, 1)): 0.186 ms for the x axis of K^dagger and the pull-back, 0.053 of them the FP64 stencil,
 // against 0.464 with FP64 sweeps; a gradient of 12 steps 5.2 ms against 8.5, its error against 64 bits 3.5e-15 against 3.3e-15
 // (4.0e-15 with the Frechet recursions before).
@@ -44,8 +43,8 @@ __device__ __forceinline__ void fx_apply_ints(const FxW& W, const i64 re[5], con
     FxVec t;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        t.re[i] = fx_op(re[i]);
-        t.im[i] = fx_op(im[i]);
+        t.re[i] = fx_split(re[i]);
+        t.im[i] = fx_split(im[i]);
     }
     fx_apply(W, t, ore, oim);
 }
@@ -62,6 +61,8 @@ struct LimbC {
     Limb re, im;
 };
 QLGA_HD LimbC fx_limbs(i64 re, i64 im) { return {fx_split(re), fx_split(im)}; }
+// a limb of -2^31 has no negative: one unit off
+QLGA_HD Limb fx_neg(Limb a) { return {-a.h, -(a.l > -0x7fffffff ? a.l : -0x7fffffff)}; }
 // s += Re / Im of conj(a) b
 QLGA_HD void fx_conj_mac(FxAcc& re, FxAcc& im, LimbC a, LimbC b) {
     fx_mac(re, a.re, b.re);
@@ -152,17 +153,14 @@ __device__ __forceinline__ bool fx_vjp_site(const cpx<double> a[5], const cpx<do
     }
     int ex = Ex - 1022 - 60, eg = Eg - 1022 - 60;
     const int np = fx_headroom(xr, xi);
-    Limb lxr[5], lxi[5];
     FxVec p;
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        lxr[i] = fx_split(fx_shift(xr[i], np));
-        lxi[i] = fx_split(fx_shift(xi[i], np));
-        p.re[i] = fx_op(lxr[i]);
-        p.im[i] = fx_op(lxi[i]);
+        p.re[i] = fx_split(fx_shift(xr[i], np));
+        p.im[i] = fx_split(fx_shift(xi[i], np));
     }
     FxForms f;
-    fx_forms(lxr, lxi, f);
+    fx_forms(p, f);
     const int et = ex + np;
     const FxBounds bd = fx_bounds(f, et, C);
     ok = ok && bd.beta <= kFxBetaMax;
@@ -173,7 +171,7 @@ __device__ __forceinline__ bool fx_vjp_site(const cpx<double> a[5], const cpx<do
     FxW W;
     fx_build_w(p, f, et, C, W);
     i64 pc, ps;
-    const bool large = fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
+    fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
 
     i64 gr[5], gi[5], hr[5], hi[5];  // ga + gb, then ga - gb
 #pragma unroll
@@ -229,8 +227,7 @@ __device__ __forceinline__ bool fx_vjp_site(const cpx<double> a[5], const cpx<do
     FxAdjSlot kept[kFxAdjSlots];
 #pragma unroll 1
     for (int r = 0; r < 2; ++r) {  // one copy of the code for both vectors
-        if (large) fx_rotate_large(pc, -ps, gr, gi);
-        else fx_rotate(pc, -ps, gr, gi);  // lambda_0 = e^{i theta} g
+        fx_rotate(pc, -ps, gr, gi);  // lambda_0 = e^{i theta} g
         // forward sweep
         i64 vr[5], vi[5];
         cpx<float> xf[5], vf[5];

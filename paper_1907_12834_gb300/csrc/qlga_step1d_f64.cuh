@@ -220,10 +220,6 @@ __global__ void __launch_bounds__(32) k_step1d_f64(const double* __restrict__ in
 // sub-partition waits for instructions half of its time on the code of the one-lane form).
 // us a step with 10 / 5 / 1 lanes: 1024 sites 4.7 / 6.0 / 11.4, 16384 13.0 / 9.9 / 12.1, 65536 43 / 25 / 19.
 
-__device__ __forceinline__ FxOp fx_shfl(FxOp v, int src) {
-    return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.hf, src), __shfl_sync(0xffffffffu, v.lf, src)};
-}
-
 __device__ __forceinline__ Limb fx_shfl(Limb v, int src) {
     return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.l, src)};
 }
@@ -280,43 +276,43 @@ __device__ __noinline__ int fx_lane_kinetic_wide(const double* in, int L, int j,
 
 // The lane's share of delta W (FxW): y_m = D x_m + conj(u_m) G + conj(up) x_{m+1} + dn x_{m-1}
 struct FxWLane {
-    FxOp D, upr, upi, dnr, dni, ur, ui;
+    Limb D, upr, upi, dnr, dni, ur, ui;
     Limb R;
     float Rf;
 };
 
 // t <- -i delta W t of NV vectors, one component a lane
 template <int NV>
-__device__ __forceinline__ void fx_lane_apply(const FxWLane& W, const FxGroup& g, const FxOp (&tr)[NV], const FxOp (&ti)[NV],
+__device__ __forceinline__ void fx_lane_apply(const FxWLane& W, const FxGroup& g, const Limb (&tr)[NV], const Limb (&ti)[NV],
                                               i64 (&outr)[NV], i64 (&outi)[NV]) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        const FxOp ar = fx_shfl(tr[v], g.up()), ai = fx_shfl(ti[v], g.up());
-        const FxOp br = fx_shfl(tr[v], g.down()), bi = fx_shfl(ti[v], g.down());
-        FxAccF dr = {0, 0.f}, di = {0, 0.f};
+        const Limb ar = fx_shfl(tr[v], g.up()), ai = fx_shfl(ti[v], g.up());
+        const Limb br = fx_shfl(tr[v], g.down()), bi = fx_shfl(ti[v], g.down());
+        FxAcc dr = fx_zero<60>(), dn = {0, 0}, di = fx_zero<60>();
         fx_mac(dr, W.ur, tr[v]);
-        fx_mac(dr, fx_neg(W.ui), ti[v]);
+        fx_mac(dn, W.ui, ti[v]);
         fx_mac(di, W.ur, ti[v]);
         fx_mac(di, W.ui, tr[v]);
-        const FxOp Gr = fx_op(fx_mul_full<55>(W.R, fx_split(g.sum(fx_sum<60, 1>(dr)))));
-        const FxOp Gi = fx_op(fx_mul_full<55>(W.R, fx_split(g.sum(fx_sum<60, 1>(di)))));
-        FxAccF yr = {0, 0.f}, yi = {0, 0.f};
+        const Limb Gr = fx_split(fx_mul_full<55>(W.R, fx_split(g.sum(fx_sum<60>(dr - dn)))));
+        const Limb Gi = fx_split(fx_mul_full<55>(W.R, fx_split(g.sum(fx_sum<60>(di)))));
+        FxAcc yr = fx_zero<61>(), yi = fx_zero<61>(), nr = {0, 0}, ni = {0, 0};
         fx_mac(yr, W.D, tr[v]);
         fx_mac(yi, W.D, ti[v]);
         fx_mac(yr, W.ur, Gr);
         fx_mac(yr, W.ui, Gi);
         fx_mac(yi, W.ur, Gi);
-        fx_mac(yi, W.ui, fx_neg(Gr));
+        fx_mac(ni, W.ui, Gr);
         fx_mac(yr, W.upr, ar);
         fx_mac(yr, W.upi, ai);
         fx_mac(yi, W.upr, ai);
-        fx_mac(yi, fx_neg(W.upi), ar);
+        fx_mac(ni, W.upi, ar);
         fx_mac(yr, W.dnr, br);
-        fx_mac(yr, fx_neg(W.dni), bi);
+        fx_mac(nr, W.dni, bi);
         fx_mac(yi, W.dnr, bi);
         fx_mac(yi, W.dni, br);
-        outr[v] = fx_sum<61, 2>(yi);
-        outi[v] = -fx_sum<61, 2>(yr);
+        outr[v] = fx_sum<61>(yi - ni);
+        outi[v] = -fx_sum<61>(yr - nr);
     }
 }
 
@@ -388,7 +384,6 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
     const int nd = nd0 + 1 > np ? nd0 + 1 : np;
     int e = E - 1022 - 55;
     const Limb lpr = fx_split(fx_shift(pr, np)), lpi = fx_split(fx_shift(pi, np));
-    const FxOp opr = fx_op(lpr), opi = fx_op(lpi);
     FxForms f;
     FxAcc nn = fx_zero<60>();
     fx_mac(nn, lpr, lpr);
@@ -400,12 +395,12 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
     const Limb r32m1 = fx_split(kFxR32m1);
     {
         const Limb ur = fx_shfl(lpr, g.up()), ui = fx_shfl(lpi, g.up());
-        FxAcc a = fx_zero<60>(), b = fx_zero<60>();
+        FxAcc a = fx_zero<60>(), b = fx_zero<60>(), n = {0, 0};
         fx_mac(a, lpr, ur);
         fx_mac(a, lpi, ui);
         fx_mac(b, lpr, ui);
-        fx_mac(b, fx_neg(lpi), ur);
-        i64 fr = fx_sum<60>(a), fi = fx_sum<60>(b);
+        fx_mac(n, lpi, ur);
+        i64 fr = fx_sum<60>(a), fi = fx_sum<60>(b - n);
         if (g.m == 1 || g.m == 2) {
             fr += fx_mul(r32m1, fx_split(fr));
             fi += fx_mul(r32m1, fx_split(fi));
@@ -422,21 +417,22 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
     FxWLane W;
     {
         const i64 gz = fx_coupled(C.fx.dz, f.Fz, et, 0), g2r = fx_coupled(C.fx.dr, f.rho, et, 0);
-        W.D = fx_op((2 - g.m) * gz - g2r);
+        W.D = fx_split((2 - g.m) * gz - g2r);
         const i64 er = fx_coupled(C.fx.e0, f.Fpr, et, 1), ei = fx_coupled(C.fx.e0, f.Fpi, et, 1);
         const i64 er1 = er + fx_mul(r32m1, fx_split(er)), ei1 = ei + fx_mul(r32m1, fx_split(ei));
         const bool s_up = g.m == 0 || g.m == 3, s_dn = g.m == 1 || g.m == 4;
-        W.upr = fx_op(g.m == 4 ? 0 : (s_up ? er : er1));
-        W.upi = fx_op(g.m == 4 ? 0 : (s_up ? ei : ei1));
-        W.dnr = fx_op(g.m == 0 ? 0 : (s_dn ? er : er1));
-        W.dni = fx_op(g.m == 0 ? 0 : (s_dn ? ei : ei1));
-        const FxOp mr = fx_shfl(opr, g.base + 4 - g.m), mi = fx_shfl(opi, g.base + 4 - g.m);
-        W.ur = (g.m & 1) ? fx_neg(mr) : mr;
-        W.ui = (g.m & 1) ? fx_neg(mi) : mi;
+        W.upr = fx_split(g.m == 4 ? 0 : (s_up ? er : er1));
+        W.upi = fx_split(g.m == 4 ? 0 : (s_up ? ei : ei1));
+        W.dnr = fx_split(g.m == 0 ? 0 : (s_dn ? er : er1));
+        W.dni = fx_split(g.m == 0 ? 0 : (s_dn ? ei : ei1));
+        const Limb mr = fx_shfl(lpr, g.base + 4 - g.m), mi = fx_shfl(lpi, g.base + 4 - g.m);
+        auto turned = [&](Limb v) { return (g.m & 1) ? fx_split(-(v.h * (i64(1) << 32) + v.l)) : v; };
+        W.ur = turned(mr);
+        W.ui = turned(mi);
         fx_singlet(C.fx, et, W.R, W.Rf);
     }
     i64 pc, ps;
-    const bool large = fx_site_phase(f.rho, et, bd.theta, C.fx, pc, ps);
+    fx_site_phase(f.rho, et, bd.theta, C.fx, pc, ps);
     i64 xr[NV], xi[NV];
     if constexpr (NV == 2) {
         xr[0] = fx_shift(pr, nd);
@@ -447,30 +443,27 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
         xr[0] = fx_shift(chain ? dr : pr, nd);
         xi[0] = fx_shift(chain ? di : pi, nd);
     }
-    FxOp tr[NV], ti[NV];
+    Limb tr[NV], ti[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-        tr[i] = fx_op(xr[i]);
-        ti[i] = fx_op(xi[i]);
+        tr[i] = fx_split(xr[i]);
+        ti[i] = fx_split(xi[i]);
     }
 #pragma unroll 1
     for (int k = 1; k <= kA; ++k) {
         i64 nr[NV], ni[NV];
         fx_lane_apply<NV>(W, g, tr, ti, nr, ni);
-        const FxOp fk = fx_op(fx_inv_fact(k));
+        const Limb fk = fx_inv_fact(k);
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-            tr[i] = fx_op(nr[i]);
-            ti[i] = fx_op(ni[i]);
+            tr[i] = fx_split(nr[i]);
+            ti[i] = fx_split(ni[i]);
             if (k <= 2) {
                 xr[i] += k == 1 ? nr[i] : (nr[i] + 1) >> 1;
                 xi[i] += k == 1 ? ni[i] : (ni[i] + 1) >> 1;
             } else {
-                FxAccF a = {0, 0.f}, b = {0, 0.f};
-                fx_mac(a, fk, tr[i]);
-                fx_mac(b, fk, ti[i]);
-                xr[i] += fx_sum<61, 0>(a);
-                xi[i] += fx_sum<61, 0>(b);
+                xr[i] += fx_mul(fk, tr[i]);
+                xi[i] += fx_mul(fk, ti[i]);
             }
         }
     }
@@ -514,8 +507,7 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
     }
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-        if (large) fx_rotate_large<1>(pc, ps, &xr[i], &xi[i]);
-        else fx_rotate<1>(pc, ps, &xr[i], &xi[i]);
+        fx_rotate<1>(pc, ps, &xr[i], &xi[i]);
     }
     e += nd - 5;  // 0.5 / 16
     double2* dst = reinterpret_cast<double2*>(out) + 2 * (int64_t(g.m) * L + j);

@@ -19,13 +19,13 @@ double host_density(const double* psi) {
         im[i] = fx_from_double<60>(psi[2 * i + 1], E);
     }
     const int n = fx_headroom(re, im);
-    Limb lr[5], li[5];
+    FxVec p;
     for (int i = 0; i < 5; ++i) {
-        lr[i] = fx_split(fx_shift(re[i], n));
-        li[i] = fx_split(fx_shift(im[i], n));
+        p.re[i] = fx_split(fx_shift(re[i], n));
+        p.im[i] = fx_split(fx_shift(im[i], n));
     }
     FxForms f;
-    fx_forms(lr, li, f);
+    fx_forms(p, f);
     return std::ldexp(double(f.rho), 2 * (E - 1022 - 60 + n) + 60);
 }
 

@@ -120,3 +120,20 @@ def test_density_is_not_biased(lib):
     rho, _, _ = forms(p.astype(np.clongdouble))
     err = ((got - rho) / rho).astype(np.float64)
     assert abs(err.mean()) <= 2.0 ** -55, err.mean()
+
+
+@pytest.mark.parametrize("g", [(1.0, 0.0, 0.0), (1.0, 0.1, 1.0), (0.0, 0.8, -0.6)])
+def test_sites_of_one_density_share_no_phase(lib, g):
+    """The mean phase of U's error over 400 sites of one density: a rounding of the phase or of W's diagonal that sites
+    share would add up over a run's steps.  Tolerance 1.2e-17: the couplings' own rounding, up to four products of 2^-54
+    of themselves at theta and beta below 0.03 (7e-18), and twice the mean's scatter (2^-54 / sqrt(4000))."""
+    rng = np.random.default_rng(17)
+    for rho in np.exp(rng.uniform(np.log(0.002), np.log(0.02), 12)):
+        x = sites(rng, 400)
+        p = x.sum(axis=2, keepdims=True)
+        x = (0.5 * p + 0.25 * (x - x[:, :, ::-1])) * np.sqrt(rho / (np.abs(p) ** 2).sum(axis=(1, 2), keepdims=True))
+        got, ok = potential(lib, x, g)
+        ref = reference(x, g)
+        assert ok.all()
+        phase = float((ref.conj() * (got - ref)).imag.sum() / (np.abs(ref) ** 2).sum())
+        assert abs(phase) <= 1.2e-17, (rho, phase)
