@@ -1382,10 +1382,11 @@ void step1d_f64_launch(const TileArgs& a) {
     auto launch_lanes = [&](auto kernel, int sites) {
         kernel<<<(L + sites - 1) / sites, 32, 0, a.stream>>>(static_cast<const double*>(a.in), static_cast<double*>(a.out), L, pc, a.status);
     };
-    // us a step (two solitons, g = (1, 0.8, -0.6)) with 10 / 5 / 1 lanes per site: 1024 sites 4.7 / 6.0 / 11.4,
-    // 4096 5.6 / 5.7 / 12.2, 6000 6.9 / 6.3 / 12.0, 16384 13.0 / 9.9 / 12.1, 24000 17.6 / 11.8 / 12.1, 32768 22.6 / 14.8 / 13.0
+    // us a step (two solitons, g = (1, 0.8, -0.6)) with 10 / 5 / 1 lanes per site: 1024 sites 6.6 / 7.8 / 18.1,
+    // 4096 7.3 / 7.8 / 18.5, 6000 9.8 / 8.0 / 18.5, 16384 18.6 / 13.2 / 18.8, 24000 25.9 / 16.3 / 19.5, 32768 33.4 / 20.4 / 20.6,
+    // 65536 64 / 36 / 30
     if (a.pot && L <= 4096) a.variant == 0 ? launch_lanes(k_step1d_f64_lanes<0, 10>, 3) : launch_lanes(k_step1d_f64_lanes<1, 10>, 3);
-    else if (a.pot && L <= 24000) a.variant == 0 ? launch_lanes(k_step1d_f64_lanes<0, 5>, 6) : launch_lanes(k_step1d_f64_lanes<1, 5>, 6);
+    else if (a.pot && L <= 32000) a.variant == 0 ? launch_lanes(k_step1d_f64_lanes<0, 5>, 6) : launch_lanes(k_step1d_f64_lanes<1, 5>, 6);
     else if (a.variant == 0) a.pot ? launch(k_step1d_f64<0, true>) : launch(k_step1d_f64<0, false>);
     else a.pot ? launch(k_step1d_f64<1, true>) : launch(k_step1d_f64<1, false>);
 }

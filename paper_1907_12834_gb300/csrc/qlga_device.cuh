@@ -285,7 +285,7 @@ struct PotConst<double> : PotConstBase<double> {
     FixPot fx;  // the same for the fixed-point form
     PotConst() = default;
     __host__ explicit PotConst(const PotParams& P)
-        : PotConstBase<double>(P), fx(cphase, dz, dr, e0, R, b1, b2) {}
+        : PotConstBase<double>(P), fx(cphase, dz, dr, e0, R) {}
 };
 
 // 1/k, k = 0..kTaylorMax+1 (entry 0 unused): Taylor coefficients without divisions.

@@ -3,26 +3,31 @@
 // GB300 issues one FP64 instruction per SM sub-partition every 64-76 cycles (measured: DFMA 64, DADD and
 // DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4, a
 // 64-bit addition every 2.4 and an FP32 multiply-add every cycle.  A product of two fixed-point numbers
-// takes three of the first, so U on a site costs a quarter of its FP64 form, at a finer
-// resolution: relative to the site's largest component the operands carry 2^-58, where FP64 rounds
+// takes three of the first, so U on a site costs 40% of its FP64 form (1024^2 sites of a vortex lattice: 0.71 ms,
+// against about 1.7), at a finer resolution: the operands carry 2^-57 of their level, where FP64 rounds
 // every operation at 2^-53 of its own result.
 //
-// Numbers.  A site's psi = a + b and d = a - b are int64 with one exponent per vector, psi's largest
-// component in [2^57, 2^58).  An operand of a product is split as v = h 2^32 + l, l the low word
+// Numbers.  Level m of the vectors psi = a + b and d = a - b is a pair of int64 in units of 2^(T_m - 57), with one
+// exponent T_m for both vectors: their moduli lie below 2^T_m.  delta W acts between the scaled levels, entry (m, j)
+// times 2^(T_j - T_m), in 2^61 = 1; its entries come from psi's own mantissas and exponents, so that no level
+// takes its resolution from another (seeds of spin mixing lie many orders of magnitude below the field; with one
+// exponent for the site a level at 1e-10 of it kept 1e-7 of its own size).  Where W would add more to a
+// level than it holds, T_m is raised to that (fx_budget): FP64, too, rounds the level at what it receives.
+// An operand of a product is split as v = h 2^32 + l, l the low word
 // taken as signed; h h' and h l' + l h' are summed in 64-bit accumulators, and l l' (zero mean,
-// below 2^62) is dropped but in the squares of the density.  The entries of delta W and the phase are fixed point with
-// 2^61 = 1.  (Cross terms in FP32 are 13% of a 1024^2 step, 5.65 against 6.54 ms for ten with load and read-out, but round the
-// low limb of an entry to 24 bits: the phase and W's diagonal, which sites of one density share, were
+// below 2^62) is dropped but in the squares of the density.  (Cross terms in FP32 rounded the low limb of an
+// entry to 24 bits: the phase and W's diagonal, which sites of one density share, were
 // off by up to 2^-55 whatever their size, 7e-17 a step of a run's phase.)
+// The error of a level is 0.36 of 2^-53 (root mean square, of its size and what reaches it), that of the same sum in
+// FP64 0.46, from levels of one size to seeds of 1e-40.
 //
 // U = e^{-i delta c} exp(-i delta W) as in potential_site, by the plain Taylor sum: the terms
-// T_k = (-i delta W)^k x are formed in fixed point up to the order k0 - 1 whose successor is bounded
-// by beta^k0 / k0! <= 2^-31 and added as T_k / k!; the terms from k0 on, so small that FP32 carries
-// them to 2^-54 of the site, continue in FP32 to a bound of 2^-57.  The phase is applied as v + (e^{-i delta c} - 1) v.
+// T_k = (-i delta W)^k x are formed in fixed point until the next one is below 2^-31 and added as T_k / k!; the terms from
+// there on, so small that FP32 carries them to 2^-54 of the level, continue in FP32 to a bound of 2^-57.  The phase is
+// applied as v + (e^{-i delta c} - 1) v.
 //
-// Domain.  beta <= 0.25 and finite components below 2^60; a warp with a lane outside it (among them
-// every site that the status word reports) takes the FP64 code.  Components below 2^-59 of the
-// site's largest one, and sites below 2^-850, round to zero.
+// Domain.  The scaled delta W has a norm of at most 1, components are finite and below 2^60, and a level is empty
+// or above 2^-930; a warp with a lane outside it (among them every site that the status word reports) takes the FP64 code.
 #pragma once
 
 #include <cmath>
@@ -42,6 +47,7 @@ struct Limb {
     int h, l;  // h 2^32 + l
 };
 
+QLGA_HD i64 fx_join(Limb a) { return a.h * (i64(1) << 32) + a.l; }
 QLGA_HD Limb fx_split(i64 v) {  // the low limb is the low word as it stands, the high one takes its sign
     return {int(v >> 32) + int(unsigned(v) >> 31), int(unsigned(v))};
 }
@@ -128,14 +134,14 @@ struct FxConst {
     }
 };
 
-// The potential's constants (those of PotConst, qlga_device.cuh) for the fixed-point form.
+// The potential's constants (those of PotConst, qlga_device.cuh) for the fixed-point form
 struct FixPot {
     FxConst cphase, dz, dr, e0, R;
-    float b1, b2, cphase_f, R_f;
+    float cphase_f, dz_f, dr_f, R_log;
     FixPot() = default;
-    __host__ FixPot(double cphase_, double dz_, double dr_, double e0_, double R_, double b1_, double b2_)
-        : cphase(cphase_), dz(dz_), dr(dr_), e0(e0_), R(R_), b1(float(b1_)), b2(float(b2_)), cphase_f(float(cphase_)),
-          R_f(float(R_)) {}
+    __host__ FixPot(double cphase_, double dz_, double dr_, double e0_, double R_)
+        : cphase(cphase_), dz(dz_), dr(dr_), e0(e0_), R(R_), cphase_f(float(cphase_)), dz_f(float(dz_)), dr_f(float(dr_)),
+          R_log(R_ == 0.0 ? -100000.f : float(std::log2(std::fabs(R_)))) {}
 };
 
 struct FxCpxF {
@@ -210,7 +216,7 @@ QLGA_HD double fx_pow2(int e) { return fx_bits(unsigned(e + 1023) << 20, 0u); } 
 
 // The biased exponent that a set of doubles is converted with: m is the largest high word without
 // sign; every |x| < 2^(E - 1022).  kFxMinExp: smaller sets round to zero.
-constexpr int kFxMinExp = 1022 - 850;
+constexpr int kFxMinExp = 1022 - 930;
 QLGA_HD int fx_exponent(unsigned m) {
     const int e = int(m >> 20);
     return e > kFxMinExp ? e : kFxMinExp;
@@ -262,37 +268,60 @@ struct FxVec {
     Limb re[5], im[5];
 };
 
-// Shift that brings the largest of the ten components of (re, im) to [2^57, 2^58): v -> v 2^(-n).
-// Returns n (components below 2^62; all zero: -57).
-QLGA_HD int fx_headroom(const i64 re[5], const i64 im[5]) {
-    unsigned long long m = 0;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) m |= static_cast<unsigned long long>(re[i] ^ (re[i] >> 63)) | static_cast<unsigned long long>(im[i] ^ (im[i] >> 63));
-    return m ? 6 - fx_clz(m) : -57;  // 64 - clz bits now, 58 wanted
-}
-QLGA_HD i64 fx_shift(i64 v, int n) { return fx_scale(v, -n); }  // v 2^(-n), n in [-57, 5] (|v| < 2^(58 + n) and 2^62)
+constexpr int kFxNone = -100000;  // the exponent of an empty level
+constexpr int kFxFloor = -950;    // the smallest exponent of a level of a vector
 
-// delta W of a site in fixed point (2^61 = 1)
+// Bits of the larger of two integers' magnitudes (one's complement)
+QLGA_HD int fx_bits_of(i64 a, i64 b) {
+    const i64 m = (a ^ (a >> 63)) | (b ^ (b >> 63));
+    return m ? 64 - fx_clz(m) : 0;
+}
+QLGA_HD int fx_max(int a, int b) { return a > b ? a : b; }
+QLGA_HD int fx_clamp(int n, int lo, int hi) { return n < lo ? lo : (n > hi ? hi : n); }
+QLGA_HD float fx_pow2f(int n) {  // 2^n, clamped to the normal range
+    n = fx_clamp(n, -126, 127);
+    union {
+        unsigned u;
+        float f;
+    } p;
+    p.u = unsigned(n + 127) << 23;
+    return p.f;
+}
+// v 2^n for any n (the caller knows that it fits)
+QLGA_HD i64 fx_scale_any(i64 v, int n) { return fx_scale(v, fx_max(n, -63)); }
+
+// A field by levels: psi_m = (re, im) 2^(e - 58), the mantissas below 2^58 and the larger one in [2^57, 2^58)
+struct FxLevels {
+    FxVec p;
+    int e[5];
+};
+QLGA_HD void fx_level(i64 re, i64 im, int unit, Limb& lr, Limb& li, int& e) {  // of (re, im) 2^unit, below 2^62
+    const int b = fx_bits_of(re, im);
+    lr = fx_split(fx_scale(re, 58 - b));
+    li = fx_split(fx_scale(im, 58 - b));
+    e = b ? unit + b : kFxNone;
+}
+
+// delta W of a site, between vectors whose level m is (re, im) 2^(T_m - 57): entry (m, j) times 2^(T_j - T_m), in
+// 2^61 = 1.  The singlet term is conj(u_m) times the sum of v_j x_j (2^58 = 1).
 struct FxW {
     Limb D[5];
-    Limb e0r, e0i, e1r, e1i;  // delta g1 F_+ times 1 and sqrt(3/2)
-    FxVec u;                  // u_j = (-1)^j psi_{4-j}
-    Limb R;                   // delta g2 / 5: G = R dot / 2^55
-    float Rf;
+    Limb upr[4], upi[4];  // row m + 1, from m: delta g1 c F_+
+    Limb dnr[4], dni[4];  // row m, from m + 1: its conjugate
+    FxVec u, v;
 };
 
 // t <- -i delta W t
 QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
-    FxAcc tp = fx_zero<60>(), tn = {0, 0}, ti = fx_zero<60>();
+    FxAcc tp = fx_zero<58>(), tn = {0, 0}, ti = fx_zero<58>();
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-        fx_mac(tp, W.u.re[j], t.re[j]);
-        fx_mac(tn, W.u.im[j], t.im[j]);
-        fx_mac(ti, W.u.re[j], t.im[j]);
-        fx_mac(ti, W.u.im[j], t.re[j]);
+        fx_mac(tp, W.v.re[j], t.re[j]);
+        fx_mac(tn, W.v.im[j], t.im[j]);
+        fx_mac(ti, W.v.re[j], t.im[j]);
+        fx_mac(ti, W.v.im[j], t.re[j]);
     }
-    const Limb Gr = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(tp - tn))));
-    const Limb Gi = fx_split(fx_mul_full<55>(W.R, fx_split(fx_sum<60>(ti))));
+    const Limb Gr = fx_split(fx_sum<58>(tp - tn)), Gi = fx_split(fx_sum<58>(ti));
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         // y = (W t)_i; o = -i y: o.re = y.im, o.im = -y.re
@@ -303,21 +332,17 @@ QLGA_HD void fx_apply(const FxW& W, const FxVec& t, i64 ore[5], i64 oim[5]) {
         fx_mac(yr, W.u.im[i], Gi);
         fx_mac(yi, W.u.re[i], Gi);
         fx_mac(ni, W.u.im[i], Gr);
-        if (i > 0) {  // e t_{i-1}
-            const bool s = i == 1 || i == 4;
-            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
-            fx_mac(yr, er, t.re[i - 1]);
-            fx_mac(nr, ei, t.im[i - 1]);
-            fx_mac(yi, er, t.im[i - 1]);
-            fx_mac(yi, ei, t.re[i - 1]);
+        if (i > 0) {
+            fx_mac(yr, W.upr[i - 1], t.re[i - 1]);
+            fx_mac(nr, W.upi[i - 1], t.im[i - 1]);
+            fx_mac(yi, W.upr[i - 1], t.im[i - 1]);
+            fx_mac(yi, W.upi[i - 1], t.re[i - 1]);
         }
-        if (i < 4) {  // conj(e) t_{i+1}
-            const bool s = i == 0 || i == 3;
-            const Limb er = s ? W.e0r : W.e1r, ei = s ? W.e0i : W.e1i;
-            fx_mac(yr, er, t.re[i + 1]);
-            fx_mac(yr, ei, t.im[i + 1]);
-            fx_mac(yi, er, t.im[i + 1]);
-            fx_mac(ni, ei, t.re[i + 1]);
+        if (i < 4) {  // the entry is the conjugate
+            fx_mac(yr, W.dnr[i], t.re[i + 1]);
+            fx_mac(yr, W.dni[i], t.im[i + 1]);
+            fx_mac(yi, W.dnr[i], t.im[i + 1]);
+            fx_mac(ni, W.dni[i], t.re[i + 1]);
         }
         ore[i] = fx_sum<61>(yi - ni);
         oim[i] = -fx_sum<61>(yr - nr);
@@ -344,14 +369,14 @@ QLGA_HD float fx_inv(int k) {
 #endif
 }
 
-constexpr float kFxBetaMax = 0.25f;
+constexpr float kFxNormMax = 1.f;  // of delta W between the scaled vectors
 // Truncation of the Taylor sums, relative to the site: the same terms are missing from step to step, so
 // the bound is a sixteenth of FP64's 2^-53 (a term of the FP32 part costs 2% of U).  Orders whose bound is
 // above kFxTolF run in fixed point.
 constexpr float kFxTol = 6.9388939e-18f;   // 2^-57
 constexpr float kFxTolF = 4.6566129e-10f;  // 2^-31
 
-// Smallest K with beta^(K+1)/(K+1)! <= tol (beta <= 1: at most 19 for 2^-57)
+// Smallest K with beta^(K+1)/(K+1)! <= tol (beta <= 1: at most 19 for 2^-57, 12 for 2^-31)
 QLGA_HD int fx_degree(float beta, float tol) {
     int K = 0;
     float term = beta;
@@ -362,46 +387,74 @@ QLGA_HD int fx_degree(float beta, float tol) {
     return K;
 }
 
-// t <- (-i / k) delta W t in FP32
-QLGA_HD void fx_apply_f(const FxW& W, const FxCpxF u[5], const FxCpxF t[5], FxCpxF o[5], float ik) {
-    float ar = 0.f, ai = 0.f;
+// The same matrix in FP32
+struct FxWF {
+    float D[5];
+    FxCpxF up[4], dn[4], u[5], v[5];
+    QLGA_HD explicit FxWF(const FxW& W) {
+        const float s58 = 3.4694470e-18f, s61 = 4.3368087e-19f;  // 2^-58, 2^-61
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            D[i] = fx_float(W.D[i], s61);
+            u[i] = {fx_float(W.u.re[i], s61), fx_float(W.u.im[i], s61)};
+            v[i] = {fx_float(W.v.re[i], s58), fx_float(W.v.im[i], s58)};
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            up[i] = {fx_float(W.upr[i], s61), fx_float(W.upi[i], s61)};
+            dn[i] = {fx_float(W.dnr[i], s61), fx_float(W.dni[i], s61)};
+        }
+    }
+};
+QLGA_HD FxCpxF fx_dot_f(const FxWF& W, const FxCpxF t[5]) {
+    FxCpxF a = {0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-        ar = fmaf(u[j].re, t[j].re, fmaf(-u[j].im, t[j].im, ar));
-        ai = fmaf(u[j].re, t[j].im, fmaf(u[j].im, t[j].re, ai));
+        a.re = fmaf(W.v[j].re, t[j].re, fmaf(-W.v[j].im, t[j].im, a.re));
+        a.im = fmaf(W.v[j].re, t[j].im, fmaf(W.v[j].im, t[j].re, a.im));
     }
-    const float gr = W.Rf * ar, gi = W.Rf * ai;
-    const float s61 = 4.3368087e-19f;  // 2^-61
-    const float e0rf = fx_float(W.e0r, s61), e0if = fx_float(W.e0i, s61);
-    const float e1rf = fx_float(W.e1r, s61), e1if = fx_float(W.e1i, s61);
+    return a;
+}
+// o <- (-i ik) delta W t, with the dot product of v and t
+QLGA_HD void fx_apply_f(const FxWF& W, const FxCpxF t[5], FxCpxF g, FxCpxF o[5], float ik) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const float Df = fx_float(W.D[i], s61);
-        float yr = fmaf(Df, t[i].re, fmaf(u[i].re, gr, u[i].im * gi));
-        float yi = fmaf(Df, t[i].im, fmaf(u[i].re, gi, -u[i].im * gr));
+        float yr = fmaf(W.D[i], t[i].re, fmaf(W.u[i].re, g.re, W.u[i].im * g.im));
+        float yi = fmaf(W.D[i], t[i].im, fmaf(W.u[i].re, g.im, -W.u[i].im * g.re));
         if (i > 0) {
-            const bool s = i == 1 || i == 4;
-            const float er = s ? e0rf : e1rf, ei = s ? e0if : e1if;
-            yr = fmaf(er, t[i - 1].re, fmaf(-ei, t[i - 1].im, yr));
-            yi = fmaf(er, t[i - 1].im, fmaf(ei, t[i - 1].re, yi));
+            const FxCpxF e = W.up[i - 1];
+            yr = fmaf(e.re, t[i - 1].re, fmaf(-e.im, t[i - 1].im, yr));
+            yi = fmaf(e.re, t[i - 1].im, fmaf(e.im, t[i - 1].re, yi));
         }
         if (i < 4) {
-            const bool s = i == 0 || i == 3;
-            const float er = s ? e0rf : e1rf, ei = s ? e0if : e1if;
-            yr = fmaf(er, t[i + 1].re, fmaf(ei, t[i + 1].im, yr));
-            yi = fmaf(er, t[i + 1].im, fmaf(-ei, t[i + 1].re, yi));
+            const FxCpxF e = W.dn[i];
+            yr = fmaf(e.re, t[i + 1].re, fmaf(e.im, t[i + 1].im, yr));
+            yi = fmaf(e.re, t[i + 1].im, fmaf(-e.im, t[i + 1].re, yi));
         }
         o[i] = {ik * yi, -ik * yr};
     }
 }
 
-// The quadratic forms of psi (unit 2^(2 e + 60) for components of unit 2^e)
+// The quadratic forms of psi: rho and F_z in units of 2^(en - 56), F_+ / 2 = (fr, fi) 2^(fe - 56) and
+// delta g1 F_+ = (er, ei) 2^(ee - 60), the larger of the two in [2^59, 2^60) in magnitude.  Each is good to 2^-57 of the
+// largest of its terms.
 struct FxForms {
-    i64 rho, Fz, Fpr, Fpi;  // F_+ = 2 (Fpr + i Fpi)
+    i64 rho, Fz, fr, fi, er, ei;
+    int en, fe, ee;
 };
+QLGA_HD void fx_coupled_spin(const FxConst& e0, FxForms& f) {  // (er, ei) from (fr, fi), below 2^60
+    f.er = fx_mul_full<60>(e0.m, fx_split(f.fr));
+    f.ei = fx_mul_full<60>(e0.m, fx_split(f.fi));
+    const int b = fx_bits_of(f.er, f.ei);
+    f.er = fx_scale(f.er, 60 - b);
+    f.ei = fx_scale(f.ei, 60 - b);
+    f.ee = b ? b + e0.ex + f.fe - 55 : kFxNone;
+}
 
-QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
-    const Limb *re = p.re, *im = p.im;
+QLGA_HD void fx_forms(const FxLevels& psi, const FixPot& C, FxForms& f) {
+    const Limb *re = psi.p.re, *im = psi.p.im;
+    const int* e = psi.e;
+    f.en = 2 * fx_max(fx_max(fx_max(e[0], e[1]), fx_max(e[2], e[3])), e[4]);
     i64 n[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {  // with l l': of a square it has no zero mean
@@ -409,39 +462,30 @@ QLGA_HD void fx_forms(const FxVec& p, FxForms& f) {
         fx_mac(s, re[i], re[i]);
         fx_mac(s, im[i], im[i]);
         s.mid += (fx_mad(re[i].l, re[i].l, 0) >> 32) + (fx_mad(im[i].l, im[i].l, 0) >> 32);
-        n[i] = fx_sum<60>(s);
+        n[i] = fx_scale_any(fx_sum<60>(s), 2 * e[i] - f.en);
     }
     f.rho = (n[0] + n[1]) + (n[2] + n[3]) + n[4];
     f.Fz = 2 * (n[0] - n[4]) + (n[1] - n[3]);
-    i64 fr[2], fi[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {  // conj(p0) p1 + conj(p3) p4, then conj(p1) p2 + conj(p2) p3
-        const int a = q, b = q == 0 ? 3 : 2;
-        FxAcc r = fx_zero<60>(), i = fx_zero<60>(), n = {0, 0};
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int j = k ? b : a;
-            fx_mac(r, re[j], re[j + 1]);
-            fx_mac(r, im[j], im[j + 1]);
-            fx_mac(i, re[j], im[j + 1]);
-            fx_mac(n, im[j], re[j + 1]);
-        }
-        fr[q] = fx_sum<60>(r);
-        fi[q] = fx_sum<60>(i - n);
-    }
+    f.fe = fx_max(fx_max(e[0] + e[1], e[1] + e[2]), fx_max(e[2] + e[3], e[3] + e[4]));
     const Limb r = fx_split(kFxR32m1);
-    f.Fpr = fr[0] + fr[1] + fx_mul(r, fx_split(fr[1]));
-    f.Fpi = fi[0] + fi[1] + fx_mul(r, fx_split(fi[1]));
-}
-
-QLGA_HD float fx_pow2f(int n) {  // 2^n, clamped to the normal range
-    n = n < -126 ? -126 : (n > 127 ? 127 : n);
-    union {
-        unsigned u;
-        float f;
-    } p;
-    p.u = unsigned(n + 127) << 23;
-    return p.f;
+    f.fr = f.fi = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // c conj(psi_i) psi_{i+1}
+        FxAcc a = fx_zero<60>(), b = fx_zero<60>(), c = {0, 0};
+        fx_mac(a, re[i], re[i + 1]);
+        fx_mac(a, im[i], im[i + 1]);
+        fx_mac(b, re[i], im[i + 1]);
+        fx_mac(c, im[i], re[i + 1]);
+        const int sh = e[i] + e[i + 1] - f.fe;
+        i64 x = fx_scale_any(fx_sum<60>(a), sh), y = fx_scale_any(fx_sum<60>(b - c), sh);
+        if (i == 1 || i == 2) {
+            x += fx_mul(r, fx_split(x));
+            y += fx_mul(r, fx_split(y));
+        }
+        f.fr += x;
+        f.fi += y;
+    }
+    fx_coupled_spin(C.e0, f);
 }
 
 // e^{-i theta} - 1 = (-c, -s), theta and the results in 2^61 = 1, |theta| <= 1/4: the Taylor series of
@@ -460,76 +504,207 @@ QLGA_HD void fx_phase(i64 theta, i64& c, i64& s) {
     c = fx_mul(q, fx_split(c1));
 }
 
-// What the warp decides from: beta and theta of a lane (as upper bounds)
-struct FxBounds {
-    float beta, theta;
+// c q 2^unit in 2^61 = 1 (below 2^62 in the domain)
+QLGA_HD i64 fx_coupled(const FxConst& c, i64 q, int unit) {
+    return fx_scale(fx_mul_full<60>(c.m, fx_split(q)), fx_clamp(c.ex + unit + 61, -63, 30));
+}
+
+// Sizes as logarithms to base 2
+constexpr float kFxLogNone = -100000.f;
+QLGA_HD float fx_log2(float x) {
+#ifdef __CUDA_ARCH__
+    return __log2f(x);
+#else
+    return log2f(x);
+#endif
+}
+QLGA_HD float fx_exp2(float x) {
+#ifdef __CUDA_ARCH__
+    return exp2f(x);
+#else
+    return ::exp2f(x);
+#endif
+}
+QLGA_HD float fx_log_of(i64 re, i64 im, int e) {  // of |(re, im)| 2^e, 0: none (components below 2^62)
+    const float a = 2.1684043e-19f * float(re), b = 2.1684043e-19f * float(im), q = fmaf(a, a, b * b);  // 2^-62
+    return q > 0.f ? fmaf(0.5f, fx_log2(q), float(e + 62)) : kFxLogNone;
+}
+
+// What bounds the entries of delta W: log2 of |psi_m|, |delta g1 F_+| and |delta g2 / 5|
+struct FxSizes {
+    float p[5], e, R;
 };
-QLGA_HD FxBounds fx_bounds(const FxForms& f, int e, const FixPot& C) {
-    // the forms in 2^61 = 1, times 2^(2 e + 121)
-    const float c = 4.3368087e-19f;
-    const float rho = fx_float(fx_split(f.rho), c), fz = fx_float(fx_split(f.Fz), c);
-    const float fr = 2.f * fx_float(fx_split(f.Fpr), c), fi = 2.f * fx_float(fx_split(f.Fpi), c);
-    const float F = sqrtf(fmaf(fz, fz, fmaf(fr, fr, fi * fi)));
-    const float u = 1.00001f * fx_pow2f(2 * e + 121);
-    FxBounds b;
-    b.beta = u * fmaf(C.b1, F, C.b2 * rho);
-    b.theta = u * fabsf(C.cphase_f) * rho;
-    return b;
+// log2 of the singlet term's row factor over |psi_{-m}|: |delta g2 / 5| sum_j |psi_{-j}| 2^L_j
+QLGA_HD float fx_log_dot(const FxSizes& z, const float L[5]) {
+    float g = z.p[4] + L[0];
+#pragma unroll
+    for (int j = 1; j < 5; ++j) g = fmaxf(g, z.p[4 - j] + L[j]);
+    float v = 0.f;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) v += fx_exp2(z.p[4 - j] + L[j] - g);
+    return z.R + g + fx_log2(v);
+}
+constexpr float kFxLogR32 = 0.29248125f;  // log2 sqrt(3/2)
+QLGA_HD float fx_log_link(const FxSizes& z, int i) { return i == 0 || i == 3 ? z.e : z.e + kFxLogR32; }  // (i, i + 1)
+
+// The exponents T of a vector's levels of sizes own (moduli below 2^T), raised until every entry of delta W off the
+// diagonal times 2^(T_j - T_m) is below 2^-margin, or what the field itself allows: a weak level that a strong
+// one drives takes a few times the size of what it receives in a step, which 2^-57 of still resolves
+// better than FP64 does.  In most fields nothing changes.
+QLGA_HD void fx_budget(const FxSizes& z, const float own[5], float margin, int T[5]) {
+    float L[5], pm = z.p[0];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        L[m] = own[m];
+        pm = fmaxf(pm, z.p[m]);
+    }
+    const float ke = fmaxf(0.f, fminf(margin, -kFxLogR32 - z.e)), ks = fmaxf(0.f, fminf(margin, -z.R - 2.f * pm));
+#pragma unroll 1
+    for (int it = 0; it < 8; ++it) {
+        const float g = fx_log_dot(z, L) + ks;
+        float N[5];
+        bool raised = false;
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+            N[m] = fmaxf(L[m], g + z.p[4 - m]);
+            if (m < 4) N[m] = fmaxf(N[m], fx_log_link(z, m) + ke + L[m + 1]);
+            if (m > 0) N[m] = fmaxf(N[m], fx_log_link(z, m - 1) + ke + L[m - 1]);
+            raised = raised || N[m] > L[m] + 0.01f;
+        }
+        if (!raised) break;
+#pragma unroll
+        for (int m = 0; m < 5; ++m) L[m] = N[m];
+    }
+#pragma unroll
+    for (int m = 0; m < 5; ++m) T[m] = int(ceilf(L[m] + 0.001f));
+}
+// The exponent of the dot product of v and a vector
+QLGA_HD int fx_dot_exp(const int P[5], const int T[5]) {
+    return fx_max(fx_max(fx_max(P[4] + T[0], P[0] + T[4]), fx_max(P[3] + T[1], P[1] + T[3])), P[2] + T[2]);
 }
 
-// c q 2^(2 e + 60) in 2^61 = 1, twice that for more = 1 (below 2^62)
-QLGA_HD i64 fx_coupled(const FxConst& c, i64 q, int e, int more) {
-    FxAcc s = fx_zero<60>();
-    fx_mac(s, c.m, fx_split(q));
-    int n = c.ex + 2 * e + 121 + more;
-    n = n < -63 ? -63 : (n > 30 ? 30 : n);
-    return fx_scale(fx_sum<60>(s), n);
+// A bound of the scaled matrix: the largest row sum of the moduli, which bounds every Taylor term of a vector with
+// moduli of at most one.  Not finite, or large, where the entries would not fit their integers.
+QLGA_HD float fx_norm(const FxSizes& z, const FxForms& f, const FixPot& C, const int T[5]) {
+    const float un = fx_pow2f(f.en - 56);
+    const float gz = C.dz_f * un * float(f.Fz), g2r = C.dr_f * un * float(f.rho);
+    float L[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) L[m] = float(T[m]);
+    const float g = fx_log_dot(z, L);
+    float w = 0.f;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        float row = fabsf(fmaf(float(2 - m), gz, -g2r)) + fx_exp2(g + z.p[4 - m] - L[m]);
+        if (m < 4) row += fx_exp2(fx_log_link(z, m) + L[m + 1] - L[m]);
+        if (m > 0) row += fx_exp2(fx_log_link(z, m - 1) + L[m - 1] - L[m]);
+        w = row > w || !(row == row) ? row : w;
+    }
+    return 1.0001f * w;
 }
 
-QLGA_HD void fx_singlet(const FixPot& C, int e, Limb& R, float& Rf) {
-    // R 2^(2 e) = m 2^(ex - 60 + 2 e); G conj(u) / 2^61 = R 2^(2 e) dot 2^60 conj(u) and G = W.R dot / 2^55.
-    // |psi|^2 >= 2^114 and beta <= 0.25 bound W.R by 2^62
-    int n = C.R.ex + 2 * e + 116;
-    n = n < -63 ? -63 : (n > 30 ? 30 : n);
-    R = fx_split(fx_scale((i64(C.R.m.h) * (i64(1) << 32)) + C.R.m.l, n));
-    Rf = C.R_f * fx_pow2f(2 * e + 116);  // for u in 2^58 = 1
+// The exponents and the norm: a margin of 1 bit, up to 2 for a field too dense for it (a bit of the margin costs a
+// driven level one)
+constexpr int kFxMargins = 3;
+QLGA_HD float fx_margin(int k) { return 1.f + 0.5f * float(k); }
+QLGA_HD float fx_exponents(const FxSizes& z, const FxForms& f, const FixPot& C, const float own[5], int T[5]) {
+    float w = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < kFxMargins; ++k) {
+        fx_budget(z, own, fx_margin(k), T);
+        w = fx_norm(z, f, C, T);
+        if (w <= kFxNormMax) break;
+    }
+    return w;
 }
 
-QLGA_HD void fx_build_w(const FxVec& p, const FxForms& f, int e, const FixPot& C, FxW& W) {
-    const i64 gz = fx_coupled(C.dz, f.Fz, e, 0), g2r = fx_coupled(C.dr, f.rho, e, 0);
+QLGA_HD void fx_build_w(const FxLevels& psi, const FxForms& f, const FixPot& C, const int T[5], FxW& W) {
+    const i64 gz = fx_coupled(C.dz, f.Fz, f.en - 56), g2r = fx_coupled(C.dr, f.rho, f.en - 56);
 #pragma unroll
     for (int i = 0; i < 5; ++i) W.D[i] = fx_split((2 - i) * gz - g2r);
     const Limb r = fx_split(kFxR32m1);
-    const i64 er = fx_coupled(C.e0, f.Fpr, e, 1), ei = fx_coupled(C.e0, f.Fpi, e, 1);
-    W.e0r = fx_split(er);
-    W.e0i = fx_split(ei);
-    W.e1r = fx_split(er + fx_mul(r, fx_split(er)));
-    W.e1i = fx_split(ei + fx_mul(r, fx_split(ei)));
+    const i64 er1 = f.er + fx_mul(r, fx_split(f.er)), ei1 = f.ei + fx_mul(r, fx_split(f.ei));
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        auto turned = [&](Limb v) { return (j & 1) ? fx_split(-(v.h * (i64(1) << 32) + v.l)) : v; };
-        W.u.re[j] = turned(p.re[4 - j]);
-        W.u.im[j] = turned(p.im[4 - j]);
+    for (int i = 0; i < 4; ++i) {
+        const i64 er = i == 0 || i == 3 ? f.er : er1, ei = i == 0 || i == 3 ? f.ei : ei1;
+        const int up = fx_clamp(f.ee + T[i] - T[i + 1] + 1, -63, 2), dn = fx_clamp(f.ee + T[i + 1] - T[i] + 1, -63, 2);
+        W.upr[i] = fx_split(fx_scale(er, up));
+        W.upi[i] = fx_split(fx_scale(ei, up));
+        W.dnr[i] = fx_split(fx_scale(er, dn));
+        W.dni[i] = fx_split(fx_scale(ei, dn));
     }
-    fx_singlet(C, e, W.R, W.Rf);
+    const int g = fx_dot_exp(psi.e, T);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {  // u_j = (-1)^j psi_{4-j}
+        const Limb pr = psi.p.re[4 - j], pi = psi.p.im[4 - j];
+        const int sv = fx_clamp(psi.e[4 - j] + T[j] - g, -63, 0), su = fx_clamp(C.R.ex + psi.e[4 - j] + g - T[j] + 3, -63, 5);
+        i64 vr = fx_scale(fx_join(pr), sv), vi = fx_scale(fx_join(pi), sv);
+        i64 ur = fx_scale(fx_mul_full<60>(C.R.m, pr), su), ui = fx_scale(fx_mul_full<60>(C.R.m, pi), su);
+        if (j & 1) {
+            vr = -vr;
+            vi = -vi;
+            ur = -ur;
+            ui = -ui;
+        }
+        W.v.re[j] = fx_split(vr);
+        W.v.im[j] = fx_split(vi);
+        W.u.re[j] = fx_split(ur);
+        W.u.im[j] = fx_split(ui);
+    }
 }
 
-// x <- exp(-i delta W) x for one vector: orders 1..kA in fixed point, kA + 1..K in FP32
-QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
+// Decisions of a warp; on the host every site is a warp of its own
+QLGA_HD bool fx_warp_all(bool v) {
+#ifdef __CUDA_ARCH__
+    return __all_sync(0xffffffffu, v);
+#else
+    return v;
+#endif
+}
+QLGA_HD int fx_warp_max(int v) {
+#ifdef __CUDA_ARCH__
+    return __reduce_max_sync(0xffffffffu, v);
+#else
+    return v;
+#endif
+}
+QLGA_HD float fx_warp_max(float v) {  // v >= 0
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+#else
+    return v;
+#endif
+}
+
+// A bound of a modulus from the largest high limb of its components, which are in 2^57 = 1
+QLGA_HD float fx_size(int h) { return 4.2146848e-8f * float(h + 1); }  // sqrt(2) 2^-25
+QLGA_HD int fx_abs_limb(Limb a) { return a.h < 0 ? -a.h : a.h; }
+QLGA_HD float fx_size(const FxVec& t) {
+    int h = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) h = fx_max(h, fx_max(fx_abs_limb(t.re[i]), fx_abs_limb(t.im[i])));
+    return fx_size(h);
+}
+
+// x <- exp(-i delta W) x for one vector, w >= the warp's norm of W: the terms T_k / k! in fixed point until the next one
+// is below 2^-31, then in FP32 until it is below 2^-57.  A term is bounded by w times the one before it; the sizes of the
+// terms themselves decide, since a scaled norm is two to five times what they shrink by (bounds of w^k / k! alone
+// took one more order in fixed point, a fifth of U).
+QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], float w) {
     FxVec t;
     i64 tr[5], ti[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        tr[i] = re[i];
-        ti[i] = im[i];
+        t.re[i] = fx_split(re[i]);
+        t.im[i] = fx_split(im[i]);
     }
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        t.re[i] = fx_split(tr[i]);
-        t.im[i] = fx_split(ti[i]);
-    }
+    float q = fx_warp_max(fx_size(t));  // of T_k / k!
+    int k = 0;
+    float fact = 6.9388939e-18f;  // 2^-57 / k!
 #pragma unroll 1
-    for (int k = 1; k <= kA; ++k) {
+    while (w * q * fx_inv(k + 1) > kFxTolF && k < kFxTerms) {
+        ++k;
+        fact *= fx_inv(k);
         fx_apply(W, t, tr, ti);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
@@ -550,27 +725,29 @@ QLGA_HD void fx_taylor(const FxW& W, i64 re[5], i64 im[5], int kA, int K) {
                 im[i] += fx_mul(f, t.im[i]);
             }
         }
+        q = 1.4411519e17f * fact * fx_warp_max(fx_size(t));  // 2^57
     }
-    if (K > kA) {
-        FxCpxF tf[5], sf[5], uf[5], of[5];
-        const float s58 = 3.4694470e-18f;  // 2^-58
-        const float fact = s58 * fx_float(fx_inv_fact(kA), 4.3368087e-19f);
+    q *= w * fx_inv(k + 1);
+    if (q > kFxTol) {
+        FxCpxF tf[5], sf[5], of[5];
+        const FxWF Wf(W);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             tf[i] = {fx_float(t.re[i], fact), fx_float(t.im[i], fact)};
-            uf[i] = {fx_float(W.u.re[i], s58), fx_float(W.u.im[i], s58)};
             sf[i] = {0.f, 0.f};
         }
 #pragma unroll 1
-        for (int k = kA + 1; k <= K; ++k) {
-            fx_apply_f(W, uf, tf, of, fx_inv(k));
+        while (q > kFxTol && k < kFxDegree - 1) {
+            ++k;
+            fx_apply_f(Wf, tf, fx_dot_f(Wf, tf), of, fx_inv(k));
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
                 tf[i] = of[i];
                 sf[i] = {sf[i].re + of[i].re, sf[i].im + of[i].im};
             }
+            q *= w * fx_inv(k + 1);
         }
-        const float one = 288230376151711744.f;  // 2^58
+        const float one = 144115188075855872.f;  // 2^57
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             re[i] += fx_rint(sf[i].re * one);
@@ -596,22 +773,6 @@ QLGA_HD void fx_rotate(i64 c, i64 s, i64* re, i64* im) {
     }
 }
 
-// Decisions of a warp; on the host every site is a warp of its own
-QLGA_HD bool fx_warp_all(bool v) {
-#ifdef __CUDA_ARCH__
-    return __all_sync(0xffffffffu, v);
-#else
-    return v;
-#endif
-}
-QLGA_HD float fx_warp_max(float v) {  // v >= 0
-#ifdef __CUDA_ARCH__
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
-#else
-    return v;
-#endif
-}
-
 // e^{-i theta} - 1 = (-c, -s) for a theta of any size (fields denser than |theta| = 1/4 are rare)
 static __host__ __device__ __noinline__ void fx_phase_large(double theta, i64* c, i64* s) {
     double sn, cs;
@@ -620,57 +781,57 @@ static __host__ __device__ __noinline__ void fx_phase_large(double theta, i64* c
     *s = i64(rint(sn * 2305843009213693952.0));
 }
 
-// e^{-i theta} - 1 = (-c, -s) of a site from its density, for a warp with a lane beyond |theta| = 1/4 in FP64
-QLGA_HD void fx_site_phase(i64 rho, int et, float theta, const FixPot& C, i64& c, i64& s) {
+// e^{-i theta} - 1 = (-c, -s) of a site from its density rho 2^unit, for a warp with a lane beyond |theta| = 1/4 in FP64
+QLGA_HD void fx_site_phase(i64 rho, int unit, const FixPot& C, i64& c, i64& s) {
+    const float theta = fabsf(C.cphase_f) * fx_pow2f(unit) * float(rho);
     if (!fx_warp_all(theta <= 0.25f)) {
-        const int n = 2 * et < -900 ? -900 : 2 * et;
-        const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex + n) * double(rho);
+        const double th = ldexp(double(C.cphase.m.h) * 4294967296.0 + double(C.cphase.m.l), C.cphase.ex - 60 + fx_max(unit, -960)) * double(rho);
         fx_phase_large(th, &c, &s);
     } else {
-        fx_phase(fx_coupled(C.cphase, rho, et, 0), c, s);
+        fx_phase(fx_coupled(C.cphase, rho, unit), c, s);
     }
 }
 
-// U on one site of a warp.  In: psi and d as integers below 2^62 of unit 2^e, `true` amplitudes
+// U on one site of a warp.  In: level m of psi and d as integers below 2^62 of unit 2^e[m], `true` amplitudes
 // 2^in_log2 times that; ok = false: a lane whose input has no such form.  Out: (psi', d') =
-// (U psi, U d) as integers of the unit 2^(returned exponent), below 2^60.  Returns false, with
+// (U psi, U d) as integers of the units 2^e[m], below 2^60.  Returns false, with
 // nothing changed, if a lane of the warp lies outside the domain.  All 32 lanes take part: the
-// orders of the Taylor sums are those of the warp's largest beta.
-QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int in_log2, bool ok,
-                                           const FixPot& C) {
-    const int np = fx_headroom(pr, pi), nd0 = fx_headroom(dr, di);
-    // d goes with psi's unit or, where it is larger, its own, below 2^57 there, so that G of its sums
-    // stays below 2^62; psi's sum takes the same unit (its limbs in W have psi's own)
-    const int nd = nd0 + 1 > np ? nd0 + 1 : np;
-    FxVec p;
+// orders of the Taylor sums are those of the warp's largest norm.
+QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int e[5], int in_log2, bool ok, const FixPot& C) {
+    FxLevels psi;
+    FxSizes z;
+    float L[5];  // sizes of the levels of both vectors
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_split(fx_shift(pr[i], np));
-        p.im[i] = fx_split(fx_shift(pi[i], np));
+        fx_level(pr[i], pi[i], e[i] + in_log2, psi.p.re[i], psi.p.im[i], psi.e[i]);
+        z.p[i] = fx_log_of(pr[i], pi[i], e[i] + in_log2);
+        L[i] = fmaxf(fmaxf(z.p[i], fx_log_of(dr[i], di[i], e[i] + in_log2)), float(kFxFloor));
     }
     FxForms f;
-    fx_forms(p, f);
-    const int et = e + np + in_log2;  // exponent of the true psi
-    const FxBounds bd = fx_bounds(f, et, C);
-    ok = ok && bd.beta <= kFxBetaMax;
+    fx_forms(psi, C, f);
+    z.e = fx_log_of(f.er, f.ei, f.ee - 60);
+    z.R = C.R_log;
+    int T[5];
+    const float w = fx_exponents(z, f, C, L, T);
+    ok = ok && w <= kFxNormMax;
     if (!fx_warp_all(ok)) return false;
-    const float beta = fx_warp_max(bd.beta);
-    const int K = fx_degree(beta, kFxTol), k0 = fx_degree(beta, kFxTolF);
-    const int kA = K < k0 ? K : k0;
+    const float wmax = fx_warp_max(w);
     FxW W;
-    fx_build_w(p, f, et, C, W);
+    fx_build_w(psi, f, C, T, W);
     i64 pc, ps;
-    fx_site_phase(f.rho, et, bd.theta, C, pc, ps);
+    fx_site_phase(f.rho, f.en - 56, C, pc, ps);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        pr[i] = fx_shift(pr[i], nd);
-        pi[i] = fx_shift(pi[i], nd);
-        dr[i] = fx_shift(dr[i], nd);
-        di[i] = fx_shift(di[i], nd);
+        const int n = fx_clamp(e[i] + in_log2 + 57 - T[i], -63, 57);
+        pr[i] = fx_scale(pr[i], n);
+        pi[i] = fx_scale(pi[i], n);
+        dr[i] = fx_scale(dr[i], n);
+        di[i] = fx_scale(di[i], n);
+        e[i] = T[i] - in_log2 - 57;
     }
 #pragma unroll 1
     for (int v = 0; v < 2; ++v) {  // one copy of the code for both vectors
-        fx_taylor(W, pr, pi, kA, K);
+        fx_taylor(W, pr, pi, wmax);
         fx_rotate(pc, ps, pr, pi);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
@@ -681,8 +842,14 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
             di[i] = ti;
         }
     }
-    e += nd;
     return true;
+}
+
+// The biased exponent of a level whose largest high word is m, and whether integers can hold it: finite, below
+// 2^60, and not between nothing and 2^-930
+QLGA_HD int fx_level_exponent(unsigned m, bool& ok) {
+    ok = ok && m < (unsigned(1023 + 60) << 20) && (m == 0 || m >= (unsigned(kFxMinExp + 1) << 20));
+    return fx_exponent(m);
 }
 
 // U on the pair (a, b) of one site of a warp in FP64, by fx_unitary; the arguments are those of
@@ -691,18 +858,13 @@ QLGA_HD bool fx_unitary(i64 pr[5], i64 pi[5], i64 dr[5], i64 di[5], int& e, int 
 template <bool PQ>
 QLGA_HD bool fx_potential(double ar[5], double ai[5], double br[5], double bi[5], int in_log2,
                                              int out_log2, const FixPot& C) {
-    unsigned m = 0;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        m = fx_top(fx_top(m, ar[i]), ai[i]);
-        m = fx_top(fx_top(m, br[i]), bi[i]);
-    }
-    const bool ok = m < (unsigned(1023 + 60) << 20);  // finite, below 2^60
-    const int E = fx_exponent(m);
-    int e = E - 1022 - 60;
+    bool ok = true;
+    int e[5];
     i64 pr[5], pi[5], dr[5], di[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
+        const int E = fx_level_exponent(fx_top(fx_top(fx_top(fx_top(0, ar[i]), ai[i]), br[i]), bi[i]), ok);
+        e[i] = E - 1022 - 60;
         const i64 a0 = fx_from_double<60>(ar[i], E), a1 = fx_from_double<60>(ai[i], E);
         const i64 b0 = fx_from_double<60>(br[i], E), b1 = fx_from_double<60>(bi[i], E);
         pr[i] = a0 + b0;
@@ -711,9 +873,9 @@ QLGA_HD bool fx_potential(double ar[5], double ai[5], double br[5], double bi[5]
         di[i] = a1 - b1;
     }
     if (!fx_unitary(pr, pi, dr, di, e, in_log2, ok, C)) return false;
-    const FxToDouble to(e + out_log2);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
+        const FxToDouble to(e[i] + out_log2);
         const i64 a0 = pr[i] + dr[i], a1 = pi[i] + di[i], b0 = pr[i] - dr[i], b1 = pi[i] - di[i];
         ar[i] = to(PQ ? a0 - b1 : a0);
         ai[i] = to(PQ ? a1 + b0 : a1);

@@ -6,27 +6,18 @@ using namespace qlga;
 
 extern "C" {
 
-long long host_shift(long long v, int n) { return fx_shift(v, n); }
+long long host_shift(long long v, int n) { return fx_scale(v, -n); }
 
 // The density of a field psi[level][re, im]
 double host_density(const double* psi) {
-    unsigned m = 0;
-    for (int i = 0; i < 10; ++i) m = fx_top(m, psi[i]);
-    const int E = fx_exponent(m);
-    i64 re[5], im[5];
+    FxLevels p;
     for (int i = 0; i < 5; ++i) {
-        re[i] = fx_from_double<60>(psi[2 * i], E);
-        im[i] = fx_from_double<60>(psi[2 * i + 1], E);
-    }
-    const int n = fx_headroom(re, im);
-    FxVec p;
-    for (int i = 0; i < 5; ++i) {
-        p.re[i] = fx_split(fx_shift(re[i], n));
-        p.im[i] = fx_split(fx_shift(im[i], n));
+        const int E = fx_exponent(fx_top(fx_top(0, psi[2 * i]), psi[2 * i + 1]));
+        fx_level(fx_from_double<60>(psi[2 * i], E), fx_from_double<60>(psi[2 * i + 1], E), E - 1022 - 60, p.p.re[i], p.p.im[i], p.e[i]);
     }
     FxForms f;
-    fx_forms(p, f);
-    return std::ldexp(double(f.rho), 2 * (E - 1022 - 60 + n) + 60);
+    fx_forms(p, FixPot(0, 0, 0, 0, 0), f);
+    return std::ldexp(double(f.rho), f.en - 56);
 }
 
 // U on the pair (a, b) of a site; x[level][qubit][re, im], in place.  Returns whether the site is in the domain.
