@@ -5,20 +5,21 @@
 // applies the nine-point x stencil from shared memory and runs the four y blocks as a register pipeline.  All
 // of K's coefficients are small integers, so on integers K is exact up to one rounding between the
 // axes, and an addition costs 2 cycles per sub-partition where FP64 takes 76 (qlga_fixed.cuh): at 1024^2 the
-// pass takes 0.13 ms (K in FP64 1.36; all levels of a strip in one warp, with 255 registers and 8 warps per SM, 0.187),
-// a step of 256^2 52 us (72).
+// pass takes 0.14 ms (K in FP64 1.36; all levels of a strip in one warp, with 255 registers and 8 warps per SM, 0.187),
+// 20 us at 256^2.
 // The potential is a pass of its own (k_potential): FP64 state traffic is far
 // from the bound.
 //
 // Numbers.  A row is converted once, in place in the ring, each lane its column and an equal share of
 // the eight halo columns, to int64 with one exponent per warp: components below 2^58, the largest of
 // the last 8 to 16 rows in [2^57, 2^58) when its row was read.  The stencil's taps sum to at most 30
-// in magnitude, so its sums fit; they are rounded to 2^-8 of their unit, and the y blocks (taps at
-// most 44) then end below 2^61 and hold the true K X.  Where a row is larger than all before it the
-// pipeline is shifted down, where the last 16 rows are smaller it is shifted up.  The resolution is
-// thus 2^-54 of the largest component of the level in a strip of 40 columns and 8 to 16 rows.  A warp that meets a
-// column more than 2^-kKin64Spread below that (the tail of a localised state) redoes its chunk in FP64, where
-// every component keeps its own digits.
+// in magnitude, so its sums fit; they are rounded to 2^-6 of their unit, and the y blocks (taps at
+// most 44) then end below 2^63 and hold four times the true K X.  Where a row is larger than all before it the
+// pipeline is shifted down, where the last 16 rows are smaller it is shifted up.  The rounding is
+// thus 2^-57.2 (root mean square) of the largest component of the level in a strip of 40 columns and 8 to 16 rows, where
+// FP64 adds 2^-53 of what lies within the stencil.  A warp whose strip varies by more than the difference redoes
+// its chunk in FP64: one that meets four neighbouring columns more than 2^-kKin64Spread below the largest
+// (the tail of a localised state), where any nine columns hold four such neighbours.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -91,7 +92,19 @@ __device__ __forceinline__ void stream_int(i64& a, i64& bt, i64& yo, i64& wc) {
 constexpr int kKin64Warps = 4;  // of a CTA: one to a sub-partition
 constexpr int kKin64Ctas = 5;   // resident per SM
 constexpr int kKin64Stages = 3;
-constexpr int kKin64Spread = 20;
+constexpr int kKin64Spread = 4;
+// The smallest exponent of four neighbouring columns of a row (aligned with the strip), from the largest high words
+// of the lane's own column and of its halo component; 0 where such four are empty.  All lanes take part.
+__device__ __forceinline__ int strip_low(unsigned column, unsigned halo) {
+    column = max(column, __shfl_xor_sync(0xffffffffu, column, 1));
+    column = max(column, __shfl_xor_sync(0xffffffffu, column, 2));
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) halo = max(halo, __shfl_xor_sync(0xffffffffu, halo, o));  // four lanes hold a column
+    return int(__reduce_min_sync(0xffffffffu, min(column, halo)) >> 20);
+}
+// v 2^n, rounded, for the pipelines' values (up to 2^63)
+QLGA_HD i64 strip_scale(i64 v, int n) { return n > 0 ? v << n : (n < 0 ? ((v >> (-n - 1)) + 1) >> 1 : v); }
+
 constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
 
 // The chunk of one warp in FP64: rows [y_begin, y_end) of its 32 columns of one level, straight from global memory.
@@ -203,6 +216,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
     for (int k = 0; k < 4; ++k) yo[k] = wc[k] = {0, 0};
     int E = kFxMinExp;                              // the pipeline's exponent
     int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
+    int low = 2047, low_before = 2047;              // and the smallest exponents of four neighbours
     int bad_until = -1;                             // rows up to here depend on one that is not finite
 
 #pragma unroll 1
@@ -217,9 +231,8 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         const double halo = reinterpret_cast<const double*>(row + 2 * kStep2dWarpCols)[lane];
         auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
         const unsigned column = max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y)));
-        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, max(column, hi(halo))));
-        // the smallest column that is not empty (a high word of 0: nothing, or below the normal range)
-        const int low = int(__reduce_min_sync(0xffffffffu, column ? column : 0x7fffffffu) >> 20);
+        const unsigned top = __reduce_max_sync(0xffffffffu, max(column, hi(halo)));
+        int Er = fx_exponent(top);
         const bool bad = Er > kKin64MaxExp;
         if (bad) {
             Er = kFxMinExp;
@@ -228,10 +241,13 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         if ((r & 7) == 0) {
             seen_before = seen;
             seen = kFxMinExp;
+            low_before = low;
+            low = 2047;
         }
         seen = max(seen, Er);
+        if (top) low = min(low, strip_low(column, hi(halo)));  // an empty row adds nothing to any site
         const int En = max(seen, seen_before);
-        if (En - low > kKin64Spread) {  // warp-uniform
+        if (En - min(low, low_before) > kKin64Spread) {  // warp-uniform
             cp_async_wait<0>();
             kinetic_strip_f64<VARIANT>(level, out2, nx, ny, x0, y_begin, y_end, abi);
             return;
@@ -240,8 +256,8 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
             const int n = max(E - En, -63);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                yo[k] = {fx_scale(yo[k].re, n), fx_scale(yo[k].im, n)};
-                wc[k] = {fx_scale(wc[k].re, n), fx_scale(wc[k].im, n)};
+                yo[k] = {strip_scale(yo[k].re, n), strip_scale(yo[k].im, n)};
+                wc[k] = {strip_scale(wc[k].re, n), strip_scale(wc[k].im, n)};
             }
             E = En;
         }
@@ -251,15 +267,15 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         reinterpret_cast<i64*>(row + 2 * kStep2dWarpCols)[lane] = bad ? 0 : fx_from_double<58>(halo, E);
         __syncwarp();
 
-        // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-8
-        cpi xa = {128, 128}, xbt = {128, 128};
+        // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-6
+        cpi xa = {32, 32}, xbt = {32, 32};
         static_for<9>([&](auto kc) {
             constexpr int kk = decltype(kc)::value;
             stencil_tap_int<VARIANT, kk>(p[2 * kk], p[2 * kk + 1], xa, xbt);
         });
-        xa = {xa.re >> 8, xa.im >> 8};
-        xbt = {xbt.re >> 8, xbt.im >> 8};
-        // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16: the true K X)
+        xa = {xa.re >> 6, xa.im >> 6};
+        xbt = {xbt.re >> 6, xbt.im >> 6};
+        // y axis: I'_2 I'_2 then I'_1 I'_1 as a streaming pipeline (x16: four times the true K X)
         static_for<4>([&](auto kc) {
             constexpr int kk = decltype(kc)::value;
             stream_int<kk < 2 ? 1 : 0, VARIANT>(xa.re, xbt.re, yo[kk].re, wc[kk].re);
@@ -271,7 +287,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
                 const double nan = fx_bits(0x7ff80000u, 0u);
                 p2[0] = p2[1] = make_double2(nan, nan);
             } else {
-                const FxToDouble to(E - 1022 - 58);
+                const FxToDouble to(E - 1022 - 60);
                 p2[0] = make_double2(to(xa.re), to(xa.im));
                 p2[1] = abi ? make_double2(to(xbt.im), to(-xbt.re)) : make_double2(to(xbt.re), to(xbt.im));
             }
