@@ -5,8 +5,10 @@
 // to 7 also on the eight columns beyond, the row goes to shared memory, and the adjoint nine-point stencil
 // of x reads it there.  The FP64 form was two passes of 320 FP64 instructions a site (66 cycles each): 106 us at 256^2, 27 here.
 //
-// Numbers.  As there, with components below 2^56 after conversion: the y blocks' taps (at most 44 in magnitude) keep
-// below 2^62, are rounded to 2^-6 of that, and the x stencil's sums are 2^58 times the true K^dagger g.
+// Numbers.  As there, with components below 2^57 after conversion: the y blocks' taps (at most 44 in magnitude) keep
+// below 2^63, are rounded to 2^-5 of that, and the x stencil's sums, below 2^63 again, are eight times the true K^dagger g.
+// The rounding is 2^-57.1 (root mean square) of a strip's largest, so the same spread of a strip's columns sends its
+// chunk to FP64: the cotangent of a local loss keeps its tails.
 #pragma once
 
 #include "qlga_adjoint.cuh"
@@ -17,42 +19,95 @@ namespace qlga {
 // One adjoint block C^dagger S_c C'^dagger S_c^T along y for one component (make_stencil_adjoint has the same
 // factors): input row n -> output row n - 1; yo: the other qubit of the previous row, wc: the shifted qubit after the
 // first collide of the previous row.
-template <int C, int FIRST>
-__device__ __forceinline__ void stream_adj_int(i64& a, i64& bt, i64& yo, i64& wc) {
-    const i64 ya = C == 1 ? yo : a, yb = C == 1 ? bt : yo;
+template <int C, int FIRST, class N>
+__device__ __forceinline__ void stream_adj(N& a, N& bt, N& yo, N& wc) {
+    const N ya = C == 1 ? yo : a, yb = C == 1 ? bt : yo;
     yo = C == 1 ? a : bt;
-    const i64 wa = ya - yb, wb = ya + yb;
-    const i64 za = C == 1 ? wa : wc, zb = C == 1 ? wc : wb;
+    const N wa = ya - yb, wb = ya + yb;
+    const N za = C == 1 ? wa : wc, zb = C == 1 ? wc : wb;
     wc = C == 1 ? wb : wa;
     a = FIRST == 0 ? za - zb : za + zb;
     bt = FIRST == 0 ? za + zb : zb - za;
 }
 
-struct AdjColumn {
-    cpi yo[4], wc[4];
+template <class P>
+struct AdjColumn {  // P: a pair of numbers, re and im
+    P yo[4], wc[4];
     __device__ __forceinline__ void clear() {
 #pragma unroll
         for (int k = 0; k < 4; ++k) yo[k] = wc[k] = {0, 0};
     }
+    template <int VARIANT>
+    __device__ __forceinline__ void push(P& a, P& bt) {
+        static_for<4>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value, c = kk < 2 ? 0 : 1;  // the blocks of qubit 1 first
+            stream_adj<c, VARIANT>(a.re, bt.re, yo[kk].re, wc[kk].re);
+            stream_adj<c, VARIANT>(a.im, bt.im, yo[kk].im, wc[kk].im);
+        });
+    }
+};
+struct AdjColumnInt : AdjColumn<cpi> {
     __device__ __forceinline__ void scale(int n) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            yo[k] = {fx_scale(yo[k].re, n), fx_scale(yo[k].im, n)};
-            wc[k] = {fx_scale(wc[k].re, n), fx_scale(wc[k].im, n)};
+            yo[k] = {strip_scale(yo[k].re, n), strip_scale(yo[k].im, n)};
+            wc[k] = {strip_scale(wc[k].re, n), strip_scale(wc[k].im, n)};
         }
     }
     template <int VARIANT>
-    __device__ __forceinline__ void push(longlong2& a, longlong2& bt) {
-        static_for<4>([&](auto kc) {
-            constexpr int kk = decltype(kc)::value, c = kk < 2 ? 0 : 1;  // the blocks of qubit 1 first
-            stream_adj_int<c, VARIANT>(a.x, bt.x, yo[kk].re, wc[kk].re);
-            stream_adj_int<c, VARIANT>(a.y, bt.y, yo[kk].im, wc[kk].im);
-        });
-        auto down = [](i64 v) { return (v + 32) >> 6; };
-        a = make_longlong2(down(a.x), down(a.y));
-        bt = make_longlong2(down(bt.x), down(bt.y));
+    __device__ __forceinline__ void push_rounded(longlong2& a, longlong2& bt) {
+        cpi x = {a.x, a.y}, y = {bt.x, bt.y};
+        push<VARIANT>(x, y);
+        auto down = [](i64 v) { return ((v >> 4) + 1) >> 1; };
+        a = make_longlong2(down(x.re), down(x.im));
+        bt = make_longlong2(down(y.re), down(y.im));
     }
 };
+
+// The chunk of one warp in FP64: rows [y_begin, y_end) of its 32 columns of one level, straight from global memory;
+// yrow: the warp's row in shared memory.
+template <int VARIANT>
+__device__ __noinline__ void adjoint_strip_f64(const double2* level, double2* out2, int nx, int ny, int x0, int y_begin,
+                                               int y_end, double2* yrow) {
+    constexpr KinStencil S = kStencilAdj[VARIANT];
+    const int lane = threadIdx.x & 31;
+    auto wrap = [&](int x) { return (x % nx + nx) % nx; };
+    const int xm = wrap(x0 - kStep2dHalo + lane), xh = wrap(x0 + kStep2dWarpCols - kStep2dHalo + (lane & 7));
+    AdjColumn<cpx<double>> own, beyond;
+    own.clear();
+    beyond.clear();
+    const int nrows = (y_end - y_begin) + 8;
+#pragma unroll 1
+    for (int r = 0; r < nrows; ++r) {
+        int y = y_begin - kStep2dHalo + r;
+        y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+        const double2* g = level + 2 * int64_t(y) * nx;
+        auto column = [&](AdjColumn<cpx<double>>& c, int x, int at) {
+            const double2 u = __ldg(g + 2 * x), v = __ldg(g + 2 * x + 1);
+            cpx<double> a = {u.x, u.y}, bt = {v.x, v.y};
+            c.template push<VARIANT>(a, bt);
+            yrow[2 * at] = make_double2(a.re, a.im);
+            yrow[2 * at + 1] = make_double2(bt.re, bt.im);
+        };
+        __syncwarp();  // the last row's stencil has read yrow
+        column(own, xm, lane);
+        if (lane < 2 * kStep2dHalo) column(beyond, xh, kStep2dWarpCols + lane);
+        __syncwarp();
+        if (r < 8) continue;
+        cpx<double> xa = {0.0, 0.0}, xbt = {0.0, 0.0};
+        static_for<9>([&](auto kc) {
+            constexpr int kk = decltype(kc)::value;
+            const double2 P = yrow[2 * (lane + kk)], Q = yrow[2 * (lane + kk) + 1];
+            kin_tap4<S.g[0][0][kk], S.g[0][1][kk], S.g[1][0][kk], S.g[1][1][kk]>(cpx<double>{P.x, P.y}, cpx<double>{Q.x, Q.y}, xa, xbt);
+        });
+        if (x0 + lane < nx) {
+            const double s = 1.0 / 256.0;
+            double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
+            p2[0] = make_double2(s * xa.re, s * xa.im);
+            p2[1] = make_double2(s * xbt.re, s * xbt.im);
+        }
+    }
+}
 
 constexpr int kAdj64Ctas = 4;  // resident per SM, of kKin64Warps warps
 
@@ -109,11 +164,12 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
 #pragma unroll
     for (int r = 0; r < kKin64Stages - 1; ++r) issue_row();
 
-    AdjColumn own, beyond;
+    AdjColumnInt own, beyond;
     own.clear();
     beyond.clear();
     int E = kFxMinExp;                              // the pipelines' exponent
     int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
+    int low = 2047, low_before = 2047;              // and the smallest exponents of four neighbours
     int bad_until = -1;                             // rows up to here depend on one that is not finite
 
 #pragma unroll 1
@@ -127,8 +183,9 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         double2* tail = row + 2 * kStep2dWarpCols;  // columns 32..39: the lane's component
         const double halo = reinterpret_cast<const double*>(tail)[lane];
         auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
-        const unsigned top = max(max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y))), hi(halo));
-        int Er = fx_exponent(__reduce_max_sync(0xffffffffu, top));
+        const unsigned column = max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y)));
+        const unsigned top = __reduce_max_sync(0xffffffffu, max(column, hi(halo)));
+        int Er = fx_exponent(top);
         const bool bad = Er > kKin64MaxExp;
         if (bad) {
             Er = kFxMinExp;
@@ -137,9 +194,17 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         if ((r & 7) == 0) {
             seen_before = seen;
             seen = kFxMinExp;
+            low_before = low;
+            low = 2047;
         }
         seen = max(seen, Er);
+        if (top) low = min(low, strip_low(column, hi(halo)));  // an empty row adds nothing to any site
         const int En = max(seen, seen_before);
+        if (En - min(low, low_before) > kKin64Spread) {  // warp-uniform
+            cp_async_wait<0>();
+            adjoint_strip_f64<VARIANT>(level, out2, nx, ny, x0, y_begin, y_end, reinterpret_cast<double2*>(yrow));
+            return;
+        }
         if (En != E) {  // warp-uniform, rare on smooth fields
             const int n = max(E - En, -63);
             own.scale(n);
@@ -148,18 +213,18 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         }
         longlong2 a = make_longlong2(0, 0), bt = a;
         if (!bad) {
-            a = make_longlong2(fx_from_double<56>(own0.x, E), fx_from_double<56>(own0.y, E));
-            bt = make_longlong2(fx_from_double<56>(own1.x, E), fx_from_double<56>(own1.y, E));
+            a = make_longlong2(fx_from_double<57>(own0.x, E), fx_from_double<57>(own0.y, E));
+            bt = make_longlong2(fx_from_double<57>(own1.x, E), fx_from_double<57>(own1.y, E));
         }
-        reinterpret_cast<i64*>(tail)[lane] = bad ? 0 : fx_from_double<56>(halo, E);
+        reinterpret_cast<i64*>(tail)[lane] = bad ? 0 : fx_from_double<57>(halo, E);
         __syncwarp();  // also: the last row's stencil has read yrow
-        own.push<VARIANT>(a, bt);
+        own.push_rounded<VARIANT>(a, bt);
         yrow[2 * lane] = a;
         yrow[2 * lane + 1] = bt;
         if (lane < 2 * kStep2dHalo) {
             const longlong2* h = reinterpret_cast<const longlong2*>(tail) + 2 * lane;
             longlong2 ha = h[0], hb = h[1];
-            beyond.push<VARIANT>(ha, hb);
+            beyond.push_rounded<VARIANT>(ha, hb);
             yrow[2 * (kStep2dWarpCols + lane)] = ha;
             yrow[2 * (kStep2dWarpCols + lane) + 1] = hb;
         }
@@ -181,7 +246,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
                 const double nan = fx_bits(0x7ff80000u, 0u);
                 p2[0] = p2[1] = make_double2(nan, nan);
             } else {
-                const FxToDouble to(E - 1022 - 58);
+                const FxToDouble to(E - 1022 - 60);
                 p2[0] = make_double2(to(xa.re), to(xa.im));
                 p2[1] = make_double2(to(xbt.re), to(xbt.im));
             }

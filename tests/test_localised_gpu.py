@@ -1,4 +1,4 @@
-"""K of a localised 2D FP64 state: every site keeps the digits of its own neighbourhood, as FP64 does, wherever the
+"""K and K^dagger of a localised 2D FP64 field: every site keeps the digits of its own neighbourhood, as FP64 does, wherever the
 field within the kernel's strip of 40 columns and 16 rows varies.
 
 Tolerance: 6e-15 of the largest component within reach (8 rows and columns for two steps).  An axis of K is 24 sums of
@@ -70,3 +70,17 @@ def test_kinetic(kind, nx, ny, variant):
         got = lat.get_state()
     err, near = np.abs(got - ref).max(axis=(3, 4)), _near(st, 8)
     assert np.all(err <= TOL * near), float((err / np.maximum(near, 1e-300)).max())
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("nx,ny,variant", [(96, 70, 0), (101, 64, 1), (40, 200, 0)])
+def test_kinetic_adjoint(kind, nx, ny, variant):
+    rng = np.random.default_rng(nx + len(kind))
+    st = I.random_state(rng, nx, ny, scale=0.05)
+    cot = rng.standard_normal(st.shape) * _envelope(kind, rng, nx, ny)[None, :, :, None, None]
+    ref = cot.copy()
+    oracle.vjp_kinetic(ref, oracle.make_cfg(2, nx, ny, 0.0, 0.0, 0.0, kinetic_variant=variant))
+    with qlga.Lattice(2, nx, ny, precision=64, g=(0.0, 0.0, 0.0), kinetic_variant=variant) as lat:
+        got, _ = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
+    err, near = np.abs(got.cpu().numpy() - ref).max(axis=(3, 4)), _near(cot, 4)
+    assert np.all(err <= 0.5 * TOL * near), float((err / np.maximum(near, 1e-300)).max())
