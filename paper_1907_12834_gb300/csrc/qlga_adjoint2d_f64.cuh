@@ -111,7 +111,7 @@ __device__ __noinline__ void adjoint_strip_f64(const double2* level, double2* ou
 
 constexpr int kAdj64Ctas = 4;  // resident per SM, of kKin64Warps warps
 
-// out = K^dagger in, both in the resident layout (a, bt); strips, chunks and values that are not finite as in
+// out = K^dagger in, both in the resident layout (a, bt); strips, chunks and their FP64 form as in
 // k_kinetic2d_f64.
 template <int VARIANT>
 __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
@@ -170,7 +170,6 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
     int E = kFxMinExp;                              // the pipelines' exponent
     int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
     int low = 2047, low_before = 2047;              // and the smallest exponents of four neighbours
-    int bad_until = -1;                             // rows up to here depend on one that is not finite
 
 #pragma unroll 1
     for (int r = 0; r < nrows; ++r) {
@@ -185,12 +184,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
         const unsigned column = max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y)));
         const unsigned top = __reduce_max_sync(0xffffffffu, max(column, hi(halo)));
-        int Er = fx_exponent(top);
-        const bool bad = Er > kKin64MaxExp;
-        if (bad) {
-            Er = kFxMinExp;
-            bad_until = r + 8;
-        }
+        const int Er = fx_exponent(top);
         if ((r & 7) == 0) {
             seen_before = seen;
             seen = kFxMinExp;
@@ -200,7 +194,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         seen = max(seen, Er);
         if (top) low = min(low, strip_low(column, hi(halo)));  // an empty row adds nothing to any site
         const int En = max(seen, seen_before);
-        if (En - min(low, low_before) > kKin64Spread) {  // warp-uniform
+        if (En - min(low, low_before) > kKin64Spread || En > kKin64MaxExp) {  // warp-uniform
             cp_async_wait<0>();
             adjoint_strip_f64<VARIANT>(level, out2, nx, ny, x0, y_begin, y_end, reinterpret_cast<double2*>(yrow));
             return;
@@ -211,12 +205,9 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
             beyond.scale(n);
             E = En;
         }
-        longlong2 a = make_longlong2(0, 0), bt = a;
-        if (!bad) {
-            a = make_longlong2(fx_from_double<57>(own0.x, E), fx_from_double<57>(own0.y, E));
-            bt = make_longlong2(fx_from_double<57>(own1.x, E), fx_from_double<57>(own1.y, E));
-        }
-        reinterpret_cast<i64*>(tail)[lane] = bad ? 0 : fx_from_double<57>(halo, E);
+        longlong2 a = make_longlong2(fx_from_double<57>(own0.x, E), fx_from_double<57>(own0.y, E));
+        longlong2 bt = make_longlong2(fx_from_double<57>(own1.x, E), fx_from_double<57>(own1.y, E));
+        reinterpret_cast<i64*>(tail)[lane] = fx_from_double<57>(halo, E);
         __syncwarp();  // also: the last row's stencil has read yrow
         own.push_rounded<VARIANT>(a, bt);
         yrow[2 * lane] = a;
@@ -242,14 +233,9 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kAdj64Ctas)
         });
         if (x0 + lane < nx) {  // output row y_begin + r - 8
             double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
-            if (r <= bad_until) {  // warp-uniform
-                const double nan = fx_bits(0x7ff80000u, 0u);
-                p2[0] = p2[1] = make_double2(nan, nan);
-            } else {
-                const FxToDouble to(E - 1022 - 60);
-                p2[0] = make_double2(to(xa.re), to(xa.im));
-                p2[1] = make_double2(to(xbt.re), to(xbt.im));
-            }
+            const FxToDouble to(E - 1022 - 60);
+            p2[0] = make_double2(to(xa.re), to(xa.im));
+            p2[1] = make_double2(to(xbt.re), to(xbt.im));
         }
     }
     cp_async_wait<0>();

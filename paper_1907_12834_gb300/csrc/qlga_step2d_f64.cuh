@@ -105,7 +105,7 @@ __device__ __forceinline__ int strip_low(unsigned column, unsigned halo) {
 // v 2^n, rounded, for the pipelines' values (up to 2^63)
 QLGA_HD i64 strip_scale(i64 v, int n) { return n > 0 ? v << n : (n < 0 ? ((v >> (-n - 1)) + 1) >> 1 : v); }
 
-constexpr int kKin64MaxExp = 1022 + 512;  // a component of 2^512 or more has no square: taken as not finite
+constexpr int kKin64MaxExp = 1022 + 900;  // larger components, and those that are not finite, take FP64
 
 // The chunk of one warp in FP64: rows [y_begin, y_end) of its 32 columns of one level, straight from global memory.
 template <int VARIANT>
@@ -161,8 +161,7 @@ __device__ __noinline__ void kinetic_strip_f64(const double2* level, double2* ou
 // out = K in: in held pending K as (P, Q), out the true state in the resident layout (a, bt) or,
 // with abi, the ABI's (a, b).  nx >= 32
 // of any remainder: the lanes of the last strip that lie past the row's end work on its periodic
-// image and store nothing.  A row holding a value that is not finite gives NaN wherever the strip
-// depends on it.
+// image and store nothing.
 template <int VARIANT>
 __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
     k_kinetic2d_f64(const double* __restrict__ in, double* __restrict__ out, int nx, int ny, int chunks, bool abi) {
@@ -217,7 +216,6 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
     int E = kFxMinExp;                              // the pipeline's exponent
     int seen = kFxMinExp, seen_before = kFxMinExp;  // the largest row exponents of this and the last 8 rows
     int low = 2047, low_before = 2047;              // and the smallest exponents of four neighbours
-    int bad_until = -1;                             // rows up to here depend on one that is not finite
 
 #pragma unroll 1
     for (int r = 0; r < nrows; ++r) {
@@ -232,12 +230,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         auto hi = [](double x) { return fx_hi(x) & 0x7fffffffu; };
         const unsigned column = max(max(hi(own0.x), hi(own0.y)), max(hi(own1.x), hi(own1.y)));
         const unsigned top = __reduce_max_sync(0xffffffffu, max(column, hi(halo)));
-        int Er = fx_exponent(top);
-        const bool bad = Er > kKin64MaxExp;
-        if (bad) {
-            Er = kFxMinExp;
-            bad_until = r + 8;
-        }
+        const int Er = fx_exponent(top);
         if ((r & 7) == 0) {
             seen_before = seen;
             seen = kFxMinExp;
@@ -247,7 +240,7 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         seen = max(seen, Er);
         if (top) low = min(low, strip_low(column, hi(halo)));  // an empty row adds nothing to any site
         const int En = max(seen, seen_before);
-        if (En - min(low, low_before) > kKin64Spread) {  // warp-uniform
+        if (En - min(low, low_before) > kKin64Spread || En > kKin64MaxExp) {  // warp-uniform
             cp_async_wait<0>();
             kinetic_strip_f64<VARIANT>(level, out2, nx, ny, x0, y_begin, y_end, abi);
             return;
@@ -262,9 +255,9 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
             E = En;
         }
         longlong2* p = reinterpret_cast<longlong2*>(row + 2 * lane);
-        p[0] = bad ? make_longlong2(0, 0) : make_longlong2(fx_from_double<58>(own0.x, E), fx_from_double<58>(own0.y, E));
-        p[1] = bad ? make_longlong2(0, 0) : make_longlong2(fx_from_double<58>(own1.x, E), fx_from_double<58>(own1.y, E));
-        reinterpret_cast<i64*>(row + 2 * kStep2dWarpCols)[lane] = bad ? 0 : fx_from_double<58>(halo, E);
+        p[0] = make_longlong2(fx_from_double<58>(own0.x, E), fx_from_double<58>(own0.y, E));
+        p[1] = make_longlong2(fx_from_double<58>(own1.x, E), fx_from_double<58>(own1.y, E));
+        reinterpret_cast<i64*>(row + 2 * kStep2dWarpCols)[lane] = fx_from_double<58>(halo, E);
         __syncwarp();
 
         // x axis: nine-point stencil (x16) from the held (P, Q) pairs to (a, bt), then rounded to 2^-6
@@ -283,14 +276,9 @@ __global__ void __launch_bounds__(32 * kKin64Warps, kKin64Ctas)
         });
         if (r >= 8 && x0 + lane < nx) {  // pipeline full: this is output row y_begin + r - 8
             double2* p2 = out2 + 2 * (int64_t(y_begin + r - 8) * nx + x0 + lane);
-            if (r <= bad_until) {  // warp-uniform
-                const double nan = fx_bits(0x7ff80000u, 0u);
-                p2[0] = p2[1] = make_double2(nan, nan);
-            } else {
-                const FxToDouble to(E - 1022 - 60);
-                p2[0] = make_double2(to(xa.re), to(xa.im));
-                p2[1] = abi ? make_double2(to(xbt.im), to(-xbt.re)) : make_double2(to(xbt.re), to(xbt.im));
-            }
+            const FxToDouble to(E - 1022 - 60);
+            p2[0] = make_double2(to(xa.re), to(xa.im));
+            p2[1] = abi ? make_double2(to(xbt.im), to(-xbt.re)) : make_double2(to(xbt.re), to(xbt.im));
         }
     }
     cp_async_wait<0>();

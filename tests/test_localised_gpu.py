@@ -84,3 +84,40 @@ def test_kinetic_adjoint(kind, nx, ny, variant):
         got, _ = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
     err, near = np.abs(got.cpu().numpy() - ref).max(axis=(3, 4)), _near(cot, 4)
     assert np.all(err <= 0.5 * TOL * near), float((err / np.maximum(near, 1e-300)).max())
+
+
+def _reach_of(bad, y, x):
+    """Whether the sites that are not finite lie within K's reach of (y, x), and that one among them."""
+    out = bad.copy()
+    out[y - 4:y + 5, x - 4:x + 5] = False
+    return bad[y, x] and not out.any()
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_what_is_not_finite_reaches_its_stencil_alone(value):
+    nx, ny = 70, 40
+    rng = np.random.default_rng(2)
+    st, cot = I.random_state(rng, nx, ny, scale=0.05), rng.standard_normal((5, ny, nx, 2, 2))
+    bad_st, bad_cot = st.copy(), cot.copy()
+    bad_st[1, 20, 30, 0, 1] = bad_cot[1, 20, 30, 0, 1] = value
+    with qlga.Lattice(2, nx, ny, precision=64, g=(1.0, 0.1, 1.0)) as lat:
+        dev = torch.empty(st.shape, dtype=torch.float64, device="cuda")
+        lat.load_state(torch.tensor(bad_st, device="cuda"))
+        lat.step(1)
+        got = lat.get_state(dev).cpu().numpy()
+    assert _reach_of(~np.isfinite(got).all(axis=(0, 3, 4)), 20, 30)
+    with qlga.Lattice(2, nx, ny, precision=64, g=(1.0, 0.1, 1.0)) as lat:
+        got, _ = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(bad_cot, device="cuda"))
+    assert _reach_of(~np.isfinite(got.cpu().numpy()).all(axis=(0, 3, 4)), 20, 30)
+
+
+def test_large_cotangents_are_pulled_back():
+    nx, ny = 70, 40
+    rng = np.random.default_rng(2)
+    st, cot = I.random_state(rng, nx, ny, scale=0.05), rng.standard_normal((5, ny, nx, 2, 2))
+    cot[1, 20:24, 30:34] *= 1e295
+    ref = cot.copy()
+    oracle.vjp_kinetic(ref, oracle.make_cfg(2, nx, ny, 0.0, 0.0, 0.0))
+    with qlga.Lattice(2, nx, ny, precision=64, g=(0.0, 0.0, 0.0)) as lat:
+        got, _ = lat.adjoint_step(torch.tensor(st, device="cuda"), torch.tensor(cot, device="cuda"))
+    assert np.all(np.abs(got.cpu().numpy() - ref).max(axis=(3, 4)) <= 0.5 * TOL * _near(cot, 4))
