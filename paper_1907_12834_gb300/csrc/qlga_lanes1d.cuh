@@ -70,8 +70,8 @@ struct WLane {
 // One fused step (K, then U with the lattice's constants) of a single periodic 1D lattice of L
 // sites, in -> out in the resident layout; 30 / LPS sites per warp, one warp per CTA.
 template <class T, int VARIANT, int LPS>
-__global__ void __launch_bounds__(32) k_step1d_lanes(const T* __restrict__ in, T* __restrict__ out, int L,
-                                                     PotConst<T> C, unsigned* status) {
+__device__ __forceinline__ void lanes1d_step(const T* __restrict__ in, T* __restrict__ out, int L, const PotConstBase<T>& C,
+                                             unsigned* status) {
     static_assert(LPS == 5 || LPS == 10, "five or ten lanes per site");
     constexpr int SPW = 30 / LPS;  // sites per warp
     const int lane = threadIdx.x;
@@ -212,6 +212,12 @@ __global__ void __launch_bounds__(32) k_step1d_lanes(const T* __restrict__ in, T
     const cpx<T> ph = {cs * out_scale, -sn * out_scale};  // e^{-i delta c} / (2 sigma)
     const cpx<T> na = cmul(ph, vp + vd), nb = cmul(ph, vp - vd);
     if (store) store_raw_pq(out, int64_t(m) * L + j, na, nb);  // held pending K again, as (P, Q)
+}
+
+template <class T, int VARIANT, int LPS>
+__global__ void __launch_bounds__(32) k_step1d_lanes(const T* __restrict__ in, T* __restrict__ out, int L,
+                                                     PotConst<T> C, unsigned* status) {
+    lanes1d_step<T, VARIANT, LPS>(in, out, L, C, status);
 }
 
 }  // namespace qlga

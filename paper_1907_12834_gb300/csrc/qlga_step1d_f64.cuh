@@ -24,6 +24,7 @@
 
 #include "qlga_batch1d.cuh"
 #include "qlga_device.cuh"
+#include "qlga_lanes1d.cuh"
 #include "qlga_step2d_f64.cuh"  // stencil_tap_int
 
 namespace qlga {
@@ -330,6 +331,14 @@ __device__ __forceinline__ int fx_lane_budget(const FxGroup& g, float p, float p
     return int(ceilf(L + 0.001f));
 }
 
+// The warp's step in FP64, with the lanes per site that it has: a warp's FP64 instructions cost the same on 3 sites as on
+// 32, and one site a lane has ten times as many of them (a field beyond the domain, us a step: 1024
+// sites 100, so 34, 16384 sites 431, so 137; the FP64 lane kernel 29 and 171)
+template <int VARIANT, int LPS>
+__device__ __noinline__ void step1d_lanes_f64(const double* in, double* out, int L, const PotConstBase<double>* C, unsigned* status) {
+    lanes1d_step<double, VARIANT, LPS>(in, out, L, *C, status);
+}
+
 // One fused step of a periodic 1D lattice of L sites held pending K as (P, Q); 30 / LPS sites per warp,
 // one warp per CTA.  Numbers and fallback as k_step1d_f64.
 template <int VARIANT, int LPS>
@@ -368,12 +377,9 @@ __global__ void __launch_bounds__(32) k_step1d_f64_lanes(const double* __restric
                 t = fx_top(fx_top(fx_top(fx_top(t, v[i][0].x), v[i][0].y), v[i][1].x), v[i][1].y);
         tops[m] = __reduce_max_sync(0xffffffffu, t);
     }
-    // the FP64 code takes the warp's sites one a lane
     auto in_fp64 = [&]() {
-        const int s = x0 + lane;
-        const bool own = lane < SPW && s < L;
         const PotConstBase<double> base = C;
-        step1d_site_f64<VARIANT, true>(in, out, L, own ? s : j, own, &base, status);
+        step1d_lanes_f64<VARIANT, LPS>(in, out, L, &base, status);
     };
     bool fits = true;
     int Es[5];
