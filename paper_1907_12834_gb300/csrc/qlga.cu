@@ -844,14 +844,50 @@ inline int step2d_device(Step2dDevice* out) {
     return 0;
 }
 
+// Row chunks of the FP64 fields, which are bound by the sub-partitions' FP64 pipes: a row is about 120 FP64
+// instructions and each of the two halo rows of a chunk 20; the busiest of the `units` sub-partitions has ceil(warps / units)
+// chunks, and one or two warps give its pipe 0.7 or 0.9 of its rate (640^2: 168 us with one warp each, 137 with three).
+inline int64_t fields_chunks_f64(int64_t strips, int64_t ny, int64_t units) {
+    int64_t best = 1;
+    double best_cost = -1.0;
+    for (int64_t c = 1; c <= ny && (c == 1 || strips * c <= 16 * units); ++c) {
+        const int64_t k = (strips * c + units - 1) / units;
+        const double eff = k >= 3 ? 1.0 : (k == 2 ? 0.9 : 0.7);
+        const double cost = double(k) / eff * (120.0 * double((ny + c - 1) / c) + 40.0);
+        if (best_cost < 0.0 || cost < best_cost) {
+            best = c;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+// Row chunks of the kernels that search for them, on one lattice.  The search takes up to 20 us of a host core on a
+// narrow lattice of many rows (a step of 32 x 4096 outside a graph 19.4 us, 16.3 without), so a handle makes it once.
+struct RowChunks {
+    int kin64 = 1, adj64 = 1, f32 = 1;
+    int64_t fields64 = 1;
+};
+inline RowChunks row_chunks(int64_t nx, int64_t ny) {
+    RowChunks c;
+    Step2dDevice dv;
+    if (step2d_device(&dv)) return c;  // a launch reports the error
+    c.fields64 = fields_chunks_f64((nx + kFieldsCols - 1) / kFieldsCols, ny, 4 * int64_t(dv.sms));
+    if (!step2d_strips_supported(nx, ny)) return c;
+    const int64_t strips = step2d_strips(nx);
+    auto fp64 = [](double rows) { return rows + 7.0; };  // a warm-up row costs 0.9 of a row
+    c.kin64 = step2d_level_chunks(strips, ny, dv.sms, kKin64Ctas * kKin64Warps / 5, fp64);
+    c.adj64 = step2d_level_chunks(strips, ny, dv.sms, std::max(1, kAdj64Ctas * kKin64Warps / 5), fp64);
+    c.f32 = step2d_level_chunks(strips, ny, dv.sms, kLevelsCtas, [](double rows) {
+        return 0.4 * (rows + 8.0) + 0.6 * (5.0 * std::ceil(rows / 5.0));  // K is 0.4 of a row, U runs by five rows
+    });
+    return c;
+}
+
 // FP64 (qlga_step2d_f64.cuh): K of a state held pending K, as the true state; same contract as
 // step2d_f32_launch.
-inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64_t ny, int variant, cudaStream_t stream, bool abi) {
-    Step2dDevice dv;
-    if (step2d_device(&dv)) return 1;
+inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64_t ny, int chunks, int variant, cudaStream_t stream, bool abi) {
     const int64_t strips = step2d_strips(nx);
-    // a warm-up row costs 0.9 of a row
-    const int chunks = step2d_level_chunks(strips, ny, dv.sms, kKin64Ctas * kKin64Warps / 5, [](double rows) { return rows + 7.0; });
     auto launch = [&](auto kernel) {
         kernel<<<int((5 * strips * chunks + kKin64Warps - 1) / kKin64Warps), 32 * kKin64Warps, 0, stream>>>(in, out, int(nx), int(ny), chunks, abi);
     };
@@ -862,7 +898,7 @@ inline int kinetic2d_f64_launch(const double* in, double* out, int64_t nx, int64
 
 // Returns 0 on success (errors are left in cudaGetLastError()).  pot = false applies the kinetic
 // operator alone; true_out (with pot): K X is stored there too.
-inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny, int variant, bool pot,
+inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny, int levels, int variant, bool pot,
                              PotConst<float> PC, unsigned* status, cudaStream_t stream, float* true_out = nullptr, bool abi = false) {
     Step2dDevice dv;
     if (step2d_device(&dv)) return 1;
@@ -870,9 +906,6 @@ inline int step2d_f32_launch(const float* in, float* out, int64_t nx, int64_t ny
     // by levels (qlga_step2d.cuh): us a step, one warp a strip / by levels: 128^2 7.8 / 6.1, 384 x 107 10.5 / 8.0,
     // 256^2 12.0 / 9.8, 512^2 22.3 / 23.5, 1024^2 61 / 72; K alone, 512^2 27.0 / 24.4, 1024^2 71 / 66, 2048^2 221 / 221
     if (nx * ny <= (pot ? int64_t(1) << 17 : int64_t(1) << 20)) {
-        const int levels = step2d_level_chunks(strips, ny, dv.sms, kLevelsCtas, [](double rows) {
-            return 0.4 * (rows + 8.0) + 0.6 * (5.0 * std::ceil(rows / 5.0));  // K is 0.4 of a row, U runs by five rows
-        });
         auto launch = [&](auto kernel) {
             kernel<<<int(strips * levels), kLevelsThreads, 0, stream>>>(in, out, int(nx), int(ny), levels, PC, status, true_out, abi);
         };
@@ -1090,6 +1123,7 @@ struct qlga_handle {
     int tile_lanes;   // 1D: fused steps by the lane-parallel kernel with 5 or 10 lanes per site, 0: not
     bool tile_fixed;  // 1D FP64: no forced shape, steps by the fixed-point kernel (reported as kFixed1dCand's shape)
     int step2d_mode;  // QLGA_STEP2D_AUTO / _FUSED / _TWO_PASS
+    RowChunks chunks;  // 2D
     // CUDA graphs of graph_steps fused steps starting (and ending) on buffer 0 or 1
     int graph_steps;
     int64_t graph_launches;  // kernels in one graph
@@ -1507,10 +1541,10 @@ qlga_status kinetic_into(qlga_handle* h, const void* in, void* out, void* mid, b
     if (step2d_uses_strips(h) && held) {
         const int err = h->cfg.precision == 32
             ? step2d_f32_launch(static_cast<const float*>(in), static_cast<float*>(out), h->cfg.nx, h->cfg.ny,
-                                h->cfg.kinetic_variant, pot, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
+                                h->chunks.f32, h->cfg.kinetic_variant, pot, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
                                 h->stream, nullptr, abi)
             : kinetic2d_f64_launch(static_cast<const double*>(in), static_cast<double*>(out), h->cfg.nx, h->cfg.ny,
-                                   h->cfg.kinetic_variant, h->stream, abi);
+                                   h->chunks.kin64, h->cfg.kinetic_variant, h->stream, abi);
         if (err) return cuda_fail(cudaGetLastError(), "step2d launch");
         h->launches += 1;
         return pot && h->cfg.precision == 64 ? launch_pot_held(h, out, out) : QLGA_OK;
@@ -1529,7 +1563,7 @@ qlga_status kinetic_and_step(qlga_handle* h, const void* in, void* true_out, voi
             return s == QLGA_OK ? launch_pot_held(h, true_out, out) : s;
         }
         if (step2d_f32_launch(static_cast<const float*>(in), static_cast<float*>(out), h->cfg.nx, h->cfg.ny,
-                              h->cfg.kinetic_variant, true, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
+                              h->chunks.f32, h->cfg.kinetic_variant, true, PotConst<float>(pot_params(h->cfg, 1.0)), h->status,
                               h->stream, static_cast<float*>(true_out)))
             return cuda_fail(cudaGetLastError(), "step2d launch");
         h->launches += 1;
@@ -1796,6 +1830,7 @@ static qlga_status init_handle(qlga_handle* h, const qlga_config* cfg, void* str
     h->tile_lanes = 0;
     h->tile_fixed = false;
     h->step2d_mode = QLGA_STEP2D_AUTO;
+    h->chunks = cfg->ndim == 2 ? row_chunks(cfg->nx, cfg->ny) : RowChunks();
     QLGA_CUDA(cudaMemsetAsync(h->X[0], 0, state_bytes_of(*cfg), h->stream), "state clear");
     QLGA_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream), "status clear");
     return QLGA_OK;
@@ -2201,24 +2236,6 @@ qlga_status qlga_exchange_rows(qlga_handle* src, int64_t ysrc, qlga_handle* dst,
     return QLGA_OK;
 }
 
-// Row chunks of the FP64 fields, which are bound by the sub-partitions' FP64 pipes: a row is about 120 FP64
-// instructions and each of the two halo rows of a chunk 20; the busiest of the `units` sub-partitions has ceil(warps / units)
-// chunks, and one or two warps give its pipe 0.7 or 0.9 of its rate (640^2: 168 us with one warp each, 137 with three).
-static int64_t fields_chunks_f64(int64_t strips, int64_t ny, int64_t units) {
-    int64_t best = 1;
-    double best_cost = -1.0;
-    for (int64_t c = 1; c <= ny && (c == 1 || strips * c <= 16 * units); ++c) {
-        const int64_t k = (strips * c + units - 1) / units;
-        const double eff = k >= 3 ? 1.0 : (k == 2 ? 0.9 : 0.7);
-        const double cost = double(k) / eff * (120.0 * double((ny + c - 1) / c) + 40.0);
-        if (best_cost < 0.0 || cost < best_cost) {
-            best = c;
-            best_cost = cost;
-        }
-    }
-    return best;
-}
-
 qlga_status qlga_fields(qlga_handle* h, void* dst, int where) {
     if (!h || !dst) return fail(QLGA_ERR_INVALID_ARG, "NULL argument%s");
     if (where != QLGA_HOST && where != QLGA_DEVICE) return fail(QLGA_ERR_INVALID_ARG, "where must be QLGA_HOST or QLGA_DEVICE%s");
@@ -2239,7 +2256,7 @@ qlga_status qlga_fields(qlga_handle* h, void* dst, int where) {
         const int64_t per_block = kFieldsThreads / 32, strips = (h->cfg.nx + kFieldsCols - 1) / kFieldsCols;
         const int64_t warps = per_block * (per_sm > 0 ? per_sm : 1) * device_sms();
         int64_t chunks = std::max<int64_t>(1, std::min(h->cfg.ny / 8, warps / strips));
-        if (h->cfg.precision == 64) chunks = fields_chunks_f64(strips, h->cfg.ny, 4 * int64_t(device_sms()));
+        if (h->cfg.precision == 64) chunks = h->chunks.fields64;
         const int64_t grid = (strips * chunks + per_block - 1) / per_block;
         if (h->cfg.precision == 32)
             k_fields2d<float><<<unsigned(grid), kFieldsThreads, 0, h->stream>>>(static_cast<const float*>(view), static_cast<float*>(target), int(h->cfg.nx), int(h->cfg.ny), int(chunks));
@@ -2459,10 +2476,8 @@ qlga_status adj_axis(qlga_handle* h, const void* gin, void* gout, const void* X,
 // FP64 on a 2D lattice of at least 32 columns: K^dagger in integer fixed point, then the pull-back through U.
 template <int V>
 qlga_status adj_pullback2d_f64(qlga_handle* h, const double* cot, double* tmp, double* out, const double* xk, double* partials) {
-    Step2dDevice dv;
-    if (step2d_device(&dv)) return cuda_fail(cudaGetLastError(), "2D adjoint set-up");
     const int64_t nx = h->cfg.nx, ny = h->cfg.ny, strips = step2d_strips(nx);
-    const int chunks = step2d_level_chunks(strips, ny, dv.sms, std::max(1, kAdj64Ctas * kKin64Warps / 5), [](double rows) { return rows + 7.0; });
+    const int chunks = h->chunks.adj64;
     k_adjoint2d_f64<V><<<int((5 * strips * chunks + kKin64Warps - 1) / kKin64Warps), 32 * kKin64Warps, 0, h->stream>>>(cot, tmp, int(nx), int(ny), chunks);
     QLGA_CUDA(cudaGetLastError(), "k_adjoint2d_f64 launch");
     const int blocks = grid_for_block(nsites_of(h->cfg), kAdjThreads, std::min(kAdjMaxBlocks, 8 * device_sms()));
