@@ -280,14 +280,16 @@ qlga_status qlga_get_step2d_kernel(qlga_handle* h, int32_t* kernel);
  * leave most of the GPU idle: shape (5, 0, 1), a site's five levels on five lanes, six sites per
  * warp; or (10, 0, 1), the psi and d = a - b recursions of U on separate lanes, three sites per
  * warp.  In FP32 the first fused step times the candidates on the live state and keeps the fastest per
- * step: a one-step shape or, in plain steps, a two-step shape (temporal blocking, see the
- * batches; qlga_step then takes fused steps two per launch).  FP64 steps run in fixed point, the
- * lanes per site chosen by the length, and report the shape (32, 1, 1); a forced shape takes the FP64
- * arithmetic of the tiled and lane-parallel kernels.
- * qlga_set_1d_shape forces a shape (the list of qlga_batch_set_shape, (5, 0, 1), (10, 0, 1), or
- * the (0, 0, 0) reset); qlga_get_1d_shape reports the one fused steps use (zeros before tuning).  Setting waits for the
+ * step: a one-step shape or, in plain steps, one of several steps per launch (temporal blocking, see the
+ * batches; qlga_step then takes fused steps by two, four or eight).  (128, 1, 4) and (128, 1, 8) are shapes of
+ * single lattices alone.  In FP64 the shape (32, 1, 1) stands for the steps in integer fixed point, with ten,
+ * five or one lane per site by the length; it is the default, and the others take the FP64 arithmetic of the tiled
+ * and lane-parallel kernels.
+ * qlga_set_1d_shape forces a shape (the list of qlga_batch_set_shape, (128, 1, 4), (128, 1, 8), (5, 0, 1), (10, 0, 1), or
+ * the (0, 0, 0) reset); qlga_get_1d_shape reports the one fused steps use (zeros before tuning), and setting
+ * that on another lattice of the size gives it the same kernels.  Setting waits for the
  * handle's stream and drops captured step graphs.  Errors: QLGA_ERR_UNSUPPORTED on a 2D lattice,
- * or two steps per launch in FP64 or with interleave; QLGA_ERR_INVALID_ARG for another shape. */
+ * or several steps per launch in FP64 or with interleave; QLGA_ERR_INVALID_ARG for another shape. */
 qlga_status qlga_set_1d_shape(qlga_handle* h, int32_t threads, int32_t sites_per_thread, int32_t steps);
 qlga_status qlga_get_1d_shape(qlga_handle* h, int32_t* threads, int32_t* sites_per_thread, int32_t* steps);
 

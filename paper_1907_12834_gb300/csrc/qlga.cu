@@ -1016,7 +1016,7 @@ struct BatchCand {
 constexpr int kBatchNumCands = 11;
 // ... and two that advance a single FP32 lattice four or eight steps per launch, for lattices bound by the launches
 // (16384 sites: 2.57 us a step two at a time, 1.80 now; 1024 sites 1.46; both pick four or eight up to the
-// graphs' 262144 sites); the caller cannot ask for them.
+// graphs' 262144 sites), which a batch cannot ask for.
 constexpr int kTileNumCands = kBatchNumCands + 2;
 constexpr BatchCand kBatchCands[kTileNumCands] = {
     {0, 32, 1, 1},  {1, 64, 1, 1},  {2, 128, 1, 1}, {3, 256, 1, 1}, {2, 64, 2, 1},  {3, 128, 2, 1},
@@ -1025,9 +1025,9 @@ constexpr BatchCand kBatchCands[kTileNumCands] = {
 constexpr int kFixed1dCand = 0;       // the shape of the FP64 fixed-point kernel: 32 threads, one site each, one step
 constexpr int kBatchDefaultCand = 1;  // before tuning: 64 threads, one site each
 
-// Candidate index of a shape (threads, sites per thread, steps), -1 if there is none.
-inline int batch_cand_of(int threads, int spt, int steps) {
-    for (int ci = 0; ci < kBatchNumCands; ++ci)
+// Index of a shape (threads, sites per thread, steps) among the first `cands`, -1 if there is none.
+inline int batch_cand_of(int threads, int spt, int steps, int cands = kBatchNumCands) {
+    for (int ci = 0; ci < cands; ++ci)
         if (kBatchCands[ci].threads == threads && kBatchCands[ci].spt == spt && kBatchCands[ci].steps == steps)
             return ci;
     return -1;
@@ -1121,7 +1121,7 @@ struct qlga_handle {
     int tile_cand;  // 1D: launch shape of the tiled step (index into kBatchCands), -1 untuned
     int tile_cand2;  // 1D: shape of several steps per launch when it beats tile_cand per step, else -1
     int tile_lanes;   // 1D: fused steps by the lane-parallel kernel with 5 or 10 lanes per site, 0: not
-    bool tile_fixed;  // 1D FP64: no forced shape, steps by the fixed-point kernel (reported as kFixed1dCand's shape)
+    bool tile_fixed;  // 1D FP64: steps by the fixed-point kernels (kFixed1dCand's shape, reported and asked for)
     int step2d_mode;  // QLGA_STEP2D_AUTO / _FUSED / _TWO_PASS
     RowChunks chunks;  // 2D
     // CUDA graphs of graph_steps fused steps starting (and ending) on buffer 0 or 1
@@ -1456,7 +1456,7 @@ inline void lanes_1d_launch(const TileArgs& a, int lps) {
 qlga_status tile_1d(qlga_handle* h, const void* in, void* out, bool pot, int steps = 1, bool abi = false) {
     TileArgs a{h->stream, h->cfg.precision, h->cfg.kinetic_variant, pot, in, out, nullptr, 0, nullptr,
                nullptr, h->status, h->cfg.nx, pot_params(h->cfg, 1.0), abi};
-    // FP64 without a forced shape: the fixed-point kernel at any size
+    // FP64 without a forced shape, or with theirs: the fixed-point kernels at any size
     if (h->cfg.precision == 64 && (h->tile_cand < 0 || h->tile_fixed)) {
         if (pot) {
             h->tile_fixed = true;
@@ -2317,22 +2317,24 @@ qlga_status qlga_set_1d_shape(qlga_handle* h, int32_t threads, int32_t sites_per
     if (h->cfg.ndim != 1) return fail(QLGA_ERR_UNSUPPORTED, "launch shapes are for 1D lattices%s");
     int c1 = -1, c2 = -1;
     const int lanes = (threads == 5 || threads == 10) && sites_per_thread == 0 && steps == 1 ? threads : 0;
+    bool fixed = false;
     if (lanes) {
         c1 = kBatchDefaultCand;  // read-outs of the pending state
     } else if (threads != 0 || sites_per_thread != 0 || steps != 0) {
-        const int ci = batch_cand_of(threads, sites_per_thread, steps);
+        const int ci = batch_cand_of(threads, sites_per_thread, steps, kTileNumCands);
         if (ci < 0) return fail(QLGA_ERR_INVALID_ARG, "not one of the launch shapes%s");
-        if (steps == 2 && (h->cfg.precision != 32 || h->cfg.interleave))
-            return fail(QLGA_ERR_UNSUPPORTED, "two steps per launch need FP32 plain steps%s");
-        c1 = steps == 2 ? batch_cand_of(threads, sites_per_thread, 1) : ci;
-        c2 = steps == 2 ? ci : -1;
+        if (steps > 1 && (h->cfg.precision != 32 || h->cfg.interleave))
+            return fail(QLGA_ERR_UNSUPPORTED, "several steps per launch need FP32 plain steps%s");
+        c1 = steps > 1 ? batch_cand_of(threads, sites_per_thread, 1) : ci;
+        c2 = steps > 1 ? ci : -1;
+        fixed = h->cfg.precision == 64 && ci == kFixed1dCand;
     }
     cudaStreamSynchronize(h->stream);
     graphs_release(h);
     h->tile_cand = c1;
     h->tile_cand2 = c2;
     h->tile_lanes = lanes;
-    h->tile_fixed = false;
+    h->tile_fixed = fixed;
     return QLGA_OK;
 }
 
