@@ -423,17 +423,26 @@ __global__ void __launch_bounds__(kThreads) k_observables2d(const float* __restr
     }
 }
 
-// Per-run observables of a batch: kBatchObsParts CTAs per run, each an equal part of its sites; terms in the state's
+// Per-run observables of a batch, a CTA to a part of a run's sites; terms in the state's
 // precision (compensated per-thread sums for FP32), FP64 block sums in a fixed order;
-// out[run][part][OBS_COUNT], summed by k_batch_obs_sum.  One CTA per run took as long as the longest run's serial
-// passes (256 runs of 2048 to 65536 sites: 40 steps with load and read-outs 5.75 ms, 5.66 now).
-constexpr int kBatchObsParts = 8;
+// out[part][OBS_COUNT], summed by k_batch_obs_sum where a run has several.  A CTA's block sums cost an SM 5 us (13 FP64
+// sums of eight warps), as much as 300 sites in FP32, so a run is split only to fill the GPU, or where it is longer than
+// an SM's share.  FP32, one CTA per run / eight / these, us: 4096 runs of 64 sites 247 / 1439 / 248, 256 of 16384
+// 238 / 313 / 251, 16 of 65536 347 / 115 / 147.
+struct BatchObsPart {
+    int run, begin, end;
+};
+inline int64_t batch_obs_chunk(int precision, int64_t nruns, int64_t total_sites, int64_t sms) {
+    return std::max<int64_t>(precision == 32 ? 2048 : 512, total_sites / (nruns >= sms ? sms : 4 * sms));
+}
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_batch_observables(const T* __restrict__ X,
                                                                 const BatchRun* __restrict__ runs,
+                                                                const BatchObsPart* __restrict__ obs_parts,
                                                                 const double* __restrict__ g3,
                                                                 double* __restrict__ out) {
-    const int r = blockIdx.x / kBatchObsParts, part = blockIdx.x % kBatchObsParts;
+    const BatchObsPart part = obs_parts[blockIdx.x];
+    const int r = part.run;
     const BatchRun run = runs[r];
     const int L = run.L;
     const int ny = run.ny, nx = L / ny;
@@ -444,8 +453,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_observables(const T* __restr
         const Pair4<T> p = load_raw_pair(X, run.base + int64_t(m) * L + j);
         return cpx<T>{p.v[0] + p.v[3], p.v[1] - p.v[2]};  // a + b, b = -i bt
     };
-    const int j_begin = int(int64_t(L) * part / kBatchObsParts), j_end = int(int64_t(L) * (part + 1) / kBatchObsParts);
-    for (int j = j_begin + threadIdx.x; j < j_end; j += blockDim.x) {
+    for (int j = part.begin + threadIdx.x; j < part.end; j += blockDim.x) {
         cpx<T> psi[5];
         T rho = T(0);
 #pragma unroll
@@ -494,13 +502,14 @@ __global__ void __launch_bounds__(kThreads) k_batch_observables(const T* __restr
     }
 }
 
-// out[run][k] = the parts' sums in order; one thread per run and quantity.
-__global__ void __launch_bounds__(kThreads) k_batch_obs_sum(const double* __restrict__ parts, double* __restrict__ out, int n) {
+// out[run][k] = the sums of the run's parts, first[run] .. first[run + 1], in order; one thread per run and quantity.
+__global__ void __launch_bounds__(kThreads) k_batch_obs_sum(const double* __restrict__ parts, const int* __restrict__ first,
+                                                            double* __restrict__ out, int n) {
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const int run = i / OBS_COUNT, k = i % OBS_COUNT;
     CompSum cs;
-    for (int p = 0; p < kBatchObsParts; ++p) cs.add(parts[(int64_t(run) * kBatchObsParts + p) * OBS_COUNT + k]);
+    for (int p = first[run]; p < first[run + 1]; ++p) cs.add(parts[int64_t(p) * OBS_COUNT + k]);
     out[i] = cs.s + cs.c;
 }
 
@@ -2636,7 +2645,10 @@ struct qlga_batch {
     BatchRun* runs;
     void* consts;             // PotConst<T>[nruns]
     double* g3;               // [nruns][3], device
-    double* obs_dev;          // [nruns][OBS_COUNT], then [nruns][kBatchObsParts][OBS_COUNT]
+    double* obs_dev;          // [nruns][OBS_COUNT], then [obs_nparts][OBS_COUNT]
+    BatchObsPart* obs_parts;  // the parts of the runs, run by run
+    int* obs_first;           // [nruns + 1], each run's first part
+    int obs_nparts;
     unsigned* status;
     BatchTile* tiles[kBatchNumWidths];  // tiles of the 1D runs, per tile width
     int ntiles[kBatchNumWidths];
@@ -2860,6 +2872,15 @@ qlga_status qlga_batch_create(const qlga_batch_config* cfg, void* stream, qlga_b
         runs2d[r] = Run2d{base, int(nx), int(ny)};
         base += 5 * nx * ny;
     }
+    std::vector<BatchObsPart> obs_parts;
+    std::vector<int> obs_first(1, 0);
+    const int64_t obs_chunk = batch_obs_chunk(cfg->precision, cfg->nruns, total, device_sms());
+    for (int r = 0; r < cfg->nruns; ++r) {
+        const int64_t L = runs[r].L, n = (L + obs_chunk - 1) / obs_chunk;
+        for (int64_t p = 0; p < n; ++p) obs_parts.push_back(BatchObsPart{r, int(L * p / n), int(L * (p + 1) / n)});
+        obs_first.push_back(int(obs_parts.size()));
+    }
+    b->obs_nparts = int(obs_parts.size());
     // tile tables of the 1D runs (the tiled kernel), 128-site tiles of every run (the potential)
     std::vector<BatchTile> tiles[kBatchNumWidths], tiles_pot;
     for (int r = 0; r < cfg->nruns; ++r) {
@@ -2896,7 +2917,9 @@ qlga_status qlga_batch_create(const qlga_batch_config* cfg, void* stream, qlga_b
     if (e == cudaSuccess) e = cudaMalloc(&b->runs, sizeof(BatchRun) * runs.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->consts, cbytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->g3, sizeof(double) * 3 * cfg->nruns);
-    if (e == cudaSuccess) e = cudaMalloc(&b->obs_dev, sizeof(double) * OBS_COUNT * cfg->nruns * (1 + kBatchObsParts));
+    if (e == cudaSuccess) e = cudaMalloc(&b->obs_dev, sizeof(double) * OBS_COUNT * (size_t(cfg->nruns) + obs_parts.size()));
+    if (e == cudaSuccess) e = cudaMalloc(&b->obs_parts, sizeof(BatchObsPart) * obs_parts.size());
+    if (e == cudaSuccess) e = cudaMalloc(&b->obs_first, sizeof(int) * obs_first.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->status, sizeof(unsigned));
     for (int wi = 0; wi < kBatchNumWidths && e == cudaSuccess; ++wi)
         e = cudaMalloc(&b->tiles[wi], sizeof(BatchTile) * std::max<size_t>(1, tiles[wi].size()));
@@ -2925,6 +2948,8 @@ qlga_status qlga_batch_create(const qlga_batch_config* cfg, void* stream, qlga_b
             e = cudaMemcpy(b->tiles[wi], tiles[wi].data(), sizeof(BatchTile) * tiles[wi].size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->tiles_pot, tiles_pot.data(), sizeof(BatchTile) * tiles_pot.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->obs_parts, obs_parts.data(), sizeof(BatchObsPart) * obs_parts.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->obs_first, obs_first.data(), sizeof(int) * obs_first.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->runs2d, runs2d.data(), sizeof(Run2d) * runs2d.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !tasks.empty())
         e = cudaMemcpy(b->tasks, tasks.data(), sizeof(WarpTask) * tasks.size(), cudaMemcpyHostToDevice);
@@ -3031,16 +3056,20 @@ qlga_status qlga_batch_observables(qlga_batch* b, qlga_obs* out) {
     const void* view = nullptr;
     qlga_status s = batch_materialize_view(b, &view);
     if (s != QLGA_OK) return s;
-    double* parts = b->obs_dev + size_t(b->nruns) * OBS_COUNT;
+    const bool split = b->obs_nparts > b->nruns;
+    double* parts = split ? b->obs_dev + size_t(b->nruns) * OBS_COUNT : b->obs_dev;
     if (b->precision == 32)
-        k_batch_observables<float><<<b->nruns * kBatchObsParts, kThreads, 0, b->stream>>>(static_cast<const float*>(view), b->runs, b->g3, parts);
+        k_batch_observables<float><<<b->obs_nparts, kThreads, 0, b->stream>>>(static_cast<const float*>(view), b->runs, b->obs_parts, b->g3, parts);
     else
-        k_batch_observables<double><<<b->nruns * kBatchObsParts, kThreads, 0, b->stream>>>(static_cast<const double*>(view), b->runs, b->g3, parts);
+        k_batch_observables<double><<<b->obs_nparts, kThreads, 0, b->stream>>>(static_cast<const double*>(view), b->runs, b->obs_parts, b->g3, parts);
     QLGA_CUDA(cudaGetLastError(), "k_batch_observables launch");
-    const int nsums = b->nruns * OBS_COUNT;
-    k_batch_obs_sum<<<(nsums + kThreads - 1) / kThreads, kThreads, 0, b->stream>>>(parts, b->obs_dev, nsums);
-    QLGA_CUDA(cudaGetLastError(), "k_batch_obs_sum launch");
-    b->launches += 2;
+    b->launches += 1;
+    if (split) {
+        const int nsums = b->nruns * OBS_COUNT;
+        k_batch_obs_sum<<<(nsums + kThreads - 1) / kThreads, kThreads, 0, b->stream>>>(parts, b->obs_first, b->obs_dev, nsums);
+        QLGA_CUDA(cudaGetLastError(), "k_batch_obs_sum launch");
+        b->launches += 1;
+    }
     std::vector<double> o(size_t(b->nruns) * OBS_COUNT);
     QLGA_CUDA(cudaMemcpyAsync(o.data(), b->obs_dev, sizeof(double) * o.size(), cudaMemcpyDeviceToHost, b->stream), "batch observables copy");
     QLGA_CUDA(cudaStreamSynchronize(b->stream), "batch observables sync");
@@ -3116,6 +3145,8 @@ qlga_status qlga_batch_destroy(qlga_batch* b) {
     cudaFree(b->consts);
     cudaFree(b->g3);
     cudaFree(b->obs_dev);
+    cudaFree(b->obs_parts);
+    cudaFree(b->obs_first);
     cudaFree(b->status);
     for (int wi = 0; wi < kBatchNumWidths; ++wi) cudaFree(b->tiles[wi]);
     cudaFree(b->tiles_pot);
