@@ -259,7 +259,8 @@ qlga_status qlga_set_graph_steps(qlga_handle* h, int32_t steps);
 
 /* Which kernel runs a step on a 2D lattice.  Sec. VII.B's step is the same either way; the two
  * forms differ only in how the passes are grouped, and their results agree to rounding.
- *   QLGA_STEP2D_AUTO      (default) FP32: the fused single-pass kernel from nx = 32 on (reported as
+ *   QLGA_STEP2D_AUTO      (default) FP32: the fused single-pass kernel from nx = 32 on, where its last strip of 32
+ *                         columns is not mostly empty on a small lattice (reported as
  *                         QLGA_STEP2D_FUSED where nx is a multiple of 32), else two passes;
  *                         FP64: two passes, K (both axes, in integer fixed point from nx = 32 on) and U;
  *   QLGA_STEP2D_FUSED     FP32: always the fused kernel (warp strips of 32 columns: nx % 32 == 0);

@@ -1235,11 +1235,19 @@ qlga_status launch_pot(qlga_handle* h, const void* in, void* out, double delta) 
     return h->cfg.precision == 32 ? launch_potential<float>(h, in, out, delta) : launch_potential<double>(h, in, out, delta);
 }
 
-// Whether K of this 2D lattice runs in the warp-strip kernels, from 32 columns on: the FP32 step unless
-// two passes are asked for, and FP64, where K is one pass and U the other, whatever the mode.
+// Whether the FP32 strips beat two passes on a width that is no multiple of 32: the last strip's lanes past the row's
+// end work for nothing.  Two passes / strips, us a step: 33 x 3030 14.7 / 18.2, 65 x 1538 15.0 / 16.1, 66 x 1515
+// 15.2 / 14.6; 36 x 13888 55.8 / 57.3, 38 x 13157 56.0 / 55.3; 33 x 121212 401 / 375, 100 x 40000 413 / 252.
+inline bool step2d_strips_pay(int64_t nx, int64_t ny) {
+    const int64_t sites = nx * ny, lanes = step2d_strips(nx) * kStep2dWarpCols;
+    return 100 * nx > (sites <= (int64_t(1) << 17) ? 68 : (sites <= (int64_t(1) << 20) ? 57 : 0)) * lanes;
+}
+
+// Whether K of this 2D lattice runs in the warp-strip kernels: the FP32 step unless two passes are faster or
+// asked for, and FP64 from 32 columns on, where K is one pass and U the other, whatever the mode.
 bool step2d_uses_strips(const qlga_handle* h) {
     if (h->cfg.ndim != 2 || !step2d_strips_supported(h->cfg.nx, h->cfg.ny)) return false;
-    return h->cfg.precision == 64 || h->step2d_mode != QLGA_STEP2D_TWO_PASS;
+    return h->cfg.precision == 64 || (h->step2d_mode != QLGA_STEP2D_TWO_PASS && step2d_strips_pay(h->cfg.nx, h->cfg.ny));
 }
 
 // Whether this handle holds its states pending K in the (P, Q) form: 1D lattices and the strip
