@@ -318,10 +318,10 @@ qlga_status qlga_destroy(qlga_handle* h);
  *
  * Checkpoints.  qlga_adjoint_forward() keeps the true state every C steps (x_0, x_C, ...) in the
  * workspace; qlga_adjoint_backward() recomputes each segment of C states from its checkpoint
- * (C - 1 extra state buffers) and pulls the cotangent back through it.  Checkpoints are held in the
+ * (C extra state buffers) and pulls the cotangent back through it.  Checkpoints are held in the
  * handle's precision: a recomputed segment repeats the forward arithmetic of that precision.
  * Workspace: qlga_adjoint_workspace_bytes() bytes of device memory, 256-byte aligned, owned by
- * the caller; about (ceil(n / C) + C + 3) state buffers.  The same workspace must be passed to
+ * the caller; about (ceil(n / C) + C + 4) state buffers.  The same workspace must be passed to
  * the forward and the backward call of one run, unchanged in between.
  *
  * The adjoint covers the plain step only: a handle with interleave = 1 gets

@@ -2413,9 +2413,9 @@ const char* qlga_last_error(void) { return g_last_error.c_str(); }
 //
 // Workspace of the adjoint calls, each part 256-byte aligned: the cotangent and a second
 // cotangent buffer (also the middle buffer of a two-pass 2D kinetic read-out), two buffers for
-// the post-potential states of a recomputed segment, the per-block coupling partials,
-// ceil(n / C) checkpoints (true states x_0, x_C, x_2C, ...) and C - 1 segment slots (the true
-// states x_k of the segment being pulled back, after its checkpoint).  All state-sized parts use the resident layout.
+// the post-potential states of a recomputed segment, the per-block coupling partials and their
+// sum, ceil(n / C) checkpoints (true states x_0, x_C, x_2C, ...) and C segment slots (true
+// states x_k of the segment being pulled back).  All state-sized parts use the resident layout.
 
 namespace {
 
@@ -2438,7 +2438,7 @@ AdjLayout adj_layout(const qlga_config& c, int64_t n, int64_t C, void* base) {
     AdjLayout L{};
     L.state = align256(state_bytes_of(c));
     L.nck = n > 0 ? (n + C - 1) / C : 0;
-    L.nslots = std::max<int64_t>(0, std::min(n, C) - 1);
+    L.nslots = n < C ? (n > 0 ? n : 1) : C;
     char* p = static_cast<char*>(base);
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -2451,6 +2451,7 @@ AdjLayout adj_layout(const qlga_config& c, int64_t n, int64_t C, void* base) {
     L.w1 = take(L.state);
     L.w2 = take(L.state);
     L.partials = reinterpret_cast<double*>(take(sizeof(double) * 3 * kAdjMaxBlocks));
+    take(sizeof(double) * 3);  // unused: the sums go to the handle's results
     L.ckpt = take(L.state * size_t(L.nck));
     L.slots = take(L.state * size_t(L.nslots));
     L.total = off;
@@ -2564,13 +2565,13 @@ qlga_status qlga_adjoint_step(qlga_handle* h, const void* x_device, void* cot_de
     qlga_status s = adj_check(h, 1, 1, workspace, workspace_bytes, &L);
     if (s != QLGA_OK) return s;
     if (!x_device || !cot_device) return fail(QLGA_ERR_INVALID_ARG, "NULL argument%s");
-    s = launch_convert(h, x_device, L.ckpt, true);
+    s = launch_convert(h, x_device, L.slots, true);
     if (s != QLGA_OK) return s;
     s = launch_convert(h, cot_device, L.cot, true);
     if (s != QLGA_OK) return s;
     QLGA_CUDA(cudaMemsetAsync(L.partials, 0, sizeof(double) * 3 * kAdjMaxBlocks, h->stream), "partials clear");
     void *cot = L.cot, *tmp = L.cot_tmp;
-    s = adj_pullback(h, &cot, &tmp, L.ckpt, L.partials);
+    s = adj_pullback(h, &cot, &tmp, L.slots, L.partials);
     if (s != QLGA_OK) return s;
     return adj_finish(h, L, cot, cot_device, dcoup);
 }
@@ -2621,14 +2622,14 @@ qlga_status qlga_adjoint_backward(qlga_handle* h, int64_t nsteps, int64_t checkp
             s = launch_pot_held(h, x0, y);
             if (s != QLGA_OK) return s;
             for (int64_t i = 1; i < len; ++i) {
-                void* slot = L.slots + L.state * size_t(i - 1);
+                void* slot = L.slots + L.state * size_t(i);
                 s = i + 1 < len ? kinetic_and_step(h, y, slot, y2, tmp) : kinetic_into(h, y, slot, tmp, false);
                 if (s != QLGA_OK) return s;
                 std::swap(y, y2);
             }
         }
         for (int64_t i = len - 1; i >= 0; --i) {
-            s = adj_pullback(h, &cot, &tmp, i ? L.slots + L.state * size_t(i - 1) : x0, L.partials);
+            s = adj_pullback(h, &cot, &tmp, i ? L.slots + L.state * size_t(i) : x0, L.partials);
             if (s != QLGA_OK) return s;
         }
     }
