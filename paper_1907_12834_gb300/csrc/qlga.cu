@@ -2413,9 +2413,10 @@ const char* qlga_last_error(void) { return g_last_error.c_str(); }
 //
 // Workspace of the adjoint calls, each part 256-byte aligned: the cotangent and a second
 // cotangent buffer (also the middle buffer of a two-pass 2D kinetic read-out), two buffers for
-// the post-potential states of a recomputed segment, the per-block coupling partials and their
-// sum, ceil(n / C) checkpoints (true states x_0, x_C, x_2C, ...) and C segment slots (true
-// states x_k of the segment being pulled back).  All state-sized parts use the resident layout.
+// the post-potential states of a recomputed segment, the per-block coupling partials,
+// ceil(n / C) checkpoints (true states x_0, x_C, x_2C, ...) and C segment slots (true
+// states x_k of the segment being pulled back; the first serves qlga_adjoint_step alone, since a run reads its checkpoint,
+// and stays for the documented size).  All state-sized parts use the resident layout.
 
 namespace {
 
@@ -2451,7 +2452,6 @@ AdjLayout adj_layout(const qlga_config& c, int64_t n, int64_t C, void* base) {
     L.w1 = take(L.state);
     L.w2 = take(L.state);
     L.partials = reinterpret_cast<double*>(take(sizeof(double) * 3 * kAdjMaxBlocks));
-    take(sizeof(double) * 3);  // unused: the sums go to the handle's results
     L.ckpt = take(L.state * size_t(L.nck));
     L.slots = take(L.state * size_t(L.nslots));
     L.total = off;
