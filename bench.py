@@ -158,12 +158,12 @@ def strip_comments(src):
 
 
 STEP_SOURCES = {32: ("qlga_step2d.cuh", "qlga_device.cuh"),
-                64: ("qlga_step2d_f64.cuh", "qlga_interleave.cuh", "qlga_step2d.cuh", "qlga_device.cuh")}
+                64: ("qlga_fixed.cuh", "qlga_step2d_f64.cuh", "qlga_step2d.cuh", "qlga_device.cuh")}
 STEP_COUNTERS = {32: "step2d_f32_traffic.json", 64: "step2d_f64_counters.json"}
 
 
 def kernel_source_hash(precision=32):
-    """Hash of the fused step kernel's sources, comments excluded: the committed ncu figures stay
+    """Hash of the step kernels' sources, comments excluded: the committed ncu figures stay
     valid across comment edits and lapse with any change to the code."""
     h = hashlib.sha256()
     for name in STEP_SOURCES[precision]:
@@ -173,7 +173,7 @@ def kernel_source_hash(precision=32):
 
 
 def recorded_step_counters(precision=32):
-    """The committed ncu figures of the fused step kernel (per site), or None when the summary is
+    """The committed ncu figures of the step (per site; FP64: K and U together), or None when the summary is
     missing or the kernel source changed since the capture."""
     path = os.path.join(ROOT, "profiles", STEP_COUNTERS[precision])
     try:
@@ -224,12 +224,10 @@ def recorded_traffic(n, precision=32):
     return None if d is None else float(d["dram_bytes_per_site"]) * n * n
 
 
-def alu64_roofline(sites, kernel_ms, sms):
-    """FP64-pipe view of the fused FP64 step, by the method of alu_roofline: FP64-pipe cycles per
-    site from the ncu capture (pct of peak sustained active x smsp__cycles_active.sum / sites)
-    over the live launch duration, against one FP64-pipe cycle per SM sub-partition per cycle at
-    the maximum SM clock; beside it the FP64 arithmetic rate (DFMA = 2 flops) against the nominal
-    1.25 TFLOP/s of GB300."""
+def issue64_roofline(sites, kernel_ms, sms):
+    """Issue view of the FP64 step, whose K and U run in integer fixed point: warp instructions per
+    site from the ncu captures of both kernels, over the live step time, against one instruction
+    per SM sub-partition per cycle at the maximum SM clock."""
     d = recorded_step_counters(64)
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -237,19 +235,16 @@ def alu64_roofline(sites, kernel_ms, sms):
     except (OSError, KeyError, ValueError):
         mhz, src = 2070.0, "nominal 2070 MHz"
     peak = 4.0 * sms * mhz * 1e6
-    if d is None or "fp64_pipe_cycles_per_site" not in d:
-        return {"bound": "alu", "achieved": None, "peak": peak, "unit": "FP64-pipe cycles/s",
+    if d is None or "warp_instructions_per_site" not in d:
+        return {"bound": "issue", "achieved": None, "peak": peak, "unit": "warp instructions/s",
                 "frac": None, "note": "no ncu figure for the current kernel source"}
-    per_site = float(d["fp64_pipe_cycles_per_site"])
+    per_site = float(d["warp_instructions_per_site"])
     achieved = per_site * sites / (kernel_ms * 1e-3)
-    flops = float(d["fp64_flops_per_site"]) * sites / (kernel_ms * 1e-3)
-    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "FP64-pipe cycles/s",
-            "frac": achieved / peak, "cycles_per_site": per_site,
+    return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "warp instructions/s",
+            "frac": achieved / peak, "instructions_per_site": per_site,
             "peak_source": "4 sub-partitions x %d SMs x %s" % (sms, src),
-            "fp64_tflops": flops / 1e12, "fp64_nominal_tflops": 1.25,
-            "fp64_frac_of_nominal": flops / 1.25e12,
-            "note": "FP64-pipe cycles and FP64 operations per site from an ncu capture of the fused "
-                    "FP64 step on the settled 2048^2 state"}
+            "note": "warp instructions per site of k_kinetic2d_f64 and k_potential from an ncu capture of "
+                    "one step on the settled 2048^2 state"}
 
 
 def cpu_baseline(state_f64, g, budget_s, n_sub=256):
@@ -383,11 +378,11 @@ def run_gb300(args):
                      "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind
                      if peak_kind == "measured" else "fallback 6.8 TB/s",
                      "kernel_ms": kernel_ms, "algorithmic_bytes_per_site": bytes_per_site,
-                     "note": ("the FP64 step is bound by the FP64 pipe (see alu)" if f64 else
+                     "note": ("the FP64 step is bound by the issue and latency of its integer sums (see alu)" if f64 else
                               "the fused step is limited by FP32 FMA-pipe cycles of the potential "
                               "(ncu --set full on the settled 2048^2 state: %s), "
                               "not by HBM traffic" % counters_note())},
-        "alu": alu64_roofline(sites, kernel_ms, sms) if f64 else alu_roofline(sites, kernel_ms, sms),
+        "alu": issue64_roofline(sites, kernel_ms, sms) if f64 else alu_roofline(sites, kernel_ms, sms),
         "e2e": e2e,
         "drift": drift,
         "gpu_launches": launches,
@@ -439,7 +434,7 @@ def run_paths(args, torch, qlga, inputs, state_f32, rate_fp32):
     sec = _timed_steps(torch, lat, 3)
     lat.close()
     out["plain_fp64_2d"] = {"lattice": [n, n], "site_updates_per_s": n * n / sec, "ms_per_step": sec * 1e3,
-                            "alu": alu64_roofline(n * n, sec * 1e3,
+                            "alu": issue64_roofline(n * n, sec * 1e3,
                                                   torch.cuda.get_device_properties(0).multi_processor_count)}
     out["fp32_over_fp64_2d"] = rate_fp32 / out["plain_fp64_2d"]["site_updates_per_s"]
     # plain 1D single lattices: config 1 (two-soliton scattering, 16384 sites) in FP32 and FP64,

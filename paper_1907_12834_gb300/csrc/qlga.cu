@@ -132,11 +132,11 @@ __device__ __forceinline__ void put_pq(float* X, int64_t pair, cpx<float> a, cpx
 // HELD_PQ: store the result as (P, Q) = (a + bt, a - bt), the form in which 1D lattices and the
 // fused 2D steps hold a state pending K (qlga_step2d.cuh); else in the resident layout (a, bt).
 template <class T, bool SPLIT, bool HELD_PQ = false>
-// FP64: 128 registers, so that 16 warps per SM cover the latency of the integer sums.  U is some 4000 instructions
-// of straight line around its loops, and warps that have drifted apart wait for instructions (2.5 cycles in each
-// instruction's 8.6), so a CTA's warps start each pass together: a step of 1024^2 0.76 ms, 0.86 without the barrier
-// (0.77 in CTAs of 512 threads; 0.86 and 1.0 at 255 and 168 registers without it).
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 2 : 0) k_potential(const T* in, T* out, int64_t nsites,
+// FP64: U is some 4000 instructions of straight line around its loops, and warps that have drifted apart wait for
+// instructions (2.5 cycles in each instruction's 8.6), so a CTA's warps start each pass together: a step of
+// 1024^2 0.86 ms without the barrier, 0.76 with it at 128 registers and 16 warps per SM, 0.745 at 255 and 8, which
+// spill less (0.75 in CTAs of 384 threads at 168).
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 1 : 0) k_potential(const T* in, T* out, int64_t nsites,
                                                         PotConst<T> PC, unsigned* status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t base = int64_t(blockIdx.x) * blockDim.x; base < nsites; base += stride) {

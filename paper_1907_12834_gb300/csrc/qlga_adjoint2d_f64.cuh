@@ -3,7 +3,8 @@
 // The adjoint of k_kinetic2d_f64 (qlga_step2d_f64.cuh): warp strips of one level that march along y.  K = K_y K_x, so
 // y comes first here: each lane runs the four adjoint blocks of y as a register pipeline on its column, lanes 0
 // to 7 also on the eight columns beyond, the row goes to shared memory, and the adjoint nine-point stencil
-// of x reads it there.  The FP64 form was two passes of 320 FP64 instructions a site (66 cycles each): 106 us at 256^2, 27 here.
+// of x reads it there.  The FP64 form was two passes of 320 FP64 instructions a site (66 cycles each): 106 us at 256^2, 29 here, and 78
+// where the cores of a vortex lattice send strips to FP64.
 //
 // Numbers.  As there, with components below 2^57 after conversion: the y blocks' taps (at most 44 in magnitude) keep
 // below 2^63, are rounded to 2^-5 of that, and the x stencil's sums, below 2^63 again, are eight times the true K^dagger g.

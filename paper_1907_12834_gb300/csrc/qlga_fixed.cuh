@@ -3,7 +3,7 @@
 // GB300 issues one FP64 instruction per SM sub-partition every 64-76 cycles (measured: DFMA 64, DADD and
 // DMUL 76, FP64 <-> FP32 conversions 64) but a 32 x 32 + 64-bit integer multiply-add every 4.4, a
 // 64-bit addition every 2.4 and an FP32 multiply-add every cycle.  A product of two fixed-point numbers
-// takes three of the first, so U on a site costs 40% of its FP64 form (1024^2 sites of a vortex lattice: 0.71 ms,
+// takes three of the first, so U on a site costs a third of its FP64 form (1024^2 sites of a vortex lattice: 0.60 ms,
 // against about 1.7), at a finer resolution: the operands carry 2^-57 of their level, where FP64 rounds
 // every operation at 2^-53 of its own result.
 //

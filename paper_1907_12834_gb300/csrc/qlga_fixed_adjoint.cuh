@@ -3,7 +3,7 @@
 // The FP64 pull-back (qlga_adjoint.cuh) is 2250 FP64 instructions a site in its sweeps alone, one every 66 cycles
 // (qlga_fixed.cuh).  Here both sweeps run on the numbers of fx_unitary: the vectors psi = a + b and d = a - b with an
 // exponent T to a level, the cotangents ga + gb and ga - gb with their own, G, and delta W once between vectors
-// of either scale.  Orders whose bound is below 2^-31 run in FP32, as there.  A gradient of 12 steps of 256^2 6.8 ms (8.5 with FP64
+// of either scale.  Orders whose bound is below 2^-31 run in FP32, as there.  A gradient of 12 steps of 256^2 7.5 ms (8.3 with FP64
 // sweeps), its error against 64 bits 2.7e-15 (3.3e-15).
 //
 // Magnitudes.  Vectors have moduli below 2^56 and cotangents below 2^57 of their levels' units, and grow by less

@@ -29,14 +29,6 @@
 
 namespace qlga {
 
-// Store a pair (a, b) as (P, Q) = (a + i b, a - i b) at pair index `pair` of the resident layout
-// (two double2; the FP32 form is one float4, pq_of in qlga_step2d.cuh).
-__device__ __forceinline__ void put_pq(double* X, int64_t pair, cpx<double> a, cpx<double> b) {
-    double2* p = reinterpret_cast<double2*>(X) + 2 * pair;
-    p[0] = make_double2(a.re - b.im, a.im + b.re);
-    p[1] = make_double2(a.re + b.im, a.im - b.re);
-}
-
 // acc + c x for a compile-time integer c, by shifts and additions
 template <int C>
 __device__ __forceinline__ i64 tap_int(i64 x, i64 acc) {
