@@ -131,12 +131,12 @@ __device__ __forceinline__ void put_pq(float* X, int64_t pair, cpx<float> a, cpx
 // warp-wide maximum); lanes past the end work on zeros and store nothing.
 // HELD_PQ: store the result as (P, Q) = (a + bt, a - bt), the form in which 1D lattices and the
 // fused 2D steps hold a state pending K (qlga_step2d.cuh); else in the resident layout (a, bt).
-template <class T, bool SPLIT, bool HELD_PQ = false>
+template <class T, bool SPLIT, bool HELD_PQ = false, bool ALONE = false>
 // FP64: U is some 4000 instructions of straight line around its loops, and warps that have drifted apart wait for
 // instructions (2.5 cycles in each instruction's 8.6), so a CTA's warps start each pass together: a step of
-// 1024^2 0.86 ms without the barrier, 0.76 with it at 128 registers and 16 warps per SM, 0.745 at 255 and 8, which
-// spill less (0.75 in CTAs of 384 threads at 168).
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 1 : 0) k_potential(const T* in, T* out, int64_t nsites,
+// 1024^2 0.86 ms without the barrier, 0.76 with it at 128 registers and 16 warps per SM, 0.745 at 255 and 8 (ALONE),
+// which spill less.  Lattices that 16 warps per SM hold at once take the former: 384 x 107 58 us a step against 64.
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? (ALONE ? 1 : 2) : 0) k_potential(const T* in, T* out, int64_t nsites,
                                                         PotConst<T> PC, unsigned* status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t base = int64_t(blockIdx.x) * blockDim.x; base < nsites; base += stride) {
@@ -1204,8 +1204,13 @@ template <class T, bool HELD_PQ = false>
 qlga_status launch_potential(qlga_handle* h, const void* in, void* out, double delta) {
     const int64_t n = nsites_of(h->cfg);
     const int nt = block_for(n);
-    k_potential<T, std::is_same<T, float>::value, HELD_PQ><<<grid_for_block(n, nt), nt, 0, h->stream>>>(
-        static_cast<const T*>(in), static_cast<T*>(out), n, PotConst<T>(pot_params(h->cfg, delta)), h->status);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid_for_block(n, nt), nt, 0, h->stream>>>(static_cast<const T*>(in), static_cast<T*>(out), n,
+                                                            PotConst<T>(pot_params(h->cfg, delta)), h->status);
+    };
+    constexpr bool kF32 = std::is_same<T, float>::value;
+    if (!kF32 && n > 16 * 32 * int64_t(device_sms())) launch(k_potential<T, kF32, HELD_PQ, !kF32>);
+    else launch(k_potential<T, kF32, HELD_PQ>);
     QLGA_CUDA(cudaGetLastError(), "k_potential launch");
     h->launches += 1;
     return QLGA_OK;
